@@ -191,7 +191,11 @@ int mobility_solve(bie_ctx* ctx, const bie_geometry* geom, const double* FT, dou
  * symmetric kernels (one CTA per unordered pair of 256-node tiles, each
  * difference, |r|^2 and reciprocal serving both directions of a pair; one
  * partial slot per tile), which are also the occupancy rule's plans once the
- * tile pairs fill the GPU four times over.
+ * tile pairs fill the GPU four times over.  The FP64 pair sums have symmetric
+ * plans too (tiles of 32 to 256 nodes by size), which are the occupancy rule's
+ * where the context's workspace cap allows their partial slots; a count
+ * reported for one is positive, and installing a count installs a directed
+ * plan.
  * splits (nullable): on input 0 to search, a positive count to install a
  * uniform plan without timing (rounded to the counts the source chunking
  * allows), or a negative value to install the symmetric plan (Laplace with

@@ -207,7 +207,7 @@ struct Work {
 
 void carve(Arena& A, Work& w, int N, int M, int kind, int m, bool solve, bool stage_in, bool stage_ipt,
            bool stage_load, bool stage_io, long long bj_floats = 0, int nprob = 0, const int* bs = nullptr,
-           const int* pb = nullptr) {
+           const int* pb = nullptr, bool compact = false) {
   const int comps = kind + 1;
   const long long n = (long long)M * comps;
   w.kind = kind;
@@ -262,9 +262,11 @@ void carve(Arena& A, Work& w, int N, int M, int kind, int m, bool solve, bool st
     w.plan32 = plan_pairs_batch(bs, N, pb, nprob, kind, 1);
     w.planff = plan_pairs_batch(bs, N, pb, nprob, kind, 2);
   } else {
-    w.plan64 = plan_pairs(M, kind, 0);
-    w.plan32 = plan_pairs(M, kind, 1);
-    w.planff = plan_pairs(M, kind, 2);
+    // compact: without the symmetric plans that trade partial slots for time
+    const int slots = compact ? 0 : kAnySlots;
+    w.plan64 = plan_pairs(M, kind, 0, slots);
+    w.plan32 = plan_pairs(M, kind, 1, slots);
+    w.planff = plan_pairs(M, kind, 2, slots);
   }
   // problems solved as one system share every Krylov array; nseg copies of the
   // Hessenberg and rotation arrays with one Krylov space per problem
@@ -342,6 +344,25 @@ int ensure_ws(bie_ctx* ctx, size_t need, cudaStream_t s) {
   ctx->graphs.clear();
   CK(cudaMallocAsync(reinterpret_cast<void**>(&ctx->ws), need, s));
   ctx->ws_size = need;
+  return BIE_OK;
+}
+
+// Sizes a call's workspace (carve with a null arena), makes it and carves it:
+// with the faster pair-sum plans where the context's cap allows their slots,
+// else compact.
+template <class Carve>
+int make_workspace(bie_ctx* ctx, Work& w, cudaStream_t s, const Carve& do_carve) {
+  bool compact = false;
+  Arena sz{nullptr};
+  do_carve(sz, w, compact);
+  if (ctx->cap && sz.off > ctx->cap) {
+    compact = true;
+    sz = Arena{nullptr};
+    do_carve(sz, w, compact);
+  }
+  if (int rc = ensure_ws(ctx, sz.off, s)) return rc;
+  Arena ar{ctx->ws};
+  do_carve(ar, w, compact);
   return BIE_OK;
 }
 
@@ -1027,11 +1048,11 @@ int solve_common(bie_ctx* ctx, const bie_geometry* geom, int kind, const double*
   }
   const bool use_bj = o.precond == 0 && !small;
   const long long bjf = use_bj ? bj_block_floats(bs.data(), N, kind) : 0;
-  Arena sz{nullptr};
-  carve(sz, w, N, M, kind, o.restart, true, true, has_ipt, true, false, bjf, batch ? P : 0, bs.data(), pb.data());
-  if ((rc = ensure_ws(ctx, sz.off, s))) return rc;
-  Arena ar{ctx->ws};
-  carve(ar, w, N, M, kind, o.restart, true, true, has_ipt, true, false, bjf, batch ? P : 0, bs.data(), pb.data());
+  if ((rc = make_workspace(ctx, w, s, [&](Arena& A, Work& x, bool compact) {
+        carve(A, x, N, M, kind, o.restart, true, true, has_ipt, true, false, bjf, batch ? P : 0, bs.data(), pb.data(),
+              compact);
+      })))
+    return rc;
   if (batch) {
     if ((rc = batch_setup(ctx, *batch, bs, pb, has_ipt, w, s))) return rc;
   } else if ((rc = setup(ctx, geom, bs, w, s))) {
@@ -1408,13 +1429,15 @@ size_t workspace_bytes_batch(int kind, const int* bs, int n_bodies, const int* p
   return sz.off;
 }
 
-size_t workspace_bytes_for(int kind, const int* body_start_host, int n_bodies, int restart) {
+void set_workspace_cap(bie_ctx* ctx, size_t cap) { ctx->cap = cap; }
+
+size_t workspace_bytes_for(int kind, const int* body_start_host, int n_bodies, int restart, bool compact) {
   const int n_nodes = body_start_host[n_bodies];
   Work w;
   Arena sz{nullptr};
   const int m = restart > 0 ? std::min(restart, 200) : 50;
   carve(sz, w, n_bodies, n_nodes, kind, m, true, true, true, true, false,
-        bj_block_floats(body_start_host, n_bodies, kind));
+        bj_block_floats(body_start_host, n_bodies, kind), 0, nullptr, nullptr, compact);
   return sz.off;
 }
 }  // namespace bie
@@ -1441,11 +1464,10 @@ int apply_operator_fmm_prec(bie_ctx* ctx, const bie_geometry* geom, int kind, in
   DeviceGuard dg(ctx->device);
   const int N = geom->n_bodies, M = bs[N];
   Work w;
-  Arena sz{nullptr};
-  carve(sz, w, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true);
-  if ((rc = ensure_ws(ctx, sz.off, s))) return rc;
-  Arena ar{ctx->ws};
-  carve(ar, w, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true);
+  if ((rc = make_workspace(ctx, w, s, [&](Arena& A, Work& x, bool compact) {
+        carve(A, x, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true, 0, 0, nullptr, nullptr, compact);
+      })))
+    return rc;
   if ((rc = setup(ctx, geom, bs, w, s))) return rc;
   if ((rc = fmm_setup(ctx->fmm, w.g, kind, &order, 1, s, ctx->err, fmm_schedule(M, kind, order).leaf_nodes)))
     return rc;
@@ -1548,17 +1570,16 @@ int bie_tune(bie_ctx* ctx, const bie_geometry* geom, int kind, int precision, in
     return BIE_OK;
   }
   Work w;
-  Arena sz{nullptr};
-  carve(sz, w, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true);
-  if ((rc = ensure_ws(ctx, sz.off, s))) return rc;
-  Arena ar{ctx->ws};
-  carve(ar, w, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true);
+  if ((rc = make_workspace(ctx, w, s, [&](Arena& A, Work& x, bool compact) {
+        carve(A, x, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true, 0, 0, nullptr, nullptr, compact);
+      })))
+    return rc;
   if ((rc = setup(ctx, geom, bs, w, s))) return rc;
   // candidates: uniform split counts around the occupancy rule's, chunks of
   // whole source tiles (256 sources), and two-level plans (large chunks first,
   // small chunks last, so that the last wave drains fast)
   const PairPlan P0 = occupancy_plan(M, kind, precision);
-  const int S0 = P0.S;
+  const int S0 = occupancy_plan(M, kind, precision, 0).S;  // uniform counts: around the directed kernel's
   std::vector<PairPlan> cand;
   auto add = [&](const PairPlan& p) {
     for (const PairPlan& q : cand)
@@ -1632,7 +1653,9 @@ int bie_tune(bie_ctx* ctx, const bie_geometry* geom, int kind, int precision, in
     best_ms = s0_ms;
   }
   set_tuned_plan(M, kind, precision, best);
-  if (splits) *splits = best.sym ? -best.S : best.S;
+  // only the symmetric plans that a negative count installs are reported negated
+  const bool installable = best.sym && kind == BIE_KIND_LAPLACE && precision != BIE_PREC_FP64;
+  if (splits) *splits = installable ? -best.S : best.S;
   if (ms) *ms = best_ms;
   return BIE_OK;
 }
@@ -1750,11 +1773,10 @@ int apply_operator(bie_ctx* ctx, const bie_geometry* geom, int kind, int precisi
   DeviceGuard dg(ctx->device);
   const int N = geom->n_bodies, M = bs[N];
   Work w;
-  Arena sz{nullptr};
-  carve(sz, w, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true);
-  if ((rc = ensure_ws(ctx, sz.off, s))) return rc;
-  Arena ar{ctx->ws};
-  carve(ar, w, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true);
+  if ((rc = make_workspace(ctx, w, s, [&](Arena& A, Work& x, bool compact) {
+        carve(A, x, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true, 0, 0, nullptr, nullptr, compact);
+      })))
+    return rc;
   if ((rc = setup(ctx, geom, bs, w, s))) return rc;
   const double* din;
   if ((rc = stage_in(ctx, in, w.io_in, (size_t)w.n, &din, s))) return rc;

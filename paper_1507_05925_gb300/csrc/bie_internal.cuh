@@ -175,13 +175,18 @@ struct PairPlan {
   int chunk;     // sources per split (the first S1 splits)
   int S1;        // splits of `chunk` sources
   int chunk2;    // sources per split after the first S1
-  int sym = 0;   // FP32 Laplace: the symmetric kernel (S = tiles of 256 nodes, one CTA per tile pair)
+  int sym = 0;   // a symmetric kernel: nodes a tile (S = tiles, one CTA per unordered tile pair); 0: directed
 };
 inline PairPlan uniform_plan(int S, int chunk) { return PairPlan{S, chunk, S, chunk}; }
 // the tuned split count of this shape (bie_tune) if any, else occupancy_plan:
-// one wave of blocks (target blocks x splits) over every SM
-PairPlan plan_pairs(int M, int kind, int precision);
-PairPlan occupancy_plan(int M, int kind, int precision);
+// one wave of blocks (target blocks x splits) over every SM, or a symmetric
+// plan.  max_slots bounds the partial slots of the symmetric FP64 plans (0: none
+// of them; a caller whose scratch is fixed, or whose workspace cap is met by the
+// directed plans only).
+constexpr int kAnySlots = 0x7fffffff;
+PairPlan plan_pairs(int M, int kind, int precision, int max_slots = kAnySlots);
+PairPlan occupancy_plan(int M, int kind, int precision, int max_slots = kAnySlots);
+PairPlan plan_symmetric64(int M, int kind, int max_slots);
 PairPlan plan_with_splits(int M, int S);
 // two-level plan: a fraction f of the sources in chunks of c1, the rest in chunks of c2
 PairPlan plan_two_level(int M, int c1, int c2, double f);
@@ -240,8 +245,12 @@ void fmm_signature(const FmmState* f, long long sig[2]);
 cudaError_t fmm_output(FmmState* f, const Geo& g, int kind, int p, const double* v, double* part, cudaStream_t s,
                        bool ff = false);
 
-// workspace of a solve with the given host body_start (bie_workspace_bytes assumes equal bodies)
-size_t workspace_bytes_for(int kind, const int* body_start_host, int n_bodies, int restart);
+// workspace of a solve with the given host body_start (bie_workspace_bytes assumes equal bodies);
+// compact: with the pair-sum plans of the fewest partial slots (a solve takes them
+// when its context's cap does not allow the faster ones)
+size_t workspace_bytes_for(int kind, const int* body_start_host, int n_bodies, int restart, bool compact = false);
+// the cap of a context's workspace (0: none), as at its creation
+void set_workspace_cap(bie_ctx* ctx, size_t cap);
 // workspace of a batched solve (host arrays: concatenated body_start [N+1],
 // first body of each problem [nprob+1])
 size_t workspace_bytes_batch(int kind, const int* bs, int n_bodies, const int* pb, int nprob, const bie_opts* opts);

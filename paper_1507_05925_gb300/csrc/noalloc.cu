@@ -156,7 +156,7 @@ extern "C" int apply_operator_noalloc(const bie_geometry* geom, int kind, int pr
   if (c.off > kScratchBytes) return BIE_ERR_NOMEM;  // sizing and carving disagree
 
   // the same source split as apply_operator, capped at the scratch's splits
-  PairPlan p = plan_pairs(M, kind, precision);
+  PairPlan p = plan_pairs(M, kind, precision, kNoallocMaxSplits);
   if (p.S > kNoallocMaxSplits) {
     const int tile = 256;
     int chunk = (M + kNoallocMaxSplits - 1) / kNoallocMaxSplits;

@@ -16,6 +16,19 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
+// 1/x in FP64: the hardware approximation (about 19 correct bits: it reads and
+// writes the high word only) and one third-order step of the series 1/x =
+// y0 (1 + e + e^2 + ...), e = 1 - x y0, |e|^3 < 2^-56: three FP64 operations,
+// against about nine of a correctly rounded division on a pipe that retires
+// two lanes a clock per SM.  x = 0 gives NaN (the pair sums skip r = 0).
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double e = fma(-x, y, 1.0);
+  e = fma(e, e, e);
+  return fma(y, e, y);
+}
+
 // ------------------------------------------------------------------- FP32 ----
 // Contribution of one pair from hi/lo positions (x = hi + lo): the leading
 // difference is exact, so r . n_a keeps its digits for neighbouring nodes.

@@ -164,13 +164,14 @@ __global__ void __launch_bounds__(kB64) k_pair64(Geo g, VecRef vr, const double*
         const double r2 = dx * dx + dy * dy;
         const bool skip = ta[k] == b || (BATCH && sr.straddle && !same_problem(g, ta[k], b));
         if (KIND == 0) {
-          const double s = skip ? 0.0 : q1 / r2;
+          const double s = skip ? 0.0 : q1 * rcp64(r2);
           ax[k] += dx * s;
           ay[k] += dy * s;
         } else {
           const double rq = dx * q1 + dy * q2;
           const double rn = dx * tnx[k] + dy * tny[k];
-          const double c = skip ? 0.0 : (rq * rn) / (r2 * r2);
+          const double y = rcp64(r2);
+          const double c = skip ? 0.0 : (rq * rn) * (y * y);
           ax[k] += c * dx;
           ay[k] += c * dy;
         }
@@ -629,6 +630,121 @@ __global__ void __launch_bounds__(kB32, 12) k_pair32s(Geo g, int ntile, double* 
       const float2 u = accB[l], v = accB[kTS + l];
       write_projected(g, b, ti, u.x + v.x, u.y + v.y, partial);
     }
+  }
+}
+
+// -------------------------------------------------------- symmetric FP64 ----
+// The FP64 pair sum on unordered pairs of tiles of TS = blockDim nodes, one CTA
+// a pair: r, |r|^2 and the reciprocal serve both directions.  GB300's FP64 pipe
+// bounds it (two lanes a clock per SM): Laplace 13 FP64 operations for two
+// directed pairs (the directed kernel: 10 for one, about 16 when it divided),
+// Stokes 24 (16, about 21).  Measured (GB300, whole launch): Laplace M = 25,600
+// 16.6 ms divided, 12.1 ms directed with rcp64, 7.5 ms symmetric (8.7e10
+// pairs/s, 90% of the pipe); Stokes M = 12,672 6.7, 4.65, 3.44 ms.
+// A lane holds one target of tile A (two a lane measured the same); the sources
+// of tile B sit in shared memory, visited on the diagonal schedule of
+// k_pair32s, the source's accumulator travelling by shuffle.  Warp w starts
+// at source group w (32 sources) and the warps meet at a barrier after each
+// group, so that a group's accumulators are added to by one warp at a time, in
+// a fixed order.  Partials as k_pair32s: slot j of tile A's nodes, slot i of
+// tile B's; a tile with itself runs the directed pass.  Nodes past M in the
+// last tile stand at its first node with zero strength.
+template <int KIND>
+__host__ __device__ constexpr int sym64_vals() { return KIND == 0 ? 5 : 8; }  // doubles a node in shared memory
+
+template <int KIND>
+__global__ void __launch_bounds__(256) k_pair64s(Geo g, VecRef vr, const double* __restrict__ sscale,
+                                                 double* __restrict__ partial, const int* __restrict__ stop) {
+  if (stop && *stop) return;
+  extern __shared__ __align__(16) double sm64[];
+  const double* __restrict__ v = vr.ptr();
+  const int M = g.M, TS = blockDim.x, t = threadIdx.x;
+  double *sx = sm64, *sy = sx + TS, *sq1 = sy + TS, *sbx = sq1 + TS, *sby = sbx + TS;
+  double *sq2 = sby + TS, *snx = sq2 + TS, *sny = snx + TS;  // Stokes
+  int ti, tj;
+  tri_decode(blockIdx.x, ti, tj);
+  const int A0 = ti * TS, B0 = tj * TS;
+  {
+    const int b = B0 + t < M ? B0 + t : B0;
+    const double s = B0 + t < M ? sscale[b] : 0.0;
+    sx[t] = g.x[b];
+    sy[t] = g.y[b];
+    sbx[t] = sby[t] = 0.0;
+    if (KIND == 0) {
+      sq1[t] = s * v[b];
+    } else {
+      sq1[t] = s * v[2 * b];
+      sq2[t] = s * v[2 * b + 1];
+      snx[t] = g.nx[b];
+      sny[t] = g.ny[b];
+    }
+  }
+  const int a = min(A0 + t, M - 1);
+  const double tx = g.x[a], ty = g.y[a], tnx = g.nx[a], tny = g.ny[a], ts = sscale[a];
+  const double tq1 = ts * v[KIND == 0 ? a : 2 * a], tq2 = KIND == 0 ? 0.0 : ts * v[2 * a + 1];
+  double ax = 0.0, ay = 0.0;
+  __syncthreads();
+  if (ti == tj) {
+    const int nt = min(TS, M - B0);
+#pragma unroll 4
+    for (int l = 0; l < nt; ++l) {
+      const double q1 = sq1[l], dx = tx - sx[l], dy = ty - sy[l];
+      const double y = rcp64(dx * dx + dy * dy);
+      if (KIND == 0) {
+        const double s = t == l ? 0.0 : q1 * y;
+        ax += dx * s;
+        ay += dy * s;
+      } else {
+        const double c = t == l ? 0.0 : ((dx * q1 + dy * sq2[l]) * (dx * tnx + dy * tny)) * (y * y);
+        ax += c * dx;
+        ay += c * dy;
+      }
+    }
+  } else {
+    const int lane = t & 31, warp = t >> 5, G = TS / 32;
+    for (int g0 = 0; g0 < G; ++g0) {
+      const int r0 = 32 * (g0 + warp < G ? g0 + warp : g0 + warp - G);
+      double bx = 0.0, by = 0.0;  // accumulator of the source this lane holds (travels)
+#pragma unroll 4
+      for (int k = 0; k < 32; ++k) {
+        const int l = r0 + ((lane + k) & 31);
+        const double q1 = sq1[l], dx = tx - sx[l], dy = ty - sy[l];
+        const double y = rcp64(dx * dx + dy * dy);
+        if (KIND == 0) {
+          const double sb = q1 * y, sa = tq1 * y;
+          ax += dx * sb;
+          ay += dy * sb;
+          bx -= dx * sa;  // the source gains -q_a r/|r|^2
+          by -= dy * sa;
+        } else {
+          const double y2 = y * y;
+          const double ca = ((dx * q1 + dy * sq2[l]) * (dx * tnx + dy * tny)) * y2;
+          const double cb = ((dx * tq1 + dy * tq2) * (dx * snx[l] + dy * sny[l])) * y2;
+          ax += ca * dx;
+          ay += ca * dy;
+          bx -= cb * dx;  // r, r . q_a and r . n_b all change sign
+          by -= cb * dy;
+        }
+        bx = __shfl_sync(0xffffffffu, bx, (lane + 1) & 31);
+        by = __shfl_sync(0xffffffffu, by, (lane + 1) & 31);
+      }
+      sbx[r0 + lane] += bx;  // back at its own lane: source r0 + lane
+      sby[r0 + lane] += by;
+      __syncthreads();
+    }
+    const int b = B0 + t;
+    if (b < M) {
+      if (KIND == 0)
+        partial[(long long)ti * M + b] = g.nx[b] * sbx[t] + g.ny[b] * sby[t];
+      else
+        reinterpret_cast<double2*>(partial)[(long long)ti * M + b] = make_double2(sbx[t], sby[t]);
+    }
+  }
+  if (A0 + t < M) {
+    if (KIND == 0)
+      partial[(long long)tj * M + a] = tnx * ax + tny * ay;
+    else
+      reinterpret_cast<double2*>(partial)[(long long)tj * M + a] = make_double2(ax, ay);
   }
 }
 
@@ -1425,21 +1541,52 @@ PairPlan plan_two_level(int M, int c1, int c2, double f) {
 
 PairPlan plan_symmetric(int M) {
   PairPlan p = uniform_plan((M + kTS - 1) / kTS, kTS);
-  p.sym = 1;
+  p.sym = kTS;
   return p;
 }
 
-PairPlan plan_pairs(int M, int kind, int precision) {
+// The symmetric FP64 plan: the tile size of the least estimated time.  The
+// FP64 pipe bounds the kernel, so a pair of tiles costs tile^2 times the
+// operations of two directed pairs, the SMs take tile pairs in rounds, and the
+// slots (one a tile) cost their write and their read.  Measured, tiles of 32 /
+// 64 / 128 / 256 nodes, Laplace: M = 704 23 / 39 / 74 / 234 us (directed 52),
+// M = 7,168 609 / 619 / 633 / 688 (926), M = 25,600 7.57 / 7.52 / 7.53 / 7.65
+// ms (12.1): small tiles fill the GPU at small M, large ones keep the slots few
+// at large M.  Slots beyond max_slots or 512 MB: no symmetric plan (S = 0).
+PairPlan plan_symmetric64(int M, int kind, int max_slots) {
+  const int nsm = device_sms();
+  PairPlan best{0, 0, 0, 0};
+  double best_us = 1e300;
+  for (int tile : {32, 64, 128, 256}) {
+    const long long nt = (M + tile - 1) / tile, pairs = nt * (nt + 1) / 2;
+    const double slot_mb = (double)nt * M * (kind + 1) * 8e-6;
+    if (nt > max_slots || slot_mb > 512.0) continue;
+    const double rounds = (double)((pairs + nsm - 1) / nsm);
+    const double us = rounds * tile * tile * (kind == 0 ? 13.0 : 24.0) / 4000.0 + slot_mb / 2.0;
+    if (us < best_us) {
+      best_us = us;
+      best = uniform_plan((int)nt, tile);
+      best.sym = tile;
+    }
+  }
+  return best;
+}
+
+PairPlan plan_pairs(int M, int kind, int precision, int max_slots) {
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned.find(tune_key(M, kind, precision));
-    if (it != g_tuned.end()) return it->second;
+    if (it != g_tuned.end() && (precision != 0 || !it->second.sym || it->second.S <= max_slots)) return it->second;
   }
-  return occupancy_plan(M, kind, precision);
+  return occupancy_plan(M, kind, precision, max_slots);
 }
 
-PairPlan occupancy_plan(int M, int kind, int precision) {
+PairPlan occupancy_plan(int M, int kind, int precision, int max_slots) {
   const DeviceShape& d = device_shape();
+  if (precision == 0) {
+    const PairPlan p = plan_symmetric64(M, kind, max_slots);
+    if (p.S > 0) return p;
+  }
   if ((precision == 1 || precision == 2) && kind == 0) {
     // the symmetric FP32 / float-float Laplace kernels once their tile pairs fill
     // the GPU a few times over and their partials (one slot per tile) stay
@@ -1501,7 +1648,14 @@ void launch_pairs(const Geo& g, int kind, int precision, const PairPlan& p, VecR
                   double* partial, const int* stop, cudaStream_t s) {
   if (precision == 0) {
     dim3 grid((g.M + kB64 * kT64 - 1) / (kB64 * kT64), p.S);
-    if (kind == 0)
+    if (!BATCH && p.sym) {
+      const long long nt = (g.M + p.sym - 1) / p.sym;
+      const unsigned pairs = (unsigned)(nt * (nt + 1) / 2);
+      if (kind == 0)
+        k_pair64s<0><<<pairs, p.sym, p.sym * sym64_vals<0>() * sizeof(double), s>>>(g, v, sscale, partial, stop);
+      else
+        k_pair64s<1><<<pairs, p.sym, p.sym * sym64_vals<1>() * sizeof(double), s>>>(g, v, sscale, partial, stop);
+    } else if (kind == 0)
       k_pair64<0, BATCH><<<grid, kB64, 0, s>>>(g, v, sscale, p, partial, stop);
     else
       k_pair64<1, BATCH><<<grid, kB64, 0, s>>>(g, v, sscale, p, partial, stop);

@@ -33,6 +33,7 @@ struct Job {
   bie_request req;
   int64_t ticket = 0;
   size_t need = 0;
+  bool compact = false;  // need is the smaller workspace's: the solve is capped at it
   std::vector<int> bs;  // body_start (host copy)
   Clock::time_point t_submit;
   double seconds = 0.0;
@@ -148,6 +149,7 @@ void worker_main(bie_server* s) {
   std::vector<int> status;
   auto solo = [&](Job* b, bie_info* info) -> int {
     const bie_request& r = b->req;
+    bie::set_workspace_cap(ctx, b->compact ? b->need : 0);
     if (r.kind == BIE_KIND_LAPLACE)
       return elastance_solve(ctx, &r.geom, r.load, r.out, r.density, &r.opts, info, stream);
     return mobility_solve(ctx, &r.geom, r.load, r.out, r.density, &r.opts, info, stream);
@@ -180,6 +182,7 @@ void worker_main(bie_server* s) {
           loads.push_back(b->req.load);
           outs.push_back(b->req.out);
         }
+        bie::set_workspace_cap(ctx, 0);
         const int rc = j->req.kind == BIE_KIND_LAPLACE
                            ? elastance_solve_batch(ctx, P, geoms.data(), loads.data(), outs.data(), opts,
                                                    infos.data(), status.data(), stream)
@@ -255,11 +258,14 @@ int bie_server_submit(bie_server* s, const bie_request* req, int64_t* ticket) {
   for (int i = 0; i < g.n_bodies; ++i)
     if (bs[i + 1] < bs[i]) return BIE_ERR_INVALID;
   cudaSetDevice(s->device);
-  const size_t need = bie::workspace_bytes_for(req->kind, bs.data(), g.n_bodies, req->opts.restart);
+  size_t need = bie::workspace_bytes_for(req->kind, bs.data(), g.n_bodies, req->opts.restart);
+  const bool compact = s->cap && need > s->cap;  // the cap allows the smaller workspace only, or not even that
+  if (compact) need = bie::workspace_bytes_for(req->kind, bs.data(), g.n_bodies, req->opts.restart, true);
   if (s->cap && need > s->cap) return BIE_ERR_NOMEM;
   Job* j = new Job();
   j->req = *req;
   j->need = need;
+  j->compact = compact;
   j->bs.swap(bs);
   j->t_submit = Clock::now();
   {
