@@ -187,6 +187,7 @@ constexpr int kAnySlots = 0x7fffffff;
 PairPlan plan_pairs(int M, int kind, int precision, int max_slots = kAnySlots);
 PairPlan occupancy_plan(int M, int kind, int precision, int max_slots = kAnySlots);
 PairPlan plan_symmetric64(int M, int kind, int max_slots);
+PairPlan plan_symmetric32(int M, int kind, int max_slots);
 PairPlan plan_with_splits(int M, int S);
 // two-level plan: a fraction f of the sources in chunks of c1, the rest in chunks of c2
 PairPlan plan_two_level(int M, int c1, int c2, double f);

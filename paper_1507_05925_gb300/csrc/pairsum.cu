@@ -458,26 +458,42 @@ __global__ void __launch_bounds__(kB32, KIND == 0 ? 12 : 10) k_pair32(Geo g, Vec
 }
 
 // ------------------------------------------------------- symmetric FP32 ----
-// Laplace pair sums with each reciprocal used for both directions of a pair.
-// The M nodes are cut into tiles of kTS = 256 consecutive nodes; one CTA takes
-// one unordered pair of tiles (A = tile i, B = tile j, i <= j) and writes the
-// contribution of B's sources to A's targets into partial[j][A] and that of
-// A's sources to B's targets into partial[i][B]: every (source tile, target
-// tile) slot is written exactly once, and the epilogue adds the S = tiles
+// FP32 pair sums with r, |r|^2 and the reciprocal used for both directions of a
+// pair.  The M nodes are cut into tiles of TS = 2H blockDim consecutive nodes; one
+// CTA takes one unordered pair of tiles (A = tile i, B = tile j, i <= j) and
+// writes the contribution of B's sources to A's targets into partial[j][A] and
+// that of A's sources to B's targets into partial[i][B]: every (source tile,
+// target tile) slot is written exactly once, and the epilogue adds the S = tiles
 // slots of a target in a fixed order (deterministic).
 //
-// Far tile pairs (boxes at least both half-diagonals apart): with r = x_a - x_b
-// and w = 1/|r|^2, target a gains q_b r w and target b gains -q_a r w, so one
-// MUFU reciprocal and about 10 FP32 lane operations serve two directed pairs
-// (the directed kernel: one reciprocal and 7 operations for one).  Each lane
-// holds four A targets in registers (packed two by two); B's sources sit in
-// shared memory and are visited on a diagonal schedule (lane l takes source
-// (l + k) mod 32 of the current group of 32 at step k), and the accumulator of
-// B's source travels with it from lane to lane by a warp shuffle, so no two
-// lanes ever add into the same place.  Coordinates are relative to A's box
-// centre, as in the directed far tiles.  Near tile pairs (and i = j) run the
-// directed near path in both directions (exact hi/lo differences).
-constexpr int kTS = kB32 * kT32;  // 256 nodes a tile
+// With r = x_a - x_b, w = 1/|r|^2 and s = r w: Laplace target a gains q_b s and
+// target b gains -q_a s (10 FP32 lane operations and one MUFU reciprocal for two
+// directed pairs; the directed kernel: 7 and one for one pair); Stokes a gains
+// s (r . q_b)(s . n_a) and b gains -s (r . q_a)(s . n_b) (20 operations, against
+// 13 for one).  Each lane holds 2H A targets in registers (packed two by two);
+// B's sources sit in shared memory and are visited 32 at a time on a diagonal
+// schedule (lane l takes source (l + k) mod 32 of the group at step k), and the
+// accumulator of B's source travels with it from lane to lane by a warp
+// shuffle, so no two lanes ever add into the same place.
+//
+// Coordinates: a group of 32 sources is far from tile A when its box (its bodies')
+// is far from every body of A; differences are then taken in plain FP32 relative
+// to the centre of the group's box, in which sources and targets are at most a
+// few |r| from the origin (rounding <= 3 x 2^-24 |r|), else from the exact hi/lo
+// coordinates (four operations more).  The test is per body, not on the tiles'
+// boxes: tiles of several bodies in no spatial order (a random suspension) stay
+// far.  (Laplace tiles whose whole boxes are far skip the per-group work: 1.5% at
+// 100 bodies of 256 nodes.)  A tile with itself runs the directed near pass.
+// Stokes sums are kept error-free over chunks of kSymChunk sources.
+//
+// Bound by the issue of FP32 instructions (two thirds of the pipe; without the
+// shuffles, or without MUFU, 5% faster).  Measured, pair sum alone, directed ->
+// symmetric: Stokes 400 bodies of 128 nodes in random order 1,684 -> 915 us
+// (2.87e12 pairs/s), 200 of 90..165 nodes 424 -> 266 us, 64 of 128 nodes 56 -> 43
+// us; Laplace with the tiles' boxes -> per body: 400 of 128 1,026 -> 558 us, 200
+// of 90..165 291 -> 165 us, 100 of 256 156 -> 154 us.
+constexpr int kTS = kB32 * kT32;  // 256 nodes a tile of the symmetric Laplace plan
+constexpr int kSymChunk = 64;
 
 __device__ __forceinline__ void tri_decode(int t, int& i, int& j) {
   int jj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);  // then corrected exactly
@@ -498,139 +514,322 @@ __device__ __forceinline__ bool boxes_far(float4 a, float4 b) {
   return gap2 > 0.f && gap2 >= need * need;
 }
 
-// partial[slot][a] = n_a . (ax, ay) in float-float (the normal's hi/lo split),
-// stored as the float pair (h, l): no FP64 pipe in the kernel
-__device__ __forceinline__ void write_projected(const Geo& g, int a, int slot, float ax, float ay,
-                                                double* __restrict__ partial) {
-  const float4 n = g.nff[a];
-  float p1, e1, p2, e2, h, l;
-  ff_mul(n.x, n.y, ax, 0.f, p1, e1);
-  ff_mul(n.z, n.w, ay, 0.f, p2, e2);
-  two_sum(p1, p2, h, l);
-  reinterpret_cast<float2*>(partial)[(long long)slot * g.M + a] = make_float2(h, l + (e1 + e2));
+// The slot entry of target a from its sum (ax + ex, ay + ey): Laplace n_a . sum in
+// float-float (the normal's hi/lo split), stored as the float pair (h, l);
+// Stokes both components as float pairs.  No FP64 pipe in the kernel.
+template <int KIND>
+__device__ __forceinline__ void write_slot(const Geo& g, int a, int slot, float ax, float ex, float ay, float ey,
+                                           double* __restrict__ partial) {
+  if (KIND == 0) {
+    const float4 n = g.nff[a];
+    float p1, e1, p2, e2, h, l;
+    ff_mul(n.x, n.y, ax, ex, p1, e1);
+    ff_mul(n.z, n.w, ay, ey, p2, e2);
+    two_sum(p1, p2, h, l);
+    reinterpret_cast<float2*>(partial)[(long long)slot * g.M + a] = make_float2(h, l + (e1 + e2));
+  } else {
+    reinterpret_cast<float4*>(partial)[(long long)slot * g.M + a] = make_float4(ax, ex, ay, ey);
+  }
 }
 
-// Directed near pass: targets [t0, t0 + kTS) gain the sources [s0, s1) (one
-// tile, exact hi/lo differences), written to partial[slot].
-template <bool DIAG>
-__device__ __forceinline__ void sym_near_pass(const Geo& g, int t0, int s0, int s1, int slot,
-                                              double* __restrict__ partial, float4* sp, float2* sq) {
-  const int M = g.M, nt = s1 - s0;
-  __syncthreads();  // the tile buffers may still be read
-  for (int l = threadIdx.x; l < nt; l += kB32) {
-    sp[l] = g.pf[s0 + l];
-    sq[l] = make_float2(g.qf[s0 + l], 0.f);
+// One group of 32 sources (shared-memory entries sX[0..32)) against this lane's
+// four targets: their sums into AX, AY (targets 0, 1 and 2, 3 packed) and the
+// sources' sums, returned at the lane that holds the source.  FAR: TX, TY and
+// the sources are relative to the group's centre; else TXL, TYL are the low
+// parts and sL the sources'.  Sources are stored negated.
+template <int KIND, bool FAR, int H>
+__device__ __forceinline__ float2 sym_group(const float4* __restrict__ sX, const float2* __restrict__ sL,
+                                            const float2* __restrict__ sN, const float2* TX, const float2* TY,
+                                            const float2* TXL, const float2* TYL, const float2* Q1, const float2* Q2,
+                                            const float2* NX, const float2* NY, float2* AX, float2* AY) {
+  const int lane = threadIdx.x & 31;
+  float bx = 0.f, by = 0.f;  // accumulator of the source this lane holds (travels)
+#pragma unroll(FAR ? 8 : 4)
+  for (int k = 0; k < 32; ++k) {
+    const int l = (lane + k) & 31;
+    const float4 src = sX[l];
+    const float2 sx = make_float2(src.x, src.x), sy = make_float2(src.y, src.y);
+    const float2 q1 = make_float2(src.z, src.z), q2 = make_float2(src.w, src.w);
+    float2 lo = make_float2(0.f, 0.f), nb = lo;
+    if (!FAR) lo = sL[l];
+    if (KIND == 1) nb = sN[l];
+    float2 ux, uy;
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      float2 dx = __fadd2_rn(TX[h], sx), dy = __fadd2_rn(TY[h], sy);
+      if (!FAR) {
+        dx = __fadd2_rn(dx, __fadd2_rn(TXL[h], make_float2(lo.x, lo.x)));
+        dy = __fadd2_rn(dy, __fadd2_rn(TYL[h], make_float2(lo.y, lo.y)));
+      }
+      const float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
+      const float2 w = make_float2(rcp_approx(r2.x), rcp_approx(r2.y));
+      if (KIND == 0) {
+        const float2 sb = __fmul2_rn(q1, w), sa = __fmul2_rn(Q1[h], w);
+        AX[h] = __ffma2_rn(dx, sb, AX[h]);
+        AY[h] = __ffma2_rn(dy, sb, AY[h]);
+        ux = h == 0 ? __fmul2_rn(dx, sa) : __ffma2_rn(dx, sa, ux);
+        uy = h == 0 ? __fmul2_rn(dy, sa) : __ffma2_rn(dy, sa, uy);
+      } else {
+        const float2 ex = __fmul2_rn(dx, w), ey = __fmul2_rn(dy, w);
+        const float2 ca = __fmul2_rn(__ffma2_rn(dx, q1, __fmul2_rn(dy, q2)),
+                                     __ffma2_rn(ex, NX[h], __fmul2_rn(ey, NY[h])));
+        const float2 cb = __fmul2_rn(__ffma2_rn(dx, Q1[h], __fmul2_rn(dy, Q2[h])),
+                                     __ffma2_rn(ex, make_float2(nb.x, nb.x), __fmul2_rn(ey, make_float2(nb.y, nb.y))));
+        AX[h] = __ffma2_rn(ca, ex, AX[h]);
+        AY[h] = __ffma2_rn(ca, ey, AY[h]);
+        ux = h == 0 ? __fmul2_rn(cb, ex) : __ffma2_rn(cb, ex, ux);
+        uy = h == 0 ? __fmul2_rn(cb, ey) : __ffma2_rn(cb, ey, uy);
+      }
+    }
+    bx -= ux.x + ux.y;
+    by -= uy.x + uy.y;
+    // hand the accumulator to the lane that takes this source next
+    bx = __shfl_sync(0xffffffffu, bx, (lane + 1) & 31);
+    by = __shfl_sync(0xffffffffu, by, (lane + 1) & 31);
   }
+  return make_float2(bx, by);  // back at its own lane
+}
+
+// Adds the targets' sums of a chunk of sources to their error-free sums over
+// the chunks (shared memory, each thread its own entries) and clears them.
+template <int H>
+__device__ __forceinline__ void sym_flush(float4* __restrict__ sAcc, float2* AX, float2* AY) {
+  const int t = threadIdx.x, B = blockDim.x;
+#pragma unroll
+  for (int k = 0; k < 2 * H; ++k) {
+    float4 c = sAcc[t + k * B];
+    comp_add(c.x, c.y, k & 1 ? AX[k >> 1].y : AX[k >> 1].x);
+    comp_add(c.z, c.w, k & 1 ? AY[k >> 1].y : AY[k >> 1].x);
+    sAcc[t + k * B] = c;
+  }
+#pragma unroll
+  for (int h = 0; h < H; ++h) AX[h] = AY[h] = make_float2(0.f, 0.f);
+}
+
+// The sources' sums [warps][TS] of tile B into their slots: the warps in order,
+// error-free.
+template <int KIND>
+__device__ __forceinline__ void sym_write_sources(const Geo& g, int B0, int TS, int slot,
+                                                  const float2* __restrict__ accB, double* __restrict__ partial) {
   __syncthreads();
-  float ax[kT32], ay[kT32], tnx[kT32], tny[kT32];
-#pragma unroll
-  for (int k = 0; k < kT32; ++k) ax[k] = ay[k] = tnx[k] = tny[k] = 0.f;
-  tile_near<0, DIAG>(g.pf, sp, sq, nt, s0, t0 + threadIdx.x, M, tnx, tny, ax, ay);
-#pragma unroll
-  for (int k = 0; k < kT32; ++k) {
-    const int a = t0 + threadIdx.x + k * kB32;
-    if (a < M) write_projected(g, a, slot, ax[k], ay[k], partial);
+  for (int l = threadIdx.x; l < TS; l += blockDim.x) {
+    const int b = B0 + l;
+    if (b >= g.M) continue;
+    float2 u = accB[l];
+    float ex = 0.f, ey = 0.f;
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) {
+      const float2 v = accB[w * TS + l];
+      comp_add(u.x, ex, v.x);
+      comp_add(u.y, ey, v.y);
+    }
+    write_slot<KIND>(g, b, slot, u.x, ex, u.y, ey, partial);
   }
 }
 
-__global__ void __launch_bounds__(kB32, 12) k_pair32s(Geo g, int ntile, double* __restrict__ partial,
-                                                      const int* __restrict__ stop) {
+// Shared memory of one CTA, bytes a node: far and near positions with the
+// strengths, near low parts, the Stokes normal and the Stokes targets' sums, the
+// warps' accumulators; per group its box and far flag.
+template <int KIND, int H>
+__host__ __device__ constexpr size_t sym32_smem(int threads) {
+  const size_t TS = 2 * H * (size_t)threads;
+  return TS * (16 + 16 + 8 + (KIND == 1 ? 8 + 16 : 0)) + (threads / 32) * TS * 8 + TS / 32 * (16 + 4);
+}
+
+template <int KIND, int H>
+__global__ void __launch_bounds__(64, KIND == 0 ? 10 : (H == 2 ? 8 : 6)) k_pair32s(Geo g, double* __restrict__ partial,
+                                                                      const int* __restrict__ stop) {
   if (stop && *stop) return;
-  __shared__ __align__(16) unsigned char sm_raw[kTS * 32];  // far: sources + 2 accumulator rows; near: sp, sq
-  const int M = g.M;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const int M = g.M, B = blockDim.x, TS = 2 * H * B, G = TS / 32;
+  float4* sF = reinterpret_cast<float4*>(sm_raw);  // far: (-x', -y', q1, q2)
+  float4* sH = sF + TS;                            // near: (-x_hi, -y_hi, q1, q2)
+  float4* sBox = sH + TS;                          // [G]
+  float4* sAcc = sBox + G;                         // Stokes: [TS] (sx, ex, sy, ey) of the targets
+  float2* sL = reinterpret_cast<float2*>(sAcc + (KIND == 1 ? TS : 0));  // near: (-x_lo, -y_lo)
+  float2* accB = sL + TS;                          // [warps][TS]
+  float2* sN = accB + (B / 32) * TS;               // Stokes normals
+  int* sFar = reinterpret_cast<int*>(sN + (KIND == 1 ? TS : 0));  // [G]
   int ti, tj;
   tri_decode(blockIdx.x, ti, tj);
-  const int A0 = ti * kTS, A1 = min(M, A0 + kTS), B0 = tj * kTS, B1 = min(M, B0 + kTS);
-  const float4 boxA = body_range_box(g.bbox, g.body_of[A0], g.body_of[A1 - 1]);
-  const float4 boxB = body_range_box(g.bbox, g.body_of[B0], g.body_of[B1 - 1]);
-  if (ti == tj || !boxes_far(boxA, boxB)) {
-    float4* sp = reinterpret_cast<float4*>(sm_raw);
-    float2* sq = reinterpret_cast<float2*>(sm_raw + kTS * sizeof(float4));
-    if (ti == tj) {
-      sym_near_pass<true>(g, A0, B0, B1, tj, partial, sp, sq);
-    } else {
-      sym_near_pass<false>(g, A0, B0, B1, tj, partial, sp, sq);
-      sym_near_pass<false>(g, B0, A0, A1, ti, partial, sp, sq);
-    }
-    return;
-  }
-  float4* sB = reinterpret_cast<float4*>(sm_raw);                    // (-x', -y', q, 0) per source
-  float2* accB = reinterpret_cast<float2*>(sm_raw + kTS * sizeof(float4));  // [2 warps][kTS]
-  const float cx = 0.5f * (boxA.x + boxA.z), cy = 0.5f * (boxA.y + boxA.w);
-  constexpr float kAway = 1e15f;  // padding: far from everything, zero strength
-  for (int l = threadIdx.x; l < kTS; l += kB32) {
-    const int b = B0 + l;
-    float4 v = make_float4(-kAway, -kAway, 0.f, 0.f);
-    if (b < M) {
-      const float4 p = g.pf[b];
-      v = make_float4(-((p.x - cx) + p.z), -((p.y - cy) + p.w), g.qf[b], 0.f);
-    }
-    sB[l] = v;
-  }
-  // four A targets per lane, packed two by two: (t0, t1) and (t2, t3)
-  float tx[kT32], ty[kT32], qa[kT32];
+  const int A0 = ti * TS, B0 = tj * TS;
+  const int t = threadIdx.x;
+  if constexpr (KIND == 0) {
+    // Laplace: tiles whose whole boxes are far (bodies of whole tiles, or in
+    // spatial order) need one centre: no per-group targets
+    const float4 boxA = body_range_box(g.bbox, g.body_of[A0], g.body_of[min(A0 + TS, M) - 1]);
+    const float4 boxB = body_range_box(g.bbox, g.body_of[B0], g.body_of[min(B0 + TS, M) - 1]);
+    if (ti != tj && boxes_far(boxA, boxB)) {
+      const float cx = 0.5f * (boxA.x + boxA.z), cy = 0.5f * (boxA.y + boxA.w);
+      for (int l = t; l < TS; l += B) {
+        const int b = min(B0 + l, M - 1);  // past the end: the last node with zero strength
+        const float4 p = g.pf[b];
+        sF[l] = make_float4(-((p.x - cx) + p.z), -((p.y - cy) + p.w), B0 + l < M ? g.qf[b] : 0.f, 0.f);
+      }
+      float2 TX[H], TY[H], Q[H], AX[H], AY[H];
 #pragma unroll
-  for (int k = 0; k < kT32; ++k) {
-    const int a = A0 + threadIdx.x + k * kB32;
-    tx[k] = ty[k] = kAway;
-    qa[k] = 0.f;
-    if (a < M) {
-      const float4 p = g.pf[a];
-      tx[k] = (p.x - cx) + p.z;
-      ty[k] = (p.y - cy) + p.w;
-      qa[k] = g.qf[a];
+      for (int h = 0; h < H; ++h) {
+        const int a0 = A0 + t + 2 * h * B, a1 = a0 + B;
+        const float4 p0 = g.pf[a0], p1 = g.pf[a1];
+        TX[h] = make_float2((p0.x - cx) + p0.z, (p1.x - cx) + p1.z);
+        TY[h] = make_float2((p0.y - cy) + p0.w, (p1.y - cy) + p1.w);
+        Q[h] = make_float2(g.qf[a0], g.qf[a1]);
+        AX[h] = AY[h] = make_float2(0.f, 0.f);
+      }
+      __syncthreads();
+      for (int o = 0; o < TS; o += 32)
+        accB[(t >> 5) * TS + o + (t & 31)] =
+            sym_group<0, true, H>(sF + o, sL, sN, TX, TY, TX, TY, Q, Q, Q, Q, AX, AY);
+#pragma unroll
+      for (int k = 0; k < 2 * H; ++k)
+        write_slot<0>(g, A0 + t + k * B, tj, k & 1 ? AX[k >> 1].y : AX[k >> 1].x, 0.f,
+                      k & 1 ? AY[k >> 1].y : AY[k >> 1].x, 0.f, partial);
+      sym_write_sources<0>(g, B0, TS, ti, accB, partial);
+      return;
     }
   }
-  const float2 TXa = make_float2(tx[0], tx[1]), TXb = make_float2(tx[2], tx[3]);
-  const float2 TYa = make_float2(ty[0], ty[1]), TYb = make_float2(ty[2], ty[3]);
-  const float2 QAa = make_float2(qa[0], qa[1]), QAb = make_float2(qa[2], qa[3]);
-  float2 AXa = make_float2(0.f, 0.f), AXb = AXa, AYa = AXa, AYb = AXa;
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int r0 = 0; r0 < kTS; r0 += 32) {
-    float bx = 0.f, by = 0.f;  // accumulator of the source this lane holds (travels)
-#pragma unroll 8
-    for (int k = 0; k < 32; ++k) {
-      const float4 src = sB[r0 + ((lane + k) & 31)];
-      const float2 sx = make_float2(src.x, src.x), sy = make_float2(src.y, src.y);
-      const float2 dxa = __fadd2_rn(TXa, sx), dxb = __fadd2_rn(TXb, sx);
-      const float2 dya = __fadd2_rn(TYa, sy), dyb = __fadd2_rn(TYb, sy);
-      const float2 r2a = __ffma2_rn(dxa, dxa, __fmul2_rn(dya, dya));
-      const float2 r2b = __ffma2_rn(dxb, dxb, __fmul2_rn(dyb, dyb));
-      const float2 ia = make_float2(rcp_approx(r2a.x), rcp_approx(r2a.y));
-      const float2 ib = make_float2(rcp_approx(r2b.x), rcp_approx(r2b.y));
-      const float2 qb = make_float2(src.z, src.z);
-      const float2 sba = __fmul2_rn(qb, ia), sbb = __fmul2_rn(qb, ib);
-      AXa = __ffma2_rn(dxa, sba, AXa);
-      AXb = __ffma2_rn(dxb, sbb, AXb);
-      AYa = __ffma2_rn(dya, sba, AYa);
-      AYb = __ffma2_rn(dyb, sbb, AYb);
-      const float2 saa = __fmul2_rn(QAa, ia), sab = __fmul2_rn(QAb, ib);
-      const float2 ux = __ffma2_rn(dxb, sab, __fmul2_rn(dxa, saa));
-      const float2 uy = __ffma2_rn(dyb, sab, __fmul2_rn(dya, saa));
-      bx -= ux.x + ux.y;  // the source gains -q_a r w
-      by -= uy.x + uy.y;
-      // hand the accumulator to the lane that takes this source next
-      bx = __shfl_sync(0xffffffffu, bx, (lane + 1) & 31);
-      by = __shfl_sync(0xffffffffu, by, (lane + 1) & 31);
+  for (int gi = t; gi < G; gi += B) {
+    const int f = min(B0 + 32 * gi, M - 1), e = min(f + 31, M - 1);
+    const float4 gb = body_range_box(g.bbox, g.body_of[f], g.body_of[e]);
+    bool far = ti != tj;
+    if (far) {
+      const int i1 = g.body_of[A0 + TS - 1];
+      for (int i = g.body_of[A0]; i <= i1; ++i) far = far && boxes_far(g.bbox[i], gb);
     }
-    accB[warp * kTS + r0 + lane] = make_float2(bx, by);  // back at its own lane: source r0 + lane
-  }
-  {
-    const int a = A0 + threadIdx.x;
-    if (a < M) write_projected(g, a, tj, AXa.x, AYa.x, partial);
-    if (a + kB32 < M) write_projected(g, a + kB32, tj, AXa.y, AYa.y, partial);
-    if (a + 2 * kB32 < M) write_projected(g, a + 2 * kB32, tj, AXb.x, AYb.x, partial);
-    if (a + 3 * kB32 < M) write_projected(g, a + 3 * kB32, tj, AXb.y, AYb.y, partial);
+    sBox[gi] = gb;
+    sFar[gi] = far;
   }
   __syncthreads();
-  for (int l = threadIdx.x; l < kTS; l += kB32) {
-    const int b = B0 + l;
-    if (b < M) {
-      const float2 u = accB[l], v = accB[kTS + l];
-      write_projected(g, b, ti, u.x + v.x, u.y + v.y, partial);
+  for (int l = t; l < TS; l += B) {
+    const int b = min(B0 + l, M - 1);  // past the end: the last node with zero strength
+    const float4 p = g.pf[b];
+    const float4 bb = sBox[l >> 5];
+    float q1 = 0.f, q2 = 0.f;
+    if (B0 + l < M) {
+      if (KIND == 0) {
+        q1 = g.qf[b];
+      } else {
+        const float2 q = reinterpret_cast<const float2*>(g.qf)[b];
+        q1 = q.x;
+        q2 = q.y;
+      }
+    }
+    const float cx = 0.5f * (bb.x + bb.z), cy = 0.5f * (bb.y + bb.w);
+    sF[l] = make_float4(-((p.x - cx) + p.z), -((p.y - cy) + p.w), q1, q2);
+    sH[l] = make_float4(-p.x, -p.y, q1, q2);
+    sL[l] = make_float2(-p.z, -p.w);
+    if (KIND == 1) {
+      sN[l] = g.nf[b];
+      sAcc[l] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
+  float2 Q1[H], Q2[H], NX[H], NY[H], AX[H], AY[H];
+  float4 P[KIND == 0 ? 2 * H : 1];  // Laplace: the targets' positions, held
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    const int a0 = min(A0 + t + 2 * h * B, M - 1), a1 = min(A0 + t + (2 * h + 1) * B, M - 1);
+    if (KIND == 0) {
+      P[2 * h] = g.pf[a0];
+      P[2 * h + 1] = g.pf[a1];
+      Q1[h] = make_float2(g.qf[a0], g.qf[a1]);
+      Q2[h] = NX[h] = NY[h] = make_float2(0.f, 0.f);  // unused
+    } else {
+      const float2 q0 = reinterpret_cast<const float2*>(g.qf)[a0], q1 = reinterpret_cast<const float2*>(g.qf)[a1];
+      const float2 n0 = g.nf[a0], n1 = g.nf[a1];
+      Q1[h] = make_float2(q0.x, q1.x);
+      Q2[h] = make_float2(q0.y, q1.y);
+      NX[h] = make_float2(n0.x, n1.x);
+      NY[h] = make_float2(n0.y, n1.y);
+    }
+    AX[h] = AY[h] = make_float2(0.f, 0.f);
+  }
+  auto target = [&](int k) { return KIND == 0 ? P[KIND == 0 ? k : 0] : g.pf[min(A0 + t + k * B, M - 1)]; };
+  __syncthreads();
+  if (ti == tj) {
+    // directed pass of the tile with itself (exact differences, r = 0 excluded)
+    const int nt = min(TS, M - B0);
+    float4 T[2 * H];
+#pragma unroll
+    for (int k = 0; k < 2 * H; ++k) T[k] = target(k);
+    for (int l0 = 0; l0 < nt; l0 += kSymChunk) {
+      const int l1 = min(nt, l0 + kSymChunk);
+#pragma unroll 2
+      for (int l = l0; l < l1; ++l) {
+        const float4 src = sH[l];
+        const float2 lo = sL[l];
+        float c[2 * H][2];
+#pragma unroll
+        for (int k = 0; k < 2 * H; ++k) {
+          const float2 n2 = NX[k >> 1], m2 = NY[k >> 1];
+          f32_pair<KIND>(T[k].x, T[k].y, T[k].z, T[k].w, k & 1 ? n2.y : n2.x, k & 1 ? m2.y : m2.x,
+                         make_float4(-src.x, -src.y, -lo.x, -lo.y), src.z, src.w, c[k][0], c[k][1]);
+          if (t + k * B == l) c[k][0] = c[k][1] = 0.f;
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          AX[h] = __fadd2_rn(AX[h], make_float2(c[2 * h][0], c[2 * h + 1][0]));
+          AY[h] = __fadd2_rn(AY[h], make_float2(c[2 * h][1], c[2 * h + 1][1]));
+        }
+      }
+      if (KIND == 1) sym_flush<H>(sAcc, AX, AY);
+    }
+  } else {
+    const int lane = t & 31, warp = t >> 5;
+    for (int gi = 0; gi < G; ++gi) {
+      const int o = 32 * gi;
+      float2 TX[H], TY[H], u;
+      if (sFar[gi]) {
+        const float4 bb = sBox[gi];
+        const float cx = 0.5f * (bb.x + bb.z), cy = 0.5f * (bb.y + bb.w);
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const float4 p0 = target(2 * h), p1 = target(2 * h + 1);
+          TX[h] = make_float2((p0.x - cx) + p0.z, (p1.x - cx) + p1.z);
+          TY[h] = make_float2((p0.y - cy) + p0.w, (p1.y - cy) + p1.w);
+        }
+        u = sym_group<KIND, true, H>(sF + o, sL + o, sN + o, TX, TY, TX, TY, Q1, Q2, NX, NY, AX, AY);
+      } else {
+        float2 TXL[H], TYL[H];
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const float4 p0 = target(2 * h), p1 = target(2 * h + 1);
+          TX[h] = make_float2(p0.x, p1.x);
+          TY[h] = make_float2(p0.y, p1.y);
+          TXL[h] = make_float2(p0.z, p1.z);
+          TYL[h] = make_float2(p0.w, p1.w);
+        }
+        u = sym_group<KIND, false, H>(sH + o, sL + o, sN + o, TX, TY, TXL, TYL, Q1, Q2, NX, NY, AX, AY);
+      }
+      accB[warp * TS + o + lane] = u;
+      if (KIND == 1 && gi % (kSymChunk / 32) == kSymChunk / 32 - 1) sym_flush<H>(sAcc, AX, AY);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 2 * H; ++k) {
+    const int a = A0 + t + k * B;
+    if (a >= M) continue;
+    if (KIND == 0) {
+      write_slot<0>(g, a, tj, k & 1 ? AX[k >> 1].y : AX[k >> 1].x, 0.f, k & 1 ? AY[k >> 1].y : AY[k >> 1].x, 0.f, partial);
+    } else {
+      const float4 c = sAcc[t + k * B];
+      write_slot<1>(g, a, tj, c.x, c.y, c.z, c.w, partial);
+    }
+  }
+  if (ti != tj) sym_write_sources<KIND>(g, B0, TS, ti, accB, partial);
+}
+
+// Tiles of 128 nodes (one warp, four targets a lane), 256 (two warps) and, Stokes,
+// 192 (one warp, six targets).
+template <int KIND>
+void launch_pair32s(const Geo& g, int tile, double* partial, const int* stop, cudaStream_t s) {
+  const long long nt = (g.M + tile - 1) / tile;
+  const unsigned pairs = (unsigned)(nt * (nt + 1) / 2);
+  if constexpr (KIND == 1) {
+    if (tile == 192) {
+      k_pair32s<1, 3><<<pairs, 32, sym32_smem<1, 3>(32), s>>>(g, partial, stop);
+      return;
+    }
+  }
+  k_pair32s<KIND, 2><<<pairs, tile / 4, sym32_smem<KIND, 2>(tile / 4), s>>>(g, partial, stop);
 }
 
 // -------------------------------------------------------- symmetric FP64 ----
@@ -1572,11 +1771,39 @@ PairPlan plan_symmetric64(int M, int kind, int max_slots) {
   return best;
 }
 
+// The symmetric FP32 plan (S = 0: the directed kernel).  Measured, Laplace, tiles
+// of 128 / 256 nodes, directed: M = 4,096 22 / 31, 22 us; M = 8,192 33 / 37, 43; M
+// = 12,800 54 / 60, 92; M = 25,600 159 / 157, 177; M = 51,200 576 / 563.  Stokes,
+// 128 / 192, directed: M = 2,048 22, 16; M = 4,096 24, 25; M = 8,192 43 / 49, 56;
+// M = 25,600 258 / 252, 305; M = 51,200 956 / 915, 1,684.
+PairPlan plan_symmetric32(int M, int kind, int max_slots) {
+  auto make = [&](int tile) {
+    PairPlan p = uniform_plan((M + tile - 1) / tile, tile);
+    p.sym = tile;
+    return p;
+  };
+  auto pairs = [&](int tile) {
+    const long long nt = (M + tile - 1) / tile;
+    return nt * (nt + 1) / 2;
+  };
+  const int nsm = device_sms();
+  PairPlan p{0, 0, 0, 0};
+  if (kind == 0) {
+    if (pairs(128) >= 6LL * nsm) p = make(pairs(256) >= 30LL * nsm ? kTS : 128);
+  } else {
+    if (pairs(128) >= 4LL * nsm) p = make(pairs(192) >= 40LL * nsm ? 192 : 128);
+  }
+  if (p.S > max_slots || (double)p.S * M * (kind + 1) * 8e-6 > 512.0) p = PairPlan{0, 0, 0, 0};
+  return p;
+}
+
 PairPlan plan_pairs(int M, int kind, int precision, int max_slots) {
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned.find(tune_key(M, kind, precision));
-    if (it != g_tuned.end() && (precision != 0 || !it->second.sym || it->second.S <= max_slots)) return it->second;
+    // (the symmetric float-float and 256-node FP32 Laplace plans are not bounded by max_slots)
+    if (it != g_tuned.end() && (!it->second.sym || it->second.S <= max_slots || (precision > 0 && it->second.sym == kTS)))
+      return it->second;
   }
   return occupancy_plan(M, kind, precision, max_slots);
 }
@@ -1585,6 +1812,10 @@ PairPlan occupancy_plan(int M, int kind, int precision, int max_slots) {
   const DeviceShape& d = device_shape();
   if (precision == 0) {
     const PairPlan p = plan_symmetric64(M, kind, max_slots);
+    if (p.S > 0) return p;
+  }
+  if (precision == 1) {
+    const PairPlan p = plan_symmetric32(M, kind, max_slots);
     if (p.S > 0) return p;
   }
   if ((precision == 1 || precision == 2) && kind == 0) {
@@ -1664,15 +1895,16 @@ void launch_pairs(const Geo& g, int kind, int precision, const PairPlan& p, VecR
     const int gs = (int)std::min<long long>(1216, (g.M + 255) / 256);
     if (kind == 0) {
       k_src32<0><<<gs, 256, 0, s>>>(g, v, sscale, stop);
-      if (!BATCH && p.sym) {
-        const long long nt = (g.M + kTS - 1) / kTS;
-        k_pair32s<<<(unsigned)(nt * (nt + 1) / 2), kB32, 0, s>>>(g, (int)nt, partial, stop);
-      } else {
+      if (!BATCH && p.sym)
+        launch_pair32s<0>(g, p.sym, partial, stop, s);
+      else
         k_pair32<0, BATCH><<<grid, kB32, 0, s>>>(g, v, sscale, p, partial, stop);
-      }
     } else {
       k_src32<1><<<gs, 256, 0, s>>>(g, v, sscale, stop);
-      k_pair32<1, BATCH><<<grid, kB32, 0, s>>>(g, v, sscale, p, partial, stop);
+      if (!BATCH && p.sym)
+        launch_pair32s<1>(g, p.sym, partial, stop, s);
+      else
+        k_pair32<1, BATCH><<<grid, kB32, 0, s>>>(g, v, sscale, p, partial, stop);
     }
     note_launches(1);
   } else {

@@ -9,7 +9,7 @@ torch = pytest.importorskip("torch")
 import synth  # noqa: E402
 from oracle import geometry, laplace, stokes  # noqa: E402
 from paper_1507_05925_gb300 import bie  # noqa: E402
-from test_gpu_parity import TOL64, TOL_SOLVE, rel2, rel_max, to_dev  # noqa: E402
+from test_gpu_parity import TOL32, TOL64, TOL_SOLVE, rel2, rel_max, to_dev  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -94,3 +94,48 @@ def test_workspace_cap_takes_the_smaller_plans(ctx):
     srv.close()
     assert rc == bie.OK and rel2(phi, ref) <= TOL_SOLVE
     assert st["peak_inflight_bytes"] <= cap
+
+
+def ragged(total, seed):
+    """Ragged bodies (8 to 300 nodes) in random order on a grid of pitch 2.6, some
+    close to each other, `total` nodes in all."""
+    rng = np.random.default_rng(seed)
+    counts = []
+    while sum(counts) < total - 400:
+        counts.append(int(rng.choice([8, 31, 32, 33, 64, 97, 128, 200, 256, 300])))
+    counts.append(total - sum(counts))
+    side = int(np.ceil(np.sqrt(len(counts))))
+    slots = rng.permutation(side * side)[:len(counts)]
+    curves = []
+    for n, s in zip(counts, slots):
+        x, y = 2.6 * (s // side), 2.6 * (s % side)
+        curves.append(synth.ellipse(x, y, 1.2, rng.uniform(0.4, 1.2), rng.uniform(0, 3), n))
+    return synth.assemble(curves)
+
+
+# tiles of 128 (the last with 1, 127 and 128 nodes), of 192 and 256
+@pytest.mark.parametrize("kind", [bie.LAPLACE, bie.STOKES])
+@pytest.mark.parametrize("M", [5505, 5631, 5632, 21505, 25857])
+def test_symmetric_fp32_operator(ctx, kind, M):
+    g = ragged(M, M)
+    assert g["x"].size == M
+    gd = to_dev(g)
+    v = np.random.default_rng(M + 1).standard_normal(M * (kind + 1))
+    vin = torch.from_numpy(v).cuda()
+    out = torch.empty_like(vin)
+    bie.tune_clear()
+    assert bie.apply_operator(ctx, gd, kind, bie.FP64, vin, out) == bie.OK
+    ref = out.cpu().numpy()
+    res = []
+    for _ in range(2):
+        out.fill_(float("nan"))
+        assert bie.apply_operator(ctx, gd, kind, bie.MIXED, vin, out) == bie.OK
+        res.append(out.cpu().numpy())
+    assert np.array_equal(res[0], res[1])  # fixed order
+    assert bie.tune(ctx, gd, kind, bie.MIXED, splits=7)[0] == bie.OK  # the directed kernel
+    assert bie.apply_operator(ctx, gd, kind, bie.MIXED, vin, out) == bie.OK
+    bie.tune_clear()
+    e_sym, e_dir = rel_max(res[0], ref), rel_max(out.cpu().numpy(), ref)
+    print(f"kind={kind} M={M}: symmetric {e_sym:.2e}, directed {e_dir:.2e}")
+    assert e_sym <= TOL32[kind]
+    assert e_dir <= TOL32[kind]
