@@ -741,13 +741,18 @@ int launch_iteration(bie_ctx* ctx, Work& w, const Op& op, cudaStream_t s) {
   CK(it.apply(op.precond ? vec(w.zbuf) : vj, vj1, &w.st->stop, s, false));
   ArnoldiArgs a{w.V,        ld,       n,      w.st,      w.arn, w.H, w.cs, w.sn, w.gv, w.g,
                 w.kind,     w.bj_off, op.precond ? w.bj_blocks : nullptr, w.zbuf};
-  a.bj64 = op.prec == 0;  // FP64 GMRES: the preconditioner applied in FP64 arithmetic
   if (w.seg.P > 1) {
+    a.bj64 = op.prec == 0;  // FP64 GMRES: the preconditioner applied in FP64 arithmetic
     CK(arnoldi_seg(a, w.seg, w.seg_grid, s));
-  } else {
+  } else if (op.prec == 1 && w.VF) {
     // the FP32 inner solves: CGS2 in FP32 against the FP32 basis
-    if (op.prec == 1 && w.VF) a.vf = w.VF;
-    CK(arnoldi(a, arnoldi_grid(n, a.vf != nullptr, w.g.N), s));
+    a.vf = w.VF;
+    CK(arnoldi(a, arnoldi_grid(n, true, w.g.N), s));
+  } else {
+    if (op.precond) a.wt = w.ytmp;  // free inside a cycle
+    CK(arnoldi(a, arnoldi_grid(n, false, w.g.N), s));
+    if (op.precond)
+      CK(bj_normalize_apply64(w.g, w.kind, w.bj_off, w.bj_blocks, w.ytmp, w.zbuf, w.V, ld, w.st, w.bj_max_nb, s));
   }
   return BIE_OK;
 }

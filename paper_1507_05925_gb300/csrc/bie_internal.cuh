@@ -297,6 +297,10 @@ void set_bj_pivot_floor(double floor);
 // z = P v (v scaled, z scaled); f64: in FP64 arithmetic on the FP16 blocks
 cudaError_t bj_apply(const Geo& g, int kind, const long long* off_dev, const bj_t* blocks, VecRef v, double* z,
                      const int* stop, int max_nb, cudaStream_t s, bool f64 = false);
+// After an Arnoldi step that left w = ||w|| v_{j+1} unnormalised (ArnoldiArgs::wt):
+// v_{j+1} into its row of V and z = P v_{j+1}, in FP64 arithmetic.
+cudaError_t bj_normalize_apply64(const Geo& g, int kind, const long long* off_dev, const bj_t* blocks, const double* w,
+                                 double* z, double* V, long long ld, const KState* st, int max_nb, cudaStream_t s);
 
 // ---------------------------------------------------------------- small.cu
 // One-launch solves of batches of small problems (one CTA per problem, the
@@ -338,7 +342,8 @@ struct ArnoldiArgs {
   const long long* off;
   const bj_t* blocks;
   double* z;
-  int bj64 = 0;            // apply the FP32 blocks in FP64 arithmetic (FP64 GMRES)
+  int bj64 = 0;            // batched step: apply the blocks in FP64 arithmetic (FP64 GMRES)
+  double* wt = nullptr;    // FP64 step: leave the new vector here, unnormalised (bj_normalize_apply64 follows)
   float* vf = nullptr;     // FP32 copy of the basis ((m + 1) x ld): CGS2 in FP32 (FP32 inner solves, wide grids)
   int fault_skip = -1;     // test hook: this CTA leaves before the first grid barrier
   long long spins = 0;     // polls before a grid barrier gives up (set by the launcher)

@@ -41,12 +41,12 @@ __device__ __forceinline__ double combine(const double* __restrict__ V, long lon
 // One Arnoldi step after w = A z_j (w = V_{j+1}) in a single cooperative
 // launch with three grid barriers: CGS2 (h1 = V^T w; w -= V h1; h2 = V^T w;
 // w -= V h2), ||w||, the Hessenberg column with its Givens rotations and the
-// residual estimate, v_{j+1} = w / ||w|| and, with the block-Jacobi
-// preconditioner, z_{j+1} = P v_{j+1}.  After each barrier every CTA adds the
-// per-CTA partials itself, in CTA order (deterministic; no atomics), so
-// nothing else synchronises the grid.  In the last phase a CTA that owns a
-// body reads that body's w, writes z and normalises v in place: every element
-// is written only by its owner, after the owner has read it.
+// residual estimate, and v_{j+1} = w / ||w||.  After each barrier every CTA adds
+// the per-CTA partials itself, in CTA order (deterministic; no atomics), so
+// nothing else synchronises the grid.  With the block-Jacobi preconditioner w is
+// left unnormalised in a.wt and the launch that follows writes v_{j+1} and
+// z_{j+1} = P v_{j+1} (bj_normalize_apply64): the blocks' FP64 arithmetic wants
+// every SM, the steps here want few CTAs at their barriers.
 
 // Partial dot products of this CTA's elements of w with V_0..V_{jc-1} into
 // out[0..jc).  NARROW (a grid of at most two CTAs per SM, few elements a
@@ -335,11 +335,9 @@ __global__ void __launch_bounds__(kBV, NARROW ? 1 : 4) k_arnoldi(ArnoldiArgs a) 
   __shared__ double sh[kBV / 32][kMaxBasis];
   __shared__ double hs1[kMaxBasis], hs2[kMaxBasis];
   __shared__ double red[kBV / 32];
-  __shared__ float ws[kBjMaxBlock];
-  __shared__ double wsd[kBjMaxBlock];
   const int j = st->j, jc = j + 1;
   const long long n = a.n, ld = a.ld;
-  double* __restrict__ w = a.V + (long long)(j + 1) * ld;
+  double* w = a.V + (long long)(j + 1) * ld;
   const long long stride = (long long)gridDim.x * kBV;
   const long long G = gridDim.x;
   double* part1 = a.part;
@@ -359,9 +357,10 @@ __global__ void __launch_bounds__(kBV, NARROW ? 1 : 4) k_arnoldi(ArnoldiArgs a) 
   arn_grid_sum(part2, jc, hs2);
   // w -= V h2; ||w||^2
   double nrm = 0.0;
+  double* wo = a.wt ? a.wt : w;
   for (long long k = blockIdx.x * (long long)kBV + threadIdx.x; k < n; k += stride) {
     const double t = w[k] - combine(a.V, ld, k, hs2, jc);
-    w[k] = t;
+    wo[k] = t;
     nrm = fma(t, t, nrm);
   }
   nrm = block_sum<kBV>(nrm, red);
@@ -375,41 +374,10 @@ __global__ void __launch_bounds__(kBV, NARROW ? 1 : 4) k_arnoldi(ArnoldiArgs a) 
   __syncthreads();
   const double hn = hn_s;
   if (blockIdx.x == 0) arn_hessenberg(a, st, j, hs1, hs2, hn);
+  if (a.wt) return;  // normalised by the preconditioner's launch
+  // v_{j+1} = w / ||w|| over this CTA's own elements
   const double inv = hn > 0.0 ? 1.0 / hn : 0.0;
-  if (!a.blocks) {
-    // v_{j+1} = w / ||w|| over this CTA's own elements
-    for (long long k = blockIdx.x * (long long)kBV + threadIdx.x; k < n; k += stride) w[k] *= inv;
-    return;
-  }
-  // per body: v = w inv (w read through L2: other CTAs wrote it), z = P v
-  __shared__ float4 red4[2 * kBV];
-  const int c = a.kind + 1;
-  for (int i = blockIdx.x; i < a.g.N; i += (int)G) {
-    const long long a0 = (long long)a.g.body_start[i] * c;
-    const int nb = (a.g.body_start[i + 1] - a.g.body_start[i]) * c;
-    if (nb > kBjMaxBlock) {
-      for (int r = threadIdx.x; r < nb; r += kBV) {
-        const double v = __ldcg(w + a0 + r) * inv;
-        w[a0 + r] = v;
-        a.z[a0 + r] = v;
-      }
-      continue;
-    }
-    for (int r = threadIdx.x; r < nb; r += kBV) {
-      const double v = __ldcg(w + a0 + r) * inv;
-      w[a0 + r] = v;
-      if (a.bj64)
-        wsd[r] = v;
-      else
-        ws[r] = (float)v;
-    }
-    __syncthreads();
-    if (a.bj64)
-      bj_body_apply64(a.blocks + a.off[i], nb, wsd, a.z + a0);
-    else
-      bj_body_apply(a.blocks + a.off[i], a.off[i], nb, ws, a.z + a0, red4);
-    __syncthreads();
-  }
+  for (long long k = blockIdx.x * (long long)kBV + threadIdx.x; k < n; k += stride) w[k] *= inv;
 }
 
 // ------------------------------------------- Arnoldi step of the FP32 solves

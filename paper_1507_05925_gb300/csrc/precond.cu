@@ -298,21 +298,16 @@ __global__ void __launch_bounds__(CS == 1 ? kMaxSingle : CS == 4 ? kMaxBlock4 : 
     }
 }
 
-// z = P v: z_i = B_i^{-1} v_i per body (identity for bodies left out).  CTA
-// (i, y) computes rows [64 y, 64 y + 64) of body i with four column groups of
-// 64 threads, reduced in shared memory; each warp reads 32 consecutive rows of
-// one column (coalesced).
-// F64: the same product in FP64 arithmetic (v not rounded to FP32), so that
-// P is one fixed linear map to FP64 rounding (FP64 GMRES).
-template <bool F64>
+// z = P v in FP32 arithmetic: z_i = B_i^{-1} v_i per body (identity for bodies
+// left out).  CTA (i, y) computes rows [64 y, 64 y + 64) of body i with four
+// column groups of 64 threads, reduced in shared memory; each warp reads 32
+// consecutive rows of one column (coalesced).
 __global__ void __launch_bounds__(kBA) k_bj_apply(Geo g, int kind, const long long* __restrict__ off,
                                                   const bj_t* __restrict__ blocks, VecRef vr, double* __restrict__ z,
                                                   const int* __restrict__ stop) {
-  using T = typename std::conditional<F64, double, float>::type;
   if (stop && *stop) return;
-  extern __shared__ __align__(16) unsigned char vs_raw[];
-  T* vs = reinterpret_cast<T*>(vs_raw);
-  __shared__ T part[kBA];
+  extern __shared__ __align__(16) float vs[];
+  __shared__ float part[kBA];
   const double* v = vr.ptr();
   const int i = blockIdx.x;
   const int c = kind + 1;
@@ -325,23 +320,95 @@ __global__ void __launch_bounds__(kBA) k_bj_apply(Geo g, int kind, const long lo
     if (grp == 0 && r < nb) z[a0 + r] = v[a0 + r];
     return;
   }
-  for (int e = threadIdx.x; e < nb; e += kBA) vs[e] = (T)v[a0 + e];
+  for (int e = threadIdx.x; e < nb; e += kBA) vs[e] = (float)v[a0 + e];
   __syncthreads();
   const bj_t* B = blocks + off[i];
-  T acc = 0;
+  float acc = 0;
   if (r < nb) {
     const int per = (nb + kApplyGroups - 1) / kApplyGroups;
     const int cb = grp * per, ce = min(nb, cb + per);
 #pragma unroll 4
-    for (int col = cb; col < ce; ++col) acc = fma((T)__half2float(B[(long long)col * nb + r]), vs[col], acc);
+    for (int col = cb; col < ce; ++col) acc = fmaf(__half2float(B[(long long)col * nb + r]), vs[col], acc);
   }
   part[threadIdx.x] = acc;
   __syncthreads();
   if (grp == 0 && r < nb) {
-    T t = part[lr];
+    float t = part[lr];
 #pragma unroll
     for (int q = 1; q < kApplyGroups; ++q) t += part[q * kApplyRows + lr];
-    z[a0 + r] = (double)(fma((T)kBjShift, vs[r], t));  // P v = 2 v + W v
+    z[a0 + r] = (double)(fmaf(kBjShift, vs[r], t));  // P v = 2 v + W v
+  }
+}
+
+// z = P v in FP64 arithmetic on the FP16 blocks (FP64 GMRES: P must be one fixed
+// linear map to FP64 rounding).  With NORM, v is the basis vector that an
+// Arnoldi step left unnormalised in `v`: v / st->hnext is written to row st->j of
+// V as well (nothing is done once the cycle has stopped).
+// Bound by the FP64 pipe (two lanes a clock per SM), so the rows of a body are
+// spread over CTAs of 32 (32 rows x 8 column groups), as many as there are; an
+// Arnoldi step that applied a body's block on one CTA took 178 us at 740 nodes in
+// four bodies of up to 600 unknowns and 139 us at 7,100 nodes in 36 bodies, with
+// this launch beside it 22 + 19 and 26 + 13 us.  An FP16 entry becomes a double
+// without the FP64 pipe (a conversion would run on it): its bits, placed in the
+// high word, are the value times 2^-1008 exactly (FP16 subnormals become FP64
+// ones); v carries 2^500 and the sum 2^508.
+constexpr int kRows64 = 32, kGroups64 = kBA / kRows64;
+
+template <bool NORM>
+__global__ void __launch_bounds__(kBA) k_bj_apply64(Geo g, int kind, const long long* __restrict__ off,
+                                                    const bj_t* __restrict__ blocks, const double* __restrict__ v,
+                                                    double* __restrict__ z, double* __restrict__ V, long long ld,
+                                                    const KState* __restrict__ st, const int* __restrict__ stop) {
+  if (stop && *stop) return;
+  extern __shared__ __align__(16) double vd[];
+  __shared__ double part[kBA];
+  const int i = blockIdx.x;
+  const int c = kind + 1;
+  const int a0 = g.body_start[i] * c, nb = (g.body_start[i + 1] - g.body_start[i]) * c;
+  const int r0 = blockIdx.y * kRows64;
+  if (r0 >= nb) return;
+  const int lr = threadIdx.x % kRows64, grp = threadIdx.x / kRows64;
+  const int r = r0 + lr;
+  const double inv = NORM ? 1.0 / st->hnext : 1.0;
+  double* vout = NORM ? V + (long long)st->j * ld + a0 : nullptr;
+  if (nb > kMaxBlock) {
+    if (grp == 0 && r < nb) {
+      const double t = v[a0 + r] * inv;
+      if (NORM) vout[r] = t;
+      z[a0 + r] = t;
+    }
+    return;
+  }
+  const double up = __hiloint2double((1023 + 500) << 20, 0), down = __hiloint2double((1023 - 500) << 20, 0);  // 2^500
+  for (int e = threadIdx.x; e < nb; e += kBA) vd[e] = v[a0 + e] * inv * up;
+  __syncthreads();
+  const unsigned short* B = reinterpret_cast<const unsigned short*>(blocks + off[i]);
+  double s0 = 0.0, s1 = 0.0;
+  if (r < nb) {
+    auto entry = [&](int col) {
+      const unsigned h = B[(long long)col * nb + r];
+      return __hiloint2double((int)(((h & 0x8000u) << 16) | ((h & 0x7fffu) << 10)), 0);
+    };
+    const int per = (nb + kGroups64 - 1) / kGroups64;
+    const int cb = grp * per, ce = min(nb, cb + per);
+    int col = cb;
+#pragma unroll 4
+    for (; col + 2 <= ce; col += 2) {
+      s0 = fma(entry(col), vd[col], s0);
+      s1 = fma(entry(col + 1), vd[col + 1], s1);
+    }
+    if (col < ce) s0 = fma(entry(col), vd[col], s0);
+  }
+  part[threadIdx.x] = s0 + s1;
+  __syncthreads();
+  if (grp == 0 && r < nb) {
+    double t = part[lr];
+#pragma unroll
+    for (int q = 1; q < kGroups64; ++q) t += part[q * kRows64 + lr];
+    t *= __hiloint2double((1023 + 508) << 20, 0);  // 2^508
+    const double x = vd[r] * down;
+    if (NORM) vout[r] = x;
+    z[a0 + r] = fma((double)kBjShift, x, t);  // P v = 2 v + W v
   }
 }
 
@@ -434,12 +501,24 @@ cudaError_t bj_setup(const Geo& g, int kind, double alpha, const int* body_start
 
 cudaError_t bj_apply(const Geo& g, int kind, const long long* off_dev, const bj_t* blocks, VecRef v, double* z,
                      const int* stop, int max_nb, cudaStream_t s, bool f64) {
-  const dim3 grid(g.N, (max_nb + kApplyRows - 1) / kApplyRows);
   const size_t nv = (size_t)std::min(max_nb, kMaxBlock);
-  if (f64)
-    k_bj_apply<true><<<grid, kBA, nv * sizeof(double), s>>>(g, kind, off_dev, blocks, v, z, stop);
-  else
-    k_bj_apply<false><<<grid, kBA, nv * sizeof(float), s>>>(g, kind, off_dev, blocks, v, z, stop);
+  if (f64) {  // (callers pass a plain vector)
+    const dim3 grid(g.N, (max_nb + kRows64 - 1) / kRows64);
+    k_bj_apply64<false><<<grid, kBA, nv * sizeof(double), s>>>(g, kind, off_dev, blocks, v.base, z, nullptr, 0, nullptr,
+                                                               stop);
+  } else {
+    const dim3 grid(g.N, (max_nb + kApplyRows - 1) / kApplyRows);
+    k_bj_apply<<<grid, kBA, nv * sizeof(float), s>>>(g, kind, off_dev, blocks, v, z, stop);
+  }
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t bj_normalize_apply64(const Geo& g, int kind, const long long* off_dev, const bj_t* blocks, const double* w,
+                                 double* z, double* V, long long ld, const KState* st, int max_nb, cudaStream_t s) {
+  const size_t nv = (size_t)std::min(max_nb, kMaxBlock);
+  const dim3 grid(g.N, (max_nb + kRows64 - 1) / kRows64);
+  k_bj_apply64<true><<<grid, kBA, nv * sizeof(double), s>>>(g, kind, off_dev, blocks, w, z, V, ld, st, &st->stop);
   note_launches(1);
   return cudaGetLastError();
 }
