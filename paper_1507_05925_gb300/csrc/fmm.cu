@@ -948,49 +948,110 @@ __global__ void __launch_bounds__(kB) k_fmm_l2l(FmmDevT<T2> f, int l, const int*
 
 // Local expansion and near field at every node of a leaf, then the kernel's
 // combination into the pair-sum partial (Laplace scalar / Stokes 2-vector).
-// NEARP = 0: the near field enters the FP64 Cauchy sums.  NEARP = 1 (FP32)
-// and 2 (float-float): the far part is combined into the kernel value in
-// FP64 and the near field is summed as the real kernel with the pair
-// arithmetic of the direct sums (exact leading coordinate differences), so
-// the accuracy follows the operator that uses it: FP32 for the inner solves,
-// float-float for residuals.
+// The near field is the real kernel, summed directly over the 3 x 3 leaves: in
+// FP64 (NEARP = 0, with rcp64), in FP32 (1, the inner solves) or in float-float
+// (2, residuals), with exact leading coordinate differences in the latter two.
+//
+// Work: the m targets at hand take L = ceil(m / TPT) threads, and the kBE threads
+// hold G = kBE / L such groups, each with every G-th source; the groups' sums are
+// added in order.  A leaf of 39 nodes (the mean at 640,000) so keeps 91-94% of
+// the lanes, against 61% with one target a thread of 64.  FP32: two targets a
+// thread, so that a staged pair of sources (packed FP32x2) serves four pairs; the
+// leaf's own sources come first, so that only they are compared with the target.
+// The local expansions are evaluated a (target, channel) a thread; Laplace needs
+// no derivative.
+// Bound by the pair arithmetic: the FP64 pipe (10 Laplace, 16 Stokes operations a
+// pair), FP32 issue and the FP32 pipe.  Measured, one target a thread of 64 (FP64:
+// as Cauchy terms with a division and F' always) -> this: FP64 Laplace, 160,000
+// nodes, order 36: 5.31 -> 1.26 ms; FP32 Stokes, 640,000 nodes, order 18: 277 ->
+// 195 us; FP32 Laplace, 25,600 nodes: 39 -> 18 us; float-float Stokes, 640,000
+// nodes, order 36: 1.74 -> 1.39 ms.
+constexpr int kBE = 128;         // threads of an evaluation block
 constexpr int kNearChunk = 256;  // near-field sources staged per round
 
+template <int NEARP>
+struct EvalNear;  // what a block stages and adds per precision
+template <>
+struct EvalNear<0> {
+  static constexpr int kTPT = 1;
+  using Sum = double2;
+};
+template <>
+struct EvalNear<1> {
+  static constexpr int kTPT = 2;
+  using Sum = float2;
+};
+template <>
+struct EvalNear<2> {
+  static constexpr int kTPT = 1;
+  using Sum = float4;  // (x_h, x_l, y_h, y_l)
+};
+
+// Values of F and s F' at one target (u relative to the leaf centre, units of s).
+template <class T2>
+__device__ __forceinline__ void horner(const T2* __restrict__ a, int p, T2 u, bool deriv, T2& h, T2& dh) {
+  h = a[p - 1];
+  dh = cx<T2>(0.0, 0.0);
+  if (deriv) {
+    for (int l = p - 2; l >= 0; --l) {
+      T2 t = h;
+      cfma(t, dh, u);
+      dh = t;
+      t = a[l];
+      cfma(t, h, u);
+      h = t;
+    }
+  } else {
+    for (int l = p - 2; l >= 0; --l) {
+      T2 t = a[l];
+      cfma(t, h, u);
+      h = t;
+    }
+  }
+}
+
 template <class T2, int NEARP>
-__global__ void __launch_bounds__(kB) k_fmm_eval(FmmDevT<T2> f, Geo g, double* __restrict__ partial, const int* stop) {
+__global__ void __launch_bounds__(kBE) k_fmm_eval(FmmDevT<T2> f, Geo g, double* __restrict__ partial, const int* stop) {
   if (stop && *stop) return;
+  using Sum = typename EvalNear<NEARP>::Sum;
+  constexpr int TPT = EvalNear<NEARP>::kTPT, NT = kBE * TPT;  // targets at hand
+  // expansions [nd][p] (float-float: split hi + lo in 16 bytes), then F and F' of
+  // the targets at hand [nd][NT][2]
   extern __shared__ __align__(16) unsigned char smraw[];
-  T2* sm = reinterpret_cast<T2*>(smraw);  // [nd][p]
-  // near-field sources of the 3 x 3 leaves, staged in rounds
-  __shared__ float4 spa[kNearChunk];  // FP32: (x_hi, y_hi, x_lo, y_lo); float-float: (xh, xm, yh, ym)
-  __shared__ float2 spb[NEARP == 2 ? kNearChunk : 1];  // float-float: (xl, yl)
-  __shared__ float4 sq[kNearChunk];   // FP32: (q1, q2, -, -); float-float: (q1h, q1l, q2h, q2l)
-  __shared__ __align__(16) int sid[kNearChunk];
+  using E = typename std::conditional<NEARP == 2, float4, T2>::type;
+  E* sm = reinterpret_cast<E*>(smraw);
+  E* FF = sm + f.nd * f.p;
+  // FP64: (x, y) and (q1, q2) as double2; FP32: pairs of sources (hi, lo, strength);
+  // float-float: (xh, xm, yh, ym), (xl, yl, -, -), strengths
+  __shared__ float4 spa[kNearChunk], spb[NEARP == 1 ? 1 : kNearChunk], sq[NEARP == 0 ? 1 : kNearChunk];
+  __shared__ Sum red[NT];
   __shared__ int lst[10], lbeg[9];
   __shared__ float cen[6];  // FP32 instance: split leaf centre, 1/s, s
+  const int t = threadIdx.x;
   const int b = blockIdx.x, bx = b % f.nb, by = b / f.nb;
   const int s0 = f.start[b], n = f.start[b + 1] - s0;
   if (n == 0) return;
+  const int nd = f.nd, p = f.p;
   const long long box = lev_off(f.L) + b;
-  if constexpr (NEARP == 2) {
-    // float-float residuals: the local expansion split into hi + lo pairs
-    float4* smf = reinterpret_cast<float4*>(smraw);
-    for (int e = threadIdx.x; e < f.nd * f.p; e += kB) {
-      const double2 a = f.lc[box * f.nd * f.p + e];
+  for (int e = t; e < nd * p; e += kBE) {
+    if constexpr (NEARP == 2) {
+      const double2 a = f.lc[box * nd * p + e];
       const float rh = (float)a.x, ih = (float)a.y;
-      smf[e] = make_float4(rh, ih, (float)(a.x - (double)rh), (float)(a.y - (double)ih));
+      sm[e] = make_float4(rh, ih, (float)(a.x - (double)rh), (float)(a.y - (double)ih));
+    } else {
+      sm[e] = f.lc[box * nd * p + e];
     }
-  } else {
-    for (int e = threadIdx.x; e < f.nd * f.p; e += kB) sm[e] = f.lc[box * f.nd * f.p + e];
   }
-  const int y0 = max(0, by - 1), y1 = min(f.nb - 1, by + 1);
-  const int x0 = max(0, bx - 1), x1 = min(f.nb - 1, bx + 1);
   if constexpr (NEARP == 1) leaf_center32(f, b, cen);
-  if (threadIdx.x == 0) {
-    int c = 0, tot = 0;
-    for (int ny = y0; ny <= y1; ++ny)
-      for (int nx = x0; nx <= x1; ++nx) {
+  if (t == 0) {
+    // the leaf itself first, then its neighbours row by row
+    int c = 1, tot = n;
+    lbeg[0] = s0;
+    lst[0] = 0;
+    for (int ny = max(0, by - 1); ny <= min(f.nb - 1, by + 1); ++ny)
+      for (int nx = max(0, bx - 1); nx <= min(f.nb - 1, bx + 1); ++nx) {
         const int nl = ny * f.nb + nx;
+        if (nl == b) continue;
         lbeg[c] = f.start[nl];
         lst[c] = tot;
         tot += f.start[nl + 1] - f.start[nl];
@@ -1000,317 +1061,314 @@ __global__ void __launch_bounds__(kB) k_fmm_eval(FmmDevT<T2> f, Geo g, double* _
   }
   __syncthreads();
   const int total = lst[9];
+  auto source = [&](int v) {  // node of entry v of the list
+    int lf = 0;
+    while (v >= lst[lf + 1]) ++lf;
+    return f.perm[lbeg[lf] + (v - lst[lf])];
+  };
   double s;
   const double2 c = box_center(f, f.L, bx, by, s);
   const double inv_s = ldexp(f.Dinv, f.L);
-  for (int j0 = 0; j0 < n; j0 += kB) {
-    const int j = j0 + threadIdx.x;
-    const bool act = j < n;
-    const int i = act ? f.perm[s0 + j] : 0;
-    double ox = 0.0, oy = 0.0;
-    float oxf = 0.f, oyf = 0.f;  // FP32 instance
-    const double nx1 = (NEARP != 1 && act) ? g.nx[i] : 0.0, ny1 = (NEARP != 1 && act) ? g.ny[i] : 0.0;
-    if (NEARP == 2 && act) {
-      // the far field in float-float on the FP32 pipe (Horner for F and F',
-      // then the kernel's combination), about the leaf centre
-      const float4* smf = reinterpret_cast<const float4*>(smraw);
-      const double ux = (g.x[i] - c.x) * inv_s, uy = (g.y[i] - c.y) * inv_s;
-      const cff U = cff_split(ux, uy);
-      const float ish = (float)inv_s, isl = (float)(inv_s - (double)ish);
-      cff F[3], dF[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        if (d < f.nd) {
-          cff h = cff_load(smf[d * f.p + f.p - 1]), dh = cff_zero();
-          for (int l = f.p - 2; l >= 0; --l) {
-            dh = cff_fma(h, dh, U);                         // h + dh u (the old h)
-            h = cff_fma(cff_load(smf[d * f.p + l]), h, U);  // a_l + h u
-          }
-          F[d] = h;
-          dF[d] = cff_scale(dh, ish, isl);
+  for (int j0 = 0; j0 < n; j0 += NT) {
+    const int m = min(NT, n - j0);
+    // ---- local expansions: F and F' (scaled by 1/s) per (channel, target)
+    for (int q = t; q < nd * m; q += kBE) {
+      const int d = q / m, tt = q - d * m;
+      const int i = f.perm[s0 + j0 + tt];
+      E* o = FF + 2 * (d * NT + tt);
+      if constexpr (NEARP == 2) {
+        // float-float on the FP32 pipe
+        const cff U = cff_split((g.x[i] - c.x) * inv_s, (g.y[i] - c.y) * inv_s);
+        cff h = cff_load(sm[d * p + p - 1]), dh = cff_zero();
+        for (int l = p - 2; l >= 0; --l) {
+          if (nd > 1) dh = cff_fma(h, dh, U);  // h + dh u (the old h)
+          h = cff_fma(cff_load(sm[d * p + l]), h, U);  // a_l + h u
         }
-      }
-      if (f.nd == 1) {
-        const double2 f0 = cff_to(F[0]);
-        ox = nx1 * f0.x - ny1 * f0.y;
+        const float ish = (float)inv_s, isl = (float)(inv_s - (double)ish);
+        o[0] = cff_store(h);
+        o[1] = cff_store(cff_scale(dh, ish, isl));
       } else {
-        const cff nu = cff_split(nx1, ny1), nub = cff_conj(nu);
-        const float slh = (float)s, sll = (float)(s - (double)slh);
-        // S3 = -F'_{q conj(z_j - c)} with c the leaf centre (channel cm holds that density / s)
-        const cff S2 = cff_neg(dF[0]), S3 = cff_neg(cff_scale(dF[2], slh, sll));
-        const cff S1 = F[0], S6 = F[1];
-        const cff zb = cff_split(g.x[i] - c.x, -(g.y[i] - c.y));
-        const cff w = cff_fma(cff_neg(S3), zb, S2);  // conj(z - c) S2 - S3
-        cff tt = cff_zero();
-        tt = cff_fma(tt, nub, cff_conj(w));
-        tt = cff_fma(tt, nu, cff_conj(S1));
-        tt = cff_fma(tt, nub, cff_conj(S6));
-        tt = cff_fma(tt, nu, S1);
-        const double2 t2 = cff_to(tt);
-        ox = 0.25 * t2.x;
-        oy = 0.25 * t2.y;
+        T2 u, h, dh;
+        if constexpr (NEARP == 1) {
+          // from the hi/lo split of z and the block's split centre (no FP64)
+          const float4 P = g.pf[i];
+          u = make_float2(((P.x - cen[0]) + (P.z - cen[2])) * cen[4], ((P.y - cen[1]) + (P.w - cen[3])) * cen[4]);
+        } else {
+          u = cx<T2>((g.x[i] - c.x) * inv_s, (g.y[i] - c.y) * inv_s);
+        }
+        horner(sm + d * p, p, u, nd > 1, h, dh);
+        using R = decltype(u.x);
+        const R is = NEARP == 1 ? (R)cen[4] : (R)inv_s;
+        dh.x *= is;
+        dh.y *= is;
+        o[0] = h;
+        o[1] = dh;
       }
     }
-    if constexpr (NEARP == 1) {
-      if (act) {
-        // FP32 throughout: u from the hi/lo split of z and the block's split
-        // centre (no FP64 instruction per target)
-        const float4 P = g.pf[i];
-        const float2 nn = g.nf[i];
-        const float dxc = (P.x - cen[0]) + (P.z - cen[2]), dyc = (P.y - cen[1]) + (P.w - cen[3]);
-        const float2 u = make_float2(dxc * cen[4], dyc * cen[4]);
-        float2 F[3], dF[3];  // nd = 1 or 3 (operator channels), unrolled: registers
+    // ---- near field
+    const int L = (m + TPT - 1) / TPT, G = max(1, kBE / L);
+    const int grp = t / L, tl = t - grp * L;
+    const bool act = grp < G;
+    int ti[TPT];  // targets (index at hand)
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          if (d < f.nd) {
-            float2 h = sm[d * f.p + f.p - 1], dh = make_float2(0.f, 0.f);
-            for (int l = f.p - 2; l >= 0; --l) {
-              dh = cadd(cmul(dh, u), h);
-              h = cadd(cmul(h, u), sm[d * f.p + l]);
+    for (int k = 0; k < TPT; ++k) ti[k] = min(tl + k * L, m - 1);
+    if constexpr (NEARP == 0) {
+      const int i = f.perm[s0 + j0 + ti[0]];
+      const double tx = g.x[i], ty = g.y[i], tnx = g.nx[i], tny = g.ny[i];
+      double ax = 0.0, ay = 0.0;
+      double2* sx2 = reinterpret_cast<double2*>(spa);
+      double2* sq2 = reinterpret_cast<double2*>(spb);
+      for (int v0 = 0; v0 < total; v0 += kNearChunk) {
+        const int mm = min(kNearChunk, total - v0);
+        __syncthreads();
+        for (int e = t; e < mm; e += kBE) {
+          const int i2 = source(v0 + e);
+          sx2[e] = make_double2(g.x[i2], g.y[i2]);
+          sq2[e] = f.Q[(long long)i2 * nd];  // Laplace (q, 0); Stokes q1 + i q2
+        }
+        __syncthreads();
+        if (act) {
+          const int self = j0 + ti[0] - v0;
+#pragma unroll 2
+          for (int e = grp; e < mm; e += G) {
+            const double2 P = sx2[e], q = sq2[e];
+            const double dx = tx - P.x, dy = ty - P.y;
+            const double y = rcp64(dx * dx + dy * dy);
+            if (nd == 1) {
+              const double w = e == self ? 0.0 : q.x * y;
+              ax += dx * w;
+              ay += dy * w;
+            } else {
+              const double w = e == self ? 0.0 : ((dx * q.x + dy * q.y) * (dx * tnx + dy * tny)) * (y * y);
+              ax += w * dx;
+              ay += w * dy;
             }
-            F[d] = h;
-            dF[d] = make_float2(dh.x * cen[4], dh.y * cen[4]);
           }
         }
-        if (f.nd == 1) {
-          oxf = nn.x * F[0].x - nn.y * F[0].y;
+      }
+      __syncthreads();  // red of the previous targets has been read
+      if (act) red[grp * L + tl] = make_double2(ax, ay);
+    } else if constexpr (NEARP == 1) {
+      // two sources a packed FP32x2 operation, staged in pairs (positions hi and
+      // lo, strengths); an odd count is padded with a zero-strength source far away
+      float4* sp2 = spa;                   // [kNearChunk / 2] (xh0, xh1, yh0, yh1), negated
+      float4* sl2 = spa + kNearChunk / 2;  // [kNearChunk / 2] (xl0, xl1, yl0, yl1), negated
+      float4* sq2 = sq;                    // [kNearChunk / 2] (q1_0, q1_1, q2_0, q2_1)
+      float4 T[TPT];
+      float2 nn[TPT], AX[TPT], AY[TPT];
+#pragma unroll
+      for (int k = 0; k < TPT; ++k) {
+        const int i = f.perm[s0 + j0 + ti[k]];
+        T[k] = g.pf[i];
+        nn[k] = g.nf[i];
+        AX[k] = AY[k] = make_float2(0.f, 0.f);
+      }
+      // one staged pair of sources; CHECK: a source may be the target itself
+      auto pairs = [&](int e2, int self0, int self1, bool check) {
+        const float4 P = sp2[e2], PL = sl2[e2], Q = sq2[e2];
+#pragma unroll
+        for (int k = 0; k < TPT; ++k) {
+          // exact leading differences
+          const float2 dx = __fadd2_rn(__fadd2_rn(make_float2(T[k].x, T[k].x), make_float2(P.x, P.y)),
+                                       __fadd2_rn(make_float2(T[k].z, T[k].z), make_float2(PL.x, PL.y)));
+          const float2 dy = __fadd2_rn(__fadd2_rn(make_float2(T[k].y, T[k].y), make_float2(P.z, P.w)),
+                                       __fadd2_rn(make_float2(T[k].w, T[k].w), make_float2(PL.z, PL.w)));
+          const float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
+          float2 w = make_float2(rcp_approx(r2.x), rcp_approx(r2.y));
+          if (check) {  // the self pair (r = 0)
+            const int self = k == 0 ? self0 : self1;
+            if (2 * e2 == self) w.x = 0.f;
+            if (2 * e2 + 1 == self) w.y = 0.f;
+          }
+          if (nd == 1) {
+            const float2 cc = __fmul2_rn(make_float2(Q.x, Q.y), w);
+            AX[k] = __ffma2_rn(cc, dx, AX[k]);
+            AY[k] = __ffma2_rn(cc, dy, AY[k]);
+          } else {
+            const float2 ex = __fmul2_rn(dx, w), ey = __fmul2_rn(dy, w);
+            const float2 rq = __ffma2_rn(dx, make_float2(Q.x, Q.y), __fmul2_rn(dy, make_float2(Q.z, Q.w)));
+            const float2 rn = __ffma2_rn(ex, make_float2(nn[k].x, nn[k].x), __fmul2_rn(ey, make_float2(nn[k].y, nn[k].y)));
+            const float2 cc = __fmul2_rn(rq, rn);
+            AX[k] = __ffma2_rn(cc, ex, AX[k]);
+            AY[k] = __ffma2_rn(cc, ey, AY[k]);
+          }
+        }
+      };
+      for (int v0 = 0; v0 < total; v0 += kNearChunk) {
+        const int mm = min(kNearChunk, total - v0), m2 = (mm + 1) >> 1;
+        __syncthreads();
+        for (int e2 = t; e2 < m2; e2 += kBE) {
+          float4 P[2];
+          float2 q[2];
+          for (int h = 0; h < 2; ++h) {
+            const int e = 2 * e2 + h;
+            P[h] = make_float4(1e15f, 1e15f, 0.f, 0.f);
+            q[h] = make_float2(0.f, 0.f);
+            if (e < mm) {
+              const int i2 = source(v0 + e);
+              P[h] = g.pf[i2];
+              q[h] = f.Qf[i2];
+            }
+          }
+          sp2[e2] = make_float4(-P[0].x, -P[1].x, -P[0].y, -P[1].y);
+          sl2[e2] = make_float4(-P[0].z, -P[1].z, -P[0].w, -P[1].w);
+          sq2[e2] = make_float4(q[0].x, q[1].x, q[0].y, q[1].y);
+        }
+        __syncthreads();
+        if (act) {
+          const int own = min(m2, max(0, (n - v0 + 1) >> 1));  // pairs with sources of the leaf itself
+          const int self0 = j0 + ti[0] - v0, self1 = j0 + ti[TPT - 1] - v0;
+          int e2 = grp;
+          for (; e2 < own; e2 += G) pairs(e2, self0, self1, true);
+#pragma unroll 2
+          for (; e2 < m2; e2 += G) pairs(e2, 0, 0, false);
+        }
+      }
+      __syncthreads();
+      if (act)
+#pragma unroll
+        for (int k = 0; k < TPT; ++k)
+          red[k * kBE + grp * L + tl] = make_float2(AX[k].x + AX[k].y, AY[k].x + AY[k].y);
+    } else {
+      // float-float: one source at a time, float-float sums
+      const int i = f.perm[s0 + j0 + ti[0]];
+      FFTarget tg;
+      {
+        const float4 pp = g.xff[i];
+        const float2 pl = g.xfl[i];
+        tg.xh = pp.x;
+        tg.xm = pp.y;
+        tg.yh = pp.z;
+        tg.ym = pp.w;
+        tg.xl = pl.x;
+        tg.yl = pl.y;
+        tg.n = g.nff[i];
+      }
+      float axh = 0.f, axl = 0.f, ayh = 0.f, ayl = 0.f;
+      for (int v0 = 0; v0 < total; v0 += kNearChunk) {
+        const int mm = min(kNearChunk, total - v0);
+        __syncthreads();
+        for (int e = t; e < mm; e += kBE) {
+          const int i2 = source(v0 + e);
+          const double2 q = f.Q[(long long)i2 * nd];
+          const float2 pl = g.xfl[i2];
+          spa[e] = g.xff[i2];
+          spb[e] = make_float4(pl.x, pl.y, 0.f, 0.f);
+          const float q1h = (float)q.x, q2h = (float)q.y;
+          sq[e] = make_float4(q1h, (float)(q.x - (double)q1h), q2h, (float)(q.y - (double)q2h));
+        }
+        __syncthreads();
+        if (act) {
+          const int self = j0 + ti[0] - v0;
+          for (int e = grp; e < mm; e += G) {
+            if (e == self) continue;
+            const float4 pb = spb[e];
+            float cxh, cxl, cyh, cyl;
+            if (nd == 1)
+              ff_pair<0>(tg, spa[e], make_float2(pb.x, pb.y), sq[e], cxh, cxl, cyh, cyl);
+            else
+              ff_pair<1>(tg, spa[e], make_float2(pb.x, pb.y), sq[e], cxh, cxl, cyh, cyl);
+            ff_acc(axh, axl, cxh, cxl);
+            ff_acc(ayh, ayl, cyh, cyl);
+          }
+        }
+      }
+      __syncthreads();
+      if (act) red[grp * L + tl] = make_float4(axh, axl, ayh, ayl);
+    }
+    __syncthreads();
+    // ---- the kernel's combination, about the leaf centre (its terms do not cancel)
+    for (int tt = t; tt < m; tt += kBE) {
+      const int i = f.perm[s0 + j0 + tt];
+      const int k = tt / L, l = tt - k * L;  // its place among the near sums
+      Sum a = red[k * kBE + l];
+      for (int q = 1; q < G; ++q) {
+        const Sum o = red[k * kBE + q * L + l];
+        if constexpr (NEARP == 2) {
+          ff_acc(a.x, a.y, o.x, o.y);
+          ff_acc(a.z, a.w, o.z, o.w);
         } else {
-          // the kernel's combination about the leaf centre, as in the FP64 instance
-          const float2 nu = nn, nub = make_float2(nn.x, -nn.y);
-          const float2 S2 = make_float2(-dF[0].x, -dF[0].y);
-          const float2 S3 = make_float2(-cen[5] * dF[2].x, -cen[5] * dF[2].y);
-          const float2 S1 = F[0], S6 = F[1];
-          float2 w = cmul(make_float2(dxc, -dyc), S2);
+          a.x += o.x;
+          a.y += o.y;
+        }
+      }
+      double ox = 0.0, oy = 0.0;
+      if constexpr (NEARP == 2) {
+        const double nx1 = g.nx[i], ny1 = g.ny[i];
+        const double nearx = (double)a.x + (double)a.y, neary = (double)a.z + (double)a.w;
+        if (nd == 1) {
+          const double2 f0 = cff_to(cff_load(FF[2 * tt]));
+          ox = nx1 * f0.x - ny1 * f0.y + nx1 * nearx + ny1 * neary;
+        } else {
+          const cff nu = cff_split(nx1, ny1), nub = cff_conj(nu);
+          const float slh = (float)s, sll = (float)(s - (double)slh);
+          // S3 = -F'_{q conj(z_j - c)} with c the leaf centre (channel cm holds that density / s)
+          const cff S2 = cff_neg(cff_load(FF[2 * tt + 1]));
+          const cff S3 = cff_neg(cff_scale(cff_load(FF[2 * (2 * NT + tt) + 1]), slh, sll));
+          const cff S1 = cff_load(FF[2 * tt]), S6 = cff_load(FF[2 * (NT + tt)]);
+          const cff zb = cff_split(g.x[i] - c.x, -(g.y[i] - c.y));
+          const cff w = cff_fma(cff_neg(S3), zb, S2);  // conj(z - c) S2 - S3
+          cff tm = cff_zero();
+          tm = cff_fma(tm, nub, cff_conj(w));
+          tm = cff_fma(tm, nu, cff_conj(S1));
+          tm = cff_fma(tm, nub, cff_conj(S6));
+          tm = cff_fma(tm, nu, S1);
+          const double2 t2 = cff_to(tm);
+          ox = 0.25 * t2.x + nearx;
+          oy = 0.25 * t2.y + neary;
+        }
+      } else {
+        using R = decltype(T2{}.x);
+        T2 nu, zb;
+        R sl;
+        if constexpr (NEARP == 1) {
+          const float4 P = g.pf[i];
+          nu = g.nf[i];
+          zb = make_float2((P.x - cen[0]) + (P.z - cen[2]), -((P.y - cen[1]) + (P.w - cen[3])));
+          sl = cen[5];
+        } else {
+          nu = cx<T2>(g.nx[i], g.ny[i]);
+          zb = cx<T2>(g.x[i] - c.x, -(g.y[i] - c.y));
+          sl = (R)s;
+        }
+        if (nd == 1) {
+          const T2 F0 = FF[2 * tt];
+          ox = (double)(nu.x * F0.x - nu.y * F0.y + (nu.x * a.x + nu.y * a.y));
+        } else {
+          const T2 nub = cconj(nu);
+          const T2 S1 = FF[2 * tt], S6 = FF[2 * (NT + tt)];
+          T2 S2 = FF[2 * tt + 1], S3 = FF[2 * (2 * NT + tt) + 1];
+          S2.x = -S2.x;
+          S2.y = -S2.y;
+          S3.x = -sl * S3.x;
+          S3.y = -sl * S3.y;
+          T2 w = cmul(zb, S2);
           w.x -= S3.x;
           w.y -= S3.y;
-          float2 tt = cmul(nub, cconj(w));
-          tt = cadd(tt, cmul(nu, cconj(S1)));
-          tt = cadd(tt, cmul(nub, cconj(S6)));
-          tt = cadd(tt, cmul(nu, S1));
-          oxf = 0.25f * tt.x;
-          oyf = 0.25f * tt.y;
+          T2 tm = cmul(nub, cconj(w));
+          tm = cadd(tm, cmul(nu, cconj(S1)));
+          tm = cadd(tm, cmul(nub, cconj(S6)));
+          tm = cadd(tm, cmul(nu, S1));
+          ox = (double)((R)0.25 * tm.x + a.x);
+          oy = (double)((R)0.25 * tm.y + a.y);
         }
       }
-    }
-    if (NEARP == 0 && act) {
-      const double2 zi = make_double2(g.x[i], g.y[i]);
-      const T2 u = cx<T2>((zi.x - c.x) * inv_s, (zi.y - c.y) * inv_s);
-      using R = decltype(u.x);
-      const R is = (R)inv_s;
-      T2 F[kMaxNd], dF[kMaxNd];
-      for (int d = 0; d < f.nd; ++d) {
-        // Horner for F and F' in u
-        T2 h = sm[d * f.p + f.p - 1], dh = cx<T2>(0.0, 0.0);
-        for (int l = f.p - 2; l >= 0; --l) {
-          dh = cadd(cmul(dh, u), h);
-          h = cadd(cmul(h, u), sm[d * f.p + l]);
-        }
-        F[d] = h;
-        dF[d] = h;
-        dF[d].x = dh.x * is;
-        dF[d].y = dh.y * is;
-      }
-      if constexpr (NEARP == 0) {
-        // near field: 3 x 3 leaves, as Cauchy terms
-        for (int ny = y0; ny <= y1; ++ny) {
-          for (int nx = x0; nx <= x1; ++nx) {
-            const int nl = ny * f.nb + nx;
-            for (int k = f.start[nl]; k < f.start[nl + 1]; ++k) {
-              const int i2 = f.perm[k];
-              if (i2 == i) continue;
-              const double rx = zi.x - g.x[i2], ry = zi.y - g.y[i2];
-              const double inv = 1.0 / (rx * rx + ry * ry);
-              const double2 r1 = make_double2(rx * inv, -ry * inv);  // 1/(z_i - z_j)
-              const double2 r2 = cmul(r1, r1);
-              for (int d = 0; d < f.nd; ++d) {
-                double2 q = f.Q[(long long)i2 * f.nd + (d == f.cm ? 0 : d)];
-                if (d == f.cm)  // leaf-relative moment density q conj(z_j - c)/s
-                  q = cmul(q, make_double2((g.x[i2] - c.x) * inv_s, -(g.y[i2] - c.y) * inv_s));
-                cfma(F[d], q, r1);
-                cfma(dF[d], make_double2(-q.x, -q.y), r2);
-              }
-            }
-          }
-        }
-      }
-      // the kernel's combination of the Cauchy sums, in the expansions' precision
-      // (about the leaf centre its terms do not cancel)
-      if (f.nd == 1) {
-        ox = (double)((R)nx1 * F[0].x - (R)ny1 * F[0].y);
-      } else {
-        const T2 nu = cx<T2>(nx1, ny1), nub = cx<T2>(nx1, -ny1);
-        const R sl = (R)s;
-        // S3 = -F'_{q conj(z_j - c)} with c the leaf centre (channel cm holds that density / s)
-        T2 S2 = dF[0], S3 = dF[2];
-        S2.x = -S2.x;
-        S2.y = -S2.y;
-        S3.x = -sl * S3.x;
-        S3.y = -sl * S3.y;
-        const T2 S1 = F[0], S6 = F[1];
-        const T2 zb = cx<T2>(zi.x - c.x, -(zi.y - c.y));
-        T2 w = cmul(zb, S2);
-        w.x -= S3.x;
-        w.y -= S3.y;
-        T2 tt = cmul(nub, cconj(w));
-        tt = cadd(tt, cmul(nu, cconj(S1)));
-        tt = cadd(tt, cmul(nub, cconj(S6)));
-        tt = cadd(tt, cmul(nu, S1));
-        ox = 0.25 * (double)tt.x;
-        oy = 0.25 * (double)tt.y;
-      }
-    }
-    if constexpr (NEARP != 0) {
-      // near field as the real kernel, sources staged through shared memory
-      float4 tp = make_float4(0.f, 0.f, 0.f, 0.f);
-      float2 tn = make_float2(0.f, 0.f);
-      FFTarget t;
-      if (act) {
-        if (NEARP == 1) {
-          tp = g.pf[i];
-          tn = g.nf[i];
-        } else {
-          const float4 pp = g.xff[i];
-          const float2 pl = g.xfl[i];
-          t.xh = pp.x;
-          t.xm = pp.y;
-          t.yh = pp.z;
-          t.ym = pp.w;
-          t.xl = pl.x;
-          t.yl = pl.y;
-          t.n = g.nff[i];
-        }
-      }
-      float ax = 0.f, ay = 0.f, axh = 0.f, axl = 0.f, ayh = 0.f, ayl = 0.f;
-      if constexpr (NEARP == 1) {
-        // FP32: two sources a packed FP32x2 operation, staged in pairs
-        // (positions hi and lo, strengths, node ids); an odd count is padded
-        // with a zero-strength source far from everything
-        float4* sp2 = spa;                  // [kNearChunk / 2] (xh0, xh1, yh0, yh1)
-        float4* sl2 = spa + kNearChunk / 2;  // [kNearChunk / 2] (xl0, xl1, yl0, yl1)
-        float4* sq2 = sq;                   // [kNearChunk / 2] (q1_0, q1_1, q2_0, q2_1)
-        int2* sid2 = reinterpret_cast<int2*>(sid);
-        const float2 TXH = make_float2(tp.x, tp.x), TYH = make_float2(tp.y, tp.y);
-        const float2 TXL = make_float2(tp.z, tp.z), TYL = make_float2(tp.w, tp.w);
-        const float2 NX = make_float2(tn.x, tn.x), NY = make_float2(tn.y, tn.y);
-        float2 AX = make_float2(0.f, 0.f), AY = AX;
-        for (int v0 = 0; v0 < total; v0 += kNearChunk) {
-          const int m = min(kNearChunk, total - v0), m2 = (m + 1) >> 1;
-          __syncthreads();
-          for (int e2 = threadIdx.x; e2 < m2; e2 += kB) {
-            float4 P[2];
-            float2 q[2];
-            int id[2];
-            for (int h = 0; h < 2; ++h) {
-              const int e = 2 * e2 + h;
-              P[h] = make_float4(1e15f, 1e15f, 0.f, 0.f);
-              q[h] = make_float2(0.f, 0.f);
-              id[h] = -1;
-              if (e < m) {
-                const int vv = v0 + e;
-                int lf = 0;
-                while (vv >= lst[lf + 1]) ++lf;
-                const int i2 = f.perm[lbeg[lf] + (vv - lst[lf])];
-                P[h] = g.pf[i2];
-                q[h] = f.Qf[i2];
-                id[h] = i2;
-              }
-            }
-            sp2[e2] = make_float4(P[0].x, P[1].x, P[0].y, P[1].y);
-            sl2[e2] = make_float4(P[0].z, P[1].z, P[0].w, P[1].w);
-            sq2[e2] = make_float4(q[0].x, q[1].x, q[0].y, q[1].y);
-            sid2[e2] = make_int2(id[0], id[1]);
-          }
-          __syncthreads();
-          if (act) {
-            for (int e2 = 0; e2 < m2; ++e2) {
-              const float4 P = sp2[e2], PL = sl2[e2], Q = sq2[e2];
-              const int2 S = sid2[e2];
-              // exact leading differences, as the scalar pair
-              const float2 dx = __fadd2_rn(__fadd2_rn(TXH, make_float2(-P.x, -P.y)),
-                                           __fadd2_rn(TXL, make_float2(-PL.x, -PL.y)));
-              const float2 dy = __fadd2_rn(__fadd2_rn(TYH, make_float2(-P.z, -P.w)),
-                                           __fadd2_rn(TYL, make_float2(-PL.z, -PL.w)));
-              const float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
-              const float2 inv = make_float2(rcp_approx(r2.x), rcp_approx(r2.y));
-              float2 cc;
-              if (f.nd == 1) {
-                cc = __fmul2_rn(make_float2(Q.x, Q.y), inv);
-              } else {
-                const float2 rq = __ffma2_rn(dx, make_float2(Q.x, Q.y), __fmul2_rn(dy, make_float2(Q.z, Q.w)));
-                const float2 rn = __ffma2_rn(dx, NX, __fmul2_rn(dy, NY));
-                cc = __fmul2_rn(__fmul2_rn(rq, rn), __fmul2_rn(inv, inv));
-              }
-              float2 cx2 = __fmul2_rn(cc, dx), cy2 = __fmul2_rn(cc, dy);
-              if (S.x == i) cx2.x = cy2.x = 0.f;  // the self pair (r = 0)
-              if (S.y == i) cx2.y = cy2.y = 0.f;
-              AX = __fadd2_rn(AX, cx2);
-              AY = __fadd2_rn(AY, cy2);
-            }
-          }
-        }
-        ax = AX.x + AX.y;
-        ay = AY.x + AY.y;
-      } else {
-        // float-float: one source at a time, float-float sums
-        for (int v0 = 0; v0 < total; v0 += kNearChunk) {
-          const int m = min(kNearChunk, total - v0);
-          __syncthreads();
-          for (int e = threadIdx.x; e < m; e += kB) {
-            const int vv = v0 + e;
-            int lf = 0;
-            while (vv >= lst[lf + 1]) ++lf;
-            const int i2 = f.perm[lbeg[lf] + (vv - lst[lf])];
-            sid[e] = i2;
-            const double2 q = f.Q[(long long)i2 * f.nd];
-            spa[e] = g.xff[i2];
-            spb[e] = g.xfl[i2];
-            const float q1h = (float)q.x, q2h = (float)q.y;
-            sq[e] = make_float4(q1h, (float)(q.x - (double)q1h), q2h, (float)(q.y - (double)q2h));
-          }
-          __syncthreads();
-          if (act) {
-            for (int e = 0; e < m; ++e) {
-              if (sid[e] == i) continue;
-              float cxh, cxl, cyh, cyl;
-              if (f.nd == 1)
-                ff_pair<0>(t, spa[e], spb[e], sq[e], cxh, cxl, cyh, cyl);
-              else
-                ff_pair<1>(t, spa[e], spb[e], sq[e], cxh, cxl, cyh, cyl);
-              ff_acc(axh, axl, cxh, cxl);
-              ff_acc(ayh, ayl, cyh, cyl);
-            }
-          }
-        }
-      }
-      if (NEARP == 2) {
-        ax = 0.f;  // unused
-        const double dax = (double)axh + (double)axl, day = (double)ayh + (double)ayl;
-        if (f.nd == 1)
-          ox += nx1 * dax + ny1 * day;
-        else {
-          ox += dax;
-          oy += day;
-        }
-      } else {
-        if (f.nd == 1) {
-          oxf += tn.x * ax + tn.y * ay;
-        } else {
-          oxf += ax;
-          oyf += ay;
-        }
-        ox = (double)oxf;
-        oy = (double)oyf;
-      }
-    }
-    if (act) {
-      if (f.nd == 1) {
+      if (nd == 1) {
         partial[i] = ox;
       } else {
         partial[2 * i] = ox;
         partial[2 * i + 1] = oy;
       }
     }
+    __syncthreads();  // FF and red are written for the next targets
   }
+}
+
+// Dynamic shared memory of an evaluation block.
+template <class T2, int NEARP>
+size_t eval_smem(int nd, int p) {
+  const size_t e = NEARP == 2 ? sizeof(float4) : sizeof(T2);
+  return e * ((size_t)nd * p + 2 * (size_t)nd * kBE * EvalNear<NEARP>::kTPT);
 }
 
 // Output densities at the boundary nodes (v = sqrt(w)-scaled total density):
@@ -1684,7 +1742,6 @@ size_t tree_smem(int nd, int p) {
 template <class T2, int NEARP>
 void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, double* partial, const int* stop, cudaStream_t s) {
   const int p = d.p, nd = d.nd;
-  const size_t sm_exp = (size_t)nd * p * sizeof(T2);
   const size_t sm_p2m = ((size_t)p * (kChunk + 1) + (size_t)kChunk * nd) * sizeof(T2);
   if constexpr (std::is_same<T2, float2>::value)
     k_fmm_p2m32<<<f->nleaf, kB, sm_p2m, s>>>(d, g, stop);
@@ -1711,7 +1768,7 @@ void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, double* partial
   }
   if (!done) launch_m2l(d, f->L, stop, s);
   for (int l = 2; l < f->L; ++l) k_fmm_l2l<T2><<<1 << (2 * (l + 1)), kB, sm_tree, s>>>(d, l, stop);
-  k_fmm_eval<T2, NEARP><<<f->nleaf, kB, sm_exp, s>>>(d, g, partial, stop);
+  k_fmm_eval<T2, NEARP><<<f->nleaf, kBE, eval_smem<T2, NEARP>(nd, p), s>>>(d, g, partial, stop);
 }
 
 }  // namespace
