@@ -457,22 +457,78 @@ __global__ void __launch_bounds__(kB) k_fmm_m2m(FmmDevT<T2> f, int l, const int*
 //   logarithm: T^log_D[l][k] = beta_l(D) P^log[l][k] alpha_k(D) for k >= 1,
 //              P^log[l][k] = C(k+l-1, l),  alpha_k = D^-k / k,  beta_l = -(-1)^l D^-l,
 //              and the a_0 column gamma_l(D) = log D (l = 0), (-1)^(l+1) D^-l / l (l >= 1).
-// P is real and the same for every offset, so a box pair costs 2 p^2 real
-// multiply-adds (the Pascal matrix times a complex vector) and 8 p for the
-// two diagonal scalings, against 4 p^2 for a complex p x p operator.  Cauchy
-// channels carry 1/s; logarithm channels add a_0 log(s) on b_0 (the level's
-// share of log d = log D + log s).
+// P is real and the same for every offset.  Cauchy channels carry 1/s;
+// logarithm channels add a_0 log(s) on b_0 (the level's share of log d = log D +
+// log s).
 //
-// One warp finds the interaction list (at most 27 boxes, in row-major order
-// of the parent's 6 x 6 neighbourhood); the sources' multipoles are staged
-// in shared memory already scaled by alpha, U[q][d][k] (q padded with zeros
-// to a multiple of 4); thread e < p nd computes coefficient l = e % p of
-// channel d = e / p over four sources at a time (four independent chains).
-// PM > 0: the thread's Pascal row is held in registers and U is zero-padded
-// to PM coefficients (p <= PM); PM = 0: the Pascal matrices are read from
-// shared memory, transposed, for any p.
-constexpr int kListPad = 28;  // the 27 interaction-list boxes rounded up to the 4-source step
+// Quarter turns: for D_r = i^r D the factors turn by powers of i, so the up to
+// four sources at D, iD, -D, -iD need one Pascal product instead of four:
+//   sum_r T_{D_r} a^(r) |_l = beta_l(D) sum_k P[l][k] alpha_k(D) A_k^((l + e + k) mod 4),
+//   A_k^(q) = sum_r i^(-rq) a_k^(r)   (e = 1 Cauchy, 0 logarithm),
+// the sources' 4-point transform (additions only), and row l uses the entries of
+// residue l + e + k.  The 27 offsets of an interaction list fall into 10 such
+// orbits (4 whole ones, 5 of two sources, 1 of one), which cuts the p x p products
+// by 2.7.  A product costs 2 p^2 real multiply-adds a channel.
+//
+// A block lists the orbits that have non-empty sources (s_src: four source boxes
+// an orbit), stages alpha_k A_k^(q) of up to nbo orbits in shared memory (U[orbit][channel,
+// k][q]), and thread (split, channel, row) adds NJ of its split's orbits at a
+// time (independent chains); the splits' sums are added in order.
+//
+// Against one product a source (the Pascal row in registers): FP64 Laplace,
+// 160,000 nodes, order 36: 1448 -> 468 us; float-float Stokes, 640,000 nodes, order
+// 36: 4100 -> 2066 us (bound by FP32 issue); FP32 Stokes, order 18: 209 -> 127 us.
 constexpr int kOffs = 49;     // offsets -3..3 x -3..3 (the 3 x 3 near ones unused)
+constexpr int kOrbits = 10;   // orbits of the others under quarter turns
+
+// The orbit of offset (x, y) and the quarter turns r from its representative (x > 0, y >= 0).
+__device__ __forceinline__ void orbit_of(int x, int y, int& id, int& r) {
+  r = 0;
+  while (!(x > 0 && y >= 0)) {  // at most three turns by -i
+    const int t = x;
+    x = y;
+    y = -t;
+    ++r;
+  }
+  id = max(x, y) == 2 ? (x == 2 ? y : 3) : (x == 3 ? 4 + y : (x == 2 ? 8 : 9));
+}
+// Offset of an orbit's representative.
+__device__ __forceinline__ int2 orbit_rep(int id) {
+  if (id < 4) return id < 3 ? make_int2(2, id) : make_int2(1, 2);
+  return id < 8 ? make_int2(3, id - 4) : make_int2(id == 8 ? 2 : 1, 3);
+}
+__device__ __forceinline__ int offset_index(int x, int y) { return (x + 3) + 7 * (y + 3); }
+
+struct OrbitList {
+  int src[kOrbits][4];  // source box (in its level) at i^r D, or -1
+  int id[kOrbits];      // the orbits with a source, in order
+  int cnt;
+};
+
+// The orbits of target box (bx, by) of level l (all threads of the block call).
+template <class T2>
+__device__ __forceinline__ void list_orbits(const FmmDevT<T2>& f, int l, int bx, int by, OrbitList& o) {
+  const int n = 1 << l, px = bx >> 1, py = by >> 1;
+  for (int c = threadIdx.x; c < 4 * kOrbits; c += blockDim.x) (&o.src[0][0])[c] = -1;
+  __syncthreads();
+  for (int c = threadIdx.x; c < 36; c += blockDim.x) {
+    const int sx = 2 * px - 2 + c % 6, sy = 2 * py - 2 + c / 6;
+    if (sx < 0 || sy < 0 || sx >= n || sy >= n || (abs(sx - bx) <= 1 && abs(sy - by) <= 1)) continue;
+    if (f.count[lev_off(l) + (long long)sy * n + sx] == 0) continue;
+    int id, r;
+    orbit_of(bx - sx, by - sy, id, r);
+    o.src[id][r] = sy * n + sx;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const int t = threadIdx.x;
+    const bool any = t < kOrbits && (o.src[t][0] >= 0 || o.src[t][1] >= 0 || o.src[t][2] >= 0 || o.src[t][3] >= 0);
+    const unsigned m = __ballot_sync(0xffffffffu, any);
+    if (any) o.id[__popc(m & ((1u << t) - 1u))] = t;
+    if (t == 0) o.cnt = __popc(m);
+  }
+  __syncthreads();
+}
 
 // Layout of the operator table of order p (complex entries): M2M and L2L
 // matrices [op][in][out], then the M2L factors alpha[2][49][p], beta[2][49][p],
@@ -485,150 +541,300 @@ __host__ __device__ inline long long tab_pascal(int p) { return tab_gamma(p) + (
 __host__ __device__ inline long long tab_size(int p) { return tab_pascal(p) + 2LL * p * p; }
 
 // w += (pp.x u.x, pp.y u.y): a real factor (duplicated in pp) times a complex value
-__device__ __forceinline__ void rfma(float2& w, float2 pp, float2 u) { w = __ffma2_rn(pp, u, w); }
 __device__ __forceinline__ void rfma(double2& w, double2 pp, double2 u) {
   w.x = fma(pp.x, u.x, w.x);
   w.y = fma(pp.y, u.y, w.y);
 }
 
-template <class T2, int PM>
-__global__ void __launch_bounds__(256) k_fmm_m2l(FmmDevT<T2> f, const int* stop) {
+// alpha_k A_k^(q), q = 0..3, of orbit id for (channel d, coefficient k): the four
+// sources' coefficients (moment channel: relative to the target centre, rho_S -
+// conj(D_r) rho_0), their 4-point transform, times alpha.
+template <class T2>
+__device__ __forceinline__ void orbit_stage(const FmmDevT<T2>& f, const OrbitList& o, int id, int l, int d, int k,
+                                            const T2* __restrict__ al, T2* __restrict__ out, T2* __restrict__ a0) {
+  const int p = f.p, nd = f.nd;
+  const int2 D = orbit_rep(id);
+  int x = D.x, y = D.y;
+  T2 v[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    v[r] = cx<T2>(0.0, 0.0);
+    if (o.src[id][r] >= 0) {
+      const T2* a = f.mp + (lev_off(l) + o.src[id][r]) * nd * p;
+      v[r] = a[d * p + k];
+      if (d == f.cm) cfma(v[r], cx<T2>((double)-x, (double)y), a[k]);
+    }
+    const int t = x;  // the next turn by i
+    x = -y;
+    y = t;
+  }
+  const T2 t0 = cadd(v[0], v[2]), t2 = cadd(v[1], v[3]);
+  T2 t1 = v[0], t3 = v[1];
+  t1.x -= v[2].x;
+  t1.y -= v[2].y;
+  t3.x -= v[3].x;
+  t3.y -= v[3].y;
+  T2 A[4];
+  A[0] = cadd(t0, t2);
+  A[1] = t1;  // t1 - i t3
+  A[1].x += t3.y;
+  A[1].y -= t3.x;
+  A[2] = t0;
+  A[2].x -= t2.x;
+  A[2].y -= t2.y;
+  A[3] = t1;  // t1 + i t3
+  A[3].x -= t3.y;
+  A[3].y += t3.x;
+  if (a0)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a0[q] = A[q];
+  const T2 w = al[(long long)offset_index(D.x, D.y) * p];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) out[q] = cmul(w, A[q]);
+}
+
+// FP64.  Threads: split x (channel, row).
+template <class T2, int NJ>
+__global__ void __launch_bounds__(256) k_fmm_m2l(FmmDevT<T2> f, int nsplit, int nbo, const int* stop) {
   using R = decltype(T2{}.x);
   if (stop && *stop) return;
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ int s_src[kListPad];
-  __shared__ int s_off[kListPad];
-  __shared__ T2 s_a0[kListPad][kMaxNd];  // raw a_0 of the logarithm channels
-  __shared__ int s_cnt;
+  __shared__ OrbitList o;
+  __shared__ T2 s_a0[kOrbits][kMaxNd][4];  // the transforms of a_0 of the logarithm channels
+  __shared__ T2 red[256];
   long long gb = blockIdx.x + lev_off(2);
   int l = 2;
   while (l < f.L && gb >= lev_off(l + 1)) ++l;
   if (f.tcount[gb] == 0) return;
-  const int p = f.p, nd = f.nd, pk = PM > 0 ? PM : p;
-  const int n = 1 << l;
-  const int b = (int)(gb - lev_off(l)), bx = b % n, by = b / n;
-  const int px = bx >> 1, py = by >> 1;
+  const int p = f.p, nd = f.nd, per = nd * p;
+  const int b = (int)(gb - lev_off(l)), bx = b & ((1 << l) - 1), by = b >> l;
   const int tid = threadIdx.x;
-  if (tid < 32) {
-    int base = 0;
-    for (int r = 0; r < 2; ++r) {
-      const int c = r * 32 + tid;
-      const int sx = 2 * px - 2 + c % 6, sy = 2 * py - 2 + c / 6;
-      bool ok = c < 36 && sx >= 0 && sy >= 0 && sx < n && sy < n && !(abs(sx - bx) <= 1 && abs(sy - by) <= 1);
-      const long long src = lev_off(l) + (long long)sy * n + sx;
-      if (ok) ok = f.count[src] != 0;
-      const unsigned m = __ballot_sync(0xffffffffu, ok);
-      if (ok) {
-        const int pos = base + __popc(m & ((1u << tid) - 1u));
-        s_src[pos] = sy * n + sx;
-        s_off[pos] = (bx - sx + 3) + 7 * (by - sy + 3);
-      }
-      base += __popc(m);
-    }
-    if (tid == 0) s_cnt = base;
-  }
-  __syncthreads();
-  const int cnt = s_cnt, cnt4 = (cnt + 3) & ~3;
-  T2* U = reinterpret_cast<T2*>(smraw);  // [cnt4][nd][pk]
-  R* Pt = reinterpret_cast<R*>(U + (long long)kListPad * nd * pk);  // PM = 0: [type][k][l]
+  list_orbits(f, l, bx, by, o);
+  T2* U = reinterpret_cast<T2*>(smraw);               // [nbo][nd p][4]
+  R* Pt = reinterpret_cast<R*>(U + (long long)nbo * per * 4);  // [type][k][l]
   const T2* alpha = f.ops + tab_alpha(p);
   const T2* beta = f.ops + tab_beta(p);
   const T2* gamma = f.ops + tab_gamma(p);
   const T2* pas = f.ops + tab_pascal(p);
   const int ntype = f.nlog > 0 ? 2 : 1;
-  if (PM == 0)
-    for (int e = tid; e < ntype * p * p; e += blockDim.x) {
-      const int t = e / (p * p), r = e % (p * p);
-      Pt[e] = pas[(long long)(f.nlog > 0 ? t : 0) * p * p + r].x;
+  for (int e = tid; e < ntype * p * p; e += blockDim.x) Pt[e] = pas[e].x;
+  const int sp = tid / per, e = tid - sp * per, d = e / p, t = e - d * p;
+  const bool act = sp < nsplit;
+  const int ty = d < f.nlog ? 1 : 0;
+  const int base = t + 1 - ty;  // the residue of the entry at k: (base + k) mod 4
+  T2 acc = cx<T2>(0.0, 0.0);
+  for (int o0 = 0; o0 < o.cnt; o0 += nbo) {
+    const int no = min(nbo, o.cnt - o0);
+    __syncthreads();
+    for (int q = tid; q < no * per; q += blockDim.x) {
+      const int oo = q / per, dk = q - oo * per, dd = dk / p, k = dk - dd * p;
+      const int tt = dd < f.nlog ? 1 : 0;
+      orbit_stage(f, o, o.id[o0 + oo], l, dd, k, alpha + (long long)tt * kOffs * p + k, U + 4LL * q,
+                  tt == 1 && k == 0 ? s_a0[o0 + oo][dd] : (T2*)nullptr);
     }
-  const int per = nd * pk;
-  // a thread keeps its (channel, coefficient) and walks the sources
-  for (int dk = tid; dk < per; dk += blockDim.x) {
-    const int d = dk / pk, k = dk % pk;
-    const int ty = d < f.nlog ? 1 : 0;
-    const T2* al = alpha + (long long)ty * kOffs * p + k;
-#pragma unroll 4
-    for (int q = 0; q < cnt4; ++q) {
-      T2 u = cx<T2>(0.0, 0.0);
-      if (q < cnt && k < p) {
-        const T2* a = f.mp + ((lev_off(l) + s_src[q]) * nd) * p;
-        const int oi = s_off[q];
-        T2 v = a[d * p + k];
-        if (d == f.cm) {
-          // source moment density relative to the target centre: rho_S - conj(D) rho_0
-          cfma(v, cx<T2>((double)(3 - oi % 7), (double)(oi / 7 - 3)), a[k]);
-        }
-        if (ty == 1 && k == 0) s_a0[q][d] = v;
-        u = cmul(al[(long long)oi * p], v);
+    __syncthreads();
+    if (!act) continue;
+    for (int q0 = sp; q0 < no; q0 += NJ * nsplit) {
+      T2 w[NJ];
+      const T2* u[NJ];
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        w[j] = cx<T2>(0.0, 0.0);
+        u[j] = U + (long long)min(q0 + j * nsplit, no - 1) * per * 4 + d * p * 4;
       }
-      U[q * per + dk] = u;
-    }
-  }
-  __syncthreads();
-  const double inv_s = ldexp(f.Dinv, l);
-  for (int e = tid; e < nd * p; e += blockDim.x) {
-    const int d = e / p, t = e % p;
-    const int ty = d < f.nlog ? 1 : 0;
-    const int tp = f.nlog > 0 ? ty : 0;  // Pascal slot of this channel
-    // log s (s = D 2^-l), on b_0 of the logarithm channels only
-    const R logs = (ty == 1 && t == 0) ? (R)(log(f.D) - l * 0.69314718055994530942) : (R)0;
-    T2 prow[PM > 0 ? PM : 1];
-    if (PM > 0) {
+      const R* pt = Pt + (long long)ty * p * p + t;
+      for (int k = 0; k < p; ++k) {
+        const R pv = pt[(long long)k * p];
+        const T2 pp = cx<T2>((double)pv, (double)pv);
+        const int at = 4 * k + ((base + k) & 3);
 #pragma unroll
-      for (int k = 0; k < (PM > 0 ? PM : 1); ++k) {
-        const R v = k < p ? pas[((long long)ty * p + k) * p + t].x : (R)0;
-        prow[k] = cx<T2>((double)v, (double)v);
-      }
-    }
-    T2 acc = cx<T2>(0.0, 0.0);
-    for (int q0 = 0; q0 < cnt; q0 += 4) {
-      T2 w[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = cx<T2>(0.0, 0.0);
-      const T2* u = U + ((long long)q0 * nd + d) * pk;
-      if (PM > 0) {
-#pragma unroll
-        for (int k = 0; k < (PM > 0 ? PM : 1); ++k)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) rfma(w[j], prow[k], u[(long long)j * per + k]);
-      } else {
-        const R* pt = Pt + (long long)tp * p * p + t;
-        for (int k = 0; k < p; ++k) {
-          const R pv = pt[(long long)k * p];
-          const T2 pp = cx<T2>((double)pv, (double)pv);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) rfma(w[j], pp, u[(long long)j * per + k]);
-        }
+        for (int j = 0; j < NJ; ++j) rfma(w[j], pp, u[j][at]);
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (q0 + j < cnt) {
-          const int oi = s_off[q0 + j];
+      for (int j = 0; j < NJ; ++j) {
+        const int q = q0 + j * nsplit;
+        if (q < no) {
+          const int id = o.id[o0 + q];
+          const int2 D = orbit_rep(id);
+          const int oi = offset_index(D.x, D.y);
           cfma(acc, beta[((long long)ty * kOffs + oi) * p + t], w[j]);
-          if (ty == 1) {
-            T2 gm = gamma[(long long)oi * p + t];
-            if (t == 0) gm.x += logs;
-            cfma(acc, gm, s_a0[q0 + j][d]);
+          if (ty == 1 && t > 0) cfma(acc, gamma[(long long)oi * p + t], s_a0[o0 + q][d][t & 3]);
+          if (ty == 1 && t == 0) {
+            // a_0 (log D_r + log s) per source, s = D 2^-l
+            const R logs = (R)(log(f.D) - l * 0.69314718055994530942);
+            int x = D.x, y = D.y;
+            for (int r = 0; r < 4; ++r) {
+              if (o.src[id][r] >= 0) {
+                T2 gm = gamma[(long long)offset_index(x, y) * p];
+                gm.x += logs;
+                cfma(acc, gm, f.mp[((lev_off(l) + o.src[id][r]) * nd + d) * p]);
+              }
+              const int z = x;
+              x = -y;
+              y = z;
+            }
           }
         }
       }
     }
+  }
+  red[tid] = acc;
+  __syncthreads();
+  if (sp == 0) {
+    for (int q = 1; q < nsplit; ++q) acc = cadd(acc, red[q * per + e]);
     // Cauchy channels carry 1/s; in the precision of the expansions
-    const R sc = ty == 1 ? (R)1 : (R)inv_s;
+    const R sc = ty == 1 ? (R)1 : (R)ldexp(f.Dinv, l);
     acc.x *= sc;
     acc.y *= sc;
-    f.lc[(gb * nd + d) * p + t] = acc;
+    f.lc[gb * per + e] = acc;
   }
 }
 
-// Shared memory of one M2L block: the staged sources and, for PM = 0, the
-// transposed Pascal matrices.
-template <class T2>
-size_t m2l_smem(int p, int nd, int nlog, int pm) {
-  const int pk = pm > 0 ? pm : p;
-  size_t b = (size_t)kListPad * nd * pk * sizeof(T2);
-  if (pm == 0) b += (size_t)(nlog > 0 ? 2 : 1) * p * p * sizeof(decltype(T2{}.x));
-  return b;
+// FP32, Cauchy channels (the inner solves' operator), ND channels of order p <= PK
+// (coefficients padded with zeros to the instance's order).  Bound by instruction
+// issue (71%), so the work around the multiply-adds is what counts:
+// - a thread takes two rows of one residue, l and l + 4: both use the same staged
+//   entries, so that a load feeds four multiply-adds; their Pascal entries come in
+//   pairs from a table of that layout (fmm_setup);
+// - all ten orbits are staged, in one pass in which a thread forms one coefficient
+//   of all channels (12 loads in flight for three), empty sources as zeros: the
+//   moment channel's shift is one multiply-add a transform instead of one a source;
+// - sizes and strides are compile-time constants (run-time ones: 241 us in place of 127).
+__host__ __device__ constexpr int m2l32_rp(int pk) { return (pk + 7) / 8; }  // row pairs of one residue
+// the instance of an order
+__host__ __device__ constexpr int m2l32_pad(int p) {
+  return p <= 12 ? 12 : p <= 16 ? 16 : p <= 20 ? 20 : p <= 24 ? 24 : p <= 32 ? 32 : p <= 48 ? 48 : 64;
+}
+
+__host__ __device__ constexpr int m2l32_splits(int nd, int pk) {
+  return 5 * nd * 4 * m2l32_rp(pk) <= 256 ? 5 : (2 * nd * 4 * m2l32_rp(pk) <= 256 ? 2 : 1);
+}
+__host__ __device__ constexpr int m2l32_threads(int nd, int pk) {
+  return (m2l32_splits(nd, pk) * nd * 4 * m2l32_rp(pk) + 31) / 32 * 32;
+}
+
+template <int ND, int PK>
+__global__ void __launch_bounds__(m2l32_threads(ND, PK)) k_fmm_m2l32(FmmDevT<float2> f, const float2* __restrict__ ptab,
+                                                                    const int* stop) {
+  if (stop && *stop) return;
+  constexpr int RP = m2l32_rp(PK), SP = m2l32_splits(ND, PK), B = m2l32_threads(ND, PK);
+  constexpr int HALF = ND * 4 * RP, NJ = 2;  // (channel, residue, pair) threads; orbits added at a time
+  constexpr int DS = 4 * PK + 4, US = ND * DS;  // channel and orbit strides: distinct banks
+  extern __shared__ __align__(16) float2 U[];   // [orbit][channel][k][4]
+  __shared__ int s_at[kOrbits * 4];             // the sources' first coefficients, or -1
+  __shared__ float4 red[B];
+  long long gb = blockIdx.x + lev_off(2);
+  int l = 2;
+  while (l < f.L && gb >= lev_off(l + 1)) ++l;
+  const int targets = f.tcount[gb];
+  const int p = f.p, n = 1 << l, tid = threadIdx.x;
+  {
+    const int b = (int)(gb - lev_off(l)), bx = b & (n - 1), by = b >> l;
+    for (int t = tid; t < 4 * kOrbits; t += B) {
+      const int2 D = orbit_rep(t >> 2);
+      const int r = t & 3, dx = r == 0 ? D.x : r == 1 ? -D.y : r == 2 ? -D.x : D.y;
+      const int dy = r == 0 ? D.y : r == 1 ? D.x : r == 2 ? -D.y : -D.x;
+      const int sx = bx - dx, sy = by - dy;  // a child of the parent's neighbours, in the level
+      const bool in = sx >= 0 && sy >= 0 && sx < n && sy < n && abs((sx >> 1) - (bx >> 1)) <= 1 &&
+                      abs((sy >> 1) - (by >> 1)) <= 1;
+      s_at[t] = in && f.count[lev_off(l) + (long long)sy * n + sx] > 0 ? (sy * n + sx) * (ND * p) : -1;
+    }
+  }
+  if (targets == 0) return;
+  __syncthreads();
+  const float2* __restrict__ mp = f.mp + lev_off(l) * ND * p;
+  for (int w = tid; w < kOrbits * p; w += B) {
+    const int oo = w / p, k = w - oo * p;
+    const int2 D = orbit_rep(oo);
+    const float2 w4 = __ldg(f.ops + tab_alpha(p) + offset_index(D.x, D.y) * p + k);
+    float2 A[ND][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int at = s_at[4 * oo + r];
+#pragma unroll
+      for (int d = 0; d < ND; ++d) A[d][r] = at >= 0 ? mp[at + d * p + k] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      const float2 t0 = cadd(A[d][0], A[d][2]), t2 = cadd(A[d][1], A[d][3]);
+      const float2 t1 = make_float2(A[d][0].x - A[d][2].x, A[d][0].y - A[d][2].y);
+      const float2 t3 = make_float2(A[d][1].x - A[d][3].x, A[d][1].y - A[d][3].y);
+      A[d][0] = cadd(t0, t2);
+      A[d][1] = make_float2(t1.x + t3.y, t1.y - t3.x);
+      A[d][2] = make_float2(t0.x - t2.x, t0.y - t2.y);
+      A[d][3] = make_float2(t1.x - t3.y, t1.y + t3.x);
+    }
+    if (ND == 3) {
+      // moment channel, relative to the target centre: rho_r - conj(i^r D) a_r, whose
+      // transform is that of rho less conj(D) times that of a, one place on
+      const float2 c = make_float2(-(float)D.x, (float)D.y);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cfma(A[ND - 1][q], c, A[0][(q + 1) & 3]);
+    }
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      float4* u4 = reinterpret_cast<float4*>(U + oo * US + d * DS + 4 * k);
+      const float2 a0 = cmul(w4, A[d][0]), a1 = cmul(w4, A[d][1]), a2 = cmul(w4, A[d][2]), a3 = cmul(w4, A[d][3]);
+      u4[0] = make_float4(a0.x, a0.y, a1.x, a1.y);
+      u4[1] = make_float4(a2.x, a2.y, a3.x, a3.y);
+    }
+  }
+  for (int w = tid; w < 2 * kOrbits * ND * (PK - p); w += B)  // the padding
+    reinterpret_cast<float4*>(U + (w / (2 * (PK - p))) * DS + 4 * p)[w % (2 * (PK - p))] = make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
+  // thread (split, channel, residue, pair): rows t0 = residue + 8 pair and t0 + 4
+  const int sp = tid / HALF, e = tid % HALF, d = e / (4 * RP), mr = e % (4 * RP), m = mr / RP;
+  const int t0 = m + 8 * (mr % RP), t1 = t0 + 4;
+  const bool act = sp < SP && t0 < p;
+  float2 acc0 = make_float2(0.f, 0.f), acc1 = acc0;
+  if (act) {
+    const int rot[4] = {(m + 1) & 3, (m + 2) & 3, (m + 3) & 3, m & 3};
+    const float2* __restrict__ beta = f.ops + tab_beta(p) + t0;
+#pragma unroll 1
+    for (int q0 = sp; q0 < kOrbits; q0 += NJ * SP) {
+      const int q1 = min(q0 + SP, kOrbits - 1);
+      const int2 Da = orbit_rep(q0), Db = orbit_rep(q1);
+      const float2* __restrict__ be = beta + offset_index(Da.x, Da.y) * p;
+      const float2* __restrict__ bf = beta + offset_index(Db.x, Db.y) * p;
+      const float2 z = make_float2(0.f, 0.f);
+      const float2 be0 = __ldg(be), be1 = t1 < p ? __ldg(be + 4) : z;
+      const float2 bf0 = q0 + SP < kOrbits ? __ldg(bf) : z, bf1 = t1 < p && q0 + SP < kOrbits ? __ldg(bf + 4) : z;
+      const float2* ua = U + q0 * US + d * DS;
+      const float2* ub = U + q1 * US + d * DS;
+      float2 a0 = z, a1 = z, b0 = z, b1 = z;
+      const float2* __restrict__ pt = ptab + mr;
+#pragma unroll
+      for (int k = 0; k < PK; ++k) {
+        const float2 P = __ldg(pt + k * 4 * RP);
+        const float2 va = ua[4 * k + rot[k & 3]], vb = ub[4 * k + rot[k & 3]];
+        a0.x = fmaf(P.x, va.x, a0.x);
+        a0.y = fmaf(P.x, va.y, a0.y);
+        a1.x = fmaf(P.y, va.x, a1.x);
+        a1.y = fmaf(P.y, va.y, a1.y);
+        b0.x = fmaf(P.x, vb.x, b0.x);
+        b0.y = fmaf(P.x, vb.y, b0.y);
+        b1.x = fmaf(P.y, vb.x, b1.x);
+        b1.y = fmaf(P.y, vb.y, b1.y);
+      }
+      cfma(acc0, be0, a0);
+      cfma(acc1, be1, a1);
+      cfma(acc0, bf0, b0);
+      cfma(acc1, bf1, b1);
+    }
+  }
+  red[tid] = make_float4(acc0.x, acc0.y, acc1.x, acc1.y);
+  __syncthreads();
+  if (sp == 0 && act) {
+#pragma unroll
+    for (int q = 1; q < SP; ++q) {
+      const float4 r = red[q * HALF + e];
+      acc0 = cadd(acc0, make_float2(r.x, r.y));
+      acc1 = cadd(acc1, make_float2(r.z, r.w));
+    }
+    const float sc = (float)ldexp(f.Dinv, l);  // Cauchy channels carry 1/s
+    f.lc[(gb * ND + d) * p + t0] = make_float2(acc0.x * sc, acc0.y * sc);
+    if (t1 < p) f.lc[(gb * ND + d) * p + t1] = make_float2(acc1.x * sc, acc1.y * sc);
+  }
 }
 
 // ---- float-float M2L: the residual operator of the float-float refinement ----
@@ -707,6 +913,16 @@ __device__ __forceinline__ cff cff_fma(cff acc, cff a, cff b) {
   ff_cfma(acc.h, acc.l, a.h, a.l, b.h, b.l);
   return acc;
 }
+// a b
+__device__ __forceinline__ cff cff_mul(cff a, cff b) {
+  cff x, y;
+  // (a_re b_re, a_re b_im) + (-a_im b_im, a_im b_re)
+  ff_mul2(make_float2(a.h.x, a.h.x), make_float2(a.l.x, a.l.x), b.h, b.l, x.h, x.l);
+  ff_mul2(make_float2(a.h.y, a.h.y), make_float2(a.l.y, a.l.y), make_float2(-b.h.y, b.h.x), make_float2(-b.l.y, b.l.x),
+          y.h, y.l);
+  ff_acc2(x.h, x.l, y.h, y.l);
+  return x;
+}
 // a (sh + sl), a real float-float factor
 __device__ __forceinline__ cff cff_scale(cff a, float sh, float sl) {
   cff r;
@@ -746,13 +962,13 @@ __global__ void __launch_bounds__(kB) k_fmm_p2m_ff(FmmDevT<double2> f, Geo g, co
       cff w = cff_split(1.0, 0.0);
       for (int k = 0; k < f.p; ++k) {
         pw[k * (kChunk + 1) + t] = cff_store(w);
-        w = cff_fma(cff_zero(), w, U);
+        w = cff_mul(w, U);
       }
       for (int d = 0; d < f.nd; ++d) {
         // channel cm: q_0 conj(u), the leaf-relative moment density
         const double2 q = f.Q[(long long)i * f.nd + (d == f.cm ? 0 : d)];
         const cff qd = cff_split(q.x, q.y);
-        qs[t * f.nd + d] = cff_store(d == f.cm ? cff_fma(cff_zero(), qd, cff_conj(U)) : qd);
+        qs[t * f.nd + d] = cff_store(d == f.cm ? cff_mul(qd, cff_conj(U)) : qd);
       }
     }
     __syncthreads();
@@ -782,128 +998,138 @@ __host__ __device__ inline long long fftab_gamma(int p) { return 4LL * kOffs * p
 __host__ __device__ inline long long fftab_pascal(int p) { return 5LL * kOffs * p; }  // in float4 units
 __host__ __device__ inline long long fftab_floats(int p) { return 20LL * kOffs * p + 4LL * p * p; }
 
-constexpr int kBFF = 128;
+// Quarter turn by -i of a complex float-float value (exact).
+__device__ __forceinline__ cff cff_turn(cff a) {
+  return cff{make_float2(a.h.y, -a.h.x), make_float2(a.l.y, -a.l.x)};
+}
+__device__ __forceinline__ cff cff_add(cff a, cff b) {
+  ff_acc2(a.h, a.l, b.h, b.l);
+  return a;
+}
 
-__global__ void __launch_bounds__(kBFF) k_fmm_m2l_ff(FmmDev f, const float4* __restrict__ mpff,
-                                                     const float* __restrict__ tab, const int* stop) {
+// Threads: split x (channel, row); orbits as in k_fmm_m2l.
+template <int NJ>
+__global__ void __launch_bounds__(256) k_fmm_m2l_ff(FmmDev f, const float4* __restrict__ mpff,
+                                                    const float* __restrict__ tab, int nsplit, int nbo,
+                                                    const int* stop) {
   if (stop && *stop) return;
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ int s_src[kListPad];
-  __shared__ int s_off[kListPad];
-  __shared__ float4 s_a0[kListPad][kMaxNd];  // a_0 of the logarithm channels
-  __shared__ int s_cnt;
+  __shared__ OrbitList o;
+  __shared__ float4 s_a0[kOrbits][kMaxNd][4];  // the transforms of a_0 of the logarithm channels
+  __shared__ float4 red[256];
   long long gb = blockIdx.x + lev_off(2);
   int l = 2;
   while (l < f.L && gb >= lev_off(l + 1)) ++l;
   if (f.tcount[gb] == 0) return;
-  const int p = f.p, nd = f.nd;
-  const int n = 1 << l;
-  const int b = (int)(gb - lev_off(l)), bx = b % n, by = b / n;
-  const int px = bx >> 1, py = by >> 1;
+  const int p = f.p, nd = f.nd, per = nd * p;
+  const int b = (int)(gb - lev_off(l)), bx = b & ((1 << l) - 1), by = b >> l;
   const int tid = threadIdx.x;
-  if (tid < 32) {
-    int base = 0;
-    for (int r = 0; r < 2; ++r) {
-      const int c = r * 32 + tid;
-      const int sx = 2 * px - 2 + c % 6, sy = 2 * py - 2 + c / 6;
-      bool ok = c < 36 && sx >= 0 && sy >= 0 && sx < n && sy < n && !(abs(sx - bx) <= 1 && abs(sy - by) <= 1);
-      const long long src = lev_off(l) + (long long)sy * n + sx;
-      if (ok) ok = f.count[src] != 0;
-      const unsigned m = __ballot_sync(0xffffffffu, ok);
-      if (ok) {
-        const int pos = base + __popc(m & ((1u << tid) - 1u));
-        s_src[pos] = sy * n + sx;
-        s_off[pos] = (bx - sx + 3) + 7 * (by - sy + 3);
-      }
-      base += __popc(m);
-    }
-    if (tid == 0) s_cnt = base;
-  }
-  __syncthreads();
-  const int cnt = s_cnt, cnt4 = (cnt + 3) & ~3;
-  float4* U = reinterpret_cast<float4*>(smraw);  // [cnt4][nd][p]
+  list_orbits(f, l, bx, by, o);
+  float4* U = reinterpret_cast<float4*>(smraw);  // [nbo][nd p][4]
   const float4* alpha = reinterpret_cast<const float4*>(tab);
   const float4* beta = alpha + fftab_beta(p);
   const float4* gamma = alpha + fftab_gamma(p);
   const float2* pas = reinterpret_cast<const float2*>(alpha + fftab_pascal(p));
-  const int per = nd * p;
-  // a thread keeps its (channel, coefficient) and walks the sources
-  for (int dk = tid; dk < per; dk += blockDim.x) {
-    const int d = dk / p, k = dk % p;
-    const int ty = d < f.nlog ? 1 : 0;
-    const float4* alk = alpha + (long long)ty * kOffs * p + k;
-#pragma unroll 2
-    for (int q = 0; q < cnt4; ++q) {
-      float2 uh = make_float2(0.f, 0.f), ul = uh;
-      if (q < cnt) {
-        const float4* a = mpff + ((lev_off(l) + s_src[q]) * nd) * p;
-        const int oi = s_off[q];
-        const float4 v = a[d * p + k];
-        float2 vh = make_float2(v.x, v.y), vl = make_float2(v.z, v.w);
-        if (d == f.cm) {
-          // source moment density relative to the target centre: rho_S - conj(D) rho_0
-          const float4 a0 = a[k];
-          ff_cfma(vh, vl, make_float2((float)(3 - oi % 7), (float)(oi / 7 - 3)), make_float2(0.f, 0.f),
-                  make_float2(a0.x, a0.y), make_float2(a0.z, a0.w));
-        }
-        if (ty == 1 && k == 0) s_a0[q][d] = make_float4(vh.x, vh.y, vl.x, vl.y);
-        const float4 al = alk[(long long)oi * p];
-        ff_cfma(uh, ul, make_float2(al.x, al.y), make_float2(al.z, al.w), vh, vl);
-      }
-      U[q * per + dk] = make_float4(uh.x, uh.y, ul.x, ul.y);
-    }
-  }
-  __syncthreads();
-  const double inv_s = ldexp(f.Dinv, l);
-  for (int e = tid; e < per; e += blockDim.x) {
-    const int d = e / p, t = e % p;
-    const int ty = d < f.nlog ? 1 : 0;
-    // log s (s = D 2^-l) on b_0 of the logarithm channels, split hi + lo
-    float lsh = 0.f, lsl = 0.f;
-    if (ty == 1 && t == 0) {
-      const double ls = log(f.D) - l * 0.69314718055994530942;
-      lsh = (float)ls;
-      lsl = (float)(ls - (double)lsh);
-    }
-    const float2* pcol = pas + (long long)ty * p * p + t;
-    float2 ah = make_float2(0.f, 0.f), al = ah;
-    for (int q0 = 0; q0 < cnt; q0 += 4) {
-      float2 sh[4], sl[4];
+  const int sp = tid / per, e = tid - sp * per, d = e / p, t = e - d * p;
+  const bool act = sp < nsplit;
+  const int ty = d < f.nlog ? 1 : 0;
+  const int base = t + 1 - ty;
+  cff acc = cff_zero();
+  for (int o0 = 0; o0 < o.cnt; o0 += nbo) {
+    const int no = min(nbo, o.cnt - o0);
+    __syncthreads();
+    for (int q = tid; q < no * per; q += blockDim.x) {
+      const int oo = q / per, dk = q - oo * per, dd = dk / p, k = dk - dd * p;
+      const int tt = dd < f.nlog ? 1 : 0, id = o.id[o0 + oo];
+      const int2 D = orbit_rep(id);
+      int x = D.x, y = D.y;
+      cff v[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) sh[j] = sl[j] = make_float2(0.f, 0.f);
-      const float4* u = U + (long long)q0 * per + d * p;
+      for (int r = 0; r < 4; ++r) {
+        v[r] = cff_zero();
+        if (o.src[id][r] >= 0) {
+          const float4* a = mpff + (lev_off(l) + o.src[id][r]) * nd * p;
+          v[r] = cff_load(a[dd * p + k]);
+          // source moment density relative to the target centre: rho_S - conj(D_r) rho_0
+          if (dd == f.cm)
+            v[r] = cff_fma(v[r], cff{make_float2((float)-x, (float)y), make_float2(0.f, 0.f)}, cff_load(a[k]));
+        }
+        const int z = x;
+        x = -y;
+        y = z;
+      }
+      const cff t0 = cff_add(v[0], v[2]), t1 = cff_add(v[0], cff_neg(v[2]));
+      const cff t2 = cff_add(v[1], v[3]), t3 = cff_turn(cff_add(v[1], cff_neg(v[3])));  // -i (a1 - a3)
+      cff A[4];
+      A[0] = cff_add(t0, t2);
+      A[1] = cff_add(t1, t3);
+      A[2] = cff_add(t0, cff_neg(t2));
+      A[3] = cff_add(t1, cff_neg(t3));
+      if (tt == 1 && k == 0)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s_a0[o0 + oo][dd][r] = cff_store(A[r]);
+      const cff al = cff_load(alpha[((long long)tt * kOffs + offset_index(D.x, D.y)) * p + k]);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) U[4 * q + r] = cff_store(cff_mul(al, A[r]));
+    }
+    __syncthreads();
+    if (!act) continue;
+    const float2* pcol = pas + (long long)ty * p * p + t;
+    for (int q0 = sp; q0 < no; q0 += NJ * nsplit) {
+      float2 sh[NJ], sl[NJ];
+      const float4* u[NJ];
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        sh[j] = sl[j] = make_float2(0.f, 0.f);
+        u[j] = U + (long long)(min(q0 + j * nsplit, no - 1) * per + d * p) * 4;
+      }
       for (int k = 0; k < p; ++k) {
         const float2 pv = __ldg(pcol + (long long)k * p);
         const float2 PH = make_float2(pv.x, pv.x), PL = make_float2(pv.y, pv.y);
+        const int at = 4 * k + ((base + k) & 3);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float4 uv = u[(long long)j * per + k];
+        for (int j = 0; j < NJ; ++j) {
+          const float4 uv = u[j][at];
           float2 ph, pl;
           ff_mul2(PH, PL, make_float2(uv.x, uv.y), make_float2(uv.z, uv.w), ph, pl);
           ff_acc2(sh[j], sl[j], ph, pl);
         }
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (q0 + j < cnt) {
-          const int oi = s_off[q0 + j];
-          const float4 be = beta[((long long)ty * kOffs + oi) * p + t];
-          ff_cfma(ah, al, make_float2(be.x, be.y), make_float2(be.z, be.w), sh[j], sl[j]);
-          if (ty == 1) {
-            // the a_0 column: gamma_l(D) a_0, and log s on b_0
-            float4 gm = gamma[(long long)oi * p + t];
-            float2 gh = make_float2(gm.x, gm.y), gl = make_float2(gm.z, gm.w);
-            ff_acc2(gh, gl, make_float2(lsh, 0.f), make_float2(lsl, 0.f));
-            const float4 a0 = s_a0[q0 + j][d];
-            ff_cfma(ah, al, gh, gl, make_float2(a0.x, a0.y), make_float2(a0.z, a0.w));
+      for (int j = 0; j < NJ; ++j) {
+        const int q = q0 + j * nsplit;
+        if (q < no) {
+          const int id = o.id[o0 + q];
+          const int2 D = orbit_rep(id);
+          const int oi = offset_index(D.x, D.y);
+          acc = cff_fma(acc, cff_load(beta[((long long)ty * kOffs + oi) * p + t]), cff{sh[j], sl[j]});
+          if (ty == 1 && t > 0)
+            acc = cff_fma(acc, cff_load(gamma[(long long)oi * p + t]), cff_load(s_a0[o0 + q][d][t & 3]));
+          if (ty == 1 && t == 0) {
+            // a_0 (log D_r + log s) per source, s = D 2^-l
+            const cff logs = cff_split(log(f.D) - l * 0.69314718055994530942, 0.0);
+            int x = D.x, y = D.y;
+            for (int r = 0; r < 4; ++r) {
+              if (o.src[id][r] >= 0)
+                acc = cff_fma(acc, cff_add(cff_load(gamma[(long long)offset_index(x, y) * p]), logs),
+                              cff_load(mpff[((lev_off(l) + o.src[id][r]) * nd + d) * p]));
+              const int z = x;
+              x = -y;
+              y = z;
+            }
           }
         }
       }
     }
+  }
+  red[tid] = cff_store(acc);
+  __syncthreads();
+  if (sp == 0) {
+    for (int q = 1; q < nsplit; ++q) acc = cff_add(acc, cff_load(red[q * per + e]));
     // Cauchy channels carry 1/s
-    const double sc = ty == 1 ? 1.0 : inv_s;
-    f.lc[(gb * nd + d) * p + t] =
-        make_double2(((double)ah.x + (double)al.x) * sc, ((double)ah.y + (double)al.y) * sc);
+    const double sc = ty == 1 ? 1.0 : ldexp(f.Dinv, l);
+    const double2 v = cff_to(acc);
+    f.lc[gb * per + e] = make_double2(v.x * sc, v.y * sc);
   }
 }
 
@@ -1664,6 +1890,15 @@ int fmm_setup(FmmState*& f, const Geo& g, int kind, const int* orders, int norde
     std::vector<float2> host32(host.size());
     for (size_t e = 0; e < host.size(); ++e)
       host32[e] = make_float2((float)host[e].real(), (float)host[e].imag());
+    // k_fmm_m2l32's Pascal table after it: [k][residue][pair] rows (l, l + 4), zeros outside the order
+    const int pk = m2l32_pad(p), rp = m2l32_rp(pk);
+    host32.resize(host.size() + (size_t)pk * 4 * rp, make_float2(0.f, 0.f));
+    for (int k = 0; k < p; ++k)
+      for (int m = 0; m < 4 * rp; ++m) {
+        const int t0 = m / rp + 8 * (m % rp);
+        const auto entry = [&](int l) { return l < p ? (float)host[(size_t)tab_pascal(p) + (size_t)k * p + l].real() : 0.f; };
+        host32[host.size() + (size_t)k * 4 * rp + m] = make_float2(entry(t0), entry(t0 + 4));
+      }
     double2* ops = nullptr;
     float2* ops32 = nullptr;
     if (!ck(cudaMallocAsync(reinterpret_cast<void**>(&ops), host.size() * sizeof(double2), s), "fmm ops") ||
@@ -1705,25 +1940,73 @@ int fmm_setup(FmmState*& f, const Geo& g, int kind, const int* orders, int norde
 
 namespace {
 
-template <class T2, int PM>
-void m2l_launch_pm(const FmmDevT<T2>& d, int L, const int* stop, cudaStream_t s) {
-  const size_t sm = m2l_smem<T2>(d.p, d.nd, d.nlog, PM);
-  const int threads = std::max(64, std::min(256, (d.nd * d.p + 31) / 32 * 32));
-  cudaFuncSetAttribute(k_fmm_m2l<T2, PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_fmm_m2l<T2, PM><<<(int)(lev_off(L + 1) - lev_off(2)), threads, sm, s>>>(d, stop);
+// The splits of the orbits that fill a block's warps best (nsplit (channel, row)
+// threads), and the orbits staged at a time (at most about 100 KB).
+struct M2lShape {
+  int nsplit, threads, nbo;
+  size_t smem;
+};
+M2lShape m2l_shape(int nd, int p, size_t entry, size_t pascal) {
+  M2lShape m{1, 0, kOrbits, 0};
+  const int per = nd * p;
+  double best = 0.0;
+  for (int s : {1, 2, 5}) {
+    const int th = (s * per + 31) / 32 * 32;
+    if (th > 256) continue;
+    const double use = (double)s * per / th;
+    if (use > best + 0.02) {
+      best = use;
+      m.nsplit = s;
+      m.threads = th;
+    }
+  }
+  while (m.nbo > 5 && (size_t)m.nbo * per * 4 * entry + pascal > 100 * 1024) m.nbo = 5;
+  m.smem = (size_t)m.nbo * per * 4 * entry + pascal;
+  return m;
 }
 
-// FP32 expansions of order <= 32 hold their Pascal rows in registers.
-template <class T2>
-void launch_m2l(const FmmDevT<T2>& d, int L, const int* stop, cudaStream_t s) {
-  if constexpr (std::is_same<T2, float2>::value) {
-    if (d.p <= 12) return m2l_launch_pm<T2, 12>(d, L, stop, s);
-    if (d.p <= 16) return m2l_launch_pm<T2, 16>(d, L, stop, s);
-    if (d.p <= 20) return m2l_launch_pm<T2, 20>(d, L, stop, s);
-    if (d.p <= 24) return m2l_launch_pm<T2, 24>(d, L, stop, s);
-    if (d.p <= 32) return m2l_launch_pm<T2, 32>(d, L, stop, s);
+template <int ND, int PK>
+void m2l32_launch(const FmmDevT<float2>& d, const float2* ptab, int L, const int* stop, cudaStream_t s) {
+  const size_t sm = (size_t)kOrbits * ND * (4 * PK + 4) * sizeof(float2);
+  if (sm > 40 * 1024) cudaFuncSetAttribute(k_fmm_m2l32<ND, PK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_fmm_m2l32<ND, PK><<<(int)(lev_off(L + 1) - lev_off(2)), m2l32_threads(ND, PK), sm, s>>>(d, ptab, stop);
+}
+
+template <int ND>
+void launch_m2l32(const FmmDevT<float2>& d, const float2* ptab, int pk, int L, const int* stop, cudaStream_t s) {
+  switch (pk) {
+    case 12: return m2l32_launch<ND, 12>(d, ptab, L, stop, s);
+    case 16: return m2l32_launch<ND, 16>(d, ptab, L, stop, s);
+    case 20: return m2l32_launch<ND, 20>(d, ptab, L, stop, s);
+    case 24: return m2l32_launch<ND, 24>(d, ptab, L, stop, s);
+    case 32: return m2l32_launch<ND, 32>(d, ptab, L, stop, s);
+    case 48: return m2l32_launch<ND, 48>(d, ptab, L, stop, s);
+    default: return m2l32_launch<ND, 64>(d, ptab, L, stop, s);
   }
-  m2l_launch_pm<T2, 0>(d, L, stop, s);
+}
+
+void launch_m2l(const FmmDev& d, int L, const int* stop, cudaStream_t s) {
+  const int grid = (int)(lev_off(L + 1) - lev_off(2));
+  const M2lShape m = m2l_shape(d.nd, d.p, sizeof(double2), (size_t)(d.nlog > 0 ? 2 : 1) * d.p * d.p * sizeof(double));
+  if (m.nsplit == 5) {
+    cudaFuncSetAttribute(k_fmm_m2l<double2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
+    k_fmm_m2l<double2, 2><<<grid, m.threads, m.smem, s>>>(d, m.nsplit, m.nbo, stop);
+  } else {
+    cudaFuncSetAttribute(k_fmm_m2l<double2, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
+    k_fmm_m2l<double2, 5><<<grid, m.threads, m.smem, s>>>(d, m.nsplit, m.nbo, stop);
+  }
+}
+
+void launch_m2l_ff(const FmmDev& d, const float4* mpff, const float* tab, int L, const int* stop, cudaStream_t s) {
+  const M2lShape m = m2l_shape(d.nd, d.p, sizeof(float4), 0);
+  const int grid = (int)(lev_off(L + 1) - lev_off(2));
+  if (m.nsplit == 5) {
+    cudaFuncSetAttribute(k_fmm_m2l_ff<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
+    k_fmm_m2l_ff<2><<<grid, m.threads, m.smem, s>>>(d, mpff, tab, m.nsplit, m.nbo, stop);
+  } else {
+    cudaFuncSetAttribute(k_fmm_m2l_ff<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
+    k_fmm_m2l_ff<5><<<grid, m.threads, m.smem, s>>>(d, mpff, tab, m.nsplit, m.nbo, stop);
+  }
 }
 
 // Shared memory of the M2M and L2L blocks: one box's expansions and one
@@ -1751,7 +2034,7 @@ void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, double* partial
     k_fmm_p2m<T2><<<f->nleaf, kB, sm_p2m, s>>>(d, g, stop);
   const size_t sm_tree = tree_smem<T2>(nd, p);
   for (int l = f->L - 1; l >= 2; --l) k_fmm_m2m<T2><<<1 << (2 * l), kB, sm_tree, s>>>(d, l, stop);
-  bool done = false;
+  [[maybe_unused]] bool done = false;
   if constexpr (std::is_same<T2, double2>::value && NEARP == 2) {
     // the float-float residual operator: float-float M2L
     const float* tab = nullptr;
@@ -1760,13 +2043,19 @@ void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, double* partial
     if (tab) {
       const long long nmp = (lev_off(f->L + 1) - lev_off(2)) * nd * p;
       k_fmm_mp_ff<<<grid_for(nmp), 256, 0, s>>>(d.mp + lev_off(2) * nd * p, nmp, f->mpff + lev_off(2) * nd * p);
-      const size_t sm = (size_t)kListPad * nd * p * sizeof(float4);
-      cudaFuncSetAttribute(k_fmm_m2l_ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      k_fmm_m2l_ff<<<(int)(lev_off(f->L + 1) - lev_off(2)), kBFF, sm, s>>>(d, f->mpff, tab, stop);
+      launch_m2l_ff(d, f->mpff, tab, f->L, stop, s);
       done = true;
     }
   }
-  if (!done) launch_m2l(d, f->L, stop, s);
+  if constexpr (std::is_same<T2, float2>::value) {
+    const float2* ptab = d.ops + tab_size(p);
+    if (nd == 1)
+      launch_m2l32<1>(d, ptab, m2l32_pad(p), f->L, stop, s);
+    else
+      launch_m2l32<3>(d, ptab, m2l32_pad(p), f->L, stop, s);
+  } else {
+    if (!done) launch_m2l(d, f->L, stop, s);
+  }
   for (int l = 2; l < f->L; ++l) k_fmm_l2l<T2><<<1 << (2 * (l + 1)), kB, sm_tree, s>>>(d, l, stop);
   k_fmm_eval<T2, NEARP><<<f->nleaf, kBE, eval_smem<T2, NEARP>(nd, p), s>>>(d, g, partial, stop);
 }
@@ -1876,9 +2165,7 @@ cudaError_t fmm_output(FmmState* f, const Geo& g, int kind, int p, const double*
     // float-float multipole-to-local step (the float-float refinement's solves)
     const long long nmp = (lev_off(f->L + 1) - lev_off(2)) * nd * p;
     k_fmm_mp_ff<<<grid_for(nmp), 256, 0, s>>>(f->mp + lev_off(2) * nd * p, nmp, f->mpff + lev_off(2) * nd * p);
-    const size_t sm = (size_t)kListPad * nd * p * sizeof(float4);
-    cudaFuncSetAttribute(k_fmm_m2l_ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_fmm_m2l_ff<<<(int)(lev_off(f->L + 1) - lev_off(2)), kBFF, sm, s>>>(d, f->mpff, tab, nullptr);
+    launch_m2l_ff(d, f->mpff, tab, f->L, nullptr, s);
     note_launches(1);
   } else {
     launch_m2l(d, f->L, nullptr, s);

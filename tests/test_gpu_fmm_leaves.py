@@ -47,3 +47,30 @@ def test_fmm_operator_uneven_leaves(kind, n_dense):
         assert bie.apply_operator_fmm_prec(ctx, g, kind, order, prec, v, out) == bie.OK
         assert np.array_equal(got, out.cpu().numpy())  # fixed order
     ctx.close()
+
+
+# Orders on both sides of the FP32 translation kernel's instances (12, 16, 20, 24,
+# 32, 48, 64) and of the numbers of splits.  The same expansions in FP64 are the
+# reference, so that only rounding differs: FP32 sums as above 2e-5; float-float
+# products (2^-46) summed in FP64, with the expansions' own FP64 rounding, 1e-11.
+@pytest.mark.parametrize("kind", [bie.LAPLACE, bie.STOKES])
+@pytest.mark.parametrize("order", [2, 7, 12, 13, 16, 17, 20, 21, 24, 25, 32, 33, 48, 49, 64])
+def test_fmm_operator_orders(kind, order):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1507_05925_gb300 import build
+    build.build()
+    ctx = bie.Context(0)
+    g = to_dev(uneven(300))
+    v = torch.from_numpy(np.random.default_rng(8).standard_normal(g["x"].numel() * (kind + 1))).cuda()
+    out = torch.empty_like(v)
+    got = {}
+    for prec in (bie.FP64, bie.MIXED_FF, bie.MIXED):
+        out.fill_(float("nan"))
+        assert bie.apply_operator_fmm_prec(ctx, g, kind, order, prec, v, out) == bie.OK, ctx.last_error()
+        got[prec] = out.cpu().numpy()
+    for prec, tol in ((bie.MIXED_FF, 1e-11), (bie.MIXED, 2e-5)):
+        err = rel_max(got[prec], got[bie.FP64])
+        print(f"kind={kind} order={order} prec={prec}: {err:.2e}")
+        assert err <= tol
+    ctx.close()
