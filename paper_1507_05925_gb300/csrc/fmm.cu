@@ -395,57 +395,167 @@ __global__ void __launch_bounds__(kB) k_fmm_p2m(FmmDevT<T2> f, Geo g, const int*
     if (t + u * kB < f.nd * f.p) f.mp[box * f.nd * f.p + t + u * kB] = acc[u];
 }
 
-// M2M into level l (parents) from level l + 1.  Per child, its multipoles and
-// the translation matrix are staged in shared memory (coalesced, one round
-// trip each); thread e < nd p computes coefficient e % p of channel e / p
-// (its terms in the order m = 0..k), summed over the children in order.
-constexpr int kAccPer = (kMaxNd * kMaxP + kB - 1) / kB;  // outputs a thread keeps
+// Shifts between a box and its children.  With u_P = u_C/2 + w_c, w_c = (+-1 +- i)/4,
+//   M2M: a'_k = sum_c sum_{m <= k} C(k, m) w_c^(k-m) 2^-m a^(c)_m,
+//   L2L: b^(c)_k = sum_{m >= k} C(m, k) w_c^(m-k) 2^-k b_m.
+// The children are quarter turns of each other, w_r = i^r w, w = |w| e^(i pi/4), so
+// one real matrix serves all four both ways: with e^(i pi m/4) = h^(m mod 2) g_m,
+// h = 2^-1/2, g_m = i^(m div 2) (1 + i)^(m mod 2) (turns and additions only), and
+//   T[m][k] = C(max, min) |w|^|k-m| 2^-min h^(m mod 2) h^(k mod 2):
+//   a'_k = g_k sum_{m <= k} T[m][k] conj(g_m) A_m^((k-m) mod 4),  A^(q)_m = sum_r i^(rq) a^(r)_m,
+//   b^(r)_k = conj(g_k) sum_j i^(rj) S_j[k],  S_j[k] = sum_{m >= k, m = k+j mod 4} T[m][k] g_m b_m.
+// That is 1/8 of the multiply-adds of four complex matrices, and no matrix to stage.
+// Both kernels, for orders p <= PK: thread (m mod 4, channel, k) keeps its column of T in
+// registers for all levels and adds the terms of its residue of m; the four sums
+// meet in shared memory.  (Run-time sizes took twice the instructions.)
+__device__ __forceinline__ int child_of_turn(int r) { return r == 0 ? 3 : r == 1 ? 2 : r == 2 ? 0 : 1; }
+__device__ __forceinline__ int turn_of_child(int c) { return c == 3 ? 0 : c == 2 ? 1 : c == 0 ? 2 : 3; }
 
+// i^j z
 template <class T2>
-__global__ void __launch_bounds__(kB) k_fmm_m2m(FmmDevT<T2> f, int l, const int* stop) {
+__device__ __forceinline__ T2 turned(T2 z, int j) {
+  T2 v = z;
+  if (j & 1) {
+    v.x = -z.y;
+    v.y = z.x;
+  }
+  if (j & 2) {
+    v.x = -v.x;
+    v.y = -v.y;
+  }
+  return v;
+}
+// g_m z and conj(g_m) z
+template <class T2>
+__device__ __forceinline__ T2 eighth(T2 z, int m) {
+  if (m & 1) {
+    const auto x = z.x;
+    z.x = x - z.y;
+    z.y = x + z.y;
+  }
+  return turned(z, (m >> 1) & 3);
+}
+template <class T2>
+__device__ __forceinline__ T2 eighth_conj(T2 z, int m) {
+  if (m & 1) {
+    const auto x = z.x;
+    z.x = x + z.y;
+    z.y = z.y - x;
+  }
+  return turned(z, -(m >> 1) & 3);
+}
+// x_r = sum_j i^(rj) v_j
+template <class T2>
+__device__ __forceinline__ void quarter_sums(T2* v) {
+  const T2 s02 = cadd(v[0], v[2]), d02 = cadd(v[0], turned(v[2], 2));
+  const T2 s13 = cadd(v[1], v[3]), d13 = turned(cadd(v[1], turned(v[3], 2)), 1);
+  v[0] = cadd(s02, s13);
+  v[1] = cadd(d02, d13);
+  v[2] = cadd(s02, turned(s13, 2));
+  v[3] = cadd(d02, turned(d13, 2));
+}
+inline int shift_threads(int nd, int p) { return (4 * nd * p + 31) / 32 * 32; }
+// of up to nc channels of order pk
+__host__ __device__ constexpr int shift_max_threads(int nc, int pk) { return (4 * nc * pk + 31) / 32 * 32; }
+// blocks an SM that the registers have to leave room for (more of them spill)
+template <class T2>
+constexpr int shift_blocks(int nc, int pk) {
+  return (sizeof(T2) == 8 ? 1536 : nc == 1 ? 640 : 1152) / shift_max_threads(nc, pk);
+}
+template <class T2>
+size_t shift_smem(int nd, int pk) {
+  return (size_t)8 * nd * (pk + 1) * sizeof(T2);
+}
+
+// M2M of all levels L-1..2 in one launch: a block forms one box of level L-1, and
+// the block that completes the last of four siblings goes on with their parent
+// (no block waits; arrive[] counts the siblings and is back at 0 at the end).
+// Each level was a launch of one 64-thread block a box, the children one after
+// the other with their matrices staged: all levels, FP32 Laplace, 1,024 leaves, order
+// 15: 31 -> 9.0 us; FP32 Stokes, 16,384 leaves, order 18: 83 -> 35 us; FP64 Stokes, order
+// 36: 995 -> 222 us (L2L: 17 -> 6.8, 49 -> 31 and 700 -> 235 us).  What is left is the
+// chain of levels (2-3 us each), in FP64 the FP64 pipe.
+template <class T2, int NC, int PK>
+__global__ void __launch_bounds__(shift_max_threads(NC, PK), shift_blocks<T2>(NC, PK))
+k_fmm_m2m(FmmDevT<T2> f, int* arrive, const int* stop) {
+  using R = decltype(T2{}.x);
   if (stop && *stop) return;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T2* sm = reinterpret_cast<T2*>(smraw);  // [nd][p]
-  T2* so = sm + f.nd * f.p;               // [p][p] the child's M2M matrix, [in][out]
-  const int n = 1 << l;
-  const int b = blockIdx.x, bx = b % n, by = b / n;
-  const long long box = lev_off(l) + b;
-  if (f.count[box] == 0) return;
-  const int t = threadIdx.x, np = f.nd * f.p, pp = f.p * f.p;
-  T2 acc[kAccPer];
+  const int p = f.p, np = f.nd * p, US = f.nd * (PK + 1), t = threadIdx.x;
+  T2* U = reinterpret_cast<T2*>(smraw);  // [q][channel][m], channels PK + 1 apart
+  T2* red = U + 4 * US;                  // [residue][channel, k]
+  __shared__ int s_last;
+  const int e = t % np, mr = t / np, d = e / p, k = e - d * p;
+  R T[PK / 4];
 #pragma unroll
-  for (int u = 0; u < kAccPer; ++u) acc[u] = cx<T2>(0.0, 0.0);
-  for (int c = 0; c < 4; ++c) {
-    const long long child = lev_off(l + 1) + (2 * by + (c >> 1)) * (2 * n) + 2 * bx + (c & 1);
-    if (f.count[child] == 0) continue;  // uniform over the block
-    __syncthreads();
-    for (int e = t; e < np; e += kB) sm[e] = f.mp[child * np + e];
-    for (int e = t; e < pp; e += kB) so[e] = f.ops[(long long)c * pp + e];
-    __syncthreads();
-    if (f.cm >= 0) {
-      // child moment density relative to the parent centre: 1/2 rho_C + gamma rho_0,
-      // gamma = conj(c_C - c_P)/(2 s_C)
-      const T2 gam = cx<T2>(0.5 * ((c & 1) - 0.5), -0.5 * ((c >> 1) - 0.5));
-      for (int m = t; m < f.p; m += kB) {
-        T2 v = cx<T2>(0.5 * (double)sm[f.cm * f.p + m].x, 0.5 * (double)sm[f.cm * f.p + m].y);
-        cfma(v, gam, sm[m]);
-        sm[f.cm * f.p + m] = v;
+  for (int i = 0; i < PK / 4; ++i) {
+    const int m = mr + 4 * i;
+    T[i] = m <= k && mr < 4 ? __ldg(reinterpret_cast<const R*>(f.ops) + m * p + k) : (R)0;
+  }
+  for (int w = t; w < 4 * f.nd * (PK + 1 - p); w += blockDim.x)  // the padding
+    U[w / (PK + 1 - p) * (PK + 1) + p + w % (PK + 1 - p)] = cx<T2>(0.0, 0.0);
+  int b = blockIdx.x;
+  for (int l = f.L - 1;; --l) {
+    const int n = 1 << l, bx = b & (n - 1), by = b >> l;
+    const long long box = lev_off(l) + b;
+    if (f.count[box] > 0) {
+      if (t < np) {
+        // other blocks of this launch wrote the children above the first level: past L1
+        T2 v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int c = child_of_turn(r);
+          const long long child = lev_off(l + 1) + (long long)(2 * by + (c >> 1)) * (2 * n) + 2 * bx + (c & 1);
+          v[r] = cx<T2>(0.0, 0.0);
+          if (f.count[child] > 0) v[r] = __ldcg(f.mp + child * np + e);
+        }
+        quarter_sums(v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) U[q * US + d * (PK + 1) + k] = eighth_conj(v[q], k);
       }
       __syncthreads();
-    }
+      if (f.cm >= 0) {
+        // child moment density relative to the parent centre: 1/2 rho_r + conj(w_r) a_r, whose
+        // transform is 1/2 that of rho plus conj(w) times that of a, one place back
+        if (t < 4 * p) {
+          const int q = t / p, m = t - q * p;
+          T2 a = U[q * US + f.cm * (PK + 1) + m];
+          a.x *= R(0.5);
+          a.y *= R(0.5);
+          cfma(a, cx<T2>(0.25, -0.25), U[((q + 3) & 3) * US + m]);
+          U[q * US + f.cm * (PK + 1) + m] = a;
+        }
+        __syncthreads();
+      }
+      if (mr < 4) {
+        T2 acc = cx<T2>(0.0, 0.0);
+        const T2* u = U + ((k - mr) & 3) * US + d * (PK + 1) + mr;
 #pragma unroll
-    for (int u = 0; u < kAccPer; ++u) {
-      const int e = t + u * kB;
-      if (e < np) {
-        const int d = e / f.p, k = e % f.p;
-        for (int m = 0; m <= k; ++m) cfma(acc[u], so[m * f.p + k], sm[d * f.p + m]);
+        for (int i = 0; i < PK / 4; ++i) {
+          const T2 x = u[4 * i];
+          acc.x = fma(T[i], x.x, acc.x);
+          acc.y = fma(T[i], x.y, acc.y);
+        }
+        red[t] = acc;
+      }
+      __syncthreads();
+      if (t < np) {
+        const T2 a = cadd(cadd(red[t], red[np + t]), cadd(red[2 * np + t], red[3 * np + t]));
+        f.mp[box * np + t] = eighth(a, k);
       }
     }
-  }
-#pragma unroll
-  for (int u = 0; u < kAccPer; ++u) {
-    const int e = t + u * kB;
-    if (e < np) f.mp[box * np + e] = acc[u];
+    if (l == 2) return;
+    __syncthreads();
+    b = (by >> 1) * (n >> 1) + (bx >> 1);
+    if (t == 0) {
+      __threadfence();  // the block's stores, ordered before it by the barrier
+      int* a = arrive + lev_off(l - 1) + b;
+      s_last = atomicAdd(a, 1) == 3;
+      if (s_last) *a = 0;
+      __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
   }
 }
 
@@ -530,11 +640,11 @@ __device__ __forceinline__ void list_orbits(const FmmDevT<T2>& f, int l, int bx,
   __syncthreads();
 }
 
-// Layout of the operator table of order p (complex entries): M2M and L2L
-// matrices [op][in][out], then the M2L factors alpha[2][49][p], beta[2][49][p],
+// Layout of the operator table of order p (complex entries): the child shifts'
+// matrix T[m][k] (p^2 reals), then the M2L factors alpha[2][49][p], beta[2][49][p],
 // gamma[49][p] and the Pascal matrices [2][k][l] (real, in the real parts);
 // type 0 = Cauchy, 1 = logarithm, offset index (Dx + 3) + 7 (Dy + 3).
-__host__ __device__ inline long long tab_alpha(int p) { return 8LL * p * p; }
+__host__ __device__ inline long long tab_alpha(int p) { return ((long long)p * p + 1) / 2; }
 __host__ __device__ inline long long tab_beta(int p) { return tab_alpha(p) + 2LL * kOffs * p; }
 __host__ __device__ inline long long tab_gamma(int p) { return tab_beta(p) + 2LL * kOffs * p; }
 __host__ __device__ inline long long tab_pascal(int p) { return tab_gamma(p) + (long long)kOffs * p; }
@@ -1133,42 +1243,91 @@ __global__ void __launch_bounds__(256) k_fmm_m2l_ff(FmmDev f, const float4* __re
   }
 }
 
-// L2L from level l to the children at level l + 1 (added to their M2L part):
-// the parent's local expansion and the child's L2L matrix staged in shared
-// memory; thread e < nd p updates coefficient e % p of channel e / p (terms
-// in the order m = k..p-1).
-template <class T2>
-__global__ void __launch_bounds__(kB) k_fmm_l2l(FmmDevT<T2> f, int l, const int* stop) {
+// L2L from level l0 down to the children of level lp (added to their M2L part), a
+// block a box of level lp: it carries the expansion down its own path l0..lp in
+// shared memory and writes the four children.  Boxes above lp are read, not
+// updated, so one launch covers several levels (fmm_l2l).
+template <class T2, int NC, int PK>
+__global__ void __launch_bounds__(shift_max_threads(NC, PK), shift_blocks<T2>(NC, PK))
+k_fmm_l2l(FmmDevT<T2> f, int l0, int lp, const int* stop) {
+  using R = decltype(T2{}.x);
   if (stop && *stop) return;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T2* sm = reinterpret_cast<T2*>(smraw);  // [nd][p]
-  T2* so = sm + f.nd * f.p;               // [p][p] the L2L matrix, [in][out]
-  const int nc = 2 << l;
-  const int b = blockIdx.x, bx = b % nc, by = b / nc;
-  const long long child = lev_off(l + 1) + b;
-  if (f.tcount[child] == 0) return;
-  const long long parent = lev_off(l) + (by >> 1) * (nc >> 1) + (bx >> 1);
-  const int c = (bx & 1) + 2 * (by & 1);
-  const int t = threadIdx.x, np = f.nd * f.p, pp = f.p * f.p;
-  for (int e = t; e < np; e += kB) sm[e] = f.lc[parent * np + e];
-  for (int e = t; e < pp; e += kB) so[e] = f.ops[(long long)(4 + c) * pp + e];
-  __syncthreads();
-  if (f.cm >= 0) {
-    // moment density relative to the child centre: 2 rho_P + delta rho_0,
-    // delta = conj(c_P - c_C)/s_C
-    const T2 del = cx<T2>(-((c & 1) - 0.5), (c >> 1) - 0.5);
-    for (int m = t; m < f.p; m += kB) {
-      T2 v = cx<T2>(2.0 * (double)sm[f.cm * f.p + m].x, 2.0 * (double)sm[f.cm * f.p + m].y);
-      cfma(v, del, sm[m]);
-      sm[f.cm * f.p + m] = v;
+  const int p = f.p, np = f.nd * p, t = threadIdx.x;
+  T2* loc = reinterpret_cast<T2*>(smraw);  // g_m b_m, [channel][m], channels PK + 1 apart
+  T2* S = loc + f.nd * (PK + 1);           // [residue of m][channel, k]
+  const int n = 1 << lp, b = blockIdx.x, bx = b & (n - 1), by = b >> lp;
+  if (f.tcount[lev_off(lp) + b] == 0) return;
+  const int e = t % np, mr = t / np, d = e / p, k = e - d * p;
+  R T[PK / 4];
+#pragma unroll
+  for (int i = 0; i < PK / 4; ++i) {
+    const int m = mr + 4 * i;
+    T[i] = m >= k && m < p && mr < 4 ? __ldg(reinterpret_cast<const R*>(f.ops) + m * p + k) : (R)0;
+  }
+  for (int w = t; w < f.nd * (PK + 1 - p); w += blockDim.x)  // the padding
+    loc[w / (PK + 1 - p) * (PK + 1) + p + w % (PK + 1 - p)] = cx<T2>(0.0, 0.0);
+  const auto at = [&](int l) {  // the path's box of level l
+    return lev_off(l) + ((long long)(by >> (lp - l)) << l) + (bx >> (lp - l));
+  };
+  // S_j, j = 0..3, of the thread's coefficient
+  const auto sums = [&](T2* x) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      x[j] = S[((k + j) & 3) * np + e];
+      if (d == f.cm) {
+        // moment density relative to the child centre: 2 rho - 2 conj(w_r) a
+        x[j].x *= R(2.0);
+        x[j].y *= R(2.0);
+        cfma(x[j], cx<T2>(-0.5, 0.5), S[((k + j + 1) & 3) * np + k]);
+      }
+    }
+  };
+  T2 next = cx<T2>(0.0, 0.0);
+  if (t < np) next = f.lc[at(l0) * np + e];
+  for (int l = l0;; ++l) {
+    if (t < np) {
+      loc[d * (PK + 1) + k] = eighth(next, k);
+      if (l < lp) next = f.lc[at(l + 1) * np + e];
     }
     __syncthreads();
+    if (mr < 4) {
+      T2 acc = cx<T2>(0.0, 0.0);
+      const T2* u = loc + d * (PK + 1) + mr;
+#pragma unroll
+      for (int i = 0; i < PK / 4; ++i) {
+        const T2 x = u[4 * i];
+        acc.x = fma(T[i], x.x, acc.x);
+        acc.y = fma(T[i], x.y, acc.y);
+      }
+      S[t] = acc;
+    }
+    __syncthreads();
+    if (l == lp) break;
+    if (t < np) {
+      const int r = turn_of_child(((bx >> (lp - l - 1)) & 1) + 2 * ((by >> (lp - l - 1)) & 1));
+      T2 x[4];
+      sums(x);
+      const T2 a = cadd(cadd(x[0], turned(x[1], r)), cadd(turned(x[2], 2 * r), turned(x[3], 3 * r)));
+      next = cadd(next, eighth_conj(a, k));
+    }
   }
-  for (int e = t; e < np; e += kB) {
-    const int d = e / f.p, k = e % f.p;
-    T2 acc = f.lc[child * np + e];
-    for (int m = k; m < f.p; ++m) cfma(acc, so[m * f.p + k], sm[d * f.p + m]);
-    f.lc[child * np + e] = acc;
+  if (t < np) {
+    T2 x[4], v[4];
+    long long box[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int c = child_of_turn(r);
+      box[r] = lev_off(lp + 1) + (long long)(2 * by + (c >> 1)) * (2 * n) + 2 * bx + (c & 1);
+      if (f.tcount[box[r]] == 0) box[r] = -1;
+      v[r] = cx<T2>(0.0, 0.0);
+      if (box[r] >= 0) v[r] = f.lc[box[r] * np + e];
+    }
+    sums(x);
+    quarter_sums(x);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (box[r] >= 0) f.lc[box[r] * np + e] = cadd(v[r], eighth_conj(x[r], k));
   }
 }
 
@@ -1716,14 +1875,14 @@ std::vector<std::complex<double>> build_ops(int p) {
     for (int b = 1; b <= a; ++b) B(a, b) = B(a - 1, b - 1) + (b <= a - 1 ? B(a - 1, b) : 0.0);
   }
   std::vector<C> ops((size_t)tab_size(p), C(0, 0));
-  auto at = [&](int o, int in, int out) -> C& { return ops[((size_t)o * p + in) * p + out]; };
-  for (int c = 0; c < 4; ++c) {
-    const C w(((c & 1) - 0.5) / 2.0, ((c >> 1) - 0.5) / 2.0);
-    for (int k = 0; k < p; ++k)
-      for (int m = 0; m <= k; ++m) at(c, m, k) = B(k, m) * std::pow(0.5, m) * std::pow(w, k - m);  // M2M
-    for (int m = 0; m < p; ++m)
-      for (int l = m; l < p; ++l) at(4 + c, l, m) = B(l, m) * std::pow(0.5, m) * std::pow(w, l - m);  // L2L
-  }
+  for (int m = 0; m < p; ++m)
+    for (int k = 0; k < p; ++k) {
+      const int hi = std::max(m, k), lo = std::min(m, k);
+      // |w| = 2^-3/2; with the factors h the exponent is a whole number: T is exact
+      const double t = B(hi, lo) * std::ldexp(1.0, -lo - (3 * (hi - lo) + (hi & 1) + (lo & 1)) / 2);
+      const int e = m * p + k;
+      ops[e / 2] = e & 1 ? C(ops[e / 2].real(), t) : C(t, 0.0);
+    }
   // M2L factors.  Cauchy: (d + u)^-(k+1) = sum_l C(k+l, l) (-1)^l u^l d^-(k+l+1).
   // Logarithm: log(d + u) = log d + sum_l (-1)^(l+1) (u/d)^l / l and
   // (d + u)^-k = sum_l C(k+l-1, l) (-1)^l u^l d^-(k+l); the log s part of log d
@@ -1764,6 +1923,7 @@ struct FmmState {
   size_t buf_size = 0;
   int *leaf = nullptr, *perm = nullptr, *tmp = nullptr, *start = nullptr, *cursor = nullptr, *count = nullptr;
   int *tcount = nullptr, *tleaf = nullptr;
+  int* arrive = nullptr;  // per box: siblings done in the upward pass (0 between launches)
   double *tx = nullptr, *ty = nullptr;
   double2 *Q = nullptr, *mp = nullptr, *lc = nullptr;
   float4* cen32 = nullptr;  // per leaf: centre split as float hi + lo (x_h, y_h, x_l, y_l)
@@ -1837,7 +1997,7 @@ int fmm_setup(FmmState*& f, const Geo& g, int kind, const int* orders, int norde
   f->pmax = pmax;
   // buffers
   auto pad = [](size_t b) { return (b + 255) & ~size_t(255); };
-  const size_t need = 3 * pad((size_t)g.M * 4) + 2 * pad(((size_t)f->nleaf + 1) * 4) + 2 * pad((size_t)f->nbox * 4) +
+  const size_t need = 3 * pad((size_t)g.M * 4) + 2 * pad(((size_t)f->nleaf + 1) * 4) + 3 * pad((size_t)f->nbox * 4) +
                       pad((size_t)g.M * nd * 16) + 3 * pad((size_t)f->nbox * nd * pmax * 16) +
                       pad((size_t)3 * g.N * 4) + 2 * pad((size_t)3 * g.N * 8) + pad((size_t)f->nleaf * 16);
   if (need > f->buf_size) {
@@ -1860,6 +2020,7 @@ int fmm_setup(FmmState*& f, const Geo& g, int kind, const int* orders, int norde
   f->cursor = (int*)take(((size_t)f->nleaf + 1) * 4);
   f->count = (int*)take((size_t)f->nbox * 4);
   f->tcount = (int*)take((size_t)f->nbox * 4);
+  f->arrive = (int*)take((size_t)f->nbox * 4);
   f->tleaf = (int*)take((size_t)3 * g.N * 4);
   f->tx = (double*)take((size_t)3 * g.N * 8);
   f->ty = (double*)take((size_t)3 * g.N * 8);
@@ -1869,7 +2030,9 @@ int fmm_setup(FmmState*& f, const Geo& g, int kind, const int* orders, int norde
   f->mpff = (float4*)take((size_t)f->nbox * nd * pmax * 16);
   f->cen32 = (float4*)take((size_t)f->nleaf * 16);
   // counting sort of the nodes by leaf, node order inside a leaf
-  if (!ck(cudaMemsetAsync(f->cursor, 0, ((size_t)f->nleaf + 1) * 4, s), "fmm memset")) return BIE_ERR_CUDA;
+  if (!ck(cudaMemsetAsync(f->cursor, 0, ((size_t)f->nleaf + 1) * 4, s), "fmm memset") ||
+      !ck(cudaMemsetAsync(f->arrive, 0, (size_t)f->nbox * 4, s), "fmm memset"))
+    return BIE_ERR_CUDA;
   k_fmm_leaf<<<grid_for(g.M), 256, 0, s>>>(g, L, f->x0, f->y0, f->D, f->leaf, f->cursor);
   k_fmm_scan<<<1, 1024, 0, s>>>(f->cursor, f->nleaf, f->start);
   cudaMemsetAsync(f->cursor, 0, ((size_t)f->nleaf + 1) * 4, s);
@@ -2009,16 +2172,53 @@ void launch_m2l_ff(const FmmDev& d, const float4* mpff, const float* tab, int L,
   }
 }
 
-// Shared memory of the M2M and L2L blocks: one box's expansions and one
-// p x p translation matrix (above the default 48 KB for FP64 at high order).
+// The instance of the shift kernels for nd channels of order p.
+template <int NC, class F>
+void for_shift_order(int p, F&& launch) {
+  using std::integral_constant;
+  const integral_constant<int, NC> nc{};
+  if (p <= 16) return launch(nc, integral_constant<int, 16>{});
+  if (p <= 20) return launch(nc, integral_constant<int, 20>{});
+  if (p <= 36) return launch(nc, integral_constant<int, 36>{});
+  launch(nc, integral_constant<int, 64>{});
+}
+template <class F>
+void for_shift(int nd, int p, F&& launch) {
+  if (nd == 1)
+    for_shift_order<1>(p, launch);
+  else
+    for_shift_order<kMaxNd>(p, launch);
+}
+
+// The downward pass.  A launch that covers several levels repeats the upper ones in
+// every block, which costs less than a launch while its lowest level has few boxes:
+// FP32 up to 1,024 (with 4,096, 43 us in place of 32 at 16,384 leaves), FP64, whose
+// pipe is 1/64 as wide, 256.
 template <class T2>
-size_t tree_smem(int nd, int p) {
-  const size_t sm = ((size_t)nd * p + (size_t)p * p) * sizeof(T2);
-  if (sm > 48 * 1024) {
-    cudaFuncSetAttribute(k_fmm_m2m<T2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_fmm_l2l<T2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+int fmm_l2l(const FmmDevT<T2>& d, const int* stop, cudaStream_t s) {
+  constexpr int kPath = std::is_same<T2, float2>::value ? 5 : 4;  // level: 4^kPath boxes
+  int n = 0;
+  for (int l0 = 2; l0 < d.L; ++n) {
+    const int lp = std::max(l0, std::min(kPath, d.L - 1));
+    const int grid = 1 << (2 * lp), threads = shift_threads(d.nd, d.p);
+    for_shift(d.nd, d.p, [&](auto nc, auto pk) {
+      constexpr int NC = decltype(nc)::value, PK = decltype(pk)::value;
+      k_fmm_l2l<T2, NC, PK><<<grid, threads, shift_smem<T2>(d.nd, PK), s>>>(d, l0, lp, stop);
+    });
+    l0 = lp + 1;
   }
-  return sm;
+  return n;
+}
+
+template <class T2>
+int fmm_m2m(const FmmDevT<T2>& d, int* arrive, const int* stop, cudaStream_t s) {
+  if (d.L <= 2) return 0;
+  for_shift(d.nd, d.p, [&](auto nc, auto pk) {
+    constexpr int NC = decltype(nc)::value, PK = decltype(pk)::value;
+    const size_t sm = shift_smem<T2>(d.nd, PK);
+    k_fmm_m2m<T2, NC, PK><<<1 << (2 * (d.L - 1)), shift_threads(d.nd, d.p), sm, s>>>(d, arrive, stop);
+  });
+  return 1;
 }
 
 // The upward pass, M2L, downward pass and evaluation with expansions of type T2.
@@ -2032,8 +2232,7 @@ void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, double* partial
     k_fmm_p2m_ff<<<f->nleaf, kB, sm_p2m, s>>>(d, g, stop);  // float4 = double2 in size
   else
     k_fmm_p2m<T2><<<f->nleaf, kB, sm_p2m, s>>>(d, g, stop);
-  const size_t sm_tree = tree_smem<T2>(nd, p);
-  for (int l = f->L - 1; l >= 2; --l) k_fmm_m2m<T2><<<1 << (2 * l), kB, sm_tree, s>>>(d, l, stop);
+  int shifts = fmm_m2m(d, f->arrive, stop, s);
   [[maybe_unused]] bool done = false;
   if constexpr (std::is_same<T2, double2>::value && NEARP == 2) {
     // the float-float residual operator: float-float M2L
@@ -2056,7 +2255,8 @@ void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, double* partial
   } else {
     if (!done) launch_m2l(d, f->L, stop, s);
   }
-  for (int l = 2; l < f->L; ++l) k_fmm_l2l<T2><<<1 << (2 * (l + 1)), kB, sm_tree, s>>>(d, l, stop);
+  shifts += fmm_l2l(d, stop, s);
+  note_launches(shifts);
   k_fmm_eval<T2, NEARP><<<f->nleaf, kBE, eval_smem<T2, NEARP>(nd, p), s>>>(d, g, partial, stop);
 }
 
@@ -2123,7 +2323,7 @@ cudaError_t fmm_pair_sum(FmmState* f, const Geo& g, int kind, int p, VecRef v, c
     else
       fmm_passes<double2, 0>(d, f, g, partial, stop, s);
   }
-  note_launches(4 + 2 * std::max(0, f->L - 2) + (near_prec == 2 ? 1 : 0));
+  note_launches(4 + (near_prec == 2 ? 1 : 0));
   return cudaGetLastError();
 }
 
@@ -2156,8 +2356,7 @@ cudaError_t fmm_output(FmmState* f, const Geo& g, int kind, int p, const double*
     k_fmm_p2m_ff<<<f->nleaf, kB, sm_p2m, s>>>(d, g, nullptr);  // float4 = double2 in size
   else
     k_fmm_p2m<double2><<<f->nleaf, kB, sm_p2m, s>>>(d, g, nullptr);
-  const size_t sm_tree = tree_smem<double2>(nd, p);
-  for (int l = f->L - 1; l >= 2; --l) k_fmm_m2m<double2><<<1 << (2 * l), kB, sm_tree, s>>>(d, l, nullptr);
+  int shifts = fmm_m2m(d, f->arrive, nullptr, s);
   const float* tab = nullptr;
   for (auto& o : f->opsff)
     if (o.first == p) tab = o.second;
@@ -2170,10 +2369,10 @@ cudaError_t fmm_output(FmmState* f, const Geo& g, int kind, int p, const double*
   } else {
     launch_m2l(d, f->L, nullptr, s);
   }
-  for (int l = 2; l < f->L; ++l) k_fmm_l2l<double2><<<1 << (2 * (l + 1)), kB, sm_tree, s>>>(d, l, nullptr);
+  shifts += fmm_l2l(d, nullptr, s);
   k_fmm_eval_targets<<<(T + kTW - 1) / kTW, 32 * kTW, 0, s>>>(d, g, kind, T, f->tx, f->ty, f->tleaf, c0x, c0y,
                                                                part);
-  note_launches(7 + f->L + 2 * std::max(0, f->L - 2));
+  note_launches(7 + f->L + shifts);
   return cudaGetLastError();
 }
 
