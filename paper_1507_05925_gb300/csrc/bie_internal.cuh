@@ -102,7 +102,7 @@ struct KState {
   int m;           // restart length
   int counter;     // last-block-done counter for grid reductions
   int pad[2];         // [0] = 1: set tol_abs from the next starting residual
-  unsigned bar_count, bar_gen;  // grid barrier of the fused Arnoldi step
+  unsigned bar_count, bar_gen;  // grid barrier of the fused Arnoldi step: arrivals, and their number before the launch
   int error;          // 1: a grid barrier gave up waiting (results invalid)
   int nactive;        // batched GMRES: problems still iterating in this cycle
 };
