@@ -16,9 +16,9 @@
 // bie_info.precond_fallbacks), so a nearly singular block can slow GMRES down
 // but never poisons it with NaN or huge entries.  A block of
 // nb <= 128 unknowns is inverted by one CTA; nb <= 448 by a cluster of four
-// CTAs and nb <= 640 by one of eight, each CTA holding a slice of the columns
-// and reading the pivot panels of the others through distributed shared
-// memory; larger blocks are left as the identity.  The inverses are stored
+// CTAs and nb <= 640 by one of eight (few bodies: larger clusters, bj_setup), each
+// CTA holding a slice of the columns and reading the pivot panels of the others
+// through L2; larger blocks are left as the identity.  The inverses are stored
 // column-major as W = B^{-1} - 2I in FP16 (half the bytes of the apply, which
 // streams every block once a GMRES iteration: 655 MB in FP32 for 10,000
 // bodies of 128 unknowns).  B^{-1} is 2I plus a compact part, so W carries
@@ -47,8 +47,8 @@ namespace {
 constexpr int kMaxSingle = 128;  // one CTA
 constexpr int kMaxBlock4 = 448;  // cluster of four CTAs
 constexpr int kMaxBlock = kBjMaxBlock;  // cluster of eight CTAs (640); larger bodies keep the identity
+constexpr int kMinCluster = 72;  // the panels' exchange fits the result's place
 constexpr int kPB = 16;          // panel width of the blocked elimination
-constexpr int kMaxThreads = 640; // one thread per row
 constexpr int kBA = 256;         // threads of an application CTA
 constexpr int kApplyRows = 64, kApplyGroups = kBA / kApplyRows;
 
@@ -62,7 +62,7 @@ __host__ __device__ __forceinline__ int gj_cols(int nb, int cs) {
 }
 __host__ __device__ __forceinline__ size_t gj_smem_floats(int nb, int cs) {
   const int h = gj_cols(nb, cs);
-  return (size_t)gj_ld(nb) * h + (size_t)h * kPB + 2 * kPB + 8 * (size_t)h;
+  return (size_t)gj_ld(nb) * h + (size_t)h * kPB + (cs > 1 ? 3 : 2) * kPB * kPB;
 }
 
 // Entry (row r, column c) of the operator's diagonal block of body i
@@ -76,10 +76,15 @@ struct BlockRow {
   float4 pa;  // (x_hi, y_hi, x_lo, y_lo) of the row's node
   float nxa, nya, swa, ka, pa0, pa1;
   int al;
-  __device__ BlockRow(const Geo& g, int kind_, int i, int r, double alpha) : kind(kind_) {
+  // weights of the completion of body i (FP64 divisions: by one thread)
+  __device__ static float2 completion(const Geo& g, int kind, int i, double alpha) {
+    return make_float2(alpha > 0.0 ? (float)(alpha / g.len[i]) : 1.0f,
+                       kind == 1 ? (alpha > 0.0 ? (float)(alpha / g.W[i]) : 1.0f) : 0.f);
+  }
+  __device__ BlockRow(const Geo& g, int kind_, int i, int r, float2 weights) : kind(kind_) {
     const int a0 = g.body_start[i];
-    cf = alpha > 0.0 ? (float)(alpha / g.len[i]) : 1.0f;
-    ct = kind == 1 ? (alpha > 0.0 ? (float)(alpha / g.W[i]) : 1.0f) : 0.f;
+    cf = weights.x;
+    ct = weights.y;
     a = a0 + (kind == 1 ? r >> 1 : r);
     al = kind == 1 ? r & 1 : 0;
     pa = g.pf[a];
@@ -91,106 +96,167 @@ struct BlockRow {
     pa0 = (float)(-(g.y[a] - g.yc[i]));
     pa1 = (float)(g.x[a] - g.xc[i]);
   }
+  // 1/x to a rounding, without the branches of the division (which kept the entries of a
+  // row from overlapping: assembly 25,000 clocks at 256 rows)
+  __device__ static float reciprocal(float x) {
+    float y;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return fmaf(fmaf(-x, y, 1.0f), y, y);
+  }
   // column data: cp = (x_hi, y_hi, x_lo, y_lo), cw = (sqrt(w), p_1, p_2, node index)
-  __device__ float entry(int r, int c, float4 cp, float4 cw) const {
+  __device__ float entry(int r, int c, float4 cp, float4 cw) const {  // Laplace
     const int b = __float_as_int(cw.w);
-    const float swb = cw.x;
     const float rx = (pa.x - cp.x) + (pa.z - cp.z), ry = (pa.y - cp.y) + (pa.w - cp.w);
-    float k;
-    if (kind == 0) {
-      if (a == b) {
-        k = -ka * (float)kInv4Pi;
-      } else {
-        k = -(float)kInv2Pi * (rx * nxa + ry * nya) / (rx * rx + ry * ry);
-      }
-      return (r == c ? 0.5f : 0.f) + swa * swb * (k + cf);
-    }
-    const int be = c & 1;
-    if (a == b) {
-      const float t = al == 0 ? -nya : nxa, u = be == 0 ? -nya : nxa;
-      k = -0.5f * (float)kInvPi * ka * t * u;
-    } else {
-      const float r2 = rx * rx + ry * ry;
-      const float rn = rx * nxa + ry * nya;
-      k = -(float)kInvPi * (al == 0 ? rx : ry) * (be == 0 ? rx : ry) * rn / (r2 * r2);
-    }
-    const float pb = be == 0 ? cw.y : cw.z;
-    const float pa_ = al == 0 ? pa0 : pa1;
-    return (r == c ? 0.5f : 0.f) + swa * swb * (k + (al == be ? cf : 0.f) + ct * pa_ * pb);
+    const float i2 = reciprocal(a == b ? 1.f : rx * rx + ry * ry);
+    const float k = a == b ? -ka * (float)kInv4Pi : -(float)kInv2Pi * ((rx * nxa + ry * nya) * i2);
+    return (r == c ? 0.5f : 0.f) + swa * cw.x * (k + cf);
+  }
+  // Stokes: columns c (even) and c + 1, the two components of one node
+  __device__ float2 entry2(int r, int c, float4 cp, float4 cw) const {
+    const int b = __float_as_int(cw.w);
+    const float rx = (pa.x - cp.x) + (pa.z - cp.z), ry = (pa.y - cp.y) + (pa.w - cp.w);
+    const bool self = a == b;
+    const float i2 = reciprocal(self ? 1.f : rx * rx + ry * ry);
+    const float t = self ? -0.5f * (float)kInvPi * ka * (al == 0 ? -nya : nxa)
+                         : -(float)kInvPi * (al == 0 ? rx : ry) * ((rx * nxa + ry * nya) * i2);
+    const float k0 = t * (self ? -nya : rx * i2), k1 = t * (self ? nxa : ry * i2);
+    const float q = ct * (al == 0 ? pa0 : pa1), sw = swa * cw.x;
+    return make_float2((r == c ? 0.5f : 0.f) + sw * (k0 + (al == 0 ? cf : 0.f) + q * cw.y),
+                       (r == c + 1 ? 0.5f : 0.f) + sw * (k1 + (al == 1 ? cf : 0.f) + q * cw.z));
   }
 };
 
-// A_:j += F G_j for the local columns [j0, j1) of row r (F = this row of the
-// panel minus E_K, G_j = rows K of column j).
-__device__ __forceinline__ void rank_update(float* __restrict__ A, const float* __restrict__ G, int h, int ld, int r,
-                                            const float (&fr)[kPB], int j0, int j1) {
-  // G is [kPB][h] (panel row t of the local columns): one 16-byte load gives
-  // four columns of one row, added with packed FP32x2 multiply-adds; each
-  // column's terms in the order t = 0, 1, ..., as one column at a time
-  int j = j0;
-  for (; j < j1 && (j & 3); ++j) {
-    float acc = A[j * ld + r];
+constexpr int kRPT = 2;  // rows a thread of the update
+// Threads a row group of the update needs for nb rows, and column groups.
+__host__ __device__ __forceinline__ int gj_rows(int nb) { return (nb + 32 * kRPT - 1) / (32 * kRPT) * 32; }
+
+// A_:j = A_:j + F G_j (START and the rows with fresh set: A_:j = F G_j) for the local columns
+// j0, j0 + step, ... (four each) of the thread's rows.  G is [kPB][h]: one 16-byte load
+// gives four columns of one row and feeds 4 kRPT multiply-adds (a load takes the
+// shared-memory pipe four clocks; with one row a thread it bound the update, with four
+// the registers spill: 100 blocks of 256 223 us against 186); each column's terms in the
+// order t = 0, 1, ...
+// SHARE: the columns also go to out (column j at out + j nb).
+template <bool START, bool SHARE>
+__device__ __forceinline__ void rank_update(float* __restrict__ A, const float* __restrict__ G, int h, int ld, int row0,
+                                            int stride, int nb, int fresh, const float (&fr)[kRPT][kPB], int j0, int j1,
+                                            int step, float* __restrict__ out = nullptr) {
+#pragma unroll 1
+  for (int j = j0; j < j1; j += step) {
+    float2 a01[kRPT], a23[kRPT];
 #pragma unroll
-    for (int t = 0; t < kPB; ++t) acc = fmaf(fr[t], G[t * h + j], acc);
-    A[j * ld + r] = acc;
-  }
-  for (; j + 4 <= j1; j += 4) {
-    float2 a01 = make_float2(A[j * ld + r], A[(j + 1) * ld + r]);
-    float2 a23 = make_float2(A[(j + 2) * ld + r], A[(j + 3) * ld + r]);
+    for (int s = 0; s < kRPT; ++s) {
+      const int r = row0 + s * stride;
+      a01[s] = a23[s] = make_float2(0.f, 0.f);
+      if (!START && r < nb && !(fresh >> s & 1)) {
+        a01[s] = make_float2(A[j * ld + r], A[(j + 1) * ld + r]);
+        a23[s] = make_float2(A[(j + 2) * ld + r], A[(j + 3) * ld + r]);
+      }
+    }
 #pragma unroll
     for (int t = 0; t < kPB; ++t) {
       const float4 g = *reinterpret_cast<const float4*>(G + t * h + j);
-      const float2 f = make_float2(fr[t], fr[t]);
-      a01 = __ffma2_rn(f, make_float2(g.x, g.y), a01);
-      a23 = __ffma2_rn(f, make_float2(g.z, g.w), a23);
-    }
-    A[j * ld + r] = a01.x;
-    A[(j + 1) * ld + r] = a01.y;
-    A[(j + 2) * ld + r] = a23.x;
-    A[(j + 3) * ld + r] = a23.y;
-  }
-  for (; j < j1; ++j) {
-    float acc = A[j * ld + r];
 #pragma unroll
-    for (int t = 0; t < kPB; ++t) acc = fmaf(fr[t], G[t * h + j], acc);
-    A[j * ld + r] = acc;
+      for (int s = 0; s < kRPT; ++s) {
+        const float2 f = make_float2(fr[s][t], fr[s][t]);
+        a01[s] = __ffma2_rn(f, make_float2(g.x, g.y), a01[s]);
+        a23[s] = __ffma2_rn(f, make_float2(g.z, g.w), a23[s]);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < kRPT; ++s) {
+      const int r = row0 + s * stride;
+      if (r < nb) {
+        A[j * ld + r] = a01[s].x;
+        A[(j + 1) * ld + r] = a01[s].y;
+        A[(j + 2) * ld + r] = a23[s].x;
+        A[(j + 3) * ld + r] = a23[s].y;
+        if (SHARE) {
+          out[j * nb + r] = a01[s].x;
+          out[(j + 1) * nb + r] = a01[s].y;
+          out[(j + 2) * nb + r] = a23[s].x;
+          out[(j + 3) * nb + r] = a23[s].y;
+        }
+      }
+    }
   }
+}
+
+// Inverse of a 16 x 16 pivot block by one warp, in registers: lane t0 + 16 half holds
+// the columns 8 half + u of row t0.  Gauss-Jordan, the pivot row by shuffles, no
+// branches (100 clocks a pivot).  Every pivot is checked.
+__device__ __forceinline__ void invert_panel(float (&a)[kPB / 2], float* inv, float floor, int* bad) {
+  constexpr int H = kPB / 2;
+  const int lane = threadIdx.x & 31, t0 = lane & (kPB - 1), half = lane / kPB;
+  bool ok = true;
+#pragma unroll 1
+  for (int tb = 0; tb < 2; ++tb)
+#pragma unroll
+    for (int u0 = 0; u0 < H; ++u0) {
+      const int t = H * tb + u0;
+      const float pv = __shfl_sync(0xffffffffu, a[u0], t + kPB * tb);
+      const float m = __shfl_sync(0xffffffffu, a[u0], t0 + kPB * tb);
+      const float ip = __frcp_rn(pv);
+      ok &= fabsf(pv) >= floor && isfinite(pv);
+      const bool piv = t0 == t;
+      const float f = piv ? ip : -m * ip;
+#pragma unroll
+      for (int u = 0; u < H; ++u) {
+        const float q = __shfl_sync(0xffffffffu, a[u], t + kPB * half);
+        a[u] = fmaf(f, q, piv ? 0.f : a[u]);
+      }
+      if (half == tb) a[u0] = f;
+    }
+  if (!ok) *bad = 1;
+  float4* o = reinterpret_cast<float4*>(inv + t0 * kPB + H * half);
+  o[0] = make_float4(a[0], a[1], a[2], a[3]);
+  o[1] = make_float4(a[4], a[5], a[6], a[7]);
 }
 
 // Assembly and in-place inversion of one diagonal block by a cluster of CS CTAs
 // (CS = 1: one CTA).  CTA q holds the columns [q h, min(nb, (q+1) h)) and all
-// rows, one thread per row.  Blocked Gauss-Jordan without pivoting: for each
-// panel K of kPB pivots, the owning CTA eliminates the panel's own columns in
-// registers, after which its columns hold [inv(A_KK); -A_RK inv(A_KK)]; every
-// CTA then applies the rank-kPB update A_:j += (panel - E_K) A_Kj to its other
-// columns, reading the panel from the owner's shared memory.  The panel stays
-// unchanged until the owner's next update, which follows the next panel's
-// cluster barrier, which no CTA reaches before it is done reading.
-// Launch bounds per cluster size: one thread per row of the largest block the
-// instance takes; the clusters of four keep at least two CTAs of 448 threads
-// (three of 256) on an SM.
-template <int CS>
-__global__ void __launch_bounds__(CS == 1 ? kMaxSingle : CS == 4 ? kMaxBlock4 : kMaxThreads, CS == 4 ? 2 : 1)
-    k_bj_factor(Geo g, int kind, double alpha,
-                                                           const int* __restrict__ list,
-                                                           const long long* __restrict__ off,
-                                                           bj_t* __restrict__ blocks, float floor,
-                                                           int* __restrict__ fallbacks) {
-  extern __shared__ float sm[];
+// rows; T threads share the rows (kRPT each), and the groups of T threads the columns;
+// one more warp inverts.  Blocked Gauss-Jordan without pivoting, for each
+// panel K of kPB pivots: with I = inv(A_KK), G_j = I A_Kj, every CTA sets
+//   A_Rj -= A_RK G_j, A_Kj = G_j  (its columns j outside K),
+//   A_RK = -A_RK I, A_KK = I      (the panel's owner),
+// reading I from the owner's shared memory and A_RK through L2: the owner writes the
+// next panel to the place of the result in memory (two panels in turn; a cluster's
+// other CTAs read 20 bytes a clock together from one SM's shared memory, which was
+// 25,000 clocks a panel of 256 rows).  One cluster barrier a panel.
+// What bounds it is the chain of panels and the shared-memory pipe.  The serial part, I, is
+// 16 x 16 by one warp, formed one panel ahead: the warp adds this panel's update to the
+// 16 x 16 next pivots itself and inverts them while the others update.  (An
+// elimination of the whole panel by all rows took a block barrier and a division a
+// column, while the other CTAs waited.)  A panel of a block of 256 takes 10,000 clocks
+// (25,000 before).  Bodies of nb unknowns: four of 128 77 -> 43 us, 10,000 of 128 3085 ->
+// 2444; 100 of 256 213 -> 186, 400 of 256 748 -> 645; 236, 286, 482 and 482 560 -> 254.
+template <int CS, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS <= 160 ? 3 : CS == 1 ? 2 : 1)
+    k_bj_factor(Geo g, int kind, double alpha, const int* __restrict__ list, const long long* __restrict__ off,
+                bj_t* __restrict__ blocks, float floor, int* __restrict__ fallbacks, int T) {
+  extern __shared__ __align__(16) float sm[];
   __shared__ int bad_s;  // this CTA met a bad pivot or a non-finite entry
   const int rank = CS > 1 ? (int)cg::this_cluster().block_rank() : 0;
   const int i = list[blockIdx.x / CS];
   const int nb = (g.body_start[i + 1] - g.body_start[i]) * (kind + 1);
   const int ld = gj_ld(nb), h = gj_cols(nb, CS);
-  const int c0 = min(nb, rank * h), nc = min(nb, c0 + h) - c0;
-  float* A = sm;                 // ld x h, column-major
-  float* G = A + (size_t)ld * h; // kPB x h: rows K of the local columns
-  float* rowbuf = G + (size_t)h * kPB;  // [2][kPB] pivot rows of the panel steps
-  float4* colp = reinterpret_cast<float4*>(rowbuf + 2 * kPB);  // [h] column node positions
-  float4* colw = colp + h;                                       // [h] column node data
-  const int r = threadIdx.x;
-  const bool live = r < nb;
+  const int c0 = min(nb, rank * h), nc = min(nb, c0 + h) - c0, nc4 = (nc + 3) & ~3;
+  float* A = sm;                         // ld x h, column-major
+  float* G = A + (size_t)ld * h;         // kPB x h: G_j of the local columns
+  float* pub = G + (size_t)h * kPB;      // [2] I of this and the next panel (the owner's)
+  float* copy = pub + 2 * kPB * kPB;     // CS > 1: this CTA's copy of I
+  float4* colp = reinterpret_cast<float4*>(G);  // [h] column node positions (assembly)
+  float4* colw = colp + h;                      // [h] column node data
+  bj_t* B = blocks + off[i];
+  // CS > 1 (nb >= kMinCluster): the panels' exchange, 2 x 16 columns of 4 nb bytes of the 2 nb^2
+  float* xch = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(B) + 15) & ~uintptr_t(15));
+  const int work = blockDim.x - 32, CG = work / T;  // threads and column groups of the update
+  const bool inverter = (int)threadIdx.x >= work;
+  const int row0 = (int)threadIdx.x % T, cgrp = (int)threadIdx.x / T;  // (not the inverter's)
+  __shared__ float2 weights;
   if (threadIdx.x == 0) bad_s = 0;
+  if ((int)threadIdx.x == work) weights = BlockRow::completion(g, kind, i, alpha);
   {
     const int a0 = g.body_start[i];
     const double xc = g.xc[i], yc = g.yc[i];
@@ -202,79 +268,149 @@ __global__ void __launch_bounds__(CS == 1 ? kMaxSingle : CS == 4 ? kMaxBlock4 : 
     }
   }
   __syncthreads();
-  if (live) {
-    const BlockRow br(g, kind, i, r, alpha);
-    for (int j = 0; j < nc; ++j) A[j * ld + r] = br.entry(r, c0 + j, colp[j], colw[j]);
-  }
-  __syncthreads();
-  for (int k0 = 0; k0 < nb; k0 += kPB) {
-    const int bsz = min(kPB, nb - k0);
-    const int owner = k0 / h;
-    if (rank == owner) {
-      // panel elimination in registers: thread r holds row r of the panel
-      const int lj = k0 - c0;
-      float pr[kPB];
-#pragma unroll
-      for (int t = 0; t < kPB; ++t) pr[t] = (live && t < bsz) ? A[(lj + t) * ld + r] : 0.f;
-#pragma unroll
-      for (int t = 0; t < kPB; ++t) {
-        if (t < bsz) {
-          float* rb = rowbuf + (t & 1) * kPB;
-          if (r == k0 + t) {
-#pragma unroll
-            for (int u = 0; u < kPB; ++u) rb[u] = pr[u];
-          }
-          __syncthreads();
-          const float pv = rb[t];
-          if (threadIdx.x == 0 && !(fabsf(pv) >= floor && isfinite(pv))) bad_s = 1;
-          const float ip = 1.0f / pv;
-          if (r == k0 + t) {
-#pragma unroll
-            for (int u = 0; u < kPB; ++u) pr[u] = (u == t) ? ip : pr[u] * ip;
-          } else {
-            const float fr = pr[t] * ip;
-#pragma unroll
-            for (int u = 0; u < kPB; ++u) pr[u] = (u == t) ? -fr : fmaf(-fr, rb[u], pr[u]);
-          }
+  if (!inverter) {
+    // a row a thread, as many column groups as there are threads for
+    const int rows = (nb + 31) / 32 * 32, cgs = max(1, work / rows);
+    for (int q = threadIdx.x; q < cgs * rows; q += work) {
+      const int r = q % rows, cgp = q / rows;
+      if (r >= nb) continue;
+      const BlockRow br(g, kind, i, r, weights);
+      if (kind == 0) {
+#pragma unroll 4
+        for (int j = cgp; j < nc; j += cgs) A[j * ld + r] = br.entry(r, c0 + j, colp[j], colw[j]);
+      } else {
+#pragma unroll 4
+        for (int j = 2 * cgp; j < nc; j += 2 * cgs) {
+          const float2 e = br.entry2(r, c0 + j, colp[j], colw[j]);
+          A[j * ld + r] = e.x;
+          A[(j + 1) * ld + r] = e.y;
         }
       }
-      if (live) {
+      if (cgp == 0)
+        for (int j = nc; j < nc4; ++j) A[j * ld + r] = 0.f;
+    }
+  }
+  __syncthreads();
+  if (CS > 1 && rank == 0)
+    for (int e = threadIdx.x; e < min(kPB, nb) * nb; e += blockDim.x) xch[e] = A[e / nb * ld + e % nb];
+  // the inverter's lane: row t0, columns 8 half.. of a pivot block
+  const int t0 = threadIdx.x & (kPB - 1), uh = ((threadIdx.x & 31) / kPB) * (kPB / 2);
+  if (rank == 0 && inverter) {
+    float a[kPB / 2];
 #pragma unroll
-        for (int t = 0; t < kPB; ++t)
-          if (t < bsz) A[(lj + t) * ld + r] = pr[t];
-      }
-    }
-    // rows K of the local columns, before any of them changes
-    for (int e = threadIdx.x; e < nc * bsz; e += blockDim.x) {
-      const int j = e / bsz, t = e % bsz;
-      G[t * h + j] = A[j * ld + k0 + t];
-    }
+    for (int u = 0; u < kPB / 2; ++u) a[u] = t0 < nb && uh + u < nb ? A[(uh + u) * ld + t0] : (t0 == uh + u ? 1.f : 0.f);
+    invert_panel(a, pub, floor, &bad_s);
+  }
+  if constexpr (CS > 1)
+    cg::this_cluster().sync();
+  else
+    __syncthreads();
+  int parity = 0;
+  for (int k0 = 0; k0 < nb; k0 += kPB, parity ^= 1) {
+    const int bsz = min(kPB, nb - k0), owner = k0 / h, lj = k0 - c0;
+    const int k1 = k0 + kPB, n0 = k1 - c0;
+    const bool ahead = k1 < nb && k1 / h == rank;  // this CTA has the next panel
+    const float* P = CS > 1 ? xch + parity * kPB * nb : A + k0 * ld;
+    const int pld = CS > 1 ? nb : ld;
+    const auto panel = [&](int t, int r) { return CS > 1 ? __ldcg(P + t * pld + r) : P[t * pld + r]; };
+    const float* inv = pub + parity * kPB * kPB;
     if constexpr (CS > 1) {
-      cg::this_cluster().sync();
-    } else {
-      __syncthreads();
+      const float* I = cg::this_cluster().map_shared_rank(inv, owner);
+      for (int e = threadIdx.x; e < kPB * kPB; e += blockDim.x) copy[e] = I[e];
+      inv = copy;
     }
-    if (live) {
-      const float* P = A + (k0 - owner * h) * ld;  // the panel in the owner's shared memory
-      if constexpr (CS > 1) P = cg::this_cluster().map_shared_rank(P, owner);
-      float fr[kPB];
+    // the thread's rows of the panel, negated (rows K: the unit vectors, so that F G_j = G_j);
+    // the inverter: its row in fr[0] and the next pivot block.  Loads first, at clamped
+    // indexes, then selections: a load inside a condition is waited for one by one
+    float fr[kRPT][kPB], a[kPB / 2];
+    int fresh = 0;
+    if (!inverter) {
 #pragma unroll
-      for (int t = 0; t < kPB; ++t) fr[t] = t < bsz ? P[t * ld + r] - (r == k0 + t ? 1.f : 0.f) : 0.f;
-      // all local columns but the panel's own (owner: [k0 - c0, k0 - c0 + bsz))
-      const int s0 = rank == owner ? k0 - c0 : nc, s1 = rank == owner ? k0 - c0 + bsz : nc;
-      rank_update(A, G, h, ld, r, fr, 0, s0);
-      rank_update(A, G, h, ld, r, fr, s1, nc);
+      for (int s = 0; s < kRPT; ++s)
+#pragma unroll
+        for (int t = 0; t < kPB; ++t) fr[s][t] = panel(min(t, bsz - 1), min(row0 + s * T, nb - 1));
+#pragma unroll
+      for (int s = 0; s < kRPT; ++s) {
+        const int r = row0 + s * T;
+        const bool in = r >= k0 && r < k0 + bsz;
+        fresh |= in ? 1 << s : 0;
+#pragma unroll
+        for (int t = 0; t < kPB; ++t) fr[s][t] = in ? (r - k0 == t ? 1.f : 0.f) : t < bsz ? -fr[s][t] : 0.f;
+      }
+    } else if (ahead) {
+      const int r = min(k1 + t0, nb - 1);
+#pragma unroll
+      for (int t = 0; t < kPB; ++t) fr[0][t] = panel(t, r);  // (a panel with a next one is full)
+#pragma unroll
+      for (int u = 0; u < kPB / 2; ++u) a[u] = A[min(n0 + uh + u, nc - 1) * ld + r];
+#pragma unroll
+      for (int t = 0; t < kPB; ++t) fr[0][t] = k1 + t0 < nb ? -fr[0][t] : 0.f;
+#pragma unroll
+      for (int u = 0; u < kPB / 2; ++u)
+        if (k1 + t0 >= nb || n0 + uh + u >= nc) a[u] = t0 == uh + u ? 1.f : 0.f;
     }
     __syncthreads();
+    // G_j = I A_Kj (the panel's own columns: I), four rows of a column a thread
+    for (int e = threadIdx.x; e < 4 * nc4; e += blockDim.x) {
+      const int uq = e / nc4, j = e - uq * nc4;
+      const bool own = rank == owner && j >= lj && j < lj + bsz;
+      float c[kPB];
+#pragma unroll
+      for (int t = 0; t < kPB; ++t) c[t] = A[j * ld + k0 + min(t, bsz - 1)];
+#pragma unroll
+      for (int t = 0; t < kPB; ++t) c[t] = own ? (j - lj == t ? 1.f : 0.f) : t < bsz ? c[t] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float v = 0.f;
+#pragma unroll
+        for (int t = 0; t < kPB; t += 4) {
+          const float4 q = *reinterpret_cast<const float4*>(inv + (4 * uq + u) * kPB + t);
+          v = fmaf(q.w, c[t + 3], fmaf(q.z, c[t + 2], fmaf(q.y, c[t + 1], fmaf(q.x, c[t], v))));
+        }
+        G[(4 * uq + u) * h + j] = v;
+      }
+    }
+    __syncthreads();
+    // all local columns but the panel's own (owner: [lj, lj + kPB))
+    const int s0 = rank == owner ? lj : nc4, s1 = rank == owner ? min(nc4, lj + kPB) : nc4;
+    if (!inverter) {
+      int b0 = s0, b1 = s1;
+      if (CS > 1 && ahead) {
+        // the next panel's columns first; it follows this one where both are here
+        const int n1 = min(nc4, n0 + kPB);
+        rank_update<false, true>(A, G, h, ld, row0, T, nb, fresh, fr, n0 + 4 * cgrp, n1, 4 * CG,
+                                 xch + ((parity ^ 1) * kPB - n0) * nb);
+        b0 = min(s0, n0);
+        b1 = n1;
+      }
+      rank_update<false, false>(A, G, h, ld, row0, T, nb, fresh, fr, 4 * cgrp, b0, 4 * CG);
+      rank_update<false, false>(A, G, h, ld, row0, T, nb, fresh, fr, b1 + 4 * cgrp, nc4, 4 * CG);
+    } else if (ahead) {
+#pragma unroll
+      for (int t = 0; t < kPB; ++t)
+#pragma unroll
+        for (int u = 0; u < kPB / 2; ++u) {
+          const float q = G[t * h + min(n0 + uh + u, nc - 1)];
+          a[u] = fmaf(n0 + uh + u < nc ? fr[0][t] : 0.f, q, a[u]);
+        }
+      invert_panel(a, pub + (parity ^ 1) * kPB * kPB, floor, &bad_s);
+    }
+    // the panel (every thread read its rows before the barriers above)
+    if (!inverter && rank == owner) rank_update<true, false>(A, G, h, ld, row0, T, nb, fresh, fr, s0 + 4 * cgrp, s1, 4 * CG);
+    if constexpr (CS > 1)
+      cg::this_cluster().sync();
+    else
+      __syncthreads();
   }
   // an entry that overflowed in the updates, or whose W = B^{-1} - 2I entry
   // lies outside FP16's range, also rejects the block
-  if (live) {
+  if (!inverter) {
     bool nf = false;
-    for (int j = 0; j < nc; ++j) {
-      const float a = A[j * ld + r] - (c0 + j == r ? kBjShift : 0.f);
-      nf |= !(fabsf(a) <= 65000.f);
-    }
+    for (int r = row0; r < nb; r += T)
+      for (int j = cgrp; j < nc; j += CG) {
+        const float a = A[j * ld + r] - (c0 + j == r ? kBjShift : 0.f);
+        nf |= !(fabsf(a) <= 65000.f);
+      }
     if (nf) bad_s = 1;
   }
   // every CTA of the cluster learns whether any of them rejected the block
@@ -290,11 +426,12 @@ __global__ void __launch_bounds__(CS == 1 ? kMaxSingle : CS == 4 ? kMaxBlock4 : 
     bad = bad_s;
   }
   if (bad && rank == 0 && threadIdx.x == 0) atomicAdd(fallbacks, 1);
-  bj_t* B = blocks + off[i];
-  if (live)
-    for (int j = 0; j < nc; ++j) {
-      const float d = c0 + j == r ? kBjShift : 0.f;  // W = B^{-1} - 2I; the identity: W = -I
-      B[(long long)(c0 + j) * nb + r] = __float2half_rn(bad ? (c0 + j == r ? 1.f : 0.f) - d : A[j * ld + r] - d);
+  if (inverter) return;
+  for (int r = row0; r < nb; r += T)
+    for (int j = cgrp; j < nc; j += CG) {
+      const bool diag = c0 + j == r;
+      const float d = diag ? kBjShift : 0.f;  // W = B^{-1} - 2I; the identity: W = -I
+      B[(long long)(c0 + j) * nb + r] = __float2half_rn(bad ? (diag ? 1.f : 0.f) - d : A[j * ld + r] - d);
     }
 }
 
@@ -425,14 +562,18 @@ long long bj_block_floats(const int* body_start_host, int N, int kind) {
 
 namespace {
 
-// Launch of k_bj_factor<CS> over count bodies of list, one thread per row.
+// Launch of k_bj_factor<CS, THREADS> over count bodies of list.
 float g_pivot_floor = 0.f;  // test hook (0: the default floor)
 constexpr float kPivotFloor = 1e-3f;
 
-template <int CS>
-cudaError_t launch_factor(const Geo& g, int kind, double alpha, const int* list, int count, int threads, size_t smem,
+template <int CS, int THREADS>
+cudaError_t launch_factor(const Geo& g, int kind, double alpha, const int* list, int count, int max_nb, size_t smem,
                           const long long* off, bj_t* blocks, int* fallbacks, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_bj_factor<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the update's threads, and one warp for the pivots (column groups read the panel each:
+  // nb = 256 in clusters of four 186 us for 100 bodies with one, 334 with two; nb <= 446, 155 bodies,
+  // 1296 and 895; clusters of eight have no registers for two: 32 bodies of 512 731 and 790)
+  const int T = gj_rows(max_nb), groups = T > 128 ? (CS == 4 ? 2 : 1) : (CS == 1 ? 256 : 128) / T, threads = groups * T + 32;
+  cudaError_t e = cudaFuncSetAttribute(k_bj_factor<CS, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(CS * count);
@@ -447,7 +588,7 @@ cudaError_t launch_factor(const Geo& g, int kind, double alpha, const int* list,
   cfg.attrs = attr;
   cfg.numAttrs = CS > 1 ? 1 : 0;
   const float floor = g_pivot_floor > 0.f ? g_pivot_floor : kPivotFloor;
-  e = cudaLaunchKernelEx(&cfg, k_bj_factor<CS>, g, kind, alpha, list, off, blocks, floor, fallbacks);
+  e = cudaLaunchKernelEx(&cfg, k_bj_factor<CS, THREADS>, g, kind, alpha, list, off, blocks, floor, fallbacks, T);
   note_launches(1);
   return e;
 }
@@ -458,8 +599,20 @@ void set_bj_pivot_floor(double floor) { g_pivot_floor = floor > 0.0 ? (float)flo
 
 cudaError_t bj_setup(const Geo& g, int kind, double alpha, const int* body_start_host, long long* off_dev,
                      int* list_dev, bj_t* blocks, int* fallbacks, cudaStream_t s) {
-  // bodies by kernel: one CTA (nb <= 128), clusters of four (<= 448) and eight (<= 640) CTAs
-  constexpr int kCs[3] = {1, 4, 8};
+  // Bodies by kernel: one CTA (nb <= 128), clusters of four (<= 448) and eight (<= 640) CTAs.
+  // Few bodies take larger clusters, and one launch: four of nb = 128 45 us in clusters of
+  // four against 70 in single CTAs; nb = 236, 286, 482, 482 254 us in one launch of
+  // clusters of eight against 158 + 254 in two.
+  int large = 0, small = 0, min_nb = kMaxBlock;
+  for (int i = 0; i < g.N; ++i) {
+    const int nb = (body_start_host[i + 1] - body_start_host[i]) * (kind + 1);
+    large += nb > kMaxSingle && nb <= kMaxBlock;
+    small += nb <= kMaxSingle;
+    if (nb <= kMaxSingle) min_nb = std::min(min_nb, nb);
+  }
+  const int sms = device_sms();
+  const int max4 = 8 * large <= sms ? kMaxSingle : kMaxBlock4;
+  const int kCs[3] = {4 * small <= sms && min_nb >= kMinCluster ? 4 : 1, 4, 8};
   std::vector<long long> off(g.N + 1, 0);
   std::vector<int> lists[3];
   int max_nb[3] = {0, 0, 0};
@@ -467,7 +620,7 @@ cudaError_t bj_setup(const Geo& g, int kind, double alpha, const int* body_start
   for (int i = 0; i < g.N; ++i) {
     const int nb = (body_start_host[i + 1] - body_start_host[i]) * (kind + 1);
     off[i + 1] = off[i] + (nb <= kMaxBlock ? (long long)nb * nb : 0);
-    const int c = nb <= kMaxSingle ? 0 : nb <= kMaxBlock4 ? 1 : nb <= kMaxBlock ? 2 : -1;
+    const int c = nb <= kMaxSingle ? 0 : nb <= max4 ? 1 : nb <= kMaxBlock ? 2 : -1;
     if (c < 0) continue;
     lists[c].push_back(i);
     max_nb[c] = std::max(max_nb[c], nb);
@@ -487,11 +640,12 @@ cudaError_t bj_setup(const Geo& g, int kind, double alpha, const int* body_start
   for (int c = 0; c < 3; ++c) {
     const int count = (int)lists[c].size();
     if (count == 0) continue;
-    const int threads = (max_nb[c] + 31) / 32 * 32;
     const int* l = list_dev + at;
-    e = c == 0   ? launch_factor<1>(g, kind, alpha, l, count, threads, smem[c], off_dev, blocks, fallbacks, s)
-        : c == 1 ? launch_factor<4>(g, kind, alpha, l, count, threads, smem[c], off_dev, blocks, fallbacks, s)
-                 : launch_factor<8>(g, kind, alpha, l, count, threads, smem[c], off_dev, blocks, fallbacks, s);
+    const auto launch = kCs[c] == 1                 ? launch_factor<1, 288>
+                        : kCs[c] == 8               ? launch_factor<8, 352>
+                        : gj_rows(max_nb[c]) <= 128 ? launch_factor<4, 160>
+                                                    : launch_factor<4, 480>;
+    e = launch(g, kind, alpha, l, count, max_nb[c], smem[c], off_dev, blocks, fallbacks, s);
     if (e != cudaSuccess) return e;
     at += count;
   }

@@ -1,6 +1,7 @@
 """The FP32 Arnoldi step of the refinement's inner solves in its three forms: blocks
 fetched into shared memory (fewer bodies than SMs), one body a CTA without the
-fetch, and more bodies than CTAs; block sizes that the fetch takes and leaves
+fetch, and more bodies than CTAs (with the clusters of the block inversion for
+few and for many bodies); block sizes that the fetch takes and leaves
 (bytes no multiple of 16, above 313 rows, above the largest block), against the
 oracle or, with hundreds of bodies, the FP64 solve."""
 import numpy as np
@@ -52,7 +53,7 @@ def test_blocks(kind, counts):
         assert e <= TOL_SOLVE
 
 
-@pytest.mark.parametrize("kind,rows,cols,n", [(0, 10, 15, 32), (0, 8, 19, 32), (0, 20, 20, 32), (1, 25, 25, 16),
+@pytest.mark.parametrize("kind,rows,cols,n", [(0, 10, 15, 32), (0, 8, 19, 32), (0, 20, 20, 32), (1, 25, 25, 16), (0, 4, 6, 160), (1, 4, 6, 130),
                                               (1, 10, 15, 40)])
 def test_many_bodies(kind, rows, cols, n):
     if not torch.cuda.is_available():
