@@ -3,8 +3,11 @@
 // passes off the per-iteration hot loop.
 #include <math.h>
 
+#include <algorithm>
+
 #include "bie_internal.cuh"
 #include "logtab.cuh"
+#include "pair_math.cuh"
 #include "reduce.cuh"
 
 namespace bie {
@@ -326,35 +329,49 @@ __global__ void __launch_bounds__(kB) k_out_lap(Geo g, const double* __restrict_
 
 // Stokes single layer (Stokeslet G_ij = (1/4pi)[-log r d_ij + r_i r_j / r^2]) at
 // the three stencil points of body i: t = 3i + s, s = 0: z0, 1: z0 + delta e1,
-// 2: z0 + delta e2.
+// 2: z0 + delta e2.  Bound by the FP64 pipe.  A block sums all three, which share the
+// source's strength and two of the four coordinate differences; with a reciprocal of
+// three operations (rcp64) for the division 30 FP64 operations a pair in place of 43.
+// 1,200 targets, 51,200 sources: MEASURE_OS.
 __global__ void __launch_bounds__(kB) k_out_stk(Geo g, const double* __restrict__ v,
                                                 double* __restrict__ part, int P) {
   __shared__ double sh[kB / 32];
   __shared__ double2 ltab[kLogTab];
   log_table_fill(ltab);
   __syncthreads();
-  const int t = blockIdx.x, p = blockIdx.y;
-  const int i = t / 3, s = t % 3;
+  const int i = blockIdx.x, p = blockIdx.y;
   const double d = g.delta[i];
-  const double zx = g.zx[i] + (s == 1 ? d : 0.0), zy = g.zy[i] + (s == 2 ? d : 0.0);
+  const double zx = g.zx[i], zy = g.zy[i], zxd = zx + d, zyd = zy + d;
   const int s0 = g.prange ? g.prange[i].x : 0, s1 = g.prange ? g.prange[i].y : g.M;
   const int chunk = (s1 - s0 + P - 1) / P;
   const int b0 = s0 + p * chunk, b1 = min(s1, b0 + chunk);
-  double u1 = 0.0, u2 = 0.0;
+  double l1[3] = {0.0, 0.0, 0.0}, l2[3] = {0.0, 0.0, 0.0};  // sums of log r^2 f
+  double u1[3] = {0.0, 0.0, 0.0}, u2[3] = {0.0, 0.0, 0.0};  // sums of r (r . f) / r^2
   for (int b = b0 + threadIdx.x; b < b1; b += kB) {
-    const double rx = zx - g.x[b], ry = zy - g.y[b];
-    const double r2 = rx * rx + ry * ry;
-    const double f1 = g.sw[b] * v[2 * b], f2 = g.sw[b] * v[2 * b + 1];
-    const double lg = -0.5 * log_tab(r2, ltab);
-    const double c = (rx * f1 + ry * f2) / r2;
-    u1 += lg * f1 + c * rx;
-    u2 += lg * f2 + c * ry;
+    const double bx = g.x[b], by = g.y[b], sw = g.sw[b];
+    const double2 vb = reinterpret_cast<const double2*>(v)[b];
+    const double f1 = sw * vb.x, f2 = sw * vb.y;
+    const double rx = zx - bx, ry = zy - by, rxd = zxd - bx, ryd = zyd - by;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      const double qx = s == 1 ? rxd : rx, qy = s == 2 ? ryd : ry;
+      const double r2 = fma(qx, qx, qy * qy);
+      const double lg = log_tab(r2, ltab);
+      const double c = fma(qx, f1, qy * f2) * rcp64(r2);
+      l1[s] = fma(lg, f1, l1[s]);
+      l2[s] = fma(lg, f2, l2[s]);
+      u1[s] = fma(c, qx, u1[s]);
+      u2[s] = fma(c, qy, u2[s]);
+    }
   }
-  u1 = block_sum<kB>(u1, sh);
-  u2 = block_sum<kB>(u2, sh);
-  if (threadIdx.x == 0) {
-    part[((long long)p * 3 * g.N + t) * 2] = u1;
-    part[((long long)p * 3 * g.N + t) * 2 + 1] = u2;
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    const double a1 = block_sum<kB>(fma(-0.5, l1[s], u1[s]), sh), a2 = block_sum<kB>(fma(-0.5, l2[s], u2[s]), sh);
+    if (threadIdx.x == 0) {
+      double* o = part + ((long long)p * 3 * g.N + 3 * i + s) * 2;
+      o[0] = a1;
+      o[1] = a2;
+    }
   }
 }
 
@@ -453,8 +470,10 @@ cudaError_t incident_density_scaled(const Geo& g, int kind, const double* load, 
 }
 
 int output_splits(const Geo& g, int kind) {
-  const int targets = kind == 0 ? g.N : 3 * g.N;
-  int P = (4 * device_sms() + targets - 1) / targets;
+  // blocks (a body's three Stokes targets are one): four an SM, Stokes, whose blocks are
+  // three times as long, eight, so that the last ones leave no SM much longer than the mean
+  int P = ((kind == 0 ? 4 : 8) * device_sms() + g.N - 1) / g.N;
+  if (kind == 1 && P > 12) P = std::max(12, (4 * device_sms() + 3 * g.N - 1) / (3 * g.N));  // one thread adds the splits
   const int maxP = (g.M + 255) / 256;
   if (P > maxP) P = maxP;
   if (P < 1) P = 1;
@@ -488,7 +507,7 @@ cudaError_t evaluate_output(const Geo& g, int kind, const double* v, const doubl
   if (kind == 0)
     k_out_lap<<<dim3(g.N, P), kB, 0, s>>>(g, v, partial, P);
   else
-    k_out_stk<<<dim3(3 * g.N, P), kB, 0, s>>>(g, v, partial, P);
+    k_out_stk<<<dim3(g.N, P), kB, 0, s>>>(g, v, partial, P);
   note_launches(1);
   return finalize_output(g, kind, v, load, partial, P, out, cres, s);
 }

@@ -32,8 +32,8 @@ __device__ __forceinline__ void log_table_fill(double2* tab) {
 }
 
 __device__ __forceinline__ double log_tab(double x, const double2* tab) {
-  if (!(x >= 2.2250738585072014e-308) || !(x <= 1.7976931348623157e308)) return log(x);
   const int hi = __double2hiint(x), lo = __double2loint(x);
+  if ((unsigned)hi - 0x00100000u >= 0x7fe00000u) return log(x);  // not positive, normal and finite
   const int e = ((hi >> 20) & 0x7ff) - 1023;
   const int j = (hi >> 13) & 0x7f;
   const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, lo);
