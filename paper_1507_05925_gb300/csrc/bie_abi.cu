@@ -2,6 +2,7 @@
 // drivers (restarted GMRES in FP64, and FP64 iterative refinement around
 // GMRES with FP32 pair sums).  Every step of the path runs in the kernels of
 // this library; the host only orders launches and reads the convergence state.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -139,6 +140,65 @@ bool foreign_device_ptr(const void* p, int dev) {
   }
   return at.type == cudaMemoryTypeDevice && at.device != dev;
 }
+
+// Where the arrays of one call lie.  A batch passes about ten arrays a problem, most of
+// them in a few allocations (a caller's memory pool), and a query takes 0.3 us: each
+// allocation of device memory is asked about once, with its address range, which
+// answers for the call's other arrays in it.  Everything else (host memory, managed
+// memory, a range that cannot be had) is asked about array by array.
+class PtrQuery {
+ public:
+  bool device(const void* p) {
+    const Range* r = range(p);
+    return r ? true : is_device_ptr(p);
+  }
+  bool foreign(const void* p, int dev) {
+    if (!p) return false;
+    const Range* r = range(p);
+    return r ? r->dev != dev : foreign_device_ptr(p, dev);
+  }
+
+ private:
+  struct Range {
+    uintptr_t lo, hi;
+    int dev;
+  };
+  using Fn = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static Fn entry() {
+    static const Fn fn = [] {
+      void* f = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+          q != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        f = nullptr;
+      }
+      return reinterpret_cast<Fn>(f);
+    }();
+    return fn;
+  }
+  const Range* range(const void* p) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    for (const Range& r : ranges_)
+      if (a >= r.lo && a < r.hi) return &r;
+    const Fn fn = entry();
+    if (!fn || !p) return nullptr;
+    CUpointer_attribute at[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                 CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned type = 0, managed = 1;
+    int dev = -1;
+    unsigned long long lo = 0;
+    size_t size = 0;
+    void* out[5] = {&type, &dev, &managed, &lo, &size};
+    if (fn(5, at, out, a) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || (managed & 0xff) || dev < 0 || a < lo ||
+        a - lo >= size)
+      return nullptr;
+    ranges_.push_back(Range{(uintptr_t)lo, (uintptr_t)(lo + size), dev});
+    return &ranges_.back();
+  }
+  std::vector<Range> ranges_;
+};
 
 int check_local(bie_ctx* ctx, std::initializer_list<const void*> ptrs, const char* what) {
   for (const void* p : ptrs)
@@ -437,7 +497,7 @@ struct BatchIn {
 // Stage the problems one after another (host or device inputs) and the tables
 // that keep every pair and output sum inside its own problem.
 int batch_setup(bie_ctx* ctx, const BatchIn& b, const std::vector<int>& bs, const std::vector<int>& pb,
-                bool ipt, Work& w, cudaStream_t s) {
+                bool ipt, Work& w, PtrQuery& where, cudaStream_t s) {
   const int N = (int)bs.size() - 1, P = b.P, c = w.kind + 1;
   const long long M = bs[N];
   const int per = w.kind == 0 ? 1 : 3;  // load entries per body
@@ -453,7 +513,7 @@ int batch_setup(bie_ctx* ctx, const BatchIn& b, const std::vector<int>& bs, cons
   std::vector<CopySeg> segs;
   auto take = [&](int slot, const double* src, double* to, long long count, long long pack_at) {
     if (count <= 0) return;
-    if (is_device_ptr(src)) {
+    if (where.device(src)) {
       segs.push_back(CopySeg{src, to, 2 * count});
     } else {
       if (pack.empty()) pack.resize(load_off + (size_t)per * N);
@@ -542,19 +602,22 @@ int batch_setup(bie_ctx* ctx, const BatchIn& b, const std::vector<int>& bs, cons
 // body_start (body offsets) and first body of each problem.  Device body_start
 // arrays are gathered by one kernel and read back once.
 int validate_batch(bie_ctx* ctx, const BatchIn& b, std::vector<int>& bs, std::vector<int>& pb, bool& has_ipt,
-                   cudaStream_t s) {
+                   PtrQuery& where, cudaStream_t s) {
   const int P = b.P;
   std::vector<long long> roff(P + 1, 0);
+  const auto who = [](int p) { return "problem " + std::to_string(p) + ": "; };
   for (int p = 0; p < P; ++p) {
     const bie_geometry& g = b.geoms[p];
-    const std::string who = "problem " + std::to_string(p) + ": ";
-    if (g.n_bodies < 1) return fail(ctx, BIE_ERR_INVALID, who + "n_bodies must be >= 1");
+    if (g.n_bodies < 1) return fail(ctx, BIE_ERR_INVALID, who(p) + "n_bodies must be >= 1");
     if (!g.body_start || !g.x || !g.y || !g.dx || !g.dy || !g.ddx || !g.ddy)
-      return fail(ctx, BIE_ERR_INVALID, who + "a geometry array is NULL");
-    if (!b.loads[p] || !b.outs[p]) return fail(ctx, BIE_ERR_INVALID, who + "a load or output is NULL");
-    if (int rc = check_local(ctx, {g.body_start, g.x, g.y, g.dx, g.dy, g.ddx, g.ddy, g.interior_pt, b.loads[p],
-                                   b.outs[p]}, (who + "an array").c_str()))
-      return rc;
+      return fail(ctx, BIE_ERR_INVALID, who(p) + "a geometry array is NULL");
+    if (!b.loads[p] || !b.outs[p]) return fail(ctx, BIE_ERR_INVALID, who(p) + "a load or output is NULL");
+    for (const void* q : {(const void*)g.body_start, (const void*)g.x, (const void*)g.y, (const void*)g.dx,
+                          (const void*)g.dy, (const void*)g.ddx, (const void*)g.ddy, (const void*)g.interior_pt,
+                          (const void*)b.loads[p], (const void*)b.outs[p]})
+      if (where.foreign(q, ctx->device))
+        return fail(ctx, BIE_ERR_INVALID,
+                    who(p) + "an array is device memory of another device than the context's");
     if (p > 0 && (g.interior_pt != nullptr) != has_ipt)
       return fail(ctx, BIE_ERR_INVALID, "batch: interior points for all problems or for none");
     has_ipt = g.interior_pt != nullptr;
@@ -566,7 +629,7 @@ int validate_batch(bie_ctx* ctx, const BatchIn& b, std::vector<int>& bs, std::ve
   std::vector<int> on_device;
   for (int p = 0; p < P; ++p) {
     const bie_geometry& g = b.geoms[p];
-    if (is_device_ptr(g.body_start)) {
+    if (where.device(g.body_start)) {
       segs.push_back(CopySeg{g.body_start, nullptr, g.n_bodies + 1});
       on_device.push_back(p);
     } else {
@@ -592,11 +655,10 @@ int validate_batch(bie_ctx* ctx, const BatchIn& b, std::vector<int>& bs, std::ve
   for (int p = 0; p < P; ++p) {
     const int* q = raw.data() + roff[p];
     const int Np = b.geoms[p].n_bodies;
-    const std::string who = "problem " + std::to_string(p) + ": ";
-    if (q[0] != 0) return fail(ctx, BIE_ERR_INVALID, who + "body_start[0] must be 0");
+    if (q[0] != 0) return fail(ctx, BIE_ERR_INVALID, who(p) + "body_start[0] must be 0");
     for (int i = 0; i < Np; ++i)
       if (q[i + 1] - q[i] < 8)
-        return fail(ctx, BIE_ERR_INVALID, who + "body " + std::to_string(i) + " has fewer than 8 nodes");
+        return fail(ctx, BIE_ERR_INVALID, who(p) + "body " + std::to_string(i) + " has fewer than 8 nodes");
     const int off = bs.back();
     if ((long long)off + q[Np] > 0x3fffffffLL) return fail(ctx, BIE_ERR_INVALID, "batch: too many nodes");
     for (int i = 1; i <= Np; ++i) bs.push_back(off + q[i]);
@@ -1010,12 +1072,13 @@ int solve_common(bie_ctx* ctx, const bie_geometry* geom, int kind, const double*
   std::vector<int> bs, pb;
   bool has_ipt = false;
   int rc;
+  PtrQuery where;  // batches
   if (batch) {
     if (!ctx) return BIE_ERR_INVALID;
     if (batch->P < 1 || batch->P > 65535 || !batch->geoms || !batch->loads || !batch->outs)
       return fail(ctx, BIE_ERR_INVALID, "batch: count outside 1..65535 or a NULL array");
     if (density) return fail(ctx, BIE_ERR_INVALID, "batch: no density output");
-    if ((rc = validate_batch(ctx, *batch, bs, pb, has_ipt, s))) return rc;
+    if ((rc = validate_batch(ctx, *batch, bs, pb, has_ipt, where, s))) return rc;
   } else {
     if ((rc = validate(ctx, geom, bs))) return rc;
     if (!load || !out) return fail(ctx, BIE_ERR_INVALID, "load or output pointer is NULL");
@@ -1059,7 +1122,7 @@ int solve_common(bie_ctx* ctx, const bie_geometry* geom, int kind, const double*
       })))
     return rc;
   if (batch) {
-    if ((rc = batch_setup(ctx, *batch, bs, pb, has_ipt, w, s))) return rc;
+    if ((rc = batch_setup(ctx, *batch, bs, pb, has_ipt, w, where, s))) return rc;
   } else if ((rc = setup(ctx, geom, bs, w, s))) {
     return rc;
   }
@@ -1294,7 +1357,7 @@ int solve_common(bie_ctx* ctx, const bie_geometry* geom, int kind, const double*
     const int per = kind == 0 ? 1 : 3;
     for (int p = 0; p < P; ++p) {
       const long long nl = (long long)(pb[p + 1] - pb[p]) * per;
-      if (is_device_ptr(batch->outs[p]))
+      if (where.device(batch->outs[p]))
         segs.push_back(CopySeg{w.outv + (long long)pb[p] * per, batch->outs[p], 2 * nl});
       else
         on_host.push_back(p);
