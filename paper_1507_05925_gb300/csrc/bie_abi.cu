@@ -317,13 +317,13 @@ void carve(Arena& A, Work& w, int N, int M, int kind, int m, bool solve, bool st
     w.io_in = A.take<double>(n);
     w.io_out = A.take<double>(n);
   }
+  // compact: without the symmetric plans that trade partial slots for time
+  const int slots = compact ? 0 : kAnySlots;
   if (nprob > 1) {
-    w.plan64 = plan_pairs_batch(bs, N, pb, nprob, kind, 0);
-    w.plan32 = plan_pairs_batch(bs, N, pb, nprob, kind, 1);
-    w.planff = plan_pairs_batch(bs, N, pb, nprob, kind, 2);
+    w.plan64 = plan_pairs_batch(bs, N, pb, nprob, kind, 0, slots);
+    w.plan32 = plan_pairs_batch(bs, N, pb, nprob, kind, 1, slots);
+    w.planff = plan_pairs_batch(bs, N, pb, nprob, kind, 2, slots);
   } else {
-    // compact: without the symmetric plans that trade partial slots for time
-    const int slots = compact ? 0 : kAnySlots;
     w.plan64 = plan_pairs(M, kind, 0, slots);
     w.plan32 = plan_pairs(M, kind, 1, slots);
     w.planff = plan_pairs(M, kind, 2, slots);

@@ -197,7 +197,8 @@ void set_tuned_plan(int M, int kind, int precision, const PairPlan& p);
 void forget_tuned_plan(int M, int kind, int precision);
 void clear_tuned_splits();
 // batched solves (host arrays: body_start [N+1], first body of each problem [P+1])
-PairPlan plan_pairs_batch(const int* body_start, int N, const int* pbody, int P, int kind, int precision);
+PairPlan plan_pairs_batch(const int* body_start, int N, const int* pbody, int P, int kind, int precision,
+                          int max_slots);
 cudaError_t pair_sum(const Geo& g, int kind, int precision, const PairPlan& p, VecRef v,
                      const double* sscale, double* partial, const int* stop, cudaStream_t s);
 

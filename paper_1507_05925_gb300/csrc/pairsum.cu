@@ -606,15 +606,15 @@ __device__ __forceinline__ void sym_flush(float4* __restrict__ sAcc, float2* AX,
   for (int h = 0; h < H; ++h) AX[h] = AY[h] = make_float2(0.f, 0.f);
 }
 
-// The sources' sums [warps][TS] of tile B into their slots: the warps in order,
-// error-free.
+// The sources' sums [warps][TS] of tile B (nodes below end) into their slots: the warps
+// in order, error-free.
 template <int KIND>
-__device__ __forceinline__ void sym_write_sources(const Geo& g, int B0, int TS, int slot,
+__device__ __forceinline__ void sym_write_sources(const Geo& g, int B0, int TS, int end, int slot,
                                                   const float2* __restrict__ accB, double* __restrict__ partial) {
   __syncthreads();
   for (int l = threadIdx.x; l < TS; l += blockDim.x) {
     const int b = B0 + l;
-    if (b >= g.M) continue;
+    if (b >= end) continue;
     float2 u = accB[l];
     float ex = 0.f, ey = 0.f;
     for (int w = 1; w < (int)blockDim.x / 32; ++w) {
@@ -635,12 +635,20 @@ __host__ __device__ constexpr size_t sym32_smem(int threads) {
   return TS * (16 + 16 + 8 + (KIND == 1 ? 8 + 16 : 0)) + (threads / 32) * TS * 8 + TS / 32 * (16 + 4);
 }
 
-template <int KIND, int H>
+// BATCH: problem blockIdx.y, its nodes cut into tiles by themselves (so no pair crosses
+// problems, and no mask is needed); a problem has as many slots as tiles.
+template <int KIND, int H, bool BATCH>
 __global__ void __launch_bounds__(64, KIND == 0 ? 10 : (H == 2 ? 8 : 6)) k_pair32s(Geo g, double* __restrict__ partial,
                                                                       const int* __restrict__ stop) {
   if (stop && *stop) return;
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  const int M = g.M, B = blockDim.x, TS = 2 * H * B, G = TS / 32;
+  const int B = blockDim.x, TS = 2 * H * B, G = TS / 32;
+  int n0 = 0, M = g.M;  // the nodes [n0, M)
+  if (BATCH) {
+    const int2 r = g.prange[g.pbody[blockIdx.y]];
+    n0 = r.x;
+    M = r.y;
+  }
   float4* sF = reinterpret_cast<float4*>(sm_raw);  // far: (-x', -y', q1, q2)
   float4* sH = sF + TS;                            // near: (-x_hi, -y_hi, q1, q2)
   float4* sBox = sH + TS;                          // [G]
@@ -651,8 +659,18 @@ __global__ void __launch_bounds__(64, KIND == 0 ? 10 : (H == 2 ? 8 : 6)) k_pair3
   int* sFar = reinterpret_cast<int*>(sN + (KIND == 1 ? TS : 0));  // [G]
   int ti, tj;
   tri_decode(blockIdx.x, ti, tj);
-  const int A0 = ti * TS, B0 = tj * TS;
+  const int A0 = n0 + ti * TS, B0 = n0 + tj * TS;
   const int t = threadIdx.x;
+  if (BATCH) {
+    if (B0 >= M) return;  // fewer tiles than the largest problem
+    if (g.ps && g.ps[blockIdx.y].stop_j <= *g.jstep) {  // stopped: zero partials, as the directed kernel
+      for (int l = t; l < TS; l += B) {
+        if (A0 + l < M) write_slot<KIND>(g, A0 + l, tj, 0.f, 0.f, 0.f, 0.f, partial);
+        if (ti != tj && B0 + l < M) write_slot<KIND>(g, B0 + l, ti, 0.f, 0.f, 0.f, 0.f, partial);
+      }
+      return;
+    }
+  }
   if constexpr (KIND == 0) {
     // Laplace: tiles whose whole boxes are far (bodies of whole tiles, or in
     // spatial order) need one centre: no per-group targets
@@ -683,7 +701,7 @@ __global__ void __launch_bounds__(64, KIND == 0 ? 10 : (H == 2 ? 8 : 6)) k_pair3
       for (int k = 0; k < 2 * H; ++k)
         write_slot<0>(g, A0 + t + k * B, tj, k & 1 ? AX[k >> 1].y : AX[k >> 1].x, 0.f,
                       k & 1 ? AY[k >> 1].y : AY[k >> 1].x, 0.f, partial);
-      sym_write_sources<0>(g, B0, TS, ti, accB, partial);
+      sym_write_sources<0>(g, B0, TS, M, ti, accB, partial);
       return;
     }
   }
@@ -814,22 +832,22 @@ __global__ void __launch_bounds__(64, KIND == 0 ? 10 : (H == 2 ? 8 : 6)) k_pair3
       write_slot<1>(g, a, tj, c.x, c.y, c.z, c.w, partial);
     }
   }
-  if (ti != tj) sym_write_sources<KIND>(g, B0, TS, ti, accB, partial);
+  if (ti != tj) sym_write_sources<KIND>(g, B0, TS, M, ti, accB, partial);
 }
 
 // Tiles of 128 nodes (one warp, four targets a lane), 256 (two warps) and, Stokes,
 // 192 (one warp, six targets).
-template <int KIND>
-void launch_pair32s(const Geo& g, int tile, double* partial, const int* stop, cudaStream_t s) {
-  const long long nt = (g.M + tile - 1) / tile;
-  const unsigned pairs = (unsigned)(nt * (nt + 1) / 2);
+template <int KIND, bool BATCH>
+void launch_pair32s(const Geo& g, const PairPlan& p, double* partial, const int* stop, cudaStream_t s) {
+  const dim3 grid((unsigned)((long long)p.S * (p.S + 1) / 2), BATCH ? g.nprob : 1);  // S tiles (the largest problem's)
+  const int tile = p.sym;
   if constexpr (KIND == 1) {
     if (tile == 192) {
-      k_pair32s<1, 3><<<pairs, 32, sym32_smem<1, 3>(32), s>>>(g, partial, stop);
+      k_pair32s<1, 3, BATCH><<<grid, 32, sym32_smem<1, 3>(32), s>>>(g, partial, stop);
       return;
     }
   }
-  k_pair32s<KIND, 2><<<pairs, tile / 4, sym32_smem<KIND, 2>(tile / 4), s>>>(g, partial, stop);
+  k_pair32s<KIND, 2, BATCH><<<grid, tile / 4, sym32_smem<KIND, 2>(tile / 4), s>>>(g, partial, stop);
 }
 
 // -------------------------------------------------------- symmetric FP64 ----
@@ -1548,8 +1566,10 @@ __global__ void __launch_bounds__(B) k_epilogue32(Geo g, VecRef vr, const double
 // target entry (1 Laplace, 2 Stokes).
 constexpr int kRT = 32, kRG = 8;
 
-__global__ void __launch_bounds__(kRT * kRG) k_reduce_slots(double* __restrict__ partial, int S, long long n,
-                                                            const int* __restrict__ stop) {
+// tile > 0: the symmetric kernel over problems, each of whose entries has as many slots
+// as its problem has tiles.
+__global__ void __launch_bounds__(kRT * kRG) k_reduce_slots(Geo g, int tile, double* __restrict__ partial, int S,
+                                                            long long n, const int* __restrict__ stop) {
   if (stop && *stop) return;
   __shared__ float sh[kRG][kRT], sl[kRG][kRT];
   const int tx = threadIdx.x % kRT, grp = threadIdx.x / kRT;
@@ -1557,6 +1577,10 @@ __global__ void __launch_bounds__(kRT * kRG) k_reduce_slots(double* __restrict__
   const float2* __restrict__ pf2 = reinterpret_cast<const float2*>(partial);
   float h = 0.f, l = 0.f, h2 = 0.f, l2 = 0.f;
   if (e < n) {
+    if (tile > 0) {
+      const int2 r = g.prange[g.body_of[n == g.M ? e : e >> 1]];
+      S = (r.y - r.x + tile - 1) / tile;
+    }
     int s = grp;
     for (; s + kRG < S; s += 2 * kRG) {
       const float2 u = pf2[(long long)s * n + e], v = pf2[(long long)(s + kRG) * n + e];
@@ -1842,7 +1866,8 @@ PairPlan occupancy_plan(int M, int kind, int precision, int max_slots) {
 // ceil(len_x / chunk) busy splits, each with about the same work whatever the
 // problem's size.  S is the smallest count whose busy blocks fill every
 // resident slot once (chunks of at least 64 sources).
-PairPlan plan_pairs_batch(const int* body_start, int N, const int* pbody, int P, int kind, int precision) {
+PairPlan plan_pairs_batch(const int* body_start, int N, const int* pbody, int P, int kind, int precision,
+                          int max_slots) {
   const DeviceShape& d = device_shape();
   const int per_block = precision == 0 ? kB64 * kT64 : (precision == 1 ? kB32 * kT32 : kBF * kTF);
   const int M = body_start[N];
@@ -1850,6 +1875,34 @@ PairPlan plan_pairs_batch(const int* body_start, int N, const int* pbody, int P,
   int src_max = 1;
   for (int p = 0; p <= P; ++p) pstart[p] = p < P ? body_start[pbody[p]] : M;
   for (int p = 0; p < P; ++p) src_max = std::max(src_max, pstart[p + 1] - pstart[p]);
+  if (precision == 1) {
+    // The symmetric kernel by the rule of single systems (plan_symmetric32) on the sum of
+    // the problems' tile pairs; problems of so different sizes that most CTAs of the grid
+    // (the largest problem's pairs for each) would be empty, and fewer slots than the
+    // slots' reduction takes, stay with the directed kernel.  Eight problems of 2,000 to
+    // 5,500 nodes, Stokes: 146 us directed, 83 symmetric.
+    const auto pairs = [&](int tile, long long& S) {
+      long long sum = 0;
+      S = 0;
+      for (int p = 0; p < P; ++p) {
+        const long long nt = (pstart[p + 1] - pstart[p] + tile - 1) / tile;
+        S = std::max(S, nt);
+        sum += nt * (nt + 1) / 2;
+      }
+      return sum;
+    };
+    const int big = kind == 0 ? kTS : 192;
+    long long S, Sbig;
+    const long long n128 = pairs(128, S), nbig = pairs(big, Sbig);
+    const bool use_big = nbig >= (kind == 0 ? 30LL : 40LL) * d.nsm;
+    if (use_big) S = Sbig;
+    if (n128 >= (kind == 0 ? 6LL : 4LL) * d.nsm && S >= kRG && S <= max_slots &&
+        P * (S * (S + 1) / 2) <= 4 * (use_big ? nbig : n128) && (double)S * M * (kind + 1) * 8e-6 <= 512.0) {
+      PairPlan p = uniform_plan((int)S, use_big ? big : 128);
+      p.sym = p.chunk;
+      return p;
+    }
+  }
   const int bx = (M + per_block - 1) / per_block;
   std::vector<int> len(bx);
   for (int x = 0; x < bx; ++x) {
@@ -1896,14 +1949,14 @@ void launch_pairs(const Geo& g, int kind, int precision, const PairPlan& p, VecR
     const int gs = (int)std::min<long long>(1216, (g.M + 255) / 256);
     if (kind == 0) {
       k_src32<0><<<gs, 256, 0, s>>>(g, v, sscale, stop);
-      if (!BATCH && p.sym)
-        launch_pair32s<0>(g, p.sym, partial, stop, s);
+      if (p.sym)
+        launch_pair32s<0, BATCH>(g, p, partial, stop, s);
       else
         k_pair32<0, BATCH><<<grid, kB32, 0, s>>>(g, v, sscale, p, partial, stop);
     } else {
       k_src32<1><<<gs, 256, 0, s>>>(g, v, sscale, stop);
-      if (!BATCH && p.sym)
-        launch_pair32s<1>(g, p.sym, partial, stop, s);
+      if (p.sym)
+        launch_pair32s<1, BATCH>(g, p, partial, stop, s);
       else
         k_pair32<1, BATCH><<<grid, kB32, 0, s>>>(g, v, sscale, p, partial, stop);
     }
@@ -1942,7 +1995,7 @@ cudaError_t epilogue(const Geo& g, int kind, const PairPlan& p, VecRef v, const 
     const long long n = (long long)g.M * (kind + 1);
     const unsigned nb = (unsigned)((n + kRT - 1) / kRT);
     if (pff)
-      k_reduce_slots<<<nb, kRT * kRG, 0, s>>>(const_cast<double*>(partial), p.S, n, stop);
+      k_reduce_slots<<<nb, kRT * kRG, 0, s>>>(g, g.prange ? p.sym : 0, const_cast<double*>(partial), p.S, n, stop);
     else
       k_reduce_slots64<<<nb, kRT * kRG, 0, s>>>(const_cast<double*>(partial), p.S, n, stop);
     note_launches(1);
