@@ -373,7 +373,7 @@ void carve(Arena& A, Work& w, int N, int M, int kind, int m, bool solve, bool st
     w.sn = A.take<double>((size_t)nseg * m);
     w.gv = A.take<double>((size_t)nseg * (m + 1));
     w.yv = A.take<double>((size_t)nseg * (m + 1));
-    w.P = output_splits(g, kind);
+    w.P = output_splits(g, kind, compact);
     const int targets = kind == 0 ? N : 3 * N;
     w.outpart = A.take<double>((size_t)w.P * targets * comps + N + 2);
     w.outv = A.take<double>(3 * N);

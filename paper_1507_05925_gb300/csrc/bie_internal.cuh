@@ -148,7 +148,7 @@ cudaError_t incident_density_scaled(const Geo& g, int kind, const double* load, 
 // the constraint residual max over bodies into *cres (device) relative to the load.
 cudaError_t evaluate_output(const Geo& g, int kind, const double* v, const double* load,
                             double* partial, int P, double* out, double* cres, cudaStream_t s);
-int output_splits(const Geo& g, int kind);
+int output_splits(const Geo& g, int kind, bool compact);
 // the second half of evaluate_output, on sums already in partial (P splits)
 cudaError_t finalize_output(const Geo& g, int kind, const double* v, const double* load, double* partial, int P,
                             double* out, double* cres, cudaStream_t s);

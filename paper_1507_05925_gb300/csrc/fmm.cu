@@ -2123,6 +2123,10 @@ namespace {
 
 // The splits of the orbits that fill a block's warps best (nsplit (channel, row)
 // threads), and the orbits staged at a time (at most about 100 KB).
+// The kernels' bound is a constant, five orbits of four channels and both Pascal
+// matrices at the largest order: with each launch's own size, another thread's
+// launch could find a smaller bound than it needs.
+constexpr int kMaxM2lSmem = 5 * kMaxNd * kMaxP * 4 * 16 + 2 * kMaxP * kMaxP * 8;
 struct M2lShape {
   int nsplit, threads, nbo;
   size_t smem;
@@ -2170,10 +2174,10 @@ void launch_m2l(const FmmDev& d, int L, const int* stop, cudaStream_t s) {
   const int grid = (int)(lev_off(L + 1) - lev_off(2));
   const M2lShape m = m2l_shape(d.nd, d.p, sizeof(double2), (size_t)(d.nlog > 0 ? 2 : 1) * d.p * d.p * sizeof(double));
   if (m.nsplit == 5) {
-    cudaFuncSetAttribute(k_fmm_m2l<double2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
+    cudaFuncSetAttribute(k_fmm_m2l<double2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
     k_fmm_m2l<double2, 2><<<grid, m.threads, m.smem, s>>>(d, m.nsplit, m.nbo, stop);
   } else {
-    cudaFuncSetAttribute(k_fmm_m2l<double2, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
+    cudaFuncSetAttribute(k_fmm_m2l<double2, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
     k_fmm_m2l<double2, 5><<<grid, m.threads, m.smem, s>>>(d, m.nsplit, m.nbo, stop);
   }
 }
@@ -2182,10 +2186,10 @@ void launch_m2l_ff(const FmmDev& d, const float4* mpff, const float* tab, int L,
   const M2lShape m = m2l_shape(d.nd, d.p, sizeof(float4), 0);
   const int grid = (int)(lev_off(L + 1) - lev_off(2));
   if (m.nsplit == 5) {
-    cudaFuncSetAttribute(k_fmm_m2l_ff<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
+    cudaFuncSetAttribute(k_fmm_m2l_ff<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
     k_fmm_m2l_ff<2><<<grid, m.threads, m.smem, s>>>(d, mpff, tab, m.nsplit, m.nbo, stop);
   } else {
-    cudaFuncSetAttribute(k_fmm_m2l_ff<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
+    cudaFuncSetAttribute(k_fmm_m2l_ff<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
     k_fmm_m2l_ff<5><<<grid, m.threads, m.smem, s>>>(d, mpff, tab, m.nsplit, m.nbo, stop);
   }
 }

@@ -469,11 +469,14 @@ cudaError_t incident_density_scaled(const Geo& g, int kind, const double* load, 
   return cudaGetLastError();
 }
 
-int output_splits(const Geo& g, int kind) {
-  // blocks (a body's three Stokes targets are one): four an SM, Stokes, whose blocks are
-  // three times as long, eight, so that the last ones leave no SM much longer than the mean
-  int P = ((kind == 0 ? 4 : 8) * device_sms() + g.N - 1) / g.N;
-  if (kind == 1 && P > 12) P = std::max(12, (4 * device_sms() + 3 * g.N - 1) / (3 * g.N));  // one thread adds the splits
+int output_splits(const Geo& g, int kind, bool compact) {
+  // Blocks (a body's three Stokes targets are one): four an SM, Stokes, whose blocks are
+  // three times as long, eight, so that the last ones leave no SM much longer than the
+  // mean, in at most twelve splits (one thread adds them).  compact: as few as fill the
+  // SMs four times with single targets.
+  const int fill = 4 * device_sms(), targets = kind == 0 ? g.N : 3 * g.N;
+  int P = (fill + targets - 1) / targets;
+  if (kind == 1 && !compact) P = std::max(P, std::min(12, (2 * fill + g.N - 1) / g.N));
   const int maxP = (g.M + 255) / 256;
   if (P > maxP) P = maxP;
   if (P < 1) P = 1;

@@ -39,8 +39,8 @@ __device__ __forceinline__ double combine(const double* __restrict__ V, long lon
 
 // ------------------------------------------------------------ fused Arnoldi
 // One Arnoldi step after w = A z_j (w = V_{j+1}) in a single cooperative
-// launch with three grid barriers: CGS2 (h1 = V^T w; w -= V h1; h2 = V^T w;
-// w -= V h2), ||w||, the Hessenberg column with its Givens rotations and the
+// launch with two grid barriers (a third where the norm cancels): CGS2 (h1 = V^T w;
+// w -= V h1; h2 = V^T w; w -= V h2), ||w||, the Hessenberg column with its Givens rotations and the
 // residual estimate, and v_{j+1} = w / ||w||.  After each barrier every CTA adds
 // the per-CTA partials itself, in CTA order (deterministic; no atomics), so
 // nothing else synchronises the grid.  With the block-Jacobi preconditioner w is

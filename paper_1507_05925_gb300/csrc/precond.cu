@@ -573,7 +573,10 @@ cudaError_t launch_factor(const Geo& g, int kind, double alpha, const int* list,
   // nb = 256 in clusters of four 186 us for 100 bodies with one, 334 with two; nb <= 446, 155 bodies,
   // 1296 and 895; clusters of eight have no registers for two: 32 bodies of 512 731 and 790)
   const int T = gj_rows(max_nb), groups = T > 128 ? (CS == 4 ? 2 : 1) : (CS == 1 ? 256 : 128) / T, threads = groups * T + 32;
-  cudaError_t e = cudaFuncSetAttribute(k_bj_factor<CS, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // a constant bound (the largest block's): with this launch's size, another thread's
+  // launch could find a smaller one than it needs
+  cudaError_t e = cudaFuncSetAttribute(k_bj_factor<CS, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(gj_smem_floats(kMaxBlock, 8) * sizeof(float)));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(CS * count);

@@ -517,13 +517,14 @@ cudaError_t small_batch_solve(const Geo& g, int kind, int P, const int* pbody, c
                               int max_iter, int max_nodes, SmallInfo* info, cudaStream_t s) {
   SmallArgs A{g, kind, pbody, pnode, f, x, r, d, rc, rin, y, V, ld, m, max_refine, max_iter, tol, inner_tol, info};
   const size_t smem = small_smem_bytes(max_nodes);
+  const int bound = (int)small_smem_bytes(kSmallMaxNodes);  // constant: other threads launch too
   cudaError_t e;
   if (kind == 0) {
-    e = cudaFuncSetAttribute(k_small_solve<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_small_solve<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bound);
     if (e != cudaSuccess) return e;
     k_small_solve<0><<<P, kSB, smem, s>>>(A);
   } else {
-    e = cudaFuncSetAttribute(k_small_solve<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_small_solve<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bound);
     if (e != cudaSuccess) return e;
     k_small_solve<1><<<P, kSB, smem, s>>>(A);
   }
