@@ -28,6 +28,7 @@
 #include "bie_internal.cuh"
 #include "pair_math.cuh"
 #include "reduce.cuh"
+#include "rotations.cuh"
 
 namespace bie {
 
@@ -95,17 +96,15 @@ __device__ void cta_moments(const Geo& g, int kind, int i0, int i1, const double
       }
     }
     m0 = warp_sum(m0);
-    m1 = warp_sum(m1);
-    m2 = warp_sum(m2);
-    if (lane == 0) {
-      if (alpha > 0.0) {
-        m0 *= alpha / g.len[i];
-        m1 *= alpha / g.len[i];
-        m2 *= alpha / g.W[i];
-      }
-      sh.mom[0][i - i0] = m0;
-      sh.mom[1][i - i0] = m1;
-      sh.mom[2][i - i0] = m2;
+    if (kind == 1) {
+      m1 = __shfl_sync(0xffffffffu, warp_sum(m1), 0);
+      m2 = __shfl_sync(0xffffffffu, warp_sum(m2), 0);
+    }
+    // lane q weights and stores moment q
+    const double m = lane == 0 ? m0 : lane == 1 ? m1 : m2;
+    if (lane < (kind == 0 ? 1 : 3)) {
+      const double weight = alpha > 0.0 ? alpha * rcp64(lane < 2 ? g.len[i] : g.W[i]) : 1.0;
+      sh.mom[lane][i - i0] = m * weight;
     }
   }
 }
@@ -252,19 +251,16 @@ __device__ void cta_apply(const Geo& g, int a0, int a1, int i0, int i1, const do
     const double wk = g.w[a] * g.kappa[a];
     if (KIND == 0) {
       const double k = g.nx[a] * k1 + g.ny[a] * k2;
-      const double mu = v[t] / os;
-      const double yv = -kInv2Pi * k - kInv4Pi * wk * mu + sh.mom[0][i];
-      out[t] = 0.5 * v[t] + os * yv;
+      // (the diagonal limit acts on v / os, times os)
+      out[t] = 0.5 * v[t] + os * (sh.mom[0][i] - kInv2Pi * k) - kInv4Pi * wk * v[t];
     } else {
-      const double mu1 = v[2 * t] / os, mu2 = v[2 * t + 1] / os;
+      const double v1 = v[2 * t], v2 = v[2 * t + 1];
       const double tx = -g.ny[a], ty = g.nx[a];
-      const double dd = -0.5 * kInvPi * wk * (tx * mu1 + ty * mu2);
+      const double dd = -0.5 * kInvPi * wk * (tx * v1 + ty * v2);
       const int ib = g.body_of[a];
       const double px = -(g.y[a] - g.yc[ib]), py = g.x[a] - g.xc[ib];
-      const double y1 = -kInvPi * k1 + dd * tx + sh.mom[0][i] + px * sh.mom[2][i];
-      const double y2 = -kInvPi * k2 + dd * ty + sh.mom[1][i] + py * sh.mom[2][i];
-      out[2 * t] = 0.5 * v[2 * t] + os * y1;
-      out[2 * t + 1] = 0.5 * v[2 * t + 1] + os * y2;
+      out[2 * t] = 0.5 * v1 + os * (sh.mom[0][i] + px * sh.mom[2][i] - kInvPi * k1) + dd * tx;
+      out[2 * t + 1] = 0.5 * v2 + os * (sh.mom[1][i] + py * sh.mom[2][i] - kInvPi * k2) + dd * ty;
     }
   }
   __syncthreads();
@@ -335,8 +331,9 @@ __device__ int cta_gmres(const SmallArgs& A, int a0, int a1, int i0, int i1, lon
       // CGS2: two passes of h = V^T w, w -= V h
       for (int pass = 0; pass < 2; ++pass) {
         double* hs = pass == 0 ? sh.h1 : sh.h2;
-        for (int i = wid; i <= j; i += kSW) {
-          const double* Vi = Vr(i);
+        // the second pass also sums ||w||^2 (as product j + 1 of w with itself)
+        for (int i = wid; i <= j + pass; i += kSW) {
+          const double* Vi = i <= j ? Vr(i) : w;
           double s0 = 0.0, s1 = 0.0;
           int k = lane;
           for (; k + 32 < n; k += 64) {
@@ -355,19 +352,29 @@ __device__ int cta_gmres(const SmallArgs& A, int a0, int a1, int i0, int i1, lon
         }
         __syncthreads();
       }
-      const double hn = sqrt(cta_dot(w, w, n, sh));
+      // ||w - V h2||^2 = ||w||^2 - ||h2||^2 while nothing cancels (k_arnoldi32), by warp 0
+      if (wid == 0) {
+        double h22 = 0.0;
+        for (int i = lane; i <= j; i += 32) h22 = fma(sh.h2[i], sh.h2[i], h22);
+        h22 = warp_sum(h22);
+        if (lane == 0) {
+          sh.scal[1] = sh.h2[j + 1] - h22;
+          sh.flag[0] = !(h22 <= 0.25 * sh.h2[j + 1]);
+        }
+      }
+      __syncthreads();
+      if (sh.flag[0]) {  // (the same in every thread)
+        const double t = cta_dot(w, w, n, sh);
+        if (threadIdx.x == 0) sh.scal[1] = t;
+      }
       if (threadIdx.x == 0) {
+        const double hn = sqrt(sh.scal[1]);
         double* Hc = sh.H + j * (m + 1);
         for (int i = 0; i <= j; ++i) Hc[i] = sh.h1[i] + sh.h2[i];
-        Hc[j + 1] = hn;
-        for (int i = 0; i < j; ++i) {
-          const double t = sh.cs[i] * Hc[i] + sh.sn[i] * Hc[i + 1];
-          Hc[i + 1] = -sh.sn[i] * Hc[i] + sh.cs[i] * Hc[i + 1];
-          Hc[i] = t;
-        }
-        const double xx = Hc[j], yy = Hc[j + 1];
-        const double rho = hypot(xx, yy);
-        const double c = rho > 0.0 ? xx / rho : 1.0, s = rho > 0.0 ? yy / rho : 0.0;
+        double c, s, rho;
+        givens(rotate_column(sh.cs, sh.sn, Hc, j), hn, c, s, rho);
+        sh.scal[1] = hn;
+        sh.scal[2] = hn > 0.0 ? 1.0 / hn : 0.0;
         sh.cs[j] = c;
         sh.sn[j] = s;
         Hc[j] = rho;
@@ -378,8 +385,7 @@ __device__ int cta_gmres(const SmallArgs& A, int a0, int a1, int i0, int i1, lon
         sh.scal[0] = fabs(s * gj);
       }
       __syncthreads();
-      const double res = sh.scal[0];
-      const double inv = hn > 0.0 ? 1.0 / hn : 0.0;
+      const double res = sh.scal[0], hn = sh.scal[1], inv = sh.scal[2];
       for (int k = threadIdx.x; k < n; k += kSB) w[k] *= inv;
       __syncthreads();
       ++total;
