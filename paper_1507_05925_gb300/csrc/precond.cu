@@ -31,7 +31,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <type_traits>
 #include <vector>
 
 #include "../../include/bie2d.h"
