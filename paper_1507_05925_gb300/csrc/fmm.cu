@@ -104,7 +104,7 @@ struct FmmDevT {
   T2* mp;
   T2* lc;
   const T2* ops;
-  const float2* Qf = nullptr;  // FP32 expansions: q per source in FP32 (channel 0), from k_fmm_density32
+  const float2* Qf = nullptr;  // FP32 expansions: q per source in FP32 (channel 0), written by k_fmm_p2m32
   const float4* cen32 = nullptr;  // FP32 expansions: leaf centres split hi + lo
   float is32 = 0.f, s32 = 0.f;    // FP32 expansions: 1/s and s of a leaf
 };
@@ -260,22 +260,6 @@ __device__ __forceinline__ void p2m_chunk(T2* acc, const T2* pw, const T2* qs, i
   }
 }
 
-// The FP32 operator's strengths: q = sqrt(w) v per source in FP32 (Laplace:
-// (q, 0); Stokes: the complex density).  The other channels (conj(q) and the
-// leaf-relative moment density) are formed where they are used, so the FP32
-// passes read 8 bytes a source and convert nothing from FP64.
-__global__ void k_fmm_density32(Geo g, int nd, VecRef vr, const double* __restrict__ sscale, float2* Qf,
-                                const int* stop) {
-  if (stop && *stop) return;
-  const double* v = vr.ptr();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.M; i += gridDim.x * blockDim.x) {
-    if (nd == 1)
-      Qf[i] = make_float2((float)(sscale[i] * v[i]), 0.f);
-    else
-      Qf[i] = make_float2((float)(sscale[i] * v[2 * i]), (float)(sscale[i] * v[2 * i + 1]));
-  }
-}
-
 // Leaf centres split as float hi + lo, once per tree (FP64 arithmetic here,
 // so that the FP32 passes form u = (z - c)/s from the hi/lo split of z in
 // FP32 with no FP64 instruction: z_hi - c_hi is exact for a node inside the
@@ -301,21 +285,30 @@ __device__ __forceinline__ void leaf_center32(const FmmDevT<float2>& f, int b, f
   }
 }
 
-// P2M of the FP32 expansions (inner solves) with no FP64 instruction per
-// source: positions from the hi/lo split, strengths from k_fmm_density32.
-__global__ void __launch_bounds__(kB) k_fmm_p2m32(FmmDevT<float2> f, Geo g, const int* stop) {
+// P2M of the FP32 expansions (inner solves): positions from the hi/lo split, and the
+// strengths q = sqrt(w) v in FP32 (Laplace: (q, 0); Stokes: the complex density; the
+// other channels are formed where they are used), formed here, where each source
+// is read once, and kept in Qf for the near field (a launch of its own was 3 us).
+// With few outputs (np = nd p <= 32) the threads are groups of np that take every
+// G-th source, added in order: FP32 Laplace, order 15, 1,024 leaves
+// 16.2 + 3.4 -> 12.3 us; Stokes, order 18, 16,384 leaves 32.7 + 8.0 -> 36.3 us.
+__global__ void __launch_bounds__(kB) k_fmm_p2m32(FmmDevT<float2> f, Geo g, VecRef vr, const double* __restrict__ sscale,
+                                                  float2* __restrict__ Qf, const int* stop) {
   if (stop && *stop) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* pw = reinterpret_cast<float2*>(smraw);  // [p][kChunk + 1]
   float2* qs = pw + f.p * (kChunk + 1);            // [kChunk][nd]
   __shared__ float cen[6];
+  __shared__ float2 red[kB];
+  const double* __restrict__ v = vr.ptr();
   const int b = blockIdx.x;
   const long long box = lev_off(f.L) + b;
   const int s0 = f.start[b], n = f.start[b + 1] - s0;
   if (n == 0) return;
   leaf_center32(f, b, cen);
   __syncthreads();
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, np = f.nd * f.p, G = kB / np;
+  const int grp = G > 1 ? t / np : 0, e = t - grp * np, d = e / f.p, k = e - d * f.p;  // G > 1
   float2 acc[kP2MAcc];
 #pragma unroll
   for (int u = 0; u < kP2MAcc; ++u) acc[u] = make_float2(0.f, 0.f);
@@ -324,13 +317,19 @@ __global__ void __launch_bounds__(kB) k_fmm_p2m32(FmmDevT<float2> f, Geo g, cons
     if (t < m) {
       const int i = f.perm[s0 + ch + t];
       const float4 P = g.pf[i];
+      const double sw = sscale[i];
+      float2 q;
+      if (f.nd == 1)
+        q = make_float2((float)(sw * v[i]), 0.f);
+      else
+        q = make_float2((float)(sw * v[2 * i]), (float)(sw * v[2 * i + 1]));
+      Qf[i] = q;
       const float2 u = make_float2(((P.x - cen[0]) + (P.z - cen[2])) * cen[4], ((P.y - cen[1]) + (P.w - cen[3])) * cen[4]);
       float2 w = make_float2(1.f, 0.f);
-      for (int k = 0; k < f.p; ++k) {
-        pw[k * (kChunk + 1) + t] = w;
+      for (int r = 0; r < f.p; ++r) {
+        pw[r * (kChunk + 1) + t] = w;
         w = cmul(w, u);
       }
-      const float2 q = f.Qf[i];
       qs[t * f.nd] = q;
       if (f.nd == 3) {
         qs[t * 3 + 1] = make_float2(q.x, -q.y);
@@ -339,12 +338,26 @@ __global__ void __launch_bounds__(kB) k_fmm_p2m32(FmmDevT<float2> f, Geo g, cons
       }
     }
     __syncthreads();
-    p2m_chunk(acc, pw, qs, f.p, f.nd, m);
+    if (G > 1) {
+      if (grp < G)
+        for (int j = grp; j < m; j += G) cfma(acc[0], pw[k * (kChunk + 1) + j], qs[j * f.nd + d]);
+    } else {
+      p2m_chunk(acc, pw, qs, f.p, f.nd, m);
+    }
     __syncthreads();
+  }
+  if (G > 1) {
+    red[t] = acc[0];
+    __syncthreads();
+    if (t < np) {
+      for (int q = 1; q < G; ++q) acc[0] = cadd(acc[0], red[q * np + t]);
+      f.mp[box * np + t] = acc[0];
+    }
+    return;
   }
 #pragma unroll
   for (int u = 0; u < kP2MAcc; ++u)
-    if (t + u * kB < f.nd * f.p) f.mp[box * f.nd * f.p + t + u * kB] = acc[u];
+    if (t + u * kB < np) f.mp[box * np + t + u * kB] = acc[u];
 }
 
 // P2M on the leaves: a_k = sum_j q_j u_j^k, u = (z - c)/s.
@@ -2247,11 +2260,12 @@ int fmm_m2m(const FmmDevT<T2>& d, int* arrive, const int* stop, cudaStream_t s) 
 
 // The upward pass, M2L, downward pass and evaluation with expansions of type T2.
 template <class T2, int NEARP>
-void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, double* partial, const int* stop, cudaStream_t s) {
+void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, [[maybe_unused]] VecRef v,
+                [[maybe_unused]] const double* sscale, double* partial, const int* stop, cudaStream_t s) {
   const int p = d.p, nd = d.nd;
   const size_t sm_p2m = ((size_t)p * (kChunk + 1) + (size_t)kChunk * nd) * sizeof(T2);
   if constexpr (std::is_same<T2, float2>::value)
-    k_fmm_p2m32<<<f->nleaf, kB, sm_p2m, s>>>(d, g, stop);
+    k_fmm_p2m32<<<f->nleaf, kB, sm_p2m, s>>>(d, g, v, sscale, const_cast<float2*>(d.Qf), stop);
   else if constexpr (NEARP == 2)
     k_fmm_p2m_ff<<<f->nleaf, kB, sm_p2m, s>>>(d, g, stop);  // float4 = double2 in size
   else
@@ -2327,7 +2341,6 @@ cudaError_t fmm_pair_sum(FmmState* f, const Geo& g, int kind, int p, VecRef v, c
     // the inner solves' operator: FP32 strengths, expansions (in the FP64
     // buffers) and near field
     float2* Qf = reinterpret_cast<float2*>(f->Q);
-    k_fmm_density32<<<grid_for(g.M), 256, 0, s>>>(g, nd, v, sscale, Qf, stop);
     FmmDevT<float2> d{f->L,     f->nb,     p,        nd,       g.M,     0,       kind == 1 ? 2 : -1,
                       f->x0,    f->y0,     f->D,     1.0 / f->D, f->leaf,  f->perm, f->start,
                       f->count, f->count,  f->Q,     reinterpret_cast<float2*>(f->mp),
@@ -2336,18 +2349,18 @@ cudaError_t fmm_pair_sum(FmmState* f, const Geo& g, int kind, int p, VecRef v, c
     d.cen32 = f->cen32;
     d.is32 = (float)ldexp(1.0 / f->D, f->L);
     d.s32 = (float)ldexp(f->D, -f->L);
-    fmm_passes<float2, 1>(d, f, g, partial, stop, s);
+    fmm_passes<float2, 1>(d, f, g, v, sscale, partial, stop, s);
   } else {
     k_fmm_density<<<grid_for(g.M), 256, 0, s>>>(g, nd, f->x0 + 0.5 * f->D, f->y0 + 0.5 * f->D, v, sscale, f->Q,
                                                  stop);
     const FmmDev d{f->L,    f->nb,    p,     nd,    g.M,   0,   kind == 1 ? 2 : -1, f->x0, f->y0, f->D, 1.0 / f->D, f->leaf,
                    f->perm, f->start, f->count, f->count, f->Q, f->mp, f->lc,  ops};
     if (near_prec == 2)
-      fmm_passes<double2, 2>(d, f, g, partial, stop, s);
+      fmm_passes<double2, 2>(d, f, g, v, sscale, partial, stop, s);
     else
-      fmm_passes<double2, 0>(d, f, g, partial, stop, s);
+      fmm_passes<double2, 0>(d, f, g, v, sscale, partial, stop, s);
   }
-  note_launches(4 + (near_prec == 2 ? 1 : 0));
+  note_launches(4 + (near_prec == 2 ? 1 : near_prec == 1 ? -1 : 0));
   return cudaGetLastError();
 }
 
