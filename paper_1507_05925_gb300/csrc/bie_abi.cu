@@ -81,7 +81,7 @@ struct bie_ctx {
   std::vector<Timing> pending;
   // CUDA graphs of one GMRES iteration, keyed by everything their kernels read
   struct IterGraph {
-    long long key[12];
+    std::vector<long long> key;
     cudaGraphExec_t exec;
     long long kernels;  // per iteration
     int last_cycle;     // iterations of the last cycle replayed from it (0: none yet)
@@ -823,31 +823,65 @@ bool capturable(cudaStream_t s) {
   return s != nullptr && s != cudaStreamLegacy && s != cudaStreamPerThread;
 }
 
-// The iteration as a CUDA graph (built once per workspace layout and operator;
-// not while pair-sum timing is on, whose events are per launch).  nullptr if
-// the stream cannot be captured.
-bie_ctx::IterGraph* iteration_graph(bie_ctx* ctx, Work& w, const Op& op, cudaStream_t s) {
-  if (ctx->prof || !capturable(s) || barrier_fault_armed()) return nullptr;
-  const PairPlan& p = op.prec == 0 ? w.plan64 : (op.prec == 1 ? w.plan32 : w.planff);
+// Everything that launch_iteration bakes into its launches: the operator, the pair-sum
+// plan, the sizes that grids and shared memory come from, and every pointer.  N, M and
+// the workspace do not imply the rest: where the arrays lie in it depends on the sum of
+// the bodies' block sizes, on interior points and on the other precisions' plans, and
+// the FP64 preconditioner's launch on the largest body.
+std::vector<long long> iteration_key(const bie_ctx* ctx, const Work& w, const Op& op) {
+  std::vector<long long> key;
+  auto num = [&](long long v) { key.push_back(v); };
+  auto ptr = [&](const void* p) { key.push_back((long long)(uintptr_t)p); };
   long long alpha_bits;
   memcpy(&alpha_bits, &op.alpha, sizeof(alpha_bits));
+  const PairPlan& p = op.prec == 0 ? w.plan64 : (op.prec == 1 ? w.plan32 : w.planff);
+  for (long long v : {(long long)op.prec, (long long)op.fmm_p, (long long)op.precond, alpha_bits, (long long)p.S,
+                      (long long)p.chunk, (long long)p.S1, (long long)p.chunk2, (long long)p.sym, (long long)w.kind,
+                      (long long)w.g.N, (long long)w.g.M, (long long)w.g.nprob, (long long)w.m, w.ld,
+                      (long long)w.bj_max_nb, (long long)w.seg.P, (long long)w.seg.nitem, (long long)w.seg_grid})
+    num(v);
+  const Geo& g = w.g;
+  for (const void* q : {(const void*)g.body_start, (const void*)g.body_of, (const void*)g.x, (const void*)g.y,
+                        (const void*)g.nx, (const void*)g.ny, (const void*)g.w, (const void*)g.sw,
+                        (const void*)g.kappa, (const void*)g.pf, (const void*)g.nf, (const void*)g.wkf,
+                        (const void*)g.len, (const void*)g.xc, (const void*)g.yc, (const void*)g.W,
+                        (const void*)g.zx, (const void*)g.zy, (const void*)g.delta, (const void*)g.wind,
+                        (const void*)g.bbox, (const void*)g.qscale, (const void*)g.xff, (const void*)g.xfl,
+                        (const void*)g.nff, (const void*)g.prange, (const void*)g.pbody, (const void*)g.qf})
+    ptr(q);
+  for (const void* q : {(const void*)w.V, (const void*)w.VF, (const void*)w.ytmp, (const void*)w.zbuf,
+                        (const void*)w.partial, (const void*)w.arn, (const void*)w.st, (const void*)w.H,
+                        (const void*)w.cs, (const void*)w.sn, (const void*)w.gv, (const void*)w.bj_off,
+                        (const void*)w.bj_blocks, (const void*)w.ps, (const void*)w.seg.pnode,
+                        (const void*)w.seg.ibeg, (const void*)w.seg.iprob, (const void*)w.seg.pitem,
+                        (const void*)w.seg.bprob})
+    ptr(q);
   // an FMM application's captured launches depend on the tree (buffers, level
   // count, bounding square), which a later setup may rebuild or reallocate
-  long long fsig[2] = {0, 0};
-  if (op.fmm_p > 0) fmm_signature(ctx->fmm, fsig);
-  const long long key[12] = {(long long)(uintptr_t)ctx->ws, (long long)ctx->ws_size, w.g.N, w.g.M,
-                             w.kind + 4LL * w.seg.P, w.m, op.prec * 1000 + op.fmm_p + (op.precond ? 500 : 0), alpha_bits,
-                             (p.S * 1000003LL + p.chunk) * 1000003LL + p.S1 * 4099LL + p.chunk2 * 2 + p.sym,
-                             w.grid + 1000003LL * w.seg.nitem, fsig[0], fsig[1]};
+  if (op.fmm_p > 0) {
+    long long fsig[2];
+    fmm_signature(ctx->fmm, fsig);
+    num(fsig[0]);
+    num(fsig[1]);
+  }
+  return key;
+}
+
+// The iteration as a CUDA graph (built once per iteration_key; not while
+// pair-sum timing is on, whose events are per launch).  nullptr if the stream
+// cannot be captured.
+bie_ctx::IterGraph* iteration_graph(bie_ctx* ctx, Work& w, const Op& op, cudaStream_t s) {
+  if (ctx->prof || !capturable(s) || barrier_fault_armed()) return nullptr;
+  const std::vector<long long> key = iteration_key(ctx, w, op);
   for (auto& gi : ctx->graphs)
-    if (memcmp(gi.key, key, sizeof(key)) == 0) return &gi;
+    if (gi.key == key) return &gi;
   auto keep = [&](cudaGraphExec_t exec, long long kernels) {
     if (ctx->graphs.size() >= 4) {
       cudaGraphExecDestroy(ctx->graphs.front().exec);
       ctx->graphs.erase(ctx->graphs.begin());
     }
     bie_ctx::IterGraph gi;
-    memcpy(gi.key, key, sizeof(key));
+    gi.key = key;
     gi.exec = exec;
     gi.kernels = kernels;
     gi.last_cycle = 0;
