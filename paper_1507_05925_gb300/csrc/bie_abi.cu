@@ -856,14 +856,7 @@ std::vector<long long> iteration_key(const bie_ctx* ctx, const Work& w, const Op
                         (const void*)w.seg.ibeg, (const void*)w.seg.iprob, (const void*)w.seg.pitem,
                         (const void*)w.seg.bprob})
     ptr(q);
-  // an FMM application's captured launches depend on the tree (buffers, level
-  // count, bounding square), which a later setup may rebuild or reallocate
-  if (op.fmm_p > 0) {
-    long long fsig[2];
-    fmm_signature(ctx->fmm, fsig);
-    num(fsig[0]);
-    num(fsig[1]);
-  }
+  if (op.fmm_p > 0) fmm_signature(ctx->fmm, key);
   return key;
 }
 

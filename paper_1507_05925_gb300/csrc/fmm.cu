@@ -2300,30 +2300,20 @@ void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, [[maybe_unused]
 
 }  // namespace
 
-void fmm_signature(const FmmState* f, long long sig[2]) {
-  if (!f) {
-    sig[0] = sig[1] = 0;
-    return;
+void fmm_signature(const FmmState* f, std::vector<long long>& key) {
+  if (!f) return;
+  for (double v : {f->x0, f->y0, f->D}) {
+    long long u;
+    memcpy(&u, &v, 8);
+    key.push_back(u);
   }
-  unsigned long long h = 1469598103934665603ULL;  // FNV-1a over the fields
-  auto mix = [&](unsigned long long v) {
-    for (int b = 0; b < 8; ++b) {
-      h ^= (v >> (8 * b)) & 0xff;
-      h *= 1099511628211ULL;
-    }
-  };
-  unsigned long long u;
-  memcpy(&u, &f->x0, 8);
-  mix(u);
-  memcpy(&u, &f->y0, 8);
-  mix(u);
-  memcpy(&u, &f->D, 8);
-  mix(u);
-  mix((unsigned long long)f->L);
-  mix((unsigned long long)f->buf_size);
-  mix((unsigned long long)f->M);
-  sig[0] = (long long)(uintptr_t)f->buf;
-  sig[1] = (long long)h;
+  for (long long v : {(long long)f->L, f->nbox, (long long)f->M, (long long)f->kind}) key.push_back(v);
+  for (const void* q : {(const void*)f->leaf, (const void*)f->perm, (const void*)f->start, (const void*)f->count,
+                        (const void*)f->arrive, (const void*)f->Q, (const void*)f->mp, (const void*)f->lc,
+                        (const void*)f->mpff, (const void*)f->cen32})
+    key.push_back((long long)(uintptr_t)q);
+  // the operator tables stay where they are as long as the state does
+  key.push_back((long long)(uintptr_t)f);
 }
 
 cudaError_t fmm_pair_sum(FmmState* f, const Geo& g, int kind, int p, VecRef v, const double* sscale,

@@ -76,3 +76,16 @@ def test_graphs_follow_the_bodies(ctx, name, kind, prec):
                 ref = (laplace.solve(g, synth.charges(N, rng))["phi"] if kind == bie.LAPLACE else
                        stokes.solve(g, synth.forces_torques(N, rng))["UW"].reshape(-1))
                 assert rel2(out, ref) <= TOL_SOLVE
+
+
+@pytest.mark.parametrize("kind", [bie.LAPLACE, bie.STOKES])
+def test_graphs_follow_the_fmm_order(ctx, kind):
+    """Outer orders 35 and 36 have one inner order, 18, but lay the tree's arrays out
+    differently in a buffer that order 38 made: the iteration captured at 35 must not be
+    replayed at 36."""
+    g = synth.assemble([synth.ellipse(3.2 * (i % 12), 3.2 * (i // 12), 1.0, 0.6, 0.3 * i, 64) for i in range(144)])
+    stream = torch.cuda.Stream()
+    opts = dict(precision=bie.MIXED_FF)
+    outs = [solve(ctx, g, kind, stream, fmm_order=p, **opts) for p in (38, 35, 36, 36)]
+    for p, out in zip((38, 35, 36, 36), outs):
+        assert np.array_equal(out, solve(ctx, g, kind, None, fmm_order=p, **opts)), p
