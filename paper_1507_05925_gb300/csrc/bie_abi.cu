@@ -265,9 +265,28 @@ struct Work {
   int P = 1, grid = 1;
 };
 
+// The pair-sum plans of a call.  They depend on the process's table of tuned plans, which
+// another thread may change at any time: a call chooses them once, and sizes and lays out
+// its workspace with the same ones.
+struct PlanSet {
+  PairPlan p64, p32, pff;
+  bool compact = false;  // without the symmetric plans that trade partial slots for time
+};
+
+PlanSet choose_plans(int kind, const std::vector<int>& bs, bool compact, int nprob = 0, const int* pb = nullptr) {
+  const int N = (int)bs.size() - 1, M = bs[N];
+  const int slots = compact ? 0 : kAnySlots;
+  PlanSet p;
+  p.compact = compact;
+  PairPlan* of[3] = {&p.p64, &p.p32, &p.pff};
+  for (int prec = 0; prec < 3; ++prec)
+    *of[prec] = nprob > 1 ? plan_pairs_batch(bs.data(), N, pb, nprob, kind, prec, slots)
+                          : plan_pairs(M, kind, prec, slots);
+  return p;
+}
+
 void carve(Arena& A, Work& w, int N, int M, int kind, int m, bool solve, bool stage_in, bool stage_ipt,
-           bool stage_load, bool stage_io, long long bj_floats = 0, int nprob = 0, const int* bs = nullptr,
-           const int* pb = nullptr, bool compact = false) {
+           bool stage_load, bool stage_io, const PlanSet& plans, long long bj_floats = 0, int nprob = 0) {
   const int comps = kind + 1;
   const long long n = (long long)M * comps;
   w.kind = kind;
@@ -317,17 +336,9 @@ void carve(Arena& A, Work& w, int N, int M, int kind, int m, bool solve, bool st
     w.io_in = A.take<double>(n);
     w.io_out = A.take<double>(n);
   }
-  // compact: without the symmetric plans that trade partial slots for time
-  const int slots = compact ? 0 : kAnySlots;
-  if (nprob > 1) {
-    w.plan64 = plan_pairs_batch(bs, N, pb, nprob, kind, 0, slots);
-    w.plan32 = plan_pairs_batch(bs, N, pb, nprob, kind, 1, slots);
-    w.planff = plan_pairs_batch(bs, N, pb, nprob, kind, 2, slots);
-  } else {
-    w.plan64 = plan_pairs(M, kind, 0, slots);
-    w.plan32 = plan_pairs(M, kind, 1, slots);
-    w.planff = plan_pairs(M, kind, 2, slots);
-  }
+  w.plan64 = plans.p64;
+  w.plan32 = plans.p32;
+  w.planff = plans.pff;
   // problems solved as one system share every Krylov array; nseg copies of the
   // Hessenberg and rotation arrays with one Krylov space per problem
   const int nseg = nprob > 1 ? nprob : 1;
@@ -373,7 +384,7 @@ void carve(Arena& A, Work& w, int N, int M, int kind, int m, bool solve, bool st
     w.sn = A.take<double>((size_t)nseg * m);
     w.gv = A.take<double>((size_t)nseg * (m + 1));
     w.yv = A.take<double>((size_t)nseg * (m + 1));
-    w.P = output_splits(g, kind, compact);
+    w.P = output_splits(g, kind, plans.compact);
     const int targets = kind == 0 ? N : 3 * N;
     w.outpart = A.take<double>((size_t)w.P * targets * comps + N + 2);
     w.outv = A.take<double>(3 * N);
@@ -410,20 +421,31 @@ int ensure_ws(bie_ctx* ctx, size_t need, cudaStream_t s) {
 // Sizes a call's workspace (carve with a null arena), makes it and carves it:
 // with the faster pair-sum plans where the context's cap allows their slots,
 // else compact.
-template <class Carve>
-int make_workspace(bie_ctx* ctx, Work& w, cudaStream_t s, const Carve& do_carve) {
-  bool compact = false;
+template <class Choose, class Carve>
+int make_workspace(bie_ctx* ctx, Work& w, cudaStream_t s, const Choose& choose, const Carve& do_carve) {
+  PlanSet plans = choose(false);
   Arena sz{nullptr};
-  do_carve(sz, w, compact);
+  do_carve(sz, w, plans);
   if (ctx->cap && sz.off > ctx->cap) {
-    compact = true;
+    plans = choose(true);
     sz = Arena{nullptr};
-    do_carve(sz, w, compact);
+    do_carve(sz, w, plans);
   }
   if (int rc = ensure_ws(ctx, sz.off, s)) return rc;
   Arena ar{ctx->ws};
-  do_carve(ar, w, compact);
+  do_carve(ar, w, plans);
   return BIE_OK;
+}
+
+// The workspace of one operator application.
+int make_operator_workspace(bie_ctx* ctx, Work& w, cudaStream_t s, const bie_geometry* geom, int kind,
+                            const std::vector<int>& bs) {
+  const int N = geom->n_bodies, M = bs[N];
+  return make_workspace(
+      ctx, w, s, [&](bool compact) { return choose_plans(kind, bs, compact); },
+      [&](Arena& A, Work& x, const PlanSet& plans) {
+        carve(A, x, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true, plans);
+      });
 }
 
 // Copies a host array into staging (or passes a device pointer through).
@@ -1143,10 +1165,12 @@ int solve_common(bie_ctx* ctx, const bie_geometry* geom, int kind, const double*
   }
   const bool use_bj = o.precond == 0 && !small;
   const long long bjf = use_bj ? bj_block_floats(bs.data(), N, kind) : 0;
-  if ((rc = make_workspace(ctx, w, s, [&](Arena& A, Work& x, bool compact) {
-        carve(A, x, N, M, kind, o.restart, true, true, has_ipt, true, false, bjf, batch ? P : 0, bs.data(), pb.data(),
-              compact);
-      })))
+  const int nprob = batch ? P : 0;
+  if ((rc = make_workspace(
+           ctx, w, s, [&](bool compact) { return choose_plans(kind, bs, compact, nprob, pb.data()); },
+           [&](Arena& A, Work& x, const PlanSet& plans) {
+             carve(A, x, N, M, kind, o.restart, true, true, has_ipt, true, false, plans, bjf, nprob);
+           })))
     return rc;
   if (batch) {
     if ((rc = batch_setup(ctx, *batch, bs, pb, has_ipt, w, where, s))) return rc;
@@ -1519,20 +1543,21 @@ size_t workspace_bytes_batch(int kind, const int* bs, int n_bodies, const int* p
   Work w;
   Arena sz{nullptr};
   const bool use_bj = o.precond == 0;
+  const std::vector<int> starts(bs, bs + n_bodies + 1);
   carve(sz, w, n_bodies, bs[n_bodies], kind, o.restart, true, true, true, true, false,
-        use_bj ? bj_block_floats(bs, n_bodies, kind) : 0, nprob, bs, pb);
+        choose_plans(kind, starts, false, nprob, pb), use_bj ? bj_block_floats(bs, n_bodies, kind) : 0, nprob);
   return sz.off;
 }
 
 void set_workspace_cap(bie_ctx* ctx, size_t cap) { ctx->cap = cap; }
 
 size_t workspace_bytes_for(int kind, const int* body_start_host, int n_bodies, int restart, bool compact) {
-  const int n_nodes = body_start_host[n_bodies];
+  const std::vector<int> bs(body_start_host, body_start_host + n_bodies + 1);
   Work w;
   Arena sz{nullptr};
   const int m = restart > 0 ? std::min(restart, 200) : 50;
-  carve(sz, w, n_bodies, n_nodes, kind, m, true, true, true, true, false,
-        bj_block_floats(body_start_host, n_bodies, kind), 0, nullptr, nullptr, compact);
+  carve(sz, w, n_bodies, bs[n_bodies], kind, m, true, true, true, true, false, choose_plans(kind, bs, compact),
+        bj_block_floats(body_start_host, n_bodies, kind));
   return sz.off;
 }
 }  // namespace bie
@@ -1559,10 +1584,7 @@ int apply_operator_fmm_prec(bie_ctx* ctx, const bie_geometry* geom, int kind, in
   DeviceGuard dg(ctx->device);
   const int N = geom->n_bodies, M = bs[N];
   Work w;
-  if ((rc = make_workspace(ctx, w, s, [&](Arena& A, Work& x, bool compact) {
-        carve(A, x, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true, 0, 0, nullptr, nullptr, compact);
-      })))
-    return rc;
+  if ((rc = make_operator_workspace(ctx, w, s, geom, kind, bs))) return rc;
   if ((rc = setup(ctx, geom, bs, w, s))) return rc;
   if ((rc = fmm_setup(ctx->fmm, w.g, kind, &order, 1, s, ctx->err, fmm_schedule(M, kind, order).leaf_nodes)))
     return rc;
@@ -1665,10 +1687,7 @@ int bie_tune(bie_ctx* ctx, const bie_geometry* geom, int kind, int precision, in
     return BIE_OK;
   }
   Work w;
-  if ((rc = make_workspace(ctx, w, s, [&](Arena& A, Work& x, bool compact) {
-        carve(A, x, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true, 0, 0, nullptr, nullptr, compact);
-      })))
-    return rc;
+  if ((rc = make_operator_workspace(ctx, w, s, geom, kind, bs))) return rc;
   if ((rc = setup(ctx, geom, bs, w, s))) return rc;
   // candidates: uniform split counts around the occupancy rule's, chunks of
   // whole source tiles (256 sources), and two-level plans (large chunks first,
@@ -1868,10 +1887,7 @@ int apply_operator(bie_ctx* ctx, const bie_geometry* geom, int kind, int precisi
   DeviceGuard dg(ctx->device);
   const int N = geom->n_bodies, M = bs[N];
   Work w;
-  if ((rc = make_workspace(ctx, w, s, [&](Arena& A, Work& x, bool compact) {
-        carve(A, x, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true, 0, 0, nullptr, nullptr, compact);
-      })))
-    return rc;
+  if ((rc = make_operator_workspace(ctx, w, s, geom, kind, bs))) return rc;
   if ((rc = setup(ctx, geom, bs, w, s))) return rc;
   const double* din;
   if ((rc = stage_in(ctx, in, w.io_in, (size_t)w.n, &din, s))) return rc;
