@@ -265,23 +265,38 @@ struct Work {
   int P = 1, grid = 1;
 };
 
-// The pair-sum plans of a call.  They depend on the process's table of tuned plans, which
+// The pair-sum plans of a call, of the precisions it sums directly (bits 1 << precision;
+// the others' partial slots would be reserved and never read: 313 MB for an FMM solve of
+// 100,000 Laplace nodes).  They depend on the process's table of tuned plans, which
 // another thread may change at any time: a call chooses them once, and sizes and lays out
 // its workspace with the same ones.
 struct PlanSet {
-  PairPlan p64, p32, pff;
+  PairPlan p64{0, 0, 0, 0}, p32{0, 0, 0, 0}, pff{0, 0, 0, 0};  // S = 0: not used
   bool compact = false;  // without the symmetric plans that trade partial slots for time
 };
+constexpr unsigned kAllSums = 7;
 
-PlanSet choose_plans(int kind, const std::vector<int>& bs, bool compact, int nprob = 0, const int* pb = nullptr) {
+// The direct pair sums of a solve.
+unsigned sums_of(const bie_opts& o) {
+  constexpr unsigned k64 = 1u << BIE_PREC_FP64, k32 = 1u << BIE_PREC_MIXED, kff = 1u << BIE_PREC_MIXED_FF;
+  unsigned u = o.formulation == 1 ? k64 : 0u;       // its right-hand side
+  if (o.precision == BIE_PREC_FP64) return u | k64;  // with the FMM: the verified residual
+  if (o.fmm_order <= 0) u |= k32;                    // the inner solves
+  if (o.fmm_order == 0) u |= o.precision == BIE_PREC_MIXED ? k64 : kff;  // the residuals
+  return u;
+}
+
+PlanSet choose_plans(int kind, const std::vector<int>& bs, unsigned sums, bool compact, int nprob = 0,
+                     const int* pb = nullptr) {
   const int N = (int)bs.size() - 1, M = bs[N];
   const int slots = compact ? 0 : kAnySlots;
   PlanSet p;
   p.compact = compact;
   PairPlan* of[3] = {&p.p64, &p.p32, &p.pff};
   for (int prec = 0; prec < 3; ++prec)
-    *of[prec] = nprob > 1 ? plan_pairs_batch(bs.data(), N, pb, nprob, kind, prec, slots)
-                          : plan_pairs(M, kind, prec, slots);
+    if (sums >> prec & 1)
+      *of[prec] = nprob > 1 ? plan_pairs_batch(bs.data(), N, pb, nprob, kind, prec, slots)
+                            : plan_pairs(M, kind, prec, slots);
   return p;
 }
 
@@ -361,7 +376,7 @@ void carve(Arena& A, Work& w, int N, int M, int kind, int m, bool solve, bool st
     w.bprob = A.take<int>(N);
     arn_units = items;
   }
-  const int S = std::max(std::max(w.plan64.S, w.plan32.S), w.planff.S);
+  const int S = std::max({1, w.plan64.S, w.plan32.S, w.planff.S});  // (1: the FMM's sums)
   w.partial = A.take<double>((size_t)S * n);
   w.grid = vec_grid(n);
   w.part = A.take<double>((size_t)w.grid * 201 + 64);
@@ -437,12 +452,12 @@ int make_workspace(bie_ctx* ctx, Work& w, cudaStream_t s, const Choose& choose, 
   return BIE_OK;
 }
 
-// The workspace of one operator application.
+// The workspace of one operator application with the direct sums `sums`.
 int make_operator_workspace(bie_ctx* ctx, Work& w, cudaStream_t s, const bie_geometry* geom, int kind,
-                            const std::vector<int>& bs) {
+                            const std::vector<int>& bs, unsigned sums) {
   const int N = geom->n_bodies, M = bs[N];
   return make_workspace(
-      ctx, w, s, [&](bool compact) { return choose_plans(kind, bs, compact); },
+      ctx, w, s, [&](bool compact) { return choose_plans(kind, bs, sums, compact); },
       [&](Arena& A, Work& x, const PlanSet& plans) {
         carve(A, x, N, M, kind, 1, false, true, geom->interior_pt != nullptr, false, true, plans);
       });
@@ -1166,8 +1181,10 @@ int solve_common(bie_ctx* ctx, const bie_geometry* geom, int kind, const double*
   const bool use_bj = o.precond == 0 && !small;
   const long long bjf = use_bj ? bj_block_floats(bs.data(), N, kind) : 0;
   const int nprob = batch ? P : 0;
+  // (the one-launch solves have pair sums of their own)
+  const unsigned sums = small ? sums_of(o) & (1u << BIE_PREC_FP64) : sums_of(o);
   if ((rc = make_workspace(
-           ctx, w, s, [&](bool compact) { return choose_plans(kind, bs, compact, nprob, pb.data()); },
+           ctx, w, s, [&](bool compact) { return choose_plans(kind, bs, sums, compact, nprob, pb.data()); },
            [&](Arena& A, Work& x, const PlanSet& plans) {
              carve(A, x, N, M, kind, o.restart, true, true, has_ipt, true, false, plans, bjf, nprob);
            })))
@@ -1545,18 +1562,20 @@ size_t workspace_bytes_batch(int kind, const int* bs, int n_bodies, const int* p
   const bool use_bj = o.precond == 0;
   const std::vector<int> starts(bs, bs + n_bodies + 1);
   carve(sz, w, n_bodies, bs[n_bodies], kind, o.restart, true, true, true, true, false,
-        choose_plans(kind, starts, false, nprob, pb), use_bj ? bj_block_floats(bs, n_bodies, kind) : 0, nprob);
+        choose_plans(kind, starts, sums_of(o), false, nprob, pb), use_bj ? bj_block_floats(bs, n_bodies, kind) : 0, nprob);
   return sz.off;
 }
 
 void set_workspace_cap(bie_ctx* ctx, size_t cap) { ctx->cap = cap; }
 
-size_t workspace_bytes_for(int kind, const int* body_start_host, int n_bodies, int restart, bool compact) {
+size_t workspace_bytes_for(int kind, const int* body_start_host, int n_bodies, int restart, const bie_opts* opts,
+                           bool compact) {
   const std::vector<int> bs(body_start_host, body_start_host + n_bodies + 1);
   Work w;
   Arena sz{nullptr};
   const int m = restart > 0 ? std::min(restart, 200) : 50;
-  carve(sz, w, n_bodies, bs[n_bodies], kind, m, true, true, true, true, false, choose_plans(kind, bs, compact),
+  carve(sz, w, n_bodies, bs[n_bodies], kind, m, true, true, true, true, false,
+        choose_plans(kind, bs, opts ? sums_of(*opts) : kAllSums, compact),
         bj_block_floats(body_start_host, n_bodies, kind));
   return sz.off;
 }
@@ -1584,7 +1603,7 @@ int apply_operator_fmm_prec(bie_ctx* ctx, const bie_geometry* geom, int kind, in
   DeviceGuard dg(ctx->device);
   const int N = geom->n_bodies, M = bs[N];
   Work w;
-  if ((rc = make_operator_workspace(ctx, w, s, geom, kind, bs))) return rc;
+  if ((rc = make_operator_workspace(ctx, w, s, geom, kind, bs, 0))) return rc;
   if ((rc = setup(ctx, geom, bs, w, s))) return rc;
   if ((rc = fmm_setup(ctx->fmm, w.g, kind, &order, 1, s, ctx->err, fmm_schedule(M, kind, order).leaf_nodes)))
     return rc;
@@ -1609,7 +1628,7 @@ size_t bie_workspace_bytes(int kind, int n_bodies, int n_nodes, int restart) {
   // preconditioner blocks sized for bodies of equal size
   std::vector<int> bs(n_bodies + 1);
   for (int i = 0; i <= n_bodies; ++i) bs[i] = (int)((long long)n_nodes * i / n_bodies);
-  return bie::workspace_bytes_for(kind, bs.data(), n_bodies, restart);
+  return bie::workspace_bytes_for(kind, bs.data(), n_bodies, restart, nullptr);
 }
 
 int bie_profile(bie_ctx* ctx, int enable, bie_profile_counters* out) {
@@ -1687,7 +1706,7 @@ int bie_tune(bie_ctx* ctx, const bie_geometry* geom, int kind, int precision, in
     return BIE_OK;
   }
   Work w;
-  if ((rc = make_operator_workspace(ctx, w, s, geom, kind, bs))) return rc;
+  if ((rc = make_operator_workspace(ctx, w, s, geom, kind, bs, 0))) return rc;
   if ((rc = setup(ctx, geom, bs, w, s))) return rc;
   // candidates: uniform split counts around the occupancy rule's, chunks of
   // whole source tiles (256 sources), and two-level plans (large chunks first,
@@ -1887,7 +1906,7 @@ int apply_operator(bie_ctx* ctx, const bie_geometry* geom, int kind, int precisi
   DeviceGuard dg(ctx->device);
   const int N = geom->n_bodies, M = bs[N];
   Work w;
-  if ((rc = make_operator_workspace(ctx, w, s, geom, kind, bs))) return rc;
+  if ((rc = make_operator_workspace(ctx, w, s, geom, kind, bs, 1u << precision))) return rc;
   if ((rc = setup(ctx, geom, bs, w, s))) return rc;
   const double* din;
   if ((rc = stage_in(ctx, in, w.io_in, (size_t)w.n, &din, s))) return rc;

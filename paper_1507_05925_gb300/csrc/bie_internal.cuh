@@ -247,10 +247,12 @@ void fmm_signature(const FmmState* f, std::vector<long long>& key);
 cudaError_t fmm_output(FmmState* f, const Geo& g, int kind, int p, const double* v, double* part, cudaStream_t s,
                        bool ff = false);
 
-// workspace of a solve with the given host body_start (bie_workspace_bytes assumes equal bodies);
-// compact: with the pair-sum plans of the fewest partial slots (a solve takes them
-// when its context's cap does not allow the faster ones)
-size_t workspace_bytes_for(int kind, const int* body_start_host, int n_bodies, int restart, bool compact = false);
+// workspace of a solve with the given host body_start (bie_workspace_bytes assumes equal bodies)
+// and these options (nullptr: of whichever needs most); compact: with the pair-sum plans of
+// the fewest partial slots (a solve takes them when its context's cap does not allow the
+// faster ones)
+size_t workspace_bytes_for(int kind, const int* body_start_host, int n_bodies, int restart, const bie_opts* opts,
+                           bool compact = false);
 // the cap of a context's workspace (0: none), as at its creation
 void set_workspace_cap(bie_ctx* ctx, size_t cap);
 // workspace of a batched solve (host arrays: concatenated body_start [N+1],

@@ -258,9 +258,10 @@ int bie_server_submit(bie_server* s, const bie_request* req, int64_t* ticket) {
   for (int i = 0; i < g.n_bodies; ++i)
     if (bs[i + 1] < bs[i]) return BIE_ERR_INVALID;
   cudaSetDevice(s->device);
-  size_t need = bie::workspace_bytes_for(req->kind, bs.data(), g.n_bodies, req->opts.restart);
+  size_t need = bie::workspace_bytes_for(req->kind, bs.data(), g.n_bodies, req->opts.restart, &req->opts);
   const bool compact = s->cap && need > s->cap;  // the cap allows the smaller workspace only, or not even that
-  if (compact) need = bie::workspace_bytes_for(req->kind, bs.data(), g.n_bodies, req->opts.restart, true);
+  if (compact)
+    need = bie::workspace_bytes_for(req->kind, bs.data(), g.n_bodies, req->opts.restart, &req->opts, true);
   if (s->cap && need > s->cap) return BIE_ERR_NOMEM;
   Job* j = new Job();
   j->req = *req;

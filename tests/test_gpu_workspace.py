@@ -1,0 +1,55 @@
+"""Device memory that a solve reserves for its pair sums' partial slots."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import synth  # noqa: E402
+from paper_1507_05925_gb300 import bie  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1507_05925_gb300 import build
+    build.build()
+
+
+def _reserved(kind, g, load, **opts):
+    """Bytes that the server reserves for a request of these options, run alone."""
+    srv = bie.Server(0, workers=1)
+    out = np.empty(load.size)
+    t = srv.submit(kind, g, load, out, opts=bie.make_opts(**opts))
+    assert t > 0
+    rc, info, _ = srv.wait(t)
+    peak = srv.stats()["peak_inflight_bytes"]
+    srv.close()
+    assert rc == bie.OK, info
+    return peak, out
+
+
+@pytest.mark.parametrize("kind", [bie.LAPLACE, bie.STOKES])
+def test_only_the_sums_of_the_call_reserve_slots(kind):
+    """160 bodies of 128 nodes: at 20,480 nodes the FP32 sums keep 107 to 160 slots, the
+    float-float and FP64 ones 5 to 160; FMM solves keep one."""
+    N, n = 160, 128
+    M = N * n
+    side = 13
+    g = synth.assemble([synth.ellipse(3.2 * (i % side), 3.2 * (i // side), 1.0, 0.7, 0.3 * i, n) for i in range(N)])
+    rng = np.random.default_rng(8)
+    load = synth.charges(N, rng) if kind == bie.LAPLACE else synth.forces_torques(N, rng).reshape(-1)
+    slot = 8 * M * (kind + 1)
+    direct, ref = _reserved(kind, g, load, precision=bie.MIXED_FF)
+    half, out_half = _reserved(kind, g, load, precision=bie.MIXED_FF, fmm_order=-36)
+    fmm, out = _reserved(kind, g, load, precision=bie.MIXED_FF, fmm_order=36)
+    assert direct - fmm >= 100 * slot
+    assert half <= direct and half - fmm >= 100 * slot  # FP32 direct sums inside
+    fmm_paper, _ = _reserved(kind, g, load, precision=bie.MIXED_FF, fmm_order=36, formulation=1)
+    assert fmm_paper > fmm  # the FP64 sum of its right-hand side
+    for o in (out_half, out):
+        assert np.linalg.norm(o - ref) <= 1e-9 * np.linalg.norm(ref)
+    whole = bie.workspace_bytes(kind, N, M)  # of whichever options need most
+    assert whole >= direct
