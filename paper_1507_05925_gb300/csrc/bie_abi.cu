@@ -415,8 +415,10 @@ void carve(Arena& A, Work& w, int N, int M, int kind, int m, bool solve, bool st
 }
 
 // Stream-ordered (cudaMallocAsync) so that growing one context's workspace
-// never synchronises the device under other contexts' work.
-int ensure_ws(bie_ctx* ctx, size_t need, cudaStream_t s) {
+// never synchronises the device under other contexts' work.  full: set if the
+// device has no room.
+int ensure_ws(bie_ctx* ctx, size_t need, cudaStream_t s, bool& full) {
+  full = false;
   if (need <= ctx->ws_size) return BIE_OK;
   if (ctx->cap && need > ctx->cap)
     return fail(ctx, BIE_ERR_NOMEM, "workspace of " + std::to_string(need) + " bytes exceeds the cap of " +
@@ -428,14 +430,17 @@ int ensure_ws(bie_ctx* ctx, size_t need, cudaStream_t s) {
   }
   for (auto& gi : ctx->graphs) cudaGraphExecDestroy(gi.exec);  // their pointers are stale
   ctx->graphs.clear();
-  CK(cudaMallocAsync(reinterpret_cast<void**>(&ctx->ws), need, s));
+  const cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&ctx->ws), need, s);
+  if (e != cudaSuccess) ctx->ws = nullptr;
+  full = e == cudaErrorMemoryAllocation;
+  CK(e);
   ctx->ws_size = need;
   return BIE_OK;
 }
 
 // Sizes a call's workspace (carve with a null arena), makes it and carves it:
-// with the faster pair-sum plans where the context's cap allows their slots,
-// else compact.
+// with the faster pair-sum plans where the context's cap and the device's free
+// memory allow their slots, else compact.
 template <class Choose, class Carve>
 int make_workspace(bie_ctx* ctx, Work& w, cudaStream_t s, const Choose& choose, const Carve& do_carve) {
   PlanSet plans = choose(false);
@@ -446,7 +451,15 @@ int make_workspace(bie_ctx* ctx, Work& w, cudaStream_t s, const Choose& choose, 
     sz = Arena{nullptr};
     do_carve(sz, w, plans);
   }
-  if (int rc = ensure_ws(ctx, sz.off, s)) return rc;
+  bool full = false;
+  int rc = ensure_ws(ctx, sz.off, s, full);
+  if (full && !plans.compact) {
+    plans = choose(true);
+    sz = Arena{nullptr};
+    do_carve(sz, w, plans);
+    rc = ensure_ws(ctx, sz.off, s, full);
+  }
+  if (rc) return rc;
   Arena ar{ctx->ws};
   do_carve(ar, w, plans);
   return BIE_OK;

@@ -53,3 +53,39 @@ def test_only_the_sums_of_the_call_reserve_slots(kind):
         assert np.linalg.norm(o - ref) <= 1e-9 * np.linalg.norm(ref)
     whole = bie.workspace_bytes(kind, N, M)  # of whichever options need most
     assert whole >= direct
+
+
+def test_full_device_takes_the_smaller_plans():
+    """With little device memory left, a call whose symmetric plan's slots do not fit runs
+    with the directed one's, as it does under a workspace cap."""
+    from test_gpu_parity import TOL64, rel_max, to_dev
+    N, n = 1000, 120
+    M = N * n
+    side = 32
+    g = to_dev(synth.assemble([synth.ellipse(3.2 * (i % side), 3.2 * (i // side), 1.0, 0.7, 0.3 * i, n)
+                               for i in range(N)]))
+    v = torch.randn(M, dtype=torch.float64, device="cuda")
+    out = torch.empty_like(v)
+    ctx = bie.Context(0)
+    assert bie.apply_operator(ctx, g, bie.LAPLACE, bie.FP64, v, out) == bie.OK
+    torch.cuda.synchronize()
+    ref = out.cpu().numpy()
+    assert bie.tune(ctx, g, bie.LAPLACE, bie.FP64, splits=1)[0] == bie.OK  # the directed kernel, now loaded too
+    assert bie.apply_operator(ctx, g, bie.LAPLACE, bie.FP64, v, out) == bie.OK
+    torch.cuda.synchronize()
+    ctx.close()
+    bie.tune_clear()
+    slots = 8 * M * 400  # the symmetric plan has more
+    torch.cuda.empty_cache()
+    held = torch.empty(torch.cuda.mem_get_info()[0] - (256 << 20), dtype=torch.uint8, device="cuda")
+    assert torch.cuda.mem_get_info()[0] < slots
+    out.fill_(float("nan"))
+    ctx = bie.Context(0)
+    rc = bie.apply_operator(ctx, g, bie.LAPLACE, bie.FP64, v, out)
+    torch.cuda.synchronize()
+    err = ctx.last_error()
+    ctx.close()
+    del held
+    torch.cuda.empty_cache()
+    assert rc == bie.OK, err
+    assert rel_max(out.cpu().numpy(), ref) <= 2 * TOL64
