@@ -187,21 +187,22 @@ int mobility_solve(bie_ctx* ctx, const bie_geometry* geom, const double* FT, dou
  * of that shape, in any context of the process, use it (the occupancy rule is
  * kept unless another plan is faster by 2%).  A different plan changes the
  * summation order, so results of that shape may change in rounding.
- * The FP32 and float-float Laplace pair sums have one more candidate, the
- * symmetric kernels (one CTA per unordered pair of 256-node tiles, each
- * difference, |r|^2 and reciprocal serving both directions of a pair; one
- * partial slot per tile), which are also the occupancy rule's plans once the
- * tile pairs fill the GPU four times over.  The FP64 pair sums have symmetric
- * plans too (tiles of 32 to 256 nodes by size), which are the occupancy rule's
- * where the context's workspace cap allows their partial slots; a count
- * reported for one is positive, and installing a count installs a directed
- * plan.
+ * Symmetric kernels (one CTA per unordered pair of tiles, each difference,
+ * |r|^2 and reciprocal serving both directions of a pair; one partial slot per
+ * tile) exist for the FP64 sums (tiles of 32 to 256 nodes), the FP32 sums (128 or
+ * 256 nodes, Stokes 128 or 192) and the float-float Laplace sums (256).  They are
+ * the occupancy rule's plans by size (FP64: always; FP32 once pairs of 128-node
+ * tiles fill the SMs six times over, Stokes four; float-float four with 256), where
+ * the context's workspace cap allows their slots.  The rule's own and, Laplace, the
+ * one of 256 nodes are candidates.
  * splits (nullable): on input 0 to search, a positive count to install a
  * uniform plan without timing (rounded to the counts the source chunking
- * allows), or a negative value to install the symmetric plan (Laplace with
- * BIE_PREC_MIXED or BIE_PREC_MIXED_FF only, else BIE_ERR_INVALID); on output
- * the number of splits of the plan kept, negated for the symmetric plan.  ms (nullable) receives its time (0 when
- * installed untimed).  Errors as for apply_operator. */
+ * allows), or a negative one to install the symmetric plan of that many tiles
+ * (FP32 and float-float Laplace: any other negative value installs the one of 256
+ * nodes; elsewhere a count that no symmetric plan has is BIE_ERR_INVALID); on output
+ * the number of splits of the plan kept, negated for a symmetric plan, so that
+ * installing it brings a uniform or symmetric plan back.  ms (nullable) receives its
+ * time (0 when installed untimed).  Errors as for apply_operator. */
 int bie_tune(bie_ctx* ctx, const bie_geometry* geom, int kind, int precision, int* splits, double* ms,
              void* stream);
 /* FMM schedule tuning (no counterpart in the paper).  Times whole solves of

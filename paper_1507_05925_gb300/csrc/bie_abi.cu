@@ -4,6 +4,7 @@
 // this library; the host only orders launches and reads the convergence state.
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 #include <stdio.h>
@@ -1710,9 +1711,13 @@ int bie_tune(bie_ctx* ctx, const bie_geometry* geom, int kind, int precision, in
   DeviceGuard dg(ctx->device);
   const int N = geom->n_bodies, M = bs[N];
   if (splits && *splits != 0) {  // install a plan, no timing
-    if (*splits < 0 && (precision == BIE_PREC_FP64 || kind != BIE_KIND_LAPLACE))
-      return fail(ctx, BIE_ERR_INVALID, "the symmetric plan exists for the FP32 and float-float Laplace pair sums only");
-    const PairPlan p = *splits > 0 ? plan_with_splits(M, *splits) : plan_symmetric(M);
+    PairPlan p = *splits > 0 ? plan_with_splits(M, *splits)
+                             : plan_with_tiles(M, kind, precision, *splits == INT_MIN ? INT_MAX : -*splits);
+    if (p.S == 0) {
+      if (precision == BIE_PREC_FP64 || kind != BIE_KIND_LAPLACE)
+        return fail(ctx, BIE_ERR_INVALID, "no symmetric plan of this many tiles");
+      p = plan_symmetric(M);  // FP32 and float-float Laplace: any negative value
+    }
     set_tuned_plan(M, kind, precision, p);
     *splits = p.sym ? -p.S : p.S;
     if (ms) *ms = 0.0;
@@ -1799,9 +1804,7 @@ int bie_tune(bie_ctx* ctx, const bie_geometry* geom, int kind, int precision, in
     best_ms = s0_ms;
   }
   set_tuned_plan(M, kind, precision, best);
-  // only the symmetric plans that a negative count installs are reported negated
-  const bool installable = best.sym && kind == BIE_KIND_LAPLACE && precision != BIE_PREC_FP64;
-  if (splits) *splits = installable ? -best.S : best.S;
+  if (splits) *splits = best.sym ? -best.S : best.S;
   if (ms) *ms = best_ms;
   return BIE_OK;
 }

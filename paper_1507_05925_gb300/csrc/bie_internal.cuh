@@ -189,6 +189,8 @@ PairPlan occupancy_plan(int M, int kind, int precision, int max_slots = kAnySlot
 PairPlan plan_symmetric64(int M, int kind, int max_slots);
 PairPlan plan_symmetric32(int M, int kind, int max_slots);
 PairPlan plan_with_splits(int M, int S);
+// the symmetric plan of that many tiles (S = 0: this kind and precision has none)
+PairPlan plan_with_tiles(int M, int kind, int precision, int tiles);
 // two-level plan: a fraction f of the sources in chunks of c1, the rest in chunks of c2
 PairPlan plan_two_level(int M, int c1, int c2, double f);
 // the symmetric FP32 Laplace pair sum (partials: one slot per 256-node tile)

@@ -1827,6 +1827,19 @@ PairPlan plan_symmetric32(int M, int kind, int max_slots) {
   return p;
 }
 
+PairPlan plan_with_tiles(int M, int kind, int precision, int tiles) {
+  const PairPlan p0 = occupancy_plan(M, kind, precision);
+  if (p0.sym && p0.S == tiles) return p0;  // (counts of small M may stand for several sizes)
+  const int sizes[3][2][4] = {{{256, 128, 64, 32}, {256, 128, 64, 32}}, {{kTS, 128}, {192, 128}}, {{kTileF}, {}}};
+  for (int tile : sizes[precision][kind]) {
+    if (tile == 0 || (M + tile - 1) / tile != tiles || (double)tiles * M * (kind + 1) * 8e-6 > 512.0) continue;
+    PairPlan p = uniform_plan(tiles, tile);
+    p.sym = tile;
+    return p;
+  }
+  return PairPlan{0, 0, 0, 0};
+}
+
 PairPlan plan_pairs(int M, int kind, int precision, int max_slots) {
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
