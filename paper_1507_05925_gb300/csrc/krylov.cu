@@ -314,11 +314,11 @@ __device__ __forceinline__ void arn_stage_rotations(const ArnoldiArgs& a, const 
 // applies the rotations; no global round trips in the chain).
 template <class R>
 __device__ __noinline__ void arn_hessenberg(const ArnoldiArgs& a, KState* st, int j, const R* hs1, const R* hs2,
-                                            R hn2, ArnRotations& q, unsigned bar) {
+                                            double hn2, ArnRotations& q, unsigned bar) {
   for (int i = threadIdx.x; i <= j; i += kBV) q.hcol[i] = (double)hs1[i] + (double)hs2[i];
   __syncthreads();
   if (threadIdx.x == 0) {
-    const double hn = sqrt((double)hn2);
+    const double hn = sqrt(hn2);
     double c, sg, r;
     givens(rotate_column(q.css, q.sns, q.hcol, j), hn, c, sg, r);
     const double res = fabs(sg * q.g);
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kBV, NARROW ? 1 : 4) k_arnoldi(ArnoldiArgs a) 
   }
   __syncthreads();
   const double h22 = h22_s;
-  if (h22 <= 0.25 * hs2[jc]) {
+  if (h22 <= kNormBySubtraction * hs2[jc]) {
     const double hn2 = hs2[jc] - h22, sc = a.wt ? 1.0 : hn2 > 0.0 ? 1.0 / sqrt(hn2) : 0.0;
     double* wo = a.wt ? a.wt : w;  // a.wt: normalised by the preconditioner's launch
     for (long long k = blockIdx.x * (long long)kBV + threadIdx.x; k < n; k += stride)
@@ -717,10 +717,10 @@ __global__ void __launch_bounds__(kBV, PREFETCH ? 1 : 4) k_arnoldi32(ArnoldiArgs
     if (i + 1 < jc) q1 = fmaf(hs2[i + 1], hs2[i + 1], q1);
   }
   const float h22 = q0 + q1;
-  if (single && h22 <= 0.25f * hs2[jc]) {
-    const float nn = hs2[jc] - h22, inv = nn > 0.f ? 1.f / sqrtf(nn) : 0.f;
+  if (single && h22 <= (float)kNormBySubtraction * hs2[jc]) {
+    const float nn = hs2[jc] - h22, inv = nn > 0.f ? rsqrt_rounded(nn, (hs2[jc] - nn) - h22) : 0.f;
     if (blockIdx.x == 0) {
-      arn_hessenberg(a, st, j, hs1, hs2, nn, rot, bar);
+      arn_hessenberg(a, st, j, hs1, hs2, (double)hs2[jc] - (double)h22, rot, bar);
       return;
     }
     if (own >= a.g.N) return;
@@ -768,8 +768,8 @@ __global__ void __launch_bounds__(kBV, PREFETCH ? 1 : 4) k_arnoldi32(ArnoldiArgs
   if (grid_barrier(st, bar, a.spins)) return;
   __shared__ float hn2[1];
   arn_grid_sum32(part3, 1, hn2);
-  if (blockIdx.x == 0) arn_hessenberg(a, st, j, hs1, hs2, hn2[0], rot, bar);
-  const float inv = hn2[0] > 0.f ? 1.f / sqrtf(hn2[0]) : 0.f;
+  if (blockIdx.x == 0) arn_hessenberg(a, st, j, hs1, hs2, (double)hn2[0], rot, bar);
+  const float inv = hn2[0] > 0.f ? rsqrt_rounded(hn2[0], 0.f) : 0.f;
   if (!a.blocks) {
     // v_{j+1} = w / ||w|| over this CTA's own elements
     for (long long c = blockIdx.x * (long long)kBV + threadIdx.x; c < n4; c += stride) {

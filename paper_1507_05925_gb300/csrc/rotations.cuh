@@ -1,4 +1,5 @@
-// Givens rotations of the GMRES steps, by one thread in FP64.
+// Scalar steps of GMRES: Givens rotations, by one thread in FP64, and the scale of the new
+// basis vector.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -33,6 +34,21 @@ __device__ __forceinline__ double rotate_column(const double* css, const double*
     x = fma(-s, x, c * y);
   }
   return x;
+}
+
+// ||w - V h||^2 = ||w||^2 - ||h||^2 stands in for the sum over the new vector while h is that
+// small a part: the rounding of ||h||^2 then is below a tenth of ||w||^2's own.
+constexpr double kNormBySubtraction = 0x1p-10;
+
+// 1/sqrt(h + l), h > 0 and l its low part, in FP32 to within (1/2 + 2^-15) ulp, as the
+// rounded quotient of the FP64 root is: one Newton step on the quotient of the rounded root (1
+// ulp off), whose residual 1 - (h + l) y^2 comes out of error-free products.  (FP64 by
+// every thread costs the narrow pipe thousands of clocks.)
+__host__ __device__ __forceinline__ float rsqrt_rounded(float h, float l) {
+  const float y = 1.f / sqrtf(h);
+  const float p = y * y, d = fmaf(y, y, -p);
+  const float e = fmaf(-l, p, fmaf(-h, d, fmaf(-h, p, 1.f)));
+  return fabsf(e) < 1e-3f ? fmaf(0.5f * y, e, y) : y;  // (y^2 outside FP32's range: no step)
 }
 
 }  // namespace bie

@@ -359,7 +359,7 @@ __device__ int cta_gmres(const SmallArgs& A, int a0, int a1, int i0, int i1, lon
         h22 = warp_sum(h22);
         if (lane == 0) {
           sh.scal[1] = sh.h2[j + 1] - h22;
-          sh.flag[0] = !(h22 <= 0.25 * sh.h2[j + 1]);
+          sh.flag[0] = !(h22 <= kNormBySubtraction * sh.h2[j + 1]);
         }
       }
       __syncthreads();
