@@ -312,6 +312,11 @@ void bie_test_arm_barrier_timeout(int skip_cta, long long spins);
  * `stream`; BIE_ERR_INVALID for NULL arrays or n < 0. */
 int bie_test_log(const double* x, double* out, long long n, void* stream);
 
+/* Test hook of the FP64 pair sums' reciprocal (no counterpart in the paper): for
+ * device arrays x [n] and out [n], out[i] = 1/x[i] as the FP64 kernels form it.
+ * Asynchronous on `stream`; BIE_ERR_INVALID for NULL arrays or n < 0. */
+int bie_test_rcp(const double* x, double* out, long long n, void* stream);
+
 /* Test hook of the block-Jacobi safeguard (no counterpart in the paper): pivots
  * of later block factorisations count as bad when |p| < floor (default 1e-3 for
  * floor <= 0), so that a test can drive every body onto the identity block and

@@ -106,6 +106,8 @@ def load():
     lib.apply_operator_fmm.restype = i32
     lib.bie_test_log.argtypes = [vp, vp, ctypes.c_int64, vp]
     lib.bie_test_log.restype = i32
+    lib.bie_test_rcp.argtypes = [vp, vp, ctypes.c_int64, vp]
+    lib.bie_test_rcp.restype = i32
     lib.apply_operator_fmm_prec.argtypes = [vp, ctypes.POINTER(BieGeometry), i32, i32, i32, vp, vp, vp]
     lib.apply_operator_fmm_prec.restype = i32
     lib.apply_operator_noalloc.argtypes = [ctypes.POINTER(BieGeometry), i32, i32, vp, vp, vp]
@@ -449,7 +451,13 @@ def test_log(x, out, stream=None) -> int:
     return load().bie_test_log(_ptr(x), _ptr(out), int(x.numel()), _stream_ptr(stream))
 
 
+def test_rcp(x, out, stream=None) -> int:
+    """bie_test_rcp: out = 1/x as the FP64 kernels form it."""
+    return load().bie_test_rcp(_ptr(x), _ptr(out), int(x.numel()), _stream_ptr(stream))
+
+
 test_log.__test__ = False
+test_rcp.__test__ = False
 
 
 def apply_operator_fmm_prec(ctx: Context, geom, kind: int, order: int, precision: int, inp, out,

@@ -589,8 +589,20 @@ __global__ void __launch_bounds__(256) k_test_log(const double* __restrict__ x, 
     out[n + i] = log(x[i]);
   }
 }
+__global__ void __launch_bounds__(256) k_test_rcp(const double* __restrict__ x, long long n, double* __restrict__ out) {
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += (long long)gridDim.x * 256) out[i] = rcp64(x[i]);
+}
 }  // namespace
 }  // namespace bie
+
+extern "C" int bie_test_rcp(const double* x, double* out, long long n, void* stream) {
+  if (!x || !out || n < 0) return BIE_ERR_INVALID;
+  if (n == 0) return BIE_OK;
+  const long long b = (n + 255) / 256;
+  bie::k_test_rcp<<<(unsigned)(b > 4096 ? 4096 : b), 256, 0, (cudaStream_t)stream>>>(x, n, out);
+  bie::note_launches(1);
+  return cudaGetLastError() == cudaSuccess ? BIE_OK : BIE_ERR_CUDA;
+}
 
 extern "C" int bie_test_log(const double* x, double* out, long long n, void* stream) {
   if (!x || !out || n < 0) return BIE_ERR_INVALID;
