@@ -312,8 +312,9 @@ void bie_test_arm_barrier_timeout(int skip_cta, long long spins);
  * `stream`; BIE_ERR_INVALID for NULL arrays or n < 0. */
 int bie_test_log(const double* x, double* out, long long n, void* stream);
 
-/* Test hook of the FP64 pair sums' reciprocal (no counterpart in the paper): for
- * device arrays x [n] and out [n], out[i] = 1/x[i] as the FP64 kernels form it.
+/* Test hook of the kernels' reciprocals (no counterpart in the paper): for device
+ * arrays x [n] and out [2n], out[i] = 1/x[i] as the FP64 pair sums form it and
+ * out[n + i] = 1/(float)x[i] as the FP32 preconditioner blocks form it.
  * Asynchronous on `stream`; BIE_ERR_INVALID for NULL arrays or n < 0. */
 int bie_test_rcp(const double* x, double* out, long long n, void* stream);
 

@@ -452,7 +452,7 @@ def test_log(x, out, stream=None) -> int:
 
 
 def test_rcp(x, out, stream=None) -> int:
-    """bie_test_rcp: out = 1/x as the FP64 kernels form it."""
+    """bie_test_rcp: out[:n] = 1/x as the FP64 pair sums form it, out[n:] as the FP32 blocks do."""
     return load().bie_test_rcp(_ptr(x), _ptr(out), int(x.numel()), _stream_ptr(stream))
 
 

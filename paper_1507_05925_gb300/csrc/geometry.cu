@@ -590,7 +590,10 @@ __global__ void __launch_bounds__(256) k_test_log(const double* __restrict__ x, 
   }
 }
 __global__ void __launch_bounds__(256) k_test_rcp(const double* __restrict__ x, long long n, double* __restrict__ out) {
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += (long long)gridDim.x * 256) out[i] = rcp64(x[i]);
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
+    out[i] = rcp64(x[i]);
+    out[n + i] = (double)rcp32((float)x[i]);
+  }
 }
 }  // namespace
 }  // namespace bie

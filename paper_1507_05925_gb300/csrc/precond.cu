@@ -35,6 +35,7 @@
 
 #include "../../include/bie2d.h"
 #include "bie_internal.cuh"
+#include "pair_math.cuh"
 #include "reduce.cuh"
 
 namespace cg = cooperative_groups;
@@ -95,18 +96,11 @@ struct BlockRow {
     pa0 = (float)(-(g.y[a] - g.yc[i]));
     pa1 = (float)(g.x[a] - g.xc[i]);
   }
-  // 1/x to a rounding, without the branches of the division (which kept the entries of a
-  // row from overlapping: assembly 25,000 clocks at 256 rows)
-  __device__ static float reciprocal(float x) {
-    float y;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return fmaf(fmaf(-x, y, 1.0f), y, y);
-  }
   // column data: cp = (x_hi, y_hi, x_lo, y_lo), cw = (sqrt(w), p_1, p_2, node index)
   __device__ float entry(int r, int c, float4 cp, float4 cw) const {  // Laplace
     const int b = __float_as_int(cw.w);
     const float rx = (pa.x - cp.x) + (pa.z - cp.z), ry = (pa.y - cp.y) + (pa.w - cp.w);
-    const float i2 = reciprocal(a == b ? 1.f : rx * rx + ry * ry);
+    const float i2 = rcp32(a == b ? 1.f : rx * rx + ry * ry);
     const float k = a == b ? -ka * (float)kInv4Pi : -(float)kInv2Pi * ((rx * nxa + ry * nya) * i2);
     return (r == c ? 0.5f : 0.f) + swa * cw.x * (k + cf);
   }
@@ -115,7 +109,7 @@ struct BlockRow {
     const int b = __float_as_int(cw.w);
     const float rx = (pa.x - cp.x) + (pa.z - cp.z), ry = (pa.y - cp.y) + (pa.w - cp.w);
     const bool self = a == b;
-    const float i2 = reciprocal(self ? 1.f : rx * rx + ry * ry);
+    const float i2 = rcp32(self ? 1.f : rx * rx + ry * ry);
     const float t = self ? -0.5f * (float)kInvPi * ka * (al == 0 ? -nya : nxa)
                          : -(float)kInvPi * (al == 0 ? rx : ry) * ((rx * nxa + ry * nya) * i2);
     const float k0 = t * (self ? -nya : rx * i2), k1 = t * (self ? nxa : ry * i2);

@@ -1,5 +1,5 @@
-"""The FP64 kernels' reciprocal (csrc/pair_math.cuh) against 1/x in extended precision,
-over mantissas and exponents, and at the ends of the range."""
+"""The kernels' reciprocals (csrc/pair_math.cuh) against 1/x in extended precision, over
+mantissas and exponents, and at the ends of the range."""
 import numpy as np
 import pytest
 
@@ -22,10 +22,11 @@ def built():
 
 def reciprocal(x):
     xd = torch.from_numpy(np.ascontiguousarray(x)).cuda()
-    out = torch.full_like(xd, float("nan"))
+    out = torch.full((2 * x.size,), float("nan"), dtype=torch.float64, device="cuda")
     assert bie.test_rcp(xd, out) == bie.OK
     torch.cuda.synchronize()
-    return out.cpu().numpy()
+    out = out.cpu().numpy()
+    return out[:x.size], out[x.size:]
 
 
 def test_reciprocal_over_mantissas_and_exponents():
@@ -35,7 +36,7 @@ def test_reciprocal_over_mantissas_and_exponents():
                         rng.uniform(1.0, 2.0, n)])
     x = np.ldexp(m, rng.integers(-1021, 1021, m.size)) * rng.choice([-1.0, 1.0], m.size)
     exact = np.longdouble(1.0) / x.astype(np.longdouble)
-    err = np.abs(reciprocal(x).astype(np.longdouble) - exact) / np.spacing(np.abs(exact).astype(np.float64))
+    err = np.abs(reciprocal(x)[0].astype(np.longdouble) - exact) / np.spacing(np.abs(exact).astype(np.float64))
     print(f"largest error {float(err.max()):.4f} ulp")
     # the last rounding, |e|^3 < 2^-57 (1/16 ulp at most), and the roundings of e, e + e^2
     assert float(err.max()) <= 0.5 + 2.0 ** -4 + 2.0 ** -15
@@ -43,9 +44,22 @@ def test_reciprocal_over_mantissas_and_exponents():
 
 def test_reciprocal_at_the_ends():
     x = np.array([np.inf, -np.inf, np.finfo(np.float64).max, 2.0 ** 1023, 0.0, -0.0, 2.0 ** -1074, np.nan])
-    r = reciprocal(x)
+    r, _ = reciprocal(x)
     assert np.array_equal(r[:4], [0.0, -0.0, 0.0, 0.0])  # (1/x of the middle two is below 2^-1022)
     assert r[4] == np.inf and r[5] == -np.inf and r[6] == np.inf and np.isnan(r[7])
+
+
+def test_fp32_reciprocal():
+    rng = np.random.default_rng(3)
+    n = 1 << 20
+    x = np.ldexp(rng.uniform(1.0, 2.0, n), rng.integers(-125, 125, n)).astype(np.float32)
+    _, r = reciprocal(x.astype(np.float64))
+    exact = 1.0 / x.astype(np.float64)
+    err = np.abs(r - exact) / np.spacing(exact.astype(np.float32))
+    print(f"largest error {err.max():.6f} ulp")
+    assert err.max() <= 0.5 + 2.0 ** -20  # the last rounding and e^2 <= 2^-44
+    _, r = reciprocal(np.array([np.inf, -np.inf, 2.0 ** -140, 0.0, np.nan]))
+    assert r[0] == 0.0 and r[1] == 0.0 and r[2] == np.inf and r[3] == np.inf and np.isnan(r[4])
 
 
 @pytest.mark.parametrize("n", [40, 300])
