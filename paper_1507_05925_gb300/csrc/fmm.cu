@@ -107,7 +107,50 @@ struct FmmDevT {
   const float2* Qf = nullptr;  // FP32 expansions: q per source in FP32 (channel 0), written by k_fmm_p2m32
   const float4* cen32 = nullptr;  // FP32 expansions: leaf centres split hi + lo
   float is32 = 0.f, s32 = 0.f;    // FP32 expansions: 1/s and s of a leaf
+  int per = 1, tper = 1;          // boxes a block goes over: of one level, of all levels (boxes_a_block)
 };
+
+// Trees of few large bodies are mostly empty (100,000 nodes on one curve: 3,300 of a
+// million leaves), and a block for every box costs more than the work: a block with a large
+// shared array holds an SM's place for a microsecond to find its box empty.  There a block
+// goes over several boxes, a grid's width apart (neighbours along a curve stay with
+// different blocks), so many that it expects an eighth of a box to do; a tree at least 1/32 full
+// keeps a block a box (at 1/16 blocks with two or three boxes cost more than the empty
+// ones: Laplace, 20 bodies of 2,000 nodes, 517 -> 548 us an application).  One Stokes body
+// of 100,000 nodes, a block a box and so: FP32 M2L 1,208 -> 74 us, float-float 3,496 -> 452,
+// FP32 M2M 442 -> 66, FP64 2,167 -> 256, FP32 evaluation 547 -> 55; a solve 82 -> 38 ms.
+inline int boxes_a_block(double used, double all) {
+  return used * 32.0 >= all ? 1 : (int)fmin(32.0, 0.125 * all / fmax(used, 1.0));
+}
+// The same for the boxes of all levels 2..L of which level l uses at most used(l).
+template <class F>
+int boxes_a_block_levels(int L, F&& used) {
+  double u = 0.0, all = 0.0;
+  for (int l = 2; l <= L; ++l) {
+    const double n = (double)(1LL << (2 * l));
+    u += fmin(n, used(l));
+    all += n;
+  }
+  return boxes_a_block(u, all);
+}
+inline unsigned blocks_for(long long boxes, int per) { return (unsigned)((boxes + per - 1) / per); }
+
+// body(box) for the block's box, or (MANY) for its boxes blockIdx.x + i gridDim.x, i < per,
+// of `boxes` that hold something.
+template <bool MANY, class F>
+__device__ __forceinline__ void for_boxes(const int* __restrict__ count, long long boxes, int per, F&& body) {
+  if (!MANY) {
+    body((long long)blockIdx.x);
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  const long long own = blockIdx.x + (long long)lane * gridDim.x;
+  unsigned todo = __ballot_sync(0xffffffffu, lane < per && own < boxes && count[own] > 0);  // the same in every warp
+  while (todo) {
+    body(blockIdx.x + (long long)(__ffs(todo) - 1) * gridDim.x);
+    todo &= todo - 1;
+  }
+}
 using FmmDev = FmmDevT<double2>;
 
 template <class T2>
@@ -480,15 +523,16 @@ size_t shift_smem(int nd, int pk) {
   return (size_t)8 * nd * (pk + 1) * sizeof(T2);
 }
 
-// M2M of all levels L-1..2 in one launch: a block forms one box of level L-1, and
-// the block that completes the last of four siblings goes on with their parent
-// (no block waits; arrive[] counts the siblings and is back at 0 at the end).
+// M2M of all levels L-1..2 in one launch: a block forms one box of level L-1 (in a mostly
+// empty tree several), and the block that completes the last of four siblings (there: of those
+// with sources) goes on with their parent (no block waits; arrive[] counts the siblings and
+// is back at 0 at the end).
 // Each level was a launch of one 64-thread block a box, the children one after
 // the other with their matrices staged: all levels, FP32 Laplace, 1,024 leaves, order
 // 15: 31 -> 9.0 us; FP32 Stokes, 16,384 leaves, order 18: 83 -> 35 us; FP64 Stokes, order
 // 36: 995 -> 222 us (L2L: 17 -> 6.8, 49 -> 31 and 700 -> 235 us).  What is left is the
 // chain of levels (2-3 us each), in FP64 the FP64 pipe.
-template <class T2, int NC, int PK>
+template <class T2, int NC, int PK, bool MANY>
 __global__ void __launch_bounds__(shift_max_threads(NC, PK), shift_blocks<T2>(NC, PK))
 k_fmm_m2m(FmmDevT<T2> f, int* arrive, const int* stop) {
   using R = decltype(T2{}.x);
@@ -507,69 +551,77 @@ k_fmm_m2m(FmmDevT<T2> f, int* arrive, const int* stop) {
   }
   for (int w = t; w < 4 * f.nd * (PK + 1 - p); w += blockDim.x)  // the padding
     U[w / (PK + 1 - p) * (PK + 1) + p + w % (PK + 1 - p)] = cx<T2>(0.0, 0.0);
-  int b = blockIdx.x;
-  for (int l = f.L - 1;; --l) {
-    const int n = 1 << l, bx = b & (n - 1), by = b >> l;
-    const long long box = lev_off(l) + b;
-    if (f.count[box] > 0) {
-      if (t < np) {
-        // other blocks of this launch wrote the children above the first level: past L1
-        T2 v[4];
+  const long long boxes = 1LL << (2 * (f.L - 1));
+  for_boxes<MANY>(f.count + lev_off(f.L - 1), boxes, f.per, [&](long long first) {
+    int b = (int)first;
+    for (int l = f.L - 1;; --l) {
+      const int n = 1 << l, bx = b & (n - 1), by = b >> l;
+      const long long box = lev_off(l) + b;
+      if (MANY || f.count[box] > 0) {
+        if (t < np) {
+          // other blocks of this launch wrote the children above the first level: past L1
+          T2 v[4];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int c = child_of_turn(r);
-          const long long child = lev_off(l + 1) + (long long)(2 * by + (c >> 1)) * (2 * n) + 2 * bx + (c & 1);
-          v[r] = cx<T2>(0.0, 0.0);
-          if (f.count[child] > 0) v[r] = __ldcg(f.mp + child * np + e);
-        }
-        quarter_sums(v);
+          for (int r = 0; r < 4; ++r) {
+            const int c = child_of_turn(r);
+            const long long child = lev_off(l + 1) + (long long)(2 * by + (c >> 1)) * (2 * n) + 2 * bx + (c & 1);
+            v[r] = cx<T2>(0.0, 0.0);
+            if (f.count[child] > 0) v[r] = __ldcg(f.mp + child * np + e);
+          }
+          quarter_sums(v);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) U[q * US + d * (PK + 1) + k] = eighth_conj(v[q], k);
-      }
-      __syncthreads();
-      if (f.cm >= 0) {
-        // child moment density relative to the parent centre: 1/2 rho_r + conj(w_r) a_r, whose
-        // transform is 1/2 that of rho plus conj(w) times that of a, one place back
-        if (t < 4 * p) {
-          const int q = t / p, m = t - q * p;
-          T2 a = U[q * US + f.cm * (PK + 1) + m];
-          a.x *= R(0.5);
-          a.y *= R(0.5);
-          cfma(a, cx<T2>(0.25, -0.25), U[((q + 3) & 3) * US + m]);
-          U[q * US + f.cm * (PK + 1) + m] = a;
+          for (int q = 0; q < 4; ++q) U[q * US + d * (PK + 1) + k] = eighth_conj(v[q], k);
         }
         __syncthreads();
-      }
-      if (mr < 4) {
-        T2 acc = cx<T2>(0.0, 0.0);
-        const T2* u = U + ((k - mr) & 3) * US + d * (PK + 1) + mr;
-#pragma unroll
-        for (int i = 0; i < PK / 4; ++i) {
-          const T2 x = u[4 * i];
-          acc.x = fma(T[i], x.x, acc.x);
-          acc.y = fma(T[i], x.y, acc.y);
+        if (f.cm >= 0) {
+          // child moment density relative to the parent centre: 1/2 rho_r + conj(w_r) a_r, whose
+          // transform is 1/2 that of rho plus conj(w) times that of a, one place back
+          if (t < 4 * p) {
+            const int q = t / p, m = t - q * p;
+            T2 a = U[q * US + f.cm * (PK + 1) + m];
+            a.x *= R(0.5);
+            a.y *= R(0.5);
+            cfma(a, cx<T2>(0.25, -0.25), U[((q + 3) & 3) * US + m]);
+            U[q * US + f.cm * (PK + 1) + m] = a;
+          }
+          __syncthreads();
         }
-        red[t] = acc;
+        if (mr < 4) {
+          T2 acc = cx<T2>(0.0, 0.0);
+          const T2* u = U + ((k - mr) & 3) * US + d * (PK + 1) + mr;
+#pragma unroll
+          for (int i = 0; i < PK / 4; ++i) {
+            const T2 x = u[4 * i];
+            acc.x = fma(T[i], x.x, acc.x);
+            acc.y = fma(T[i], x.y, acc.y);
+          }
+          red[t] = acc;
+        }
+        __syncthreads();
+        if (t < np) {
+          const T2 a = cadd(cadd(red[t], red[np + t]), cadd(red[2 * np + t], red[3 * np + t]));
+          f.mp[box * np + t] = eighth(a, k);
+        }
+      }
+      if (l == 2) return;
+      __syncthreads();
+      b = (by >> 1) * (n >> 1) + (bx >> 1);
+      if (t == 0) {
+        __threadfence();  // the block's stores, ordered before it by the barrier
+        int* a = arrive + lev_off(l - 1) + b;
+        int siblings = 4;  // the boxes that arrive
+        if (MANY) {        // only those with sources
+          const int* c = f.count + lev_off(l) + (by & ~1) * n + (bx & ~1);
+          siblings = (c[0] > 0) + (c[1] > 0) + (c[n] > 0) + (c[n + 1] > 0);
+        }
+        s_last = atomicAdd(a, 1) == siblings - 1;
+        if (s_last) *a = 0;
+        __threadfence();
       }
       __syncthreads();
-      if (t < np) {
-        const T2 a = cadd(cadd(red[t], red[np + t]), cadd(red[2 * np + t], red[3 * np + t]));
-        f.mp[box * np + t] = eighth(a, k);
-      }
+      if (!s_last) return;
     }
-    if (l == 2) return;
-    __syncthreads();
-    b = (by >> 1) * (n >> 1) + (bx >> 1);
-    if (t == 0) {
-      __threadfence();  // the block's stores, ordered before it by the barrier
-      int* a = arrive + lev_off(l - 1) + b;
-      s_last = atomicAdd(a, 1) == 3;
-      if (s_last) *a = 0;
-      __threadfence();
-    }
-    __syncthreads();
-    if (!s_last) return;
-  }
+  });
 }
 
 // M2L for the target boxes of all levels 2..L (one block per box), through
@@ -718,14 +770,12 @@ __device__ __forceinline__ void orbit_stage(const FmmDevT<T2>& f, const OrbitLis
 
 // FP64.  Threads: split x (channel, row).
 template <class T2, int NJ>
-__global__ void __launch_bounds__(256) k_fmm_m2l(FmmDevT<T2> f, int nsplit, int nbo, const int* stop) {
+__device__ __forceinline__ void m2l_box(const FmmDevT<T2>& f, long long gb, int nsplit, int nbo) {
   using R = decltype(T2{}.x);
-  if (stop && *stop) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ OrbitList o;
   __shared__ T2 s_a0[kOrbits][kMaxNd][4];  // the transforms of a_0 of the logarithm channels
   __shared__ T2 red[256];
-  long long gb = blockIdx.x + lev_off(2);
   int l = 2;
   while (l < f.L && gb >= lev_off(l + 1)) ++l;
   if (f.tcount[gb] == 0) return;
@@ -813,6 +863,13 @@ __global__ void __launch_bounds__(256) k_fmm_m2l(FmmDevT<T2> f, int nsplit, int 
   }
 }
 
+template <class T2, int NJ, bool MANY>
+__global__ void __launch_bounds__(256) k_fmm_m2l(FmmDevT<T2> f, int nsplit, int nbo, const int* stop) {
+  if (stop && *stop) return;
+  for_boxes<MANY>(f.tcount + lev_off(2), lev_off(f.L + 1) - lev_off(2), f.tper,
+                  [&](long long b) { m2l_box<T2, NJ>(f, b + lev_off(2), nsplit, nbo); });
+}
+
 // FP32, Cauchy channels (the inner solves' operator), ND channels of order p <= PK
 // (coefficients padded with zeros to the instance's order).  Bound by instruction
 // issue (71%), so the work around the multiply-adds is what counts:
@@ -837,16 +894,13 @@ __host__ __device__ constexpr int m2l32_threads(int nd, int pk) {
 }
 
 template <int ND, int PK>
-__global__ void __launch_bounds__(m2l32_threads(ND, PK)) k_fmm_m2l32(FmmDevT<float2> f, const float2* __restrict__ ptab,
-                                                                    const int* stop) {
-  if (stop && *stop) return;
+__device__ __forceinline__ void m2l32_box(const FmmDevT<float2>& f, long long gb, const float2* __restrict__ ptab) {
   constexpr int RP = m2l32_rp(PK), SP = m2l32_splits(ND, PK), B = m2l32_threads(ND, PK);
   constexpr int HALF = ND * 4 * RP, NJ = 2;  // (channel, residue, pair) threads; orbits added at a time
   constexpr int DS = 4 * PK + 4, US = ND * DS;  // channel and orbit strides: distinct banks
   extern __shared__ __align__(16) float2 U[];   // [orbit][channel][k][4]
   __shared__ int s_at[kOrbits * 4];             // the sources' first coefficients, or -1
   __shared__ float4 red[B];
-  long long gb = blockIdx.x + lev_off(2);
   int l = 2;
   while (l < f.L && gb >= lev_off(l + 1)) ++l;
   const int targets = f.tcount[gb];
@@ -958,6 +1012,14 @@ __global__ void __launch_bounds__(m2l32_threads(ND, PK)) k_fmm_m2l32(FmmDevT<flo
     f.lc[(gb * ND + d) * p + t0] = make_float2(acc0.x * sc, acc0.y * sc);
     if (t1 < p) f.lc[(gb * ND + d) * p + t1] = make_float2(acc1.x * sc, acc1.y * sc);
   }
+}
+
+template <int ND, int PK, bool MANY>
+__global__ void __launch_bounds__(m2l32_threads(ND, PK)) k_fmm_m2l32(FmmDevT<float2> f, const float2* __restrict__ ptab,
+                                                                    const int* stop) {
+  if (stop && *stop) return;
+  for_boxes<MANY>(f.tcount + lev_off(2), lev_off(f.L + 1) - lev_off(2), f.tper,
+                  [&](long long b) { m2l32_box<ND, PK>(f, b + lev_off(2), ptab); });
 }
 
 // ---- float-float M2L: the residual operator of the float-float refinement ----
@@ -1132,15 +1194,12 @@ __device__ __forceinline__ cff cff_add(cff a, cff b) {
 
 // Threads: split x (channel, row); orbits as in k_fmm_m2l.
 template <int NJ>
-__global__ void __launch_bounds__(256) k_fmm_m2l_ff(FmmDev f, const float4* __restrict__ mpff,
-                                                    const float* __restrict__ tab, int nsplit, int nbo,
-                                                    const int* stop) {
-  if (stop && *stop) return;
+__device__ __forceinline__ void m2l_ff_box(const FmmDev& f, long long gb, const float4* __restrict__ mpff,
+                                           const float* __restrict__ tab, int nsplit, int nbo) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ OrbitList o;
   __shared__ float4 s_a0[kOrbits][kMaxNd][4];  // the transforms of a_0 of the logarithm channels
   __shared__ float4 red[256];
-  long long gb = blockIdx.x + lev_off(2);
   int l = 2;
   while (l < f.L && gb >= lev_off(l + 1)) ++l;
   if (f.tcount[gb] == 0) return;
@@ -1254,6 +1313,15 @@ __global__ void __launch_bounds__(256) k_fmm_m2l_ff(FmmDev f, const float4* __re
     const double2 v = cff_to(acc);
     f.lc[gb * per + e] = make_double2(v.x * sc, v.y * sc);
   }
+}
+
+template <int NJ, bool MANY>
+__global__ void __launch_bounds__(256) k_fmm_m2l_ff(FmmDev f, const float4* __restrict__ mpff,
+                                                    const float* __restrict__ tab, int nsplit, int nbo,
+                                                    const int* stop) {
+  if (stop && *stop) return;
+  for_boxes<MANY>(f.tcount + lev_off(2), lev_off(f.L + 1) - lev_off(2), f.tper,
+                  [&](long long b) { m2l_ff_box<NJ>(f, b + lev_off(2), mpff, tab, nsplit, nbo); });
 }
 
 // L2L from level l0 down to the children of level lp (added to their M2L part), a
@@ -1409,8 +1477,7 @@ __device__ __forceinline__ void horner(const T2* __restrict__ a, int p, T2 u, bo
 }
 
 template <class T2, int NEARP>
-__global__ void __launch_bounds__(kBE) k_fmm_eval(FmmDevT<T2> f, Geo g, double* __restrict__ partial, const int* stop) {
-  if (stop && *stop) return;
+__device__ __forceinline__ void eval_leaf(const FmmDevT<T2>& f, const Geo& g, int b, double* __restrict__ partial) {
   using Sum = typename EvalNear<NEARP>::Sum;
   constexpr int TPT = EvalNear<NEARP>::kTPT, NT = kBE * TPT;  // targets at hand
   // expansions [nd][p] (float-float: split hi + lo in 16 bytes), then F and F' of
@@ -1426,7 +1493,7 @@ __global__ void __launch_bounds__(kBE) k_fmm_eval(FmmDevT<T2> f, Geo g, double* 
   __shared__ int lst[10], lbeg[9];
   __shared__ float cen[6];  // FP32 instance: split leaf centre, 1/s, s
   const int t = threadIdx.x;
-  const int b = blockIdx.x, bx = b % f.nb, by = b / f.nb;
+  const int bx = b % f.nb, by = b / f.nb;
   const int s0 = f.start[b], n = f.start[b + 1] - s0;
   if (n == 0) return;
   const int nd = f.nd, p = f.p;
@@ -1762,6 +1829,13 @@ __global__ void __launch_bounds__(kBE) k_fmm_eval(FmmDevT<T2> f, Geo g, double* 
   }
 }
 
+template <class T2, int NEARP, bool MANY>
+__global__ void __launch_bounds__(kBE) k_fmm_eval(FmmDevT<T2> f, Geo g, double* __restrict__ partial, const int* stop) {
+  if (stop && *stop) return;
+  for_boxes<MANY>(f.count + lev_off(f.L), (long long)f.nb * f.nb, f.per,
+                  [&](long long b) { eval_leaf<T2, NEARP>(f, g, (int)b, partial); });
+}
+
 // Dynamic shared memory of an evaluation block.
 template <class T2, int NEARP>
 size_t eval_smem(int nd, int p) {
@@ -1949,6 +2023,7 @@ struct FmmState {
   int L = 0, nb = 0, nleaf = 0, kind = 0, M = 0, N = 0;
   double x0 = 0, y0 = 0, D = 0;
   long long nbox = 0;
+  int per = 1, tper = 1;  // boxes that a block goes over: of the leaves (and of the level above), of all levels
   // device buffers (stream-ordered), grown on demand
   char* buf = nullptr;
   size_t buf_size = 0;
@@ -2013,10 +2088,11 @@ int fmm_setup(FmmState*& f, const Geo& g, int kind, const int* orders, int norde
   // leaf_nodes nodes (default 24); nodes on curves of total length P occupy
   // about min(4^L, 1.3 P 2^L / D) leaves
   int L = 2;
-  for (int l = 2; l <= 10; ++l) {
-    const double boxes = fmin((double)(1LL << (2 * l)), 1.3 * h[3] * (double)(1 << l) / f->D);
-    if ((double)g.M / fmax(boxes, 1.0) >= (double)leaf_nodes) L = l;
-  }
+  const auto used = [&](int l) { return fmin((double)(1LL << (2 * l)), 1.3 * h[3] * (double)(1 << l) / f->D); };
+  for (int l = 2; l <= 10; ++l)
+    if ((double)g.M / fmax(used(l), 1.0) >= (double)leaf_nodes) L = l;
+  f->per = boxes_a_block(used(L), (double)(1LL << (2 * L)));
+  f->tper = boxes_a_block_levels(L, used);
   f->L = L;
   f->nb = 1 << L;
   f->nleaf = f->nb * f->nb;
@@ -2168,8 +2244,10 @@ M2lShape m2l_shape(int nd, int p, size_t entry, size_t pascal) {
 template <int ND, int PK>
 void m2l32_launch(const FmmDevT<float2>& d, const float2* ptab, int L, const int* stop, cudaStream_t s) {
   const size_t sm = (size_t)kOrbits * ND * (4 * PK + 4) * sizeof(float2);
-  if (sm > 40 * 1024) cudaFuncSetAttribute(k_fmm_m2l32<ND, PK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_fmm_m2l32<ND, PK><<<(int)(lev_off(L + 1) - lev_off(2)), m2l32_threads(ND, PK), sm, s>>>(d, ptab, stop);
+  const unsigned grid = blocks_for(lev_off(L + 1) - lev_off(2), d.tper);
+  const auto fn = d.tper > 1 ? k_fmm_m2l32<ND, PK, true> : k_fmm_m2l32<ND, PK, false>;
+  if (sm > 40 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  fn<<<grid, m2l32_threads(ND, PK), sm, s>>>(d, ptab, stop);
 }
 
 template <int ND>
@@ -2186,27 +2264,21 @@ void launch_m2l32(const FmmDevT<float2>& d, const float2* ptab, int pk, int L, c
 }
 
 void launch_m2l(const FmmDev& d, int L, const int* stop, cudaStream_t s) {
-  const int grid = (int)(lev_off(L + 1) - lev_off(2));
+  const unsigned grid = blocks_for(lev_off(L + 1) - lev_off(2), d.tper);
   const M2lShape m = m2l_shape(d.nd, d.p, sizeof(double2), (size_t)(d.nlog > 0 ? 2 : 1) * d.p * d.p * sizeof(double));
-  if (m.nsplit == 5) {
-    cudaFuncSetAttribute(k_fmm_m2l<double2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
-    k_fmm_m2l<double2, 2><<<grid, m.threads, m.smem, s>>>(d, m.nsplit, m.nbo, stop);
-  } else {
-    cudaFuncSetAttribute(k_fmm_m2l<double2, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
-    k_fmm_m2l<double2, 5><<<grid, m.threads, m.smem, s>>>(d, m.nsplit, m.nbo, stop);
-  }
+  const auto fn = m.nsplit == 5 ? (d.tper > 1 ? k_fmm_m2l<double2, 2, true> : k_fmm_m2l<double2, 2, false>)
+                                : (d.tper > 1 ? k_fmm_m2l<double2, 5, true> : k_fmm_m2l<double2, 5, false>);
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
+  fn<<<grid, m.threads, m.smem, s>>>(d, m.nsplit, m.nbo, stop);
 }
 
 void launch_m2l_ff(const FmmDev& d, const float4* mpff, const float* tab, int L, const int* stop, cudaStream_t s) {
   const M2lShape m = m2l_shape(d.nd, d.p, sizeof(float4), 0);
-  const int grid = (int)(lev_off(L + 1) - lev_off(2));
-  if (m.nsplit == 5) {
-    cudaFuncSetAttribute(k_fmm_m2l_ff<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
-    k_fmm_m2l_ff<2><<<grid, m.threads, m.smem, s>>>(d, mpff, tab, m.nsplit, m.nbo, stop);
-  } else {
-    cudaFuncSetAttribute(k_fmm_m2l_ff<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
-    k_fmm_m2l_ff<5><<<grid, m.threads, m.smem, s>>>(d, mpff, tab, m.nsplit, m.nbo, stop);
-  }
+  const unsigned grid = blocks_for(lev_off(L + 1) - lev_off(2), d.tper);
+  const auto fn = m.nsplit == 5 ? (d.tper > 1 ? k_fmm_m2l_ff<2, true> : k_fmm_m2l_ff<2, false>)
+                                : (d.tper > 1 ? k_fmm_m2l_ff<5, true> : k_fmm_m2l_ff<5, false>);
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxM2lSmem);
+  fn<<<grid, m.threads, m.smem, s>>>(d, mpff, tab, m.nsplit, m.nbo, stop);
 }
 
 // The instance of the shift kernels for nd channels of order p.
@@ -2253,7 +2325,8 @@ int fmm_m2m(const FmmDevT<T2>& d, int* arrive, const int* stop, cudaStream_t s) 
   for_shift(d.nd, d.p, [&](auto nc, auto pk) {
     constexpr int NC = decltype(nc)::value, PK = decltype(pk)::value;
     const size_t sm = shift_smem<T2>(d.nd, PK);
-    k_fmm_m2m<T2, NC, PK><<<1 << (2 * (d.L - 1)), shift_threads(d.nd, d.p), sm, s>>>(d, arrive, stop);
+    const auto fn = d.per > 1 ? k_fmm_m2m<T2, NC, PK, true> : k_fmm_m2m<T2, NC, PK, false>;
+    fn<<<blocks_for(1LL << (2 * (d.L - 1)), d.per), shift_threads(d.nd, d.p), sm, s>>>(d, arrive, stop);
   });
   return 1;
 }
@@ -2295,7 +2368,8 @@ void fmm_passes(const FmmDevT<T2>& d, FmmState* f, const Geo& g, [[maybe_unused]
   }
   shifts += fmm_l2l(d, stop, s);
   note_launches(shifts);
-  k_fmm_eval<T2, NEARP><<<f->nleaf, kBE, eval_smem<T2, NEARP>(nd, p), s>>>(d, g, partial, stop);
+  const auto eval = d.per > 1 ? k_fmm_eval<T2, NEARP, true> : k_fmm_eval<T2, NEARP, false>;
+  eval<<<blocks_for(f->nleaf, d.per), kBE, eval_smem<T2, NEARP>(nd, p), s>>>(d, g, partial, stop);
 }
 
 }  // namespace
@@ -2307,7 +2381,9 @@ void fmm_signature(const FmmState* f, std::vector<long long>& key) {
     memcpy(&u, &v, 8);
     key.push_back(u);
   }
-  for (long long v : {(long long)f->L, f->nbox, (long long)f->M, (long long)f->kind}) key.push_back(v);
+  for (long long v : {(long long)f->L, (long long)f->per, (long long)f->tper, f->nbox, (long long)f->M,
+                      (long long)f->kind})
+    key.push_back(v);
   for (const void* q : {(const void*)f->leaf, (const void*)f->perm, (const void*)f->start, (const void*)f->count,
                         (const void*)f->arrive, (const void*)f->Q, (const void*)f->mp, (const void*)f->lc,
                         (const void*)f->mpff, (const void*)f->cen32})
@@ -2339,12 +2415,16 @@ cudaError_t fmm_pair_sum(FmmState* f, const Geo& g, int kind, int p, VecRef v, c
     d.cen32 = f->cen32;
     d.is32 = (float)ldexp(1.0 / f->D, f->L);
     d.s32 = (float)ldexp(f->D, -f->L);
+    d.per = f->per;
+    d.tper = f->tper;
     fmm_passes<float2, 1>(d, f, g, v, sscale, partial, stop, s);
   } else {
     k_fmm_density<<<grid_for(g.M), 256, 0, s>>>(g, nd, f->x0 + 0.5 * f->D, f->y0 + 0.5 * f->D, v, sscale, f->Q,
                                                  stop);
-    const FmmDev d{f->L,    f->nb,    p,     nd,    g.M,   0,   kind == 1 ? 2 : -1, f->x0, f->y0, f->D, 1.0 / f->D, f->leaf,
+    FmmDev d{f->L,    f->nb,    p,     nd,    g.M,   0,   kind == 1 ? 2 : -1, f->x0, f->y0, f->D, 1.0 / f->D, f->leaf,
                    f->perm, f->start, f->count, f->count, f->Q, f->mp, f->lc,  ops};
+    d.per = f->per;
+    d.tper = f->tper;
     if (near_prec == 2)
       fmm_passes<double2, 2>(d, f, g, v, sscale, partial, stop, s);
     else
@@ -2378,6 +2458,8 @@ cudaError_t fmm_output(FmmState* f, const Geo& g, int kind, int p, const double*
   k_fmm_out_density<<<grid_for(g.M), 256, 0, s>>>(g, nd, c0x, c0y, v, f->Q);
   FmmDev d{f->L, f->nb, p, nd, g.M, nlog, -1, f->x0, f->y0, f->D, 1.0 / f->D, f->leaf, f->perm, f->start, f->count, f->tcount,
            f->Q, f->mp, f->lc, ops};
+  d.per = f->per;
+  d.tper = boxes_a_block_levels(f->L, [&](int) { return (double)T; });
   const size_t sm_p2m = ((size_t)p * (kChunk + 1) + (size_t)kChunk * nd) * sizeof(double2);
   if (ff)
     k_fmm_p2m_ff<<<f->nleaf, kB, sm_p2m, s>>>(d, g, nullptr);  // float4 = double2 in size
