@@ -497,18 +497,18 @@ __global__ void __launch_bounds__(kBA) k_bj_apply64(Geo g, int kind, const long 
   const int a0 = g.body_start[i] * c, nb = (g.body_start[i + 1] - g.body_start[i]) * c;
   const int r0 = blockIdx.y * kRows64;
   if (r0 >= nb) return;
-  const int lr = threadIdx.x % kRows64, grp = threadIdx.x / kRows64;
-  const int r = r0 + lr;
   const double inv = NORM ? 1.0 / st->hnext : 1.0;
   double* vout = NORM ? V + (long long)st->j * ld + a0 : nullptr;
-  if (nb > kMaxBlock) {
-    if (grp == 0 && r < nb) {
-      const double t = v[a0 + r] * inv;
-      if (NORM) vout[r] = t;
-      z[a0 + r] = t;
+  if (nb > kMaxBlock) {  // the identity
+    for (long long e = blockIdx.y * kBA + threadIdx.x; e < nb; e += gridDim.y * kBA) {
+      const double t = v[a0 + e] * inv;
+      if (NORM) vout[e] = t;
+      z[a0 + e] = t;
     }
     return;
   }
+  const int lr = threadIdx.x % kRows64, grp = threadIdx.x / kRows64;
+  const int r = r0 + lr;
   const double up = __hiloint2double((1023 + 500) << 20, 0), down = __hiloint2double((1023 - 500) << 20, 0);  // 2^500
   for (int e = threadIdx.x; e < nb; e += kBA) vd[e] = v[a0 + e] * inv * up;
   __syncthreads();
@@ -649,13 +649,24 @@ cudaError_t bj_setup(const Geo& g, int kind, double alpha, const int* body_start
   return cudaStreamSynchronize(s);
 }
 
+namespace {
+// CTAs of k_bj_apply64: a body's rows of 32, and where a body is larger than the blocks,
+// which its CTAs copy in strides, so many that the bodies fill the SMs twice.
+// (By the largest body's rows, one of 20,000 unknowns among 3,000 of 16 made 1.9 million, all but
+// 7,000 of them empty, and one of 2.1 million no valid grid.)
+dim3 apply64_grid(const Geo& g, int max_nb) {
+  const int rows = (std::min(max_nb, kMaxBlock) + kRows64 - 1) / kRows64;
+  if (max_nb <= kMaxBlock) return dim3(g.N, rows);
+  return dim3(g.N, std::max(rows, std::min((max_nb + kBA - 1) / kBA, 2 * device_sms() / g.N)));
+}
+}  // namespace
+
 cudaError_t bj_apply(const Geo& g, int kind, const long long* off_dev, const bj_t* blocks, VecRef v, double* z,
                      const int* stop, int max_nb, cudaStream_t s, bool f64) {
   const size_t nv = (size_t)std::min(max_nb, kMaxBlock);
   if (f64) {  // (callers pass a plain vector)
-    const dim3 grid(g.N, (max_nb + kRows64 - 1) / kRows64);
-    k_bj_apply64<false><<<grid, kBA, nv * sizeof(double), s>>>(g, kind, off_dev, blocks, v.base, z, nullptr, 0, nullptr,
-                                                               stop);
+    k_bj_apply64<false><<<apply64_grid(g, max_nb), kBA, nv * sizeof(double), s>>>(g, kind, off_dev, blocks, v.base, z,
+                                                                                  nullptr, 0, nullptr, stop);
   } else {
     const dim3 grid(g.N, (max_nb + kApplyRows - 1) / kApplyRows);
     k_bj_apply<<<grid, kBA, nv * sizeof(float), s>>>(g, kind, off_dev, blocks, v, z, stop);
@@ -667,8 +678,8 @@ cudaError_t bj_apply(const Geo& g, int kind, const long long* off_dev, const bj_
 cudaError_t bj_normalize_apply64(const Geo& g, int kind, const long long* off_dev, const bj_t* blocks, const double* w,
                                  double* z, double* V, long long ld, const KState* st, int max_nb, cudaStream_t s) {
   const size_t nv = (size_t)std::min(max_nb, kMaxBlock);
-  const dim3 grid(g.N, (max_nb + kRows64 - 1) / kRows64);
-  k_bj_apply64<true><<<grid, kBA, nv * sizeof(double), s>>>(g, kind, off_dev, blocks, w, z, V, ld, st, &st->stop);
+  k_bj_apply64<true><<<apply64_grid(g, max_nb), kBA, nv * sizeof(double), s>>>(g, kind, off_dev, blocks, w, z, V, ld,
+                                                                               st, &st->stop);
   note_launches(1);
   return cudaGetLastError();
 }
