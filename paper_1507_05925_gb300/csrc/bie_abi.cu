@@ -65,6 +65,8 @@ struct bie_ctx {
   size_t cap = 0;
   char* ws = nullptr;
   size_t ws_size = 0;
+  char* tab = nullptr;  // batches: tables of the copies between the caller's arrays and ours (batch_tables)
+  size_t tab_size = 0;
   KState* h_state = nullptr;  // pinned mirror of the device solver state
   double* h_small = nullptr;  // pinned scratch for small read-backs
   std::string err;
@@ -477,6 +479,30 @@ int make_operator_workspace(bie_ctx* ctx, Work& w, cudaStream_t s, const bie_geo
       });
 }
 
+// Device memory for a batch's copy tables, kept by the context (twice the largest batch's, a
+// few hundred bytes a problem).  Allocating it on each call mapped fresh memory, which the
+// next synchronisation unmapped, whenever the workspace left no room in the driver's pool: a
+// batch of 73 two-disc problems 887 or 1,227 us by the size of the workspace, 872 so.
+int batch_tables(bie_ctx* ctx, size_t need, cudaStream_t s) {
+  if (need <= ctx->tab_size) return BIE_OK;
+  if (ctx->tab) cudaFreeAsync(ctx->tab, s);
+  ctx->tab = nullptr;
+  ctx->tab_size = 0;
+  need = std::max<size_t>(2 * need, 4096);
+  const cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&ctx->tab), need, s);
+  if (e != cudaSuccess) ctx->tab = nullptr;
+  CK(e);
+  ctx->tab_size = need;
+  return BIE_OK;
+}
+
+// The copies of a batch by one kernel.
+int copy_segments(bie_ctx* ctx, const std::vector<CopySeg>& segs, cudaStream_t s) {
+  if (int rc = batch_tables(ctx, segs.size() * sizeof(CopySeg), s)) return rc;
+  CK(gather_segments(segs, reinterpret_cast<CopySeg*>(ctx->tab), s));
+  return BIE_OK;
+}
+
 // Copies a host array into staging (or passes a device pointer through).
 template <class T>
 int stage_in(bie_ctx* ctx, const T* src, T* staging, size_t count, const T** out, cudaStream_t s) {
@@ -587,7 +613,7 @@ int batch_setup(bie_ctx* ctx, const BatchIn& b, const std::vector<int>& bs, cons
   if (from_host[7])
     CK(cudaMemcpyAsync(w.load, pack.data() + load_off, (size_t)per * N * sizeof(double), cudaMemcpyHostToDevice,
                        s));
-  CK(gather_segments(segs, s));
+  if (int rc = copy_segments(ctx, segs, s)) return rc;
   std::vector<int2> pr(N);
   std::vector<long long> pn(P + 1);
   for (int p = 0; p < P; ++p) {
@@ -689,15 +715,13 @@ int validate_batch(bie_ctx* ctx, const BatchIn& b, std::vector<int>& bs, std::ve
   }
   if (!segs.empty()) {
     DeviceGuard dg(ctx->device);
-    int* d = nullptr;
-    CK(cudaMallocAsync(reinterpret_cast<void**>(&d), roff[P] * sizeof(int), s));
+    const size_t table = segs.size() * sizeof(CopySeg);  // (a multiple of eight bytes)
+    if (int rc = batch_tables(ctx, table + roff[P] * sizeof(int), s)) return rc;
+    int* d = reinterpret_cast<int*>(ctx->tab + table);
     for (size_t i = 0; i < segs.size(); ++i) segs[i].dst = d + roff[on_device[i]];
     std::vector<int> tmp(roff[P]);
-    cudaError_t e = gather_segments(segs, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(tmp.data(), d, roff[P] * sizeof(int), cudaMemcpyDeviceToHost, s);
-    const cudaError_t f = cudaFreeAsync(d, s);  // on every path
-    CK(e);
-    CK(f);
+    CK(gather_segments(segs, reinterpret_cast<CopySeg*>(ctx->tab), s));
+    CK(cudaMemcpyAsync(tmp.data(), d, roff[P] * sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     for (int p : on_device) std::copy(tmp.begin() + roff[p], tmp.begin() + roff[p + 1], raw.begin() + roff[p]);
   }
@@ -1444,7 +1468,7 @@ int solve_common(bie_ctx* ctx, const bie_geometry* geom, int kind, const double*
       else
         on_host.push_back(p);
     }
-    CK(gather_segments(segs, s));
+    if (int rc = copy_segments(ctx, segs, s)) return rc;
     if (!on_host.empty()) {
       std::vector<double> h(nload);
       CK(cudaMemcpyAsync(h.data(), w.outv, nload * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1557,6 +1581,11 @@ int bie_create(bie_ctx** out, int device, size_t cap) {
 
 namespace bie {
 void release_workspace(bie_ctx* ctx, cudaStream_t s) {
+  if (ctx && ctx->tab) {
+    cudaFreeAsync(ctx->tab, s);
+    ctx->tab = nullptr;
+    ctx->tab_size = 0;
+  }
   if (ctx && ctx->ws) {
     cudaFreeAsync(ctx->ws, s);
     ctx->ws = nullptr;
@@ -1666,9 +1695,10 @@ void bie_destroy(bie_ctx* c) {
   for (cudaEvent_t e : c->pool) cudaEventDestroy(e);
   for (auto& gi : c->graphs) cudaGraphExecDestroy(gi.exec);
   if (c->fmm) bie::fmm_free(c->fmm, nullptr);
-  if (c->ws) {
+  if (c->ws || c->tab) {
     cudaDeviceSynchronize();
-    cudaFree(c->ws);
+    if (c->ws) cudaFree(c->ws);
+    if (c->tab) cudaFree(c->tab);
   }
   if (c->h_state) cudaFreeHost(c->h_state);
   if (c->h_small) cudaFreeHost(c->h_small);

@@ -540,21 +540,15 @@ cudaError_t batch_unscale(int nprob, const long long* pnode, const double* scale
   return cudaGetLastError();
 }
 
-cudaError_t gather_segments(const std::vector<CopySeg>& segs, cudaStream_t s) {
+cudaError_t gather_segments(const std::vector<CopySeg>& segs, CopySeg* table, cudaStream_t s) {
   if (segs.empty()) return cudaSuccess;
-  CopySeg* d = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&d), segs.size() * sizeof(CopySeg), s);
-  if (e != cudaSuccess) return e;
   // a pageable source: the call returns once the table is staged
-  e = cudaMemcpyAsync(d, segs.data(), segs.size() * sizeof(CopySeg), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) {
-    const int n = (int)segs.size();
-    k_gather<<<n < 1024 ? n : 1024, kB, 0, s>>>(d, n);
-    note_launches(1);
-    e = cudaGetLastError();
-  }
-  const cudaError_t f = cudaFreeAsync(d, s);
-  return e != cudaSuccess ? e : f;
+  const cudaError_t e = cudaMemcpyAsync(table, segs.data(), segs.size() * sizeof(CopySeg), cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return e;
+  const int n = (int)segs.size();
+  k_gather<<<n < 1024 ? n : 1024, kB, 0, s>>>(table, n);
+  note_launches(1);
+  return cudaGetLastError();
 }
 
 cudaError_t seg_norms(int nprob, const long long* pnode, const double* x, double* norms, cudaStream_t s) {

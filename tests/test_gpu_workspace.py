@@ -55,6 +55,31 @@ def test_only_the_sums_of_the_call_reserve_slots(kind):
     assert whole >= direct
 
 
+def test_batches_of_changing_size_and_stream():
+    """The copy tables that a context keeps between batches: larger and smaller batches, on
+    two streams, from device and host arrays, each bitwise as in a context of its own."""
+    from test_gpu_parity import to_dev
+    ctx = bie.Context(0)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for k, P in enumerate((3, 200, 5, 700, 1, 40)):
+        geoms = [synth.four_discs(seed=300 + 10 * k + p % 7, n=24 + 8 * (p % 3)) for p in range(P)]
+        loads = [synth.charges(4, np.random.default_rng(p)) for p in range(P)]
+        res = []
+        for c, stream in ((ctx, streams[k % 2]), (bie.Context(0), None)):
+            gs = [to_dev(g) if p % 3 else g for p, g in enumerate(geoms)]
+            ls = [torch.from_numpy(q).cuda() if p % 2 else q for p, q in enumerate(loads)]
+            outs = [torch.empty(4, dtype=torch.float64, device="cuda") if p % 2 else np.empty(4) for p in range(P)]
+            torch.cuda.synchronize()
+            rc, _, _ = bie.elastance_solve_batch(c, gs, ls, outs, opts=bie.make_opts(precision=bie.MIXED_FF), stream=stream)
+            torch.cuda.synchronize()
+            assert rc == bie.OK, c.last_error()
+            res.append([o.cpu().numpy() if p % 2 else o for p, o in enumerate(outs)])
+            if c is not ctx:
+                c.close()
+        assert all(np.array_equal(a, b) for a, b in zip(*res)), P
+    ctx.close()
+
+
 def test_full_device_takes_the_smaller_plans():
     """With little device memory left, a call whose symmetric plan's slots do not fit runs
     with the directed one's, as it does under a workspace cap."""
