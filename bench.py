@@ -45,7 +45,7 @@ FLOPS_PER_PAIR = {"laplace": 10.0, "stokes": 18.0}
 # capture of the current kernels (profiles/k_pair32s_laplace_stars100_M25600.md:
 # the symmetric FP32 kernel); a kernel changed since its capture must be taken
 # out of this table
-DRAM_BYTES_PER_LAUNCH = {"laplace_fp32": 1.002e6}
+DRAM_BYTES_PER_LAUNCH = {"laplace_fp32": 1.130e6}
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -64,7 +64,7 @@ def parse():
                     help="solves of the four-disc case (M = 512) per precision, host clock (0 = skip)")
     ap.add_argument("--splits", type=int, default=0,
                     help="--kernel: install this pair-sum split count instead of searching (0 = search, "
-                         "negative = the symmetric FP32 Laplace plan)")
+                         "negative = the symmetric plan of that many tiles)")
     ap.add_argument("--no-tune", action="store_true",
                     help="keep the occupancy rule's pair-sum split counts (no bie_tune before the warm-up)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
@@ -917,7 +917,7 @@ def main():
     # the pair kernel's own ALU bound, from its far-pair loop: the directed kernel
     # needs 7 FP32 lane operations and one MUFU reciprocal a pair, the
     # symmetric one (tile pairs, one reciprocal for both directions) 5.5 and 0.5
-    sym = bool(tuning and tuning["laplace_fp32"]["splits"] < 0) if tuning else M >= 8960
+    sym = bool(tuning and tuning["laplace_fp32"]["splits"] < 0) if tuning else M > 5376
     ops_pair, mufu_pair = (5.5, 0.5) if sym else (7.0, 1.0)
     lane_ops = fp32_peak * 1e12 / 2.0
     pipe_bound_pairs = min(lane_ops / ops_pair, peaks["mufu_rcp_tops"] * 1e12 / mufu_pair)

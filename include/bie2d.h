@@ -345,15 +345,17 @@ int apply_operator_fmm_prec(bie_ctx* ctx, const bie_geometry* geom, int kind, in
 
 /* Device workspace (bytes) that elastance_solve (kind 0) or mobility_solve
  * (kind 1) needs for N bodies, M nodes and GMRES restart length `restart`
- * (0 = default): the Krylov basis, the staged geometry, the partial sums and
- * the staging of host inputs.  Requires a current CUDA device. */
+ * (0 = default) with whichever options need most: the Krylov basis, the staged
+ * geometry, the partial sums and the staging of host inputs.  A smaller cap may
+ * still do: a call reserves partial sums for its own options only, and takes
+ * plans with few of them where others do not fit.  Requires a current CUDA device. */
 size_t bie_workspace_bytes(int kind, int n_bodies, int n_nodes, int restart);
 
 /* ---- Serving: continuous batching of solve requests ----
  * A server owns `workers` host threads, each with its own context and its own
  * non-blocking CUDA stream, so that the solves of concurrent requests overlap
  * on the device.  Requests wait in a queue and are admitted when a worker is
- * free and their workspace (bie_workspace_bytes) fits under hbm_cap_bytes
+ * free and their workspace (at most bie_workspace_bytes) fits under hbm_cap_bytes
  * together with the requests in flight (0 = no cap); a request may pass an
  * earlier one that does not fit yet, but not more than 64 times.  Results do
  * not depend on what else is in flight: every kernel reduces in a fixed order

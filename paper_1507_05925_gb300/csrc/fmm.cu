@@ -2281,7 +2281,13 @@ void launch_m2l_ff(const FmmDev& d, const float4* mpff, const float* tab, int L,
   fn<<<grid, m.threads, m.smem, s>>>(d, mpff, tab, m.nsplit, m.nbo, stop);
 }
 
-// The instance of the shift kernels for nd channels of order p.
+// The instance of the shift kernels for nd channels of order p, whose coefficients are
+// padded with zeros to its width: the default inner orders (15 and 18) and residual order (36)
+// have one of their own, larger ones the widest.  A whole application at order 37 takes 3%
+// (FP64) and 8% (float-float) longer than at 36 (25,600 Stokes nodes: 1,006 and 1,041 us, 482
+// and 518), so that a further instance of the four kernels would be little used for little;
+// orders 37 to 64 at 160,000 nodes run 1.3 to 3.3 times as fast as with run-time sizes (FP64
+// Stokes 14.6 -> 4.5 ms at 37, 20.4 -> 6.8 at 64; FP32 881 -> 683 us and 1,323 -> 775).
 template <int NC, class F>
 void for_shift_order(int p, F&& launch) {
   using std::integral_constant;

@@ -40,7 +40,7 @@ __device__ __forceinline__ double combine(const double* __restrict__ V, long lon
 
 // ------------------------------------------------------------ fused Arnoldi
 // One Arnoldi step after w = A z_j (w = V_{j+1}) in a single cooperative
-// launch with two grid barriers (a third where the norm cancels): CGS2 (h1 = V^T w;
+// launch with two grid barriers (a third where kNormBySubtraction asks): CGS2 (h1 = V^T w;
 // w -= V h1; h2 = V^T w; w -= V h2), ||w||, the Hessenberg column with its Givens rotations and the
 // residual estimate, and v_{j+1} = w / ||w||.  After each barrier every CTA adds
 // the per-CTA partials itself, in CTA order (deterministic; no atomics), so
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(kBV, NARROW ? 1 : 4) k_arnoldi(ArnoldiArgs a) 
   if (grid_barrier(st, bar, a.spins)) return;
   arn_grid_sum(part2, jc + 1, hs2);
   // ||w - V h2||^2 = ||w||^2 - ||h2||^2, V being orthonormal: no third barrier for
-  // the norm while nothing cancels (h2 is the rounding of the first pass)
+  // the norm while nothing is lost (kNormBySubtraction; h2 is the rounding of the first pass)
   __shared__ double h22_s;
   if (threadIdx.x < 32) {
     double t = 0.0;
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(kBV, PREFETCH ? 1 : 4) k_arnoldi32(ArnoldiArgs
   if (grid_barrier(st, bar, a.spins)) return;
   arn_grid_sum32(part2, jc + 1, hs2);
   // ||w - VF h2||^2 = ||w||^2 - ||h2||^2, VF being orthonormal: no third barrier for
-  // the norm while nothing cancels (h2 is the rounding of the first pass).  The
+  // the norm while nothing is lost (kNormBySubtraction; h2 is the rounding of the first pass).  The
   // subtraction and the preconditioner then run body by body, which is one pass
   // less where every CTA has one body at most.  With more bodies a CTA the chunks
   // are the faster order and the barrier stays (the bodies' elements are other

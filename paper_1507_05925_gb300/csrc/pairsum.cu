@@ -862,7 +862,7 @@ void launch_pair32s(const Geo& g, const PairPlan& p, double* partial, const int*
 // directed pairs (the directed kernel: 10 for one, about 16 when it divided),
 // Stokes 24 (16, about 21).  Measured (GB300, whole launch): Laplace M = 25,600
 // 16.6 ms divided, 12.1 ms directed with rcp64, 7.5 ms symmetric (8.7e10
-// pairs/s, 90% of the pipe); Stokes M = 12,672 6.7, 4.65, 3.44 ms.
+// pairs/s, 90% of the pipe); Stokes M = 12,630 6.7, 4.65, 3.43 ms.
 // A lane holds one target of tile A (two a lane measured the same); the sources
 // of tile B sit in shared memory, visited on the diagonal schedule of
 // k_pair32s, the source's accumulator travelling by shuffle.  Warp w starts

@@ -352,7 +352,7 @@ __device__ int cta_gmres(const SmallArgs& A, int a0, int a1, int i0, int i1, lon
         }
         __syncthreads();
       }
-      // ||w - V h2||^2 = ||w||^2 - ||h2||^2 while nothing cancels (k_arnoldi32), by warp 0
+      // ||w - V h2||^2 = ||w||^2 - ||h2||^2 while nothing is lost (kNormBySubtraction), by warp 0
       if (wid == 0) {
         double h22 = 0.0;
         for (int i = lane; i <= j; i += 32) h22 = fma(sh.h2[i], sh.h2[i], h22);
