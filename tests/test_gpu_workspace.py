@@ -102,15 +102,20 @@ def test_full_device_takes_the_smaller_plans():
     bie.tune_clear()
     slots = 8 * M * 400  # the symmetric plan has more
     torch.cuda.empty_cache()
-    held = torch.empty(torch.cuda.mem_get_info()[0] - (256 << 20), dtype=torch.uint8, device="cuda")
-    assert torch.cuda.mem_get_info()[0] < slots
-    out.fill_(float("nan"))
+    try:
+        held = torch.empty(torch.cuda.mem_get_info()[0] - (256 << 20), dtype=torch.uint8, device="cuda")
+    except torch.OutOfMemoryError:
+        pytest.skip("the device's free memory is not one piece")
     ctx = bie.Context(0)
-    rc = bie.apply_operator(ctx, g, bie.LAPLACE, bie.FP64, v, out)
-    torch.cuda.synchronize()
-    err = ctx.last_error()
-    ctx.close()
-    del held
-    torch.cuda.empty_cache()
+    try:
+        assert torch.cuda.mem_get_info()[0] < slots
+        out.fill_(float("nan"))
+        rc = bie.apply_operator(ctx, g, bie.LAPLACE, bie.FP64, v, out)
+        torch.cuda.synchronize()
+        err = ctx.last_error()
+    finally:
+        ctx.close()
+        del held
+        torch.cuda.empty_cache()
     assert rc == bie.OK, err
     assert rel_max(out.cpu().numpy(), ref) <= 2 * TOL64
